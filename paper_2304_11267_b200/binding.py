@@ -1,8 +1,9 @@
-"""ctypes binding of the C-ABI attention library (argument marshalling only).
+"""Binding of the C-ABI attention library (argument marshalling only).
 
-Function names mirror ``include/sd_attn.h``.  Tensors are passed as raw device addresses
-(``tensor.data_ptr()``); PyTorch only owns the memory and the streams.  There is no fallback:
-if ``libsd_attn.so`` is missing or fails to load, every call raises.
+The functions named as in ``include/*.h`` go through ctypes and take raw device addresses
+(``tensor.data_ptr()``); the calls on torch tensors (``Attention.forward``, ``geglu``, ``groupnorm``) are
+marshalled by the extension module ``_sd_torch`` (csrc/torch_binding.cpp).  PyTorch only owns the memory and the
+streams.  There is no fallback: if ``libsd_attn.so`` or the extension is missing or fails to load, every call raises.
 """
 from __future__ import annotations
 
@@ -33,6 +34,7 @@ EXPORTS = ["sd_attn_create", "sd_attn_create_ex", "sd_attn_static_query_status",
            "sd_winograd_conv3x3_forward", "sd_winograd_query_status"]
 
 _lib = None
+_torch_ext = None
 
 
 class Problem(ctypes.Structure):
@@ -128,6 +130,23 @@ def load() -> ctypes.CDLL:
     return lib
 
 
+def _ext():
+    """The extension module that marshals torch tensors (built in-tree by ``build.py``).  Raises if it is absent."""
+    global _torch_ext
+    if _torch_ext is None:
+        import importlib.machinery
+        import importlib.util
+        import torch  # noqa: F401  (its libraries must be in the process first)
+        load()
+        path = os.path.join(_PKG, "_sd_torch.so")
+        if not os.path.exists(path):
+            raise FileNotFoundError("%s not found: build it with `python -m paper_2304_11267_b200.build`" % path)
+        spec = importlib.util.spec_from_file_location(
+            "_sd_torch", path, loader=importlib.machinery.ExtensionFileLoader("_sd_torch", path))
+        _torch_ext = importlib.util.module_from_spec(spec)
+    return _torch_ext
+
+
 def status_string(status: int) -> str:
     return load().sd_attn_status_string(int(status)).decode()
 
@@ -200,20 +219,10 @@ def sd_geglu_forward(x, out, rows: int, C: int, dtype: int, stream=0) -> int:
 
 def geglu(x, out=None, stream=None):
     """Marshalling helper for torch tensors: x [..., 2C] (float16 or float32, contiguous, CUDA) -> [..., C]."""
-    import torch
-    if not x.is_cuda or not x.is_contiguous():
-        raise ValueError("x must be a contiguous CUDA tensor")
-    if x.dtype not in (torch.float16, torch.float32) or x.shape[-1] % 2:
-        raise ValueError("x must be float16 or float32 with an even last dimension")
-    C = x.shape[-1] // 2
-    if out is None:
-        out = torch.empty(x.shape[:-1] + (C,), dtype=x.dtype, device=x.device)
-    rows = x.numel() // (2 * C) if C else 0
-    s = stream if stream is not None else torch.cuda.current_stream().cuda_stream
-    rc = sd_geglu_forward(x.data_ptr(), out.data_ptr(), rows, C, F16 if x.dtype == torch.float16 else F32, s)
-    if rc != OK:
-        raise SdAttnError(rc, "sd_geglu_forward")
-    return out
+    r = (_torch_ext or _ext()).geglu(x, out, stream)
+    if r.__class__ is int:
+        raise SdAttnError(r, "sd_geglu_forward")
+    return r
 
 
 def sd_groupnorm_forward(x, gamma, beta, y, N: int, C: int, HW: int, G: int, eps: float, dtype: int, stream=0) -> int:
@@ -227,25 +236,10 @@ def sd_groupnorm_forward(x, gamma, beta, y, N: int, C: int, HW: int, G: int, eps
 
 def groupnorm(x, groups: int, eps: float = 1e-5, gamma=None, beta=None, out=None, stream=None):
     """Marshalling helper for torch tensors: x [N, C, ...] (float16 or float32, contiguous, CUDA)."""
-    import torch
-    if not x.is_cuda or not x.is_contiguous() or x.dim() < 2:
-        raise ValueError("x must be a contiguous CUDA tensor [N, C, ...]")
-    if x.dtype not in (torch.float16, torch.float32):
-        raise ValueError("x must be float16 or float32")
-    N, C = x.shape[0], x.shape[1]
-    HW = x.numel() // (N * C) if N * C else 1
-    for t in (gamma, beta):
-        if t is not None and (t.dtype != x.dtype or tuple(t.shape) != (C,) or not t.is_cuda or not t.is_contiguous()):
-            raise ValueError("gamma and beta must be contiguous CUDA tensors [C] of x's dtype")
-    if out is None:
-        out = torch.empty_like(x)
-    s = stream if stream is not None else torch.cuda.current_stream().cuda_stream
-    rc = sd_groupnorm_forward(x.data_ptr(), gamma.data_ptr() if gamma is not None else 0,
-                              beta.data_ptr() if beta is not None else 0, out.data_ptr(), N, C, HW, groups, eps,
-                              F16 if x.dtype == torch.float16 else F32, s)
-    if rc != OK:
-        raise SdAttnError(rc, "sd_groupnorm_forward")
-    return out
+    r = (_torch_ext or _ext()).groupnorm(x, groups, eps, gamma, beta, out, stream)
+    if r.__class__ is int:
+        raise SdAttnError(r, "sd_groupnorm_forward")
+    return r
 
 
 def sd_winograd_filter_elems(K: int, C: int) -> int:
@@ -404,43 +398,28 @@ class Attention:
             raise SdAttnError(rc, "sd_attn_set_mode")
 
     def forward(self, q, k, v, scale: Optional[float] = None, out=None, stream: Optional[int] = None):
+        r = (_torch_ext or _ext()).attention(self.handle, self.layout, q, k, v, scale, out, stream)
+        if r.__class__ is not int:
+            return r
+        if r == ERR_WORKSPACE:
+            self._lend_workspace(q, k)
+            r = _ext().attention(self.handle, self.layout, q, k, v, scale, out, stream)
+            if r.__class__ is not int:
+                return r
+        raise SdAttnError(r, "sd_attn_forward")
+
+    def _lend_workspace(self, q, k) -> None:
+        """Scratch for a two-pass call on q and k."""
         import torch
-        if not (q.is_cuda and k.is_cuda and v.is_cuda):
-            raise ValueError("q, k, v must be CUDA tensors")
-        if not (q.is_contiguous() and k.is_contiguous() and v.is_contiguous()):
-            raise ValueError("q, k, v must be contiguous [B,H,N,d] (or, token-major, [B,N,H,d]) tensors")
-        if q.dtype == torch.float16:
-            dtype = F16
-        elif q.dtype == torch.float32:
-            dtype = F32
-        elif q.dtype == torch.bfloat16:
-            dtype = BF16
-        else:
-            raise TypeError("float16, bfloat16 or float32 only")
         if self.layout == LAYOUT_BNHD:
-            B, Nq, H, d = q.shape
-            Nk = k.shape[1]
+            (B, Nq, H, d), Nk = q.shape, k.shape[1]
         else:
-            B, H, Nq, d = q.shape
-            Nk = k.shape[2]
-        if out is None:
-            out = torch.empty_like(q)
-        if scale is None:
-            scale = float(d) ** -0.5
-        if stream is None:
-            stream = torch.cuda.current_stream(q.device).cuda_stream
-        rc = sd_attn_forward(self.handle, q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(),
-                             B, H, Nq, Nk, d, scale, dtype, stream)
-        if rc == ERR_WORKSPACE:
-            need = sd_attn_workspace_bytes(MODE_TWOPASS, B, H, Nq, Nk, d, dtype)
-            self._workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-            rc = sd_attn_set_workspace(self.handle, self._workspace.data_ptr(), need)
-            if rc == OK:
-                rc = sd_attn_forward(self.handle, q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(),
-                                     B, H, Nq, Nk, d, scale, dtype, stream)
+            (B, H, Nq, d), Nk = q.shape, k.shape[2]
+        need = sd_attn_workspace_bytes(MODE_TWOPASS, B, H, Nq, Nk, d, F16)
+        self._workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
+        rc = sd_attn_set_workspace(self.handle, self._workspace.data_ptr(), need)
         if rc != OK:
-            raise SdAttnError(rc, "sd_attn_forward")
-        return out
+            raise SdAttnError(rc, "sd_attn_set_workspace")
 
     def check(self, stream: int = 0) -> None:
         """Synchronise and raise if a kernel reported an expired wait."""
