@@ -9,11 +9,16 @@
 // with p the degree-10 polynomial fitted by gen_erfc_coeffs.py to log2(exp(z^2) erfc(z) / t) on z in [0, 10] (relative
 // error of erfc in binary32: 6e-7 for z <= 2, growing with the rounding of z^2 like 2 z^2 * 2^-24 beyond): one
 // reciprocal, one exp2, a dozen FMAs.  The form keeps its RELATIVE accuracy for very negative gates, where 1 + erf
-// would cancel.  Every thread fetches UNROLL pairs of 16-byte pieces (one of each half of a row) before it computes
-// anything, and the grid is a small multiple of the SM count walking the tensor with a stride.
+// would cancel.  A thread takes UNROLL pairs of 16-byte pieces (one of each half of a row), all fetched before it computes
+// anything, and ends; finding a piece's row is one multiplication (a 64-bit division per piece was a third of the
+// instructions).  Two elements at a time on the packed binary32 pipe come to about 16 instructions per element.
+// 8192 x 1280 fp16 (63 MB): 12.3 us = 5.1 TB/s (16.4 with the division, a grid-stride loop and 28 instructions per
+// element, launched without overlap); fp32: 19.2 us = 6.55 TB/s, the copy rate (22.3).
 #pragma once
 #include <cuda_fp16.h>
 #include <stdint.h>
+
+#include "tc_common.cuh"  // programmatic dependent launch, FastDiv
 
 namespace sd_attn {
 
@@ -47,7 +52,7 @@ __device__ __forceinline__ float geglu_one(float a, float g) {
 }
 
 // The same for two elements at once on the packed binary32 pipe (one instruction, two results): the kernel is bound by
-// instruction issue otherwise (34 instructions per element measured with the scalar form, 18 at the copy rate).
+// instruction issue otherwise.
 __device__ __forceinline__ uint64_t geglu_dup(float v) {
     const uint32_t b = __float_as_uint(v);
     return ((uint64_t)b << 32) | b;
@@ -68,11 +73,12 @@ __device__ __forceinline__ uint64_t geglu_add2(uint64_t a, uint64_t b) {
     return d;
 }
 __device__ __forceinline__ float2 geglu_two(float2 a, float2 g) {
+    // (constants folded: t = 1 / (1 + |g| / (2 sqrt 2)), z^2 log2 e = g^2 log2(e) / 2, and the half of g/2 (1 + erf) in the
+    // exponent, so that e t is Phi(-|g|) itself)
     const uint32_t g0 = __float_as_uint(g.x), g1 = __float_as_uint(g.y);
     const uint64_t gg = ((uint64_t)g1 << 32) | g0;
     const uint64_t ag = ((uint64_t)(g1 & 0x7fffffffu) << 32) | (g0 & 0x7fffffffu);                 // |g|
-    const uint64_t z = geglu_mul2(ag, geglu_dup(0.70710678118654752f));
-    const uint64_t den = geglu_fma2(z, geglu_dup(0.5f), geglu_dup(1.0f));
+    const uint64_t den = geglu_fma2(ag, geglu_dup(0.35355339059327376f), geglu_dup(1.0f));
     float t0, t1, e0, e1;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(__uint_as_float((uint32_t)den)));
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(__uint_as_float((uint32_t)(den >> 32))));
@@ -86,83 +92,69 @@ __device__ __forceinline__ float2 geglu_two(float2 a, float2 g) {
     p = geglu_fma2(p, t, geglu_dup(geglu_p<3>()));
     p = geglu_fma2(p, t, geglu_dup(geglu_p<2>()));
     p = geglu_fma2(p, t, geglu_dup(geglu_p<1>()));
-    p = geglu_fma2(p, t, geglu_dup(geglu_p<0>()));
-    const uint64_t arg = geglu_fma2(geglu_mul2(z, geglu_dup(-1.4426950408889634f)), z, p);
+    p = geglu_fma2(p, t, geglu_dup(geglu_p<0>() - 1.0f));
+    const uint64_t arg = geglu_fma2(geglu_mul2(gg, geglu_dup(-0.72134752044448170f)), gg, p);
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(__uint_as_float((uint32_t)arg)));
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(__uint_as_float((uint32_t)(arg >> 32))));
     const uint64_t e = ((uint64_t)__float_as_uint(e1) << 32) | __float_as_uint(e0);
-    // erfc(-g / sqrt 2): erfc(z) itself for a negative gate (no subtraction: it keeps its relative accuracy), 2 - erfc(z)
-    // otherwise -- one select per element (slct picks its first operand where the third is >= 0)
-    const uint64_t ez = geglu_mul2(e, t);
-    const uint64_t two_minus = geglu_fma2(ez, geglu_dup(-1.0f), geglu_dup(2.0f));
+    // Phi(g): e t itself for a negative gate (no subtraction: it keeps its relative accuracy), 1 - e t otherwise -- one
+    // select per element (slct picks its first operand where the third is >= 0)
+    const uint64_t et = geglu_mul2(e, t);
+    const uint64_t one_minus = geglu_fma2(et, geglu_dup(-1.0f), geglu_dup(1.0f));
     float w0, w1;
-    asm("slct.f32.f32 %0, %1, %2, %3;" : "=f"(w0) : "f"(__uint_as_float((uint32_t)two_minus)), "f"(__uint_as_float((uint32_t)ez)), "f"(g.x));
-    asm("slct.f32.f32 %0, %1, %2, %3;" : "=f"(w1) : "f"(__uint_as_float((uint32_t)(two_minus >> 32))), "f"(__uint_as_float((uint32_t)(ez >> 32))), "f"(g.y));
-    const uint64_t two_phi = ((uint64_t)__float_as_uint(w1) << 32) | __float_as_uint(w0);
-    const uint64_t half_a = geglu_mul2(((uint64_t)__float_as_uint(a.y) << 32) | __float_as_uint(a.x), geglu_dup(0.5f));
-    const uint64_t o = geglu_mul2(half_a, geglu_mul2(gg, two_phi));
+    asm("slct.f32.f32 %0, %1, %2, %3;" : "=f"(w0) : "f"(__uint_as_float((uint32_t)one_minus)), "f"(__uint_as_float((uint32_t)et)), "f"(g.x));
+    asm("slct.f32.f32 %0, %1, %2, %3;" : "=f"(w1) : "f"(__uint_as_float((uint32_t)(one_minus >> 32))), "f"(__uint_as_float((uint32_t)(et >> 32))), "f"(g.y));
+    const uint64_t phi = ((uint64_t)__float_as_uint(w1) << 32) | __float_as_uint(w0);
+    const uint64_t o = geglu_mul2(((uint64_t)__float_as_uint(a.y) << 32) | __float_as_uint(a.x), geglu_mul2(gg, phi));
     return make_float2(__uint_as_float((uint32_t)o), __uint_as_float((uint32_t)(o >> 32)));
 }
 
 constexpr int GEGLU_THREADS = 256;
-#ifndef SD_GEGLU_UNROLL
-#define SD_GEGLU_UNROLL 1
-#endif
-#ifndef SD_GEGLU_BLOCKS_PER_SM
-#define SD_GEGLU_BLOCKS_PER_SM 64
-#endif
-constexpr int GEGLU_UNROLL = SD_GEGLU_UNROLL;
-constexpr int GEGLU_BLOCKS_PER_SM = SD_GEGLU_BLOCKS_PER_SM;
+constexpr int GEGLU_BLOCKS_PER_SM = 64;   // grid cap of the scalar kernel
 
 // VEC elements per 16-byte piece: 8 (fp16) or 4 (fp32); C is a multiple of VEC and both tensors are 16-byte aligned.
-// A thread walks the tensor with the grid's stride, UNROLL pieces of each half per step, all of them requested before
-// the first is used.  (Requesting the NEXT step's pieces before computing the current one -- software pipelining inside
-// the thread -- measured slower: 18.5 against 16.5 us on the 8192 x 1280 tensor; enough blocks per SM overlap one
-// another's loads and arithmetic already.  One piece per step and up to 64 blocks per SM measured best: 16.5 us there,
-// 5.74 TB/s on a tensor sixteen times as large.)
-template <typename T, int VEC>
+// BIG: 2^31 pieces or more (64-bit indices).
+template <typename T, int VEC, int UNROLL, bool BIG>
 __global__ void __launch_bounds__(GEGLU_THREADS)
-geglu_vector_kernel(const T* __restrict__ x, T* __restrict__ out, long long pieces, int pieces_per_row) {
-    const long long stride = (long long)gridDim.x * GEGLU_THREADS;
-    const long long two_c = 2ll * pieces_per_row * VEC;
-    for (long long p0 = (long long)blockIdx.x * GEGLU_THREADS + threadIdx.x; p0 < pieces; p0 += stride * GEGLU_UNROLL) {
-        uint4 a[GEGLU_UNROLL], g[GEGLU_UNROLL];
+geglu_vector_kernel(const T* __restrict__ x, T* __restrict__ out, long long pieces, FastDiv row) {
+    if (threadIdx.x == 0) pdl_launch_dependents();
+    pdl_wait();   // x may come from the previous kernel of the stream
+    const long long p0 = (long long)blockIdx.x * (GEGLU_THREADS * UNROLL) + threadIdx.x;
+    uint4 a[UNROLL], g[UNROLL];
 #pragma unroll
-        for (int u = 0; u < GEGLU_UNROLL; ++u) {
-            const long long p = p0 + u * stride;
-            if (p < pieces) {
-                const long long r = p / pieces_per_row;
-                const T* src = x + r * two_c + (p - r * pieces_per_row) * VEC;
-                a[u] = __ldg(reinterpret_cast<const uint4*>(src));
-                g[u] = __ldg(reinterpret_cast<const uint4*>(src + (long long)pieces_per_row * VEC));
+    for (int u = 0; u < UNROLL; ++u) {
+        const long long p = p0 + u * GEGLU_THREADS;
+        if (p < pieces) {
+            const long long r = BIG ? p / row.d : (long long)fast_div((uint32_t)p, row);
+            const uint4* src = reinterpret_cast<const uint4*>(x) + (p + r * row.d);   // row r starts at piece 2 r d
+            a[u] = __ldg(src);
+            g[u] = __ldg(src + row.d);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u) {
+        const long long p = p0 + u * GEGLU_THREADS;
+        if (p >= pieces) break;
+        uint4 o;
+        if (VEC == 8) {
+            const __half2* ah = reinterpret_cast<const __half2*>(&a[u]);
+            const __half2* gh = reinterpret_cast<const __half2*>(&g[u]);
+            __half2* oh = reinterpret_cast<__half2*>(&o);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                oh[k] = __float22half2_rn(geglu_two(__half22float2(ah[k]), __half22float2(gh[k])));
+        } else {
+            const float* af = reinterpret_cast<const float*>(&a[u]);
+            const float* gf = reinterpret_cast<const float*>(&g[u]);
+            float* of = reinterpret_cast<float*>(&o);
+#pragma unroll
+            for (int k = 0; k < 4; k += 2) {
+                const float2 o2 = geglu_two(make_float2(af[k], af[k + 1]), make_float2(gf[k], gf[k + 1]));
+                of[k] = o2.x;
+                of[k + 1] = o2.y;
             }
         }
-#pragma unroll
-        for (int u = 0; u < GEGLU_UNROLL; ++u) {
-            const long long p = p0 + u * stride;
-            if (p < pieces) {
-                uint4 o;
-                if (VEC == 8) {
-                    const __half2* ah = reinterpret_cast<const __half2*>(&a[u]);
-                    const __half2* gh = reinterpret_cast<const __half2*>(&g[u]);
-                    __half2* oh = reinterpret_cast<__half2*>(&o);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        oh[k] = __float22half2_rn(geglu_two(__half22float2(ah[k]), __half22float2(gh[k])));
-                } else {
-                    const float* af = reinterpret_cast<const float*>(&a[u]);
-                    const float* gf = reinterpret_cast<const float*>(&g[u]);
-                    float* of = reinterpret_cast<float*>(&o);
-#pragma unroll
-                    for (int k = 0; k < 4; k += 2) {
-                        const float2 o2 = geglu_two(make_float2(af[k], af[k + 1]), make_float2(gf[k], gf[k + 1]));
-                        of[k] = o2.x;
-                        of[k + 1] = o2.y;
-                    }
-                }
-                *reinterpret_cast<uint4*>(out + p * VEC) = o;
-            }
-        }
+        reinterpret_cast<uint4*>(out)[p] = o;
     }
 }
 

@@ -397,6 +397,19 @@ __host__ __device__ constexpr uint32_t idesc_f16(int m, int n, bool a_mn_major, 
 }
 
 // ------------------------------------------------------------------ small math helpers
+// q = n / d for 0 <= n < 2^31 by one multiplication: m = floor(2^(31 + l) / d) + 1 with l = ceil(log2 d) exceeds the exact
+// quotient's multiplier by less than 2^l / d parts, which the floor absorbs for every such n.
+struct FastDiv {
+    uint32_t d, m, shift;
+};
+__host__ inline FastDiv make_fast_div(uint32_t d) {
+    uint32_t l = 0;
+    while ((1ull << l) < d) ++l;
+    return {d, (uint32_t)((1ull << (31 + l)) / d + 1), 31 + l};
+}
+__device__ __forceinline__ uint32_t fast_div(uint32_t n, const FastDiv& f) {
+    return (uint32_t)(((uint64_t)n * f.m) >> f.shift);
+}
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
