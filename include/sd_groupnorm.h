@@ -28,9 +28,8 @@ extern "C" {
  *   eps         added to the (biased) variance under the root; finite and >= 0
  *   dtype       SD_ATTN_F16 (binary16 storage, binary32 statistics and arithmetic) or SD_ATTN_F32
  *   stream      cudaStream_t passed as void* (NULL = the legacy default stream)
- * Asynchronous and stream-ordered: enqueues one kernel (one thread block per (sample, group)), does not synchronise,
- * allocate or read back; no handle.  The FIRST call in a process raises the kernel's shared-memory limit (a host-side
- * attribute call); make it outside any stream capture.  A non-OK return means nothing was enqueued.
+ * Asynchronous and stream-ordered: enqueues one kernel (one to eight thread blocks per (sample, group)), does not
+ * synchronise, allocate or read back; no handle.  A non-OK return means nothing was enqueued.
  * Errors: INVALID_VALUE (null x or y, a size <= 0, C % G != 0, eps negative or not finite, more than 2^31 - 1 groups),
  * UNSUPPORTED (dtype), ALIGNMENT, ARCH (device not compute capability 10.x), CUDA.
  */

@@ -1,20 +1,21 @@
 // Fused group normalisation (Sec. 3.1, Eq. 1): mean, variance, normalisation and the per-channel affine of one
-// (sample, group) in one thread block, the group read from global memory ONCE.
+// (sample, group) in one kernel, the group read from global memory ONCE.
 //
 // In the model's NCHW layout a group -- C/G consecutive channels of HW values -- is one contiguous run of memory: 80 KB
-// at the 64 x 64 level of the UNet (fp16), less below.  The block copies it into shared memory while summing it, takes
-// the variance from the centred values there (two passes over shared memory: no cancellation, no second trip to DRAM)
-// and writes the result straight from shared memory.  Memory-bound: 4 bytes per fp16 element (2 read, 2 written).
-// A group that does not fit shared memory, or whose channels are not multiples of 16 bytes, takes the streaming form:
-// three passes over global memory (the second and third hit the L2).
+// at the 64 x 64 level of the UNet (fp16), less below, up to 0.7 MB (fp32, 96 x 96).  A cluster of one to eight blocks
+// takes it into registers, reduces it to mean and variance there and writes the result.  Memory-bound: 4 bytes per
+// fp16 element (2 read, 2 written).  A group that does not fit takes the streaming form: three passes over global
+// memory (the second and third hit the L2).
 #pragma once
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include "softmax_math.cuh"  // packed binary32 arithmetic
+#include "tc_common.cuh"     // programmatic dependent launch, FastDiv
+
 namespace sd_attn {
 
 constexpr int GN_THREADS = 512;
-constexpr int GN_MAX_STAGED_BYTES = 200 * 1024;
 
 __device__ __forceinline__ float gn_to_float(__half v) { return __half2float(v); }
 __device__ __forceinline__ float gn_to_float(float v) { return v; }
@@ -45,65 +46,218 @@ struct GroupNormArgs {
     float eps;
 };
 
-// Staged form.  VEC = elements per 16-byte piece; HW and the group size are multiples of VEC, so a piece never
-// straddles two channels.  The group is fetched with asynchronous 16-byte copies straight into shared memory, all of a
-// thread's copies in flight at once (with loads through registers, four at a time, the fetch of an 80 KB group was
-// three DRAM round trips long).  Every thread only ever touches the pieces it fetched itself, so no barrier separates
-// the passes; the two block-wide sums are the only meeting points.
-// (Sharing a group out among the blocks of a thread-block cluster, partial sums through distributed shared memory, was
-// measured and dropped: 8.3-8.6 us for the UNet's largest layer with 1, 2 or 4 blocks per group, 15 us with 8, and
-// slower at large batch -- the call is bound by its launch and its five dependent phases, not by one SM's bandwidth.)
+__device__ __forceinline__ uint64_t gn_pack(float lo, float hi) { return pack_b64(__float_as_uint(lo), __float_as_uint(hi)); }
+__device__ __forceinline__ float gn_sum_pair(uint64_t v) {
+    uint32_t lo, hi;
+    unpack_b64(v, lo, hi);
+    return __uint_as_float(lo) + __uint_as_float(hi);
+}
+__device__ __forceinline__ void gn_from_pair(float& d0, float& d1, uint64_t v) {   // d0, d1: neighbours in memory
+    uint32_t lo, hi;
+    unpack_b64(v, lo, hi);
+    d0 = __uint_as_float(lo);
+    d1 = __uint_as_float(hi);
+}
+__device__ __forceinline__ void gn_from_pair(__half& d0, __half&, uint64_t v) {
+    uint32_t lo, hi;
+    unpack_b64(v, lo, hi);
+    *reinterpret_cast<__half2*>(&d0) = __floats2half2_rn(__uint_as_float(lo), __uint_as_float(hi));
+}
+// x * scale + shift for the VEC values of a 16-byte piece
 template <typename T, int VEC>
-__global__ void __launch_bounds__(GN_THREADS)
-groupnorm_staged_kernel(const GroupNormArgs a) {
-    extern __shared__ uint4 gn_smem[];
-    __shared__ float scratch[GN_THREADS / 32 + 1];
-    const int cpg = a.C / a.G;
-    const long long n_elems = (long long)cpg * a.HW;
-    const int pieces = (int)(n_elems / VEC);
-    const int n = blockIdx.x / a.G, g = blockIdx.x % a.G;
-    const long long base = ((long long)n * a.C + (long long)g * cpg) * a.HW;
-    const uint4* src = reinterpret_cast<const uint4*>(static_cast<const T*>(a.x) + base);
-    uint4* dst = reinterpret_cast<uint4*>(static_cast<T*>(a.y) + base);
-
-    const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(gn_smem);
-    for (int p = threadIdx.x; p < pieces; p += GN_THREADS)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem0 + (uint32_t)p * 16u), "l"(src + p) : "memory");
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-
-    float sum = 0.f;
-    for (int p = threadIdx.x; p < pieces; p += GN_THREADS) {
-        const uint4 v = gn_smem[p];
-        const T* e = reinterpret_cast<const T*>(&v);
+__device__ __forceinline__ void gn_affine_piece(const uint4& x, float scale, float shift, uint4& y) {
+    const T* e = reinterpret_cast<const T*>(&x);
+    T* o = reinterpret_cast<T*>(&y);
+    const uint64_t ss = gn_pack(scale, scale), hh = gn_pack(shift, shift);
 #pragma unroll
-        for (int k = 0; k < VEC; ++k) sum += gn_to_float(e[k]);
+    for (int i = 0; i < VEC; i += 2)
+        gn_from_pair(o[i], o[i + 1], fma_f32x2(gn_pack(gn_to_float(e[i]), gn_to_float(e[i + 1])), ss, hh));
+}
+
+// ------------------------------------------------------------------ statistics of a set of values
+// (count, mean, sum of squared deviations from that mean).  Two sets merge without cancellation (Chan, Golub and
+// LeVeque's pairwise update), so ONE reduction delivers mean and variance: a thread takes its own values' mean and
+// deviations from registers, then warps, the block and the cluster merge triples.
+struct GnStat {
+    float n, mean, m2;
+};
+__device__ __forceinline__ GnStat gn_merge(const GnStat& a, const GnStat& b) {
+    const float n = a.n + b.n, w = n > 0.f ? __fdividef(b.n, n) : 0.f, d = b.mean - a.mean;
+    GnStat r;
+    r.n = n;
+    r.mean = fmaf(d, w, a.mean);
+    r.m2 = a.m2 + b.m2 + d * d * (a.n * w);
+    return r;
+}
+template <int LANES>
+__device__ __forceinline__ GnStat gn_merge_lanes(GnStat s) {
+#pragma unroll
+    for (int o = LANES / 2; o > 0; o >>= 1) {
+        GnStat t;
+        t.n = __shfl_xor_sync(0xffffffffu, s.n, o);
+        t.mean = __shfl_xor_sync(0xffffffffu, s.mean, o);
+        t.m2 = __shfl_xor_sync(0xffffffffu, s.m2, o);
+        s = gn_merge(s, t);
     }
-    const float mu = gn_block_sum(sum, scratch) / (float)n_elems;
-    float sq = 0.f;
-    for (int p = threadIdx.x; p < pieces; p += GN_THREADS) {
-        const uint4 v = gn_smem[p];
-        const T* e = reinterpret_cast<const T*>(&v);
+    return s;
+}
+
+// Registers form: a group is shared out among the CL blocks of a cluster, a thread holds PPT 16-byte pieces of it in
+// registers from the one read to the one write, and the blocks exchange one triple each through distributed shared
+// memory.  RAGGED: HW times the element size is no multiple of 16, so groups begin and end inside an aligned 16-byte
+// piece and pieces straddle channels.  The pieces are then those that lie whole inside the group, and the values before
+// the first and behind the last one (fewer than a piece each) go to the first block's first threads one by one.
+// What bounds it is the latency of one pass -- fetch, reduction, exchange, write -- as long as the group is shared out
+// finely enough for every SM to take part; see launch_groupnorm in sd_attn_api.cu for the split and what it measured.
+constexpr int GN_MAX_THREADS = 512;
+constexpr int GN_MAX_CLUSTER = 8;
+constexpr int GN_MAX_CPG = 1024;   // channels per group whose affine parameters the block keeps in shared memory
+
+struct GroupNormPlan {
+    int log2_cluster, pieces_per_block, cpg;   // blocks per group, 16-byte pieces of each, channels per group
+    FastDiv by_hw, by_groups;
+};
+
+__device__ __forceinline__ void gn_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void gn_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+template <typename T, int PPT, bool RAGGED>
+__global__ void __launch_bounds__(GN_MAX_THREADS)
+groupnorm_cluster_kernel(const GroupNormArgs a, const GroupNormPlan plan) {
+    const int cluster = 1 << plan.log2_cluster, pieces_per_block = plan.pieces_per_block;
+    constexpr int VEC = 16 / (int)sizeof(T);
+    __shared__ GnStat warp_stat[GN_MAX_THREADS / 32];
+    __shared__ GnStat block_stat[GN_MAX_CLUSTER];
+    __shared__ T affine[2][GN_MAX_CPG];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = (int)blockIdx.x & (cluster - 1), group = (int)blockIdx.x >> plan.log2_cluster;
+    const int cpg = plan.cpg, hw = (int)a.HW, n_elems = cpg * hw;
+    const int c0 = (group - (int)fast_div((uint32_t)group, plan.by_groups) * a.G) * cpg;
+    const long long base = (long long)group * n_elems;   // groups follow one another in memory
+    const int head = RAGGED ? (int)((VEC - (base & (VEC - 1))) & (VEC - 1)) : 0;   // values before the first whole piece
+    const int n_pieces = (n_elems - head) / VEC;                                    // (n_elems >= hw >= VEC > head)
+    const int p_end = min(n_pieces, (rank + 1) * pieces_per_block);
+    const T* src = static_cast<const T*>(a.x) + base;
+    T* dst = static_cast<T*>(a.y) + base;
+
+    if (tid == 0) pdl_launch_dependents();
+    if (cluster > 1) gn_cluster_arrive();   // every block of the cluster has started once the first wait returns
+    pdl_wait();
+
+    uint4 v[PPT];
 #pragma unroll
-        for (int k = 0; k < VEC; ++k) {
-            const float d = gn_to_float(e[k]) - mu;
-            sq = fmaf(d, d, sq);
+    for (int k = 0; k < PPT; ++k) {
+        const int p = rank * pieces_per_block + tid + k * (int)blockDim.x;
+        if (p < p_end) v[k] = *reinterpret_cast<const uint4*>(src + head + p * VEC);
+    }
+    // RAGGED: this thread's lone value, if it has one
+    const int lone = tid < head ? tid : head + n_pieces * VEC + (tid - head);
+    const bool has_lone = RAGGED && rank == 0 && tid < 2 * VEC && lone < n_elems;
+    float lone_x = has_lone ? gn_to_float(src[lone]) : 0.f;
+    for (int c = tid; c < cpg; c += (int)blockDim.x) {
+        if (a.gamma) affine[0][c] = static_cast<const T*>(a.gamma)[c0 + c];
+        if (a.beta) affine[1][c] = static_cast<const T*>(a.beta)[c0 + c];
+    }
+
+    // ---- statistics: the thread's own values, then warp, block, cluster.  One pass over the registers, about the
+    // thread's first value: as that value is one of the set, the sum of squares about it exceeds the one about the mean by
+    // at most a factor of the thread's count (and typically two), which is all the subtraction below can lose.
+    float pivot = 0.f, count = 0.f;
+    uint64_t sum2 = 0ull, sq2 = 0ull;
+#pragma unroll
+    for (int k = 0; k < PPT; ++k) {
+        const int p = rank * pieces_per_block + tid + k * (int)blockDim.x;
+        if (p >= p_end) continue;
+        const T* e = reinterpret_cast<const T*>(&v[k]);
+        if (k == 0) pivot = gn_to_float(e[0]);
+        const uint64_t pp = gn_pack(pivot, pivot);
+        count += (float)VEC;
+#pragma unroll
+        for (int i = 0; i < VEC; i += 2) {
+            const uint64_t d = sub_f32x2(gn_pack(gn_to_float(e[i]), gn_to_float(e[i + 1])), pp);
+            sum2 = add_f32x2(sum2, d);
+            sq2 = fma_f32x2(d, d, sq2);
         }
     }
-    const float var = gn_block_sum(sq, scratch) / (float)n_elems;
-    const float rstd = 1.0f / sqrtf(var + a.eps);
-    const int pieces_per_channel = (int)(a.HW / VEC);
-    const T* gamma = static_cast<const T*>(a.gamma);
-    const T* beta = static_cast<const T*>(a.beta);
-    for (int p = threadIdx.x; p < pieces; p += GN_THREADS) {
-        const int c = g * cpg + p / pieces_per_channel;
-        const float ga = gamma ? gn_to_float(gamma[c]) : 1.f, be = beta ? gn_to_float(beta[c]) : 0.f;
-        const float scale = rstd * ga, shift = fmaf(-mu, scale, be);   // y = x * scale + shift
-        uint4 v = gn_smem[p];
-        T* e = reinterpret_cast<T*>(&v);
+    if (has_lone) {
+        if (count == 0.f) pivot = lone_x;
+        const float d = lone_x - pivot;
+        count += 1.f;
+        sum2 = add_f32x2(sum2, gn_pack(d, 0.f));
+        sq2 = add_f32x2(sq2, gn_pack(d * d, 0.f));
+    }
+    GnStat s;
+    {
+        const float sum = gn_sum_pair(sum2), sq = gn_sum_pair(sq2), shift = count > 0.f ? __fdividef(sum, count) : 0.f;
+        s.n = count;
+        s.mean = pivot + shift;
+        s.m2 = fmaxf(fmaf(-sum, shift, sq), 0.f);
+    }
+    s = gn_merge_lanes<32>(s);
+    if (lane == 0) warp_stat[warp] = s;
+    __syncthreads();
+    const int warps = (int)blockDim.x >> 5;
+    s = lane < warps ? warp_stat[lane] : GnStat{0.f, 0.f, 0.f};
+    s = gn_merge_lanes<GN_MAX_THREADS / 32>(s);   // lanes 0..15 hold it all (and 16..31 nothing: lane 0 counts)
+    if (cluster > 1) {
+        gn_cluster_wait();
+        if (warp == 0 && lane < cluster) {
+            // every lane of the lower half has the block's triple; lane r stores it into block r's slot of this block
+            const GnStat mine = {__shfl_sync((1u << cluster) - 1u, s.n, 0), __shfl_sync((1u << cluster) - 1u, s.mean, 0),
+                                 __shfl_sync((1u << cluster) - 1u, s.m2, 0)};
+            const uint32_t slot = (uint32_t)__cvta_generic_to_shared(&block_stat[rank]);
+            uint32_t remote;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(slot), "r"(lane));
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(mine.n) : "memory");
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote + 4), "f"(mine.mean) : "memory");
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote + 8), "f"(mine.m2) : "memory");
+        }
+        gn_cluster_arrive();
+        gn_cluster_wait();
+        s = block_stat[0];
+        for (int r = 1; r < cluster; ++r) s = gn_merge(s, block_stat[r]);
+    } else {
+        s.mean = __shfl_sync(0xffffffffu, s.mean, 0);
+        s.m2 = __shfl_sync(0xffffffffu, s.m2, 0);
+    }
+    const float rstd = 1.0f / sqrtf(s.m2 / (float)n_elems + a.eps);
+
+    // ---- y = x * scale + shift
+    auto affine_of = [&](int c, float& scale, float& shift) {
+        const float ga = a.gamma ? gn_to_float(affine[0][c]) : 1.f, be = a.beta ? gn_to_float(affine[1][c]) : 0.f;
+        scale = rstd * ga;
+        shift = fmaf(-s.mean, scale, be);
+    };
 #pragma unroll
-        for (int k = 0; k < VEC; ++k) gn_from_float(e[k], fmaf(gn_to_float(e[k]), scale, shift));
-        dst[p] = v;
+    for (int k = 0; k < PPT; ++k) {
+        const int p = rank * pieces_per_block + tid + k * (int)blockDim.x, e0 = head + p * VEC;
+        if (p >= p_end) continue;
+        const int c = (int)fast_div((uint32_t)e0, plan.by_hw);
+        const int left = (c + 1) * hw - e0;   // values of the piece before the next channel begins
+        float scale, shift;
+        affine_of(c, scale, shift);
+        uint4 o;
+        gn_affine_piece<T, VEC>(v[k], scale, shift, o);
+        if (RAGGED && left < VEC) {
+            // a channel boundary inside (one: hw >= VEC), and another channel behind it, as the piece lies inside the group:
+            // the words behind the boundary come from a second evaluation
+            affine_of(c + 1, scale, shift);
+            uint4 o1;
+            gn_affine_piece<T, VEC>(v[k], scale, shift, o1);
+            uint32_t* w = reinterpret_cast<uint32_t*>(&o);
+            const uint32_t* w1 = reinterpret_cast<const uint32_t*>(&o1);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t m = left * (int)sizeof(T) >= 4 * i + 4 ? 0u : left * (int)sizeof(T) > 4 * i ? 0xffff0000u : 0xffffffffu;
+                w[i] = (w[i] & ~m) | (w1[i] & m);
+            }
+        }
+        *reinterpret_cast<uint4*>(dst + e0) = o;
+    }
+    if (has_lone) {
+        float scale, shift;
+        affine_of((int)fast_div((uint32_t)lone, plan.by_hw), scale, shift);
+        gn_from_float(dst[lone], fmaf(lone_x, scale, shift));
     }
 }
 

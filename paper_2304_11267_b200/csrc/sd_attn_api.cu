@@ -1247,9 +1247,61 @@ extern "C" int sd_geglu_forward(const void* x, void* out, long long rows, int C,
 }
 
 // ------------------------------------------------------------------------------------------------
-// Fused group normalisation (Sec. 3.1, Eq. 1): stateless, one kernel, one thread block per (sample, group).
-static std::mutex g_gn_mutex;
-static int g_gn_limits_raised[STATIC_MAX_DEVICES];
+// Fused group normalisation (Sec. 3.1, Eq. 1): stateless, one kernel.
+template <typename T, int PPT, bool RAGGED>
+static cudaError_t launch_groupnorm_as(const GroupNormArgs& a, const GroupNormPlan& plan, unsigned groups, int threads, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(groups << plan.log2_cluster);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1u << plan.log2_cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = plan.log2_cluster > 0 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, groupnorm_cluster_kernel<T, PPT, RAGGED>, a, plan);
+}
+
+// The registers form, or *launched = false where the group needs the streaming form.
+// Blocks per group: one as long as its 512 threads hold the group (96 KB).  A cluster of two to eight blocks with a
+// smaller share each measured slower below that, also where one block per group leaves SMs idle (2 x 320 x 64 x 64 fp16, 64
+// groups of 80 KB: 4.6 us with one block, 5.1 with two, 5.8 with four; 2 x 640 x 32 x 32: 3.6, 5.2, 5.8): a
+// cluster's launch and its barrier cost about 1.5 us.  Beyond 96 KB as few blocks of 256 threads as hold it, two of
+// which share an SM's registers (4 x 320 x 96 x 96 fp16: 14.8 us, with 512 threads 15.8).
+template <typename T>
+static cudaError_t launch_groupnorm(const GroupNormArgs& a, unsigned groups, cudaStream_t s, bool* launched) {
+    constexpr int VEC = 16 / (int)sizeof(T), MAX_PPT = 12;
+    *launched = false;
+    const long long n_elems = (long long)(a.C / a.G) * a.HW;
+    if (a.C / a.G > GN_MAX_CPG || n_elems > (long long)GN_MAX_CLUSTER * GN_MAX_THREADS * MAX_PPT * VEC) return cudaSuccess;
+    const bool ragged = a.HW % VEC != 0;
+    if (ragged && a.HW < VEC) return cudaSuccess;
+    const int pieces = (int)((n_elems + VEC - 1) / VEC);   // (a ragged group has one less)
+    int threads = pieces > 1024 ? GN_MAX_THREADS : 256, log2_cluster = 0;
+    if (pieces > GN_MAX_THREADS * MAX_PPT) {
+        threads = 256;
+        while (pieces > (threads * MAX_PPT << log2_cluster) && log2_cluster < 3) ++log2_cluster;
+        if (pieces > threads * MAX_PPT << log2_cluster) threads = GN_MAX_THREADS;
+    }
+    const int cluster = 1 << log2_cluster;
+    GroupNormPlan plan;
+    plan.log2_cluster = log2_cluster;
+    plan.pieces_per_block = (pieces + cluster - 1) / cluster;
+    plan.cpg = a.C / a.G;
+    plan.by_hw = make_fast_div((uint32_t)a.HW);
+    plan.by_groups = make_fast_div((uint32_t)a.G);
+    const int ppt = (plan.pieces_per_block + threads - 1) / threads;
+    *launched = true;
+#define SD_GN_LAUNCH(P) (ragged ? launch_groupnorm_as<T, P, true>(a, plan, groups, threads, s) : launch_groupnorm_as<T, P, false>(a, plan, groups, threads, s))
+    if (ppt <= 2) return SD_GN_LAUNCH(2);
+    if (ppt <= 4) return SD_GN_LAUNCH(4);
+    if (ppt <= 8) return SD_GN_LAUNCH(8);
+    return SD_GN_LAUNCH(MAX_PPT);
+#undef SD_GN_LAUNCH
+}
 
 extern "C" int sd_groupnorm_forward(const void* x, const void* gamma, const void* beta, void* y, int N, int C,
                                     long long HW, int G, float eps, int dtype, void* stream) {
@@ -1262,40 +1314,23 @@ extern "C" int sd_groupnorm_forward(const void* x, const void* gamma, const void
     const size_t es = dtype == SD_ATTN_F16 ? 2 : 4;
     if (((uintptr_t)x & 15u) || ((uintptr_t)y & 15u) || ((uintptr_t)gamma & (es - 1)) || ((uintptr_t)beta & (es - 1)))
         return SD_ATTN_ERR_ALIGNMENT;
-    int dev = 0, major = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
-    if (e != cudaSuccess) return cuda_fail(nullptr, e);
-    if (major != 10) return SD_ATTN_ERR_ARCH;
-    if (dev < 0 || dev >= STATIC_MAX_DEVICES) return SD_ATTN_ERR_UNSUPPORTED;
-    {
-        std::lock_guard<std::mutex> lock(g_gn_mutex);
-        if (!g_gn_limits_raised[dev]) {
-            e = raise_smem_limit(groupnorm_staged_kernel<__half, 8>, GN_MAX_STAGED_BYTES);
-            if (e == cudaSuccess) e = raise_smem_limit(groupnorm_staged_kernel<float, 4>, GN_MAX_STAGED_BYTES);
-            if (e != cudaSuccess) return cuda_fail(nullptr, e);
-            g_gn_limits_raised[dev] = 1;
-        }
-    }
+    int sms = 0;
+    const int rc = device_is_sm100(&sms);
+    if (rc != SD_ATTN_OK) return rc;
     GroupNormArgs a;
     a.x = x; a.gamma = gamma; a.beta = beta; a.y = y;
     a.C = C; a.G = G; a.HW = HW; a.eps = eps;
     cudaStream_t s = (cudaStream_t)stream;
-    const long long group_elems = (long long)(C / G) * HW;
-    const long long group_bytes = group_elems * (long long)es;
-    const int vec = (int)(16 / es);
-    const unsigned blocks = (unsigned)((long long)N * G);
-    // staged: the group fits shared memory and neither a channel nor the group ends inside a 16-byte piece
-    const bool staged = group_bytes <= GN_MAX_STAGED_BYTES && HW % vec == 0;
-    if (staged && dtype == SD_ATTN_F16) {
-        groupnorm_staged_kernel<__half, 8><<<blocks, GN_THREADS, (size_t)group_bytes, s>>>(a);
-    } else if (staged) {
-        groupnorm_staged_kernel<float, 4><<<blocks, GN_THREADS, (size_t)group_bytes, s>>>(a);
-    } else if (dtype == SD_ATTN_F16)
-        groupnorm_streaming_kernel<__half><<<blocks, GN_THREADS, 0, s>>>(a);
-    else
-        groupnorm_streaming_kernel<float><<<blocks, GN_THREADS, 0, s>>>(a);
-    e = cudaGetLastError();
+    const unsigned groups = (unsigned)((long long)N * G);
+    bool launched = false;
+    cudaError_t e = cudaSuccess;
+    if (groups < (1u << 28))
+        e = dtype == SD_ATTN_F16 ? launch_groupnorm<__half>(a, groups, s, &launched) : launch_groupnorm<float>(a, groups, s, &launched);
+    if (!launched) {
+        if (dtype == SD_ATTN_F16) groupnorm_streaming_kernel<__half><<<groups, GN_THREADS, 0, s>>>(a);
+        else groupnorm_streaming_kernel<float><<<groups, GN_THREADS, 0, s>>>(a);
+        e = cudaGetLastError();
+    }
     return e == cudaSuccess ? SD_ATTN_OK : cuda_fail(nullptr, e);
 }
 

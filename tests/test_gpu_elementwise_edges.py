@@ -1,0 +1,56 @@
+"""The edges of the dispatch rules of the group normalisation and GEGLU kernels, against the oracle (tolerances of
+test_gpu_groupnorm.py and test_gpu_geglu.py)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import test_gpu_geglu as geglu  # noqa: E402
+import test_gpu_groupnorm as gn  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def bd():
+    from paper_2304_11267_b200 import binding
+    from paper_2304_11267_b200 import build
+    build.build()
+    binding.load()
+    return binding
+
+
+# (channels per group, values per channel, groups), in values of the dtype; a 16-byte piece is 8 (fp16) or 4 (fp32) of them
+@pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
+@pytest.mark.parametrize("pieces_times", [
+    (1024, 0), (1024, 1),            # 256 threads / 512 threads
+    (6144, 0), (6144, 1),            # one block / a cluster of four
+    (12288, 1), (24576, 0), (24576, 1), (49152, 0), (49152, 1),   # clusters of eight, of larger blocks, streaming form
+])
+def test_groupnorm_group_sizes_at_the_edges_of_a_plan(bd, dtype, pieces_times):
+    pieces, more = pieces_times
+    vec = 16 // np.dtype(dtype).itemsize
+    x, gamma, beta = gn.make(pieces + more, (2, 2, (pieces + more) * vec), dtype, scale=1.3, shift=-0.7)
+    gn.check(gn.run(bd, x, 2, 1e-5, gamma, beta), x, 2, 1e-5, gamma, beta, what=str(pieces_times))
+
+
+@pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
+@pytest.mark.parametrize("C,HW,G", [(12, 9, 3), (6, 5, 1), (40, 31, 8), (10, 5525, 1), (20, 4757, 2), (64, 37, 32), (1030, 9, 1),
+                                    (2, 24577, 1), (2, 8, 2), (4, 4, 1)])
+def test_groupnorm_ragged_channels(bd, dtype, C, HW, G):
+    x, gamma, beta = gn.make(C + HW, (3, C, HW), dtype, scale=0.8, shift=5.0)
+    gn.check(gn.run(bd, x, G, 1e-5, gamma, beta), x, G, 1e-5, gamma, beta, what=str((C, HW, G)))
+
+
+@pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
+def test_groupnorm_of_an_outlier_in_front(bd, dtype):
+    """The statistics are summed about a thread's first value: a group whose first values lie far from the rest."""
+    x, gamma, beta = gn.make(5, (1, 4, 4096), dtype, scale=0.01, shift=0.0)
+    x[:, :, :8] = dtype(300.0)
+    gn.check(gn.run(bd, x, 4, 1e-5, gamma, beta), x, 4, 1e-5, gamma, beta, what="outlier")
+
+
+@pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
+@pytest.mark.parametrize("rows,C", [(1, 8), (255, 8), (257, 8), (148 * 16, 2048), (148 * 16 - 1, 2048), (4737, 1288)])
+def test_geglu_sizes_at_the_edges(bd, dtype, rows, C):
+    x = geglu.make(rows + C, rows, C, dtype)
+    geglu.check(bd.geglu(torch.from_numpy(x).cuda()).cpu().numpy(), x, what=str((rows, C)))
