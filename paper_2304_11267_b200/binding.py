@@ -1,7 +1,7 @@
 """Binding of the C-ABI attention library (argument marshalling only).
 
 The functions named as in ``include/*.h`` go through ctypes and take raw device addresses
-(``tensor.data_ptr()``); the calls on torch tensors (``Attention.forward``, ``geglu``, ``groupnorm``) are
+(``tensor.data_ptr()``); the calls on torch tensors (``Attention.forward``, ``geglu``, ``groupnorm``, ``WinogradConv3x3``) are
 marshalled by the extension module ``_sd_torch`` (csrc/torch_binding.cpp).  PyTorch only owns the memory and the
 streams.  There is no fallback: if ``libsd_attn.so`` or the extension is missing or fails to load, every call raises.
 """
@@ -31,7 +31,9 @@ EXPORTS = ["sd_attn_create", "sd_attn_create_ex", "sd_attn_static_query_status",
            "sd_attn_forward_host", "sd_attn_host_staging_bytes",
            "sd_attn_forward_twopass_static", "sd_geglu_forward", "sd_groupnorm_forward", "sd_attn_set_layout", "sd_attn_forward_batch",
            "sd_winograd_filter_elems", "sd_winograd_transform_filter", "sd_winograd_workspace_bytes",
-           "sd_winograd_conv3x3_forward", "sd_winograd_query_status"]
+           "sd_winograd_conv3x3_forward", "sd_winograd_direct_supported",
+           "sd_winograd_direct_filter_elems", "sd_winograd_direct_pack_filter", "sd_winograd_direct_forward",
+           "sd_winograd_query_status"]
 
 _lib = None
 _torch_ext = None
@@ -102,6 +104,14 @@ def load() -> ctypes.CDLL:
     lib.sd_winograd_workspace_bytes.argtypes = [ci, ci, ci, ci, ci]
     lib.sd_winograd_conv3x3_forward.restype = ci
     lib.sd_winograd_conv3x3_forward.argtypes = [vp, vp, vp, vp, vp, sz, ci, ci, ci, ci, ci, vp]
+    lib.sd_winograd_direct_supported.restype = ci
+    lib.sd_winograd_direct_supported.argtypes = [ci] * 5
+    lib.sd_winograd_direct_filter_elems.restype = sz
+    lib.sd_winograd_direct_filter_elems.argtypes = [ci, ci]
+    lib.sd_winograd_direct_pack_filter.restype = ci
+    lib.sd_winograd_direct_pack_filter.argtypes = [vp, vp, ci, ci, vp]
+    lib.sd_winograd_direct_forward.restype = ci
+    lib.sd_winograd_direct_forward.argtypes = [vp, vp, vp, vp, ci, ci, ci, ci, ci, vp]
     lib.sd_winograd_query_status.restype = ci
     lib.sd_winograd_query_status.argtypes = [vp, ctypes.POINTER(ci)]
     lib.sd_attn_set_layout.restype = ci
@@ -259,6 +269,22 @@ def sd_winograd_conv3x3_forward(x, U, bias, y, workspace, workspace_bytes, N, H,
                                               workspace_bytes, N, H, W, C, K, stream or None)
 
 
+def sd_winograd_direct_supported(N, H, W, C, K) -> bool:
+    return bool(load().sd_winograd_direct_supported(N, H, W, C, K))
+
+
+def sd_winograd_direct_filter_elems(K: int, C: int) -> int:
+    return int(load().sd_winograd_direct_filter_elems(K, C))
+
+
+def sd_winograd_direct_pack_filter(w, packed, K, C, stream) -> int:
+    return load().sd_winograd_direct_pack_filter(w or None, packed or None, K, C, stream or None)
+
+
+def sd_winograd_direct_forward(x, packed, bias, y, N, H, W, C, K, stream) -> int:
+    return load().sd_winograd_direct_forward(x or None, packed or None, bias or None, y or None, N, H, W, C, K, stream or None)
+
+
 def sd_winograd_query_status(stream=0):
     detail = (ctypes.c_int * 4)()
     rc = load().sd_winograd_query_status(stream or None, detail)
@@ -266,8 +292,11 @@ def sd_winograd_query_status(stream=0):
 
 
 class WinogradConv3x3:
-    """A layer's transformed filter plus torch-tensor marshalling: ``WinogradConv3x3(w, bias)(x)`` with
-    w [K,3,3,C], bias [K] or None, x [N,H,W,C] float16 CUDA tensors (channels-last memory) -> y [N,H,W,K]."""
+    """A layer's prepared filter plus torch-tensor marshalling: ``WinogradConv3x3(w, bias)(x)`` with
+    w [K,3,3,C], bias [K] or None, x [N,H,W,C] float16 CUDA tensors (channels-last memory) -> y [N,H,W,K].
+
+    Images the direct convolution covers go there (it is the faster one on this GPU); the others through the
+    transformed domain, whose filter ``U`` is made when the first of them comes."""
 
     def __init__(self, w, bias=None, stream: Optional[int] = None):
         import torch
@@ -275,27 +304,58 @@ class WinogradConv3x3:
             raise ValueError("w must be a contiguous float16 CUDA tensor [K,3,3,C]")
         self.K, self.C = int(w.shape[0]), int(w.shape[3])
         self.bias = bias.contiguous() if bias is not None else None
-        self.U = torch.empty(sd_winograd_filter_elems(self.K, self.C), dtype=torch.float16, device=w.device)
+        self._packed = torch.empty(sd_winograd_direct_filter_elems(self.K, self.C), dtype=torch.float16, device=w.device)
         s = stream if stream is not None else torch.cuda.current_stream(w.device).cuda_stream
-        rc = sd_winograd_transform_filter(w.data_ptr(), self.U.data_ptr(), self.K, self.C, s)
+        rc = sd_winograd_direct_pack_filter(w.data_ptr(), self._packed.data_ptr(), self.K, self.C, s)
         if rc != OK:
-            raise SdAttnError(rc, "sd_winograd_transform_filter")
+            raise SdAttnError(rc, "sd_winograd_direct_pack_filter")
+        self._U = None
         self._workspace = None
 
-    def __call__(self, x, out=None, stream: Optional[int] = None):
+    def _filter(self):
+        """The filter [K,3,3,C] back from the packed one (pieces of eight channels, swizzled by the filter's number)."""
         import torch
-        if not (x.is_cuda and x.dtype == torch.float16 and x.is_contiguous() and x.dim() == 4 and x.shape[3] == self.C):
-            raise ValueError("x must be a contiguous float16 CUDA tensor [N,H,W,%d]" % self.C)
+        p = self._packed.view(-1, 9, (self.K + 15) // 16 * 16, 8, 8)
+        at = torch.arange(8, device=p.device)[None, :] ^ (torch.arange(p.shape[2], device=p.device) & 7)[:, None]
+        p = torch.gather(p, 3, at[None, None, :, :, None].expand(p.shape))
+        return p.permute(2, 1, 0, 3, 4).reshape(p.shape[2], 3, 3, -1)[:self.K, :, :, :self.C].contiguous()
+
+    @property
+    def U(self):
+        """The filter in the transformed domain (made on the current stream at first use)."""
+        import torch
+        if self._U is None:
+            w = self._filter()
+            U = torch.empty(sd_winograd_filter_elems(self.K, self.C), dtype=torch.float16, device=w.device)
+            rc = sd_winograd_transform_filter(w.data_ptr(), U.data_ptr(), self.K, self.C,
+                                              torch.cuda.current_stream(w.device).cuda_stream)
+            if rc != OK:
+                raise SdAttnError(rc, "sd_winograd_transform_filter")
+            self._U = U
+        return self._U
+
+    def __call__(self, x, out=None, stream: Optional[int] = None):
+        r = (_torch_ext or _ext()).conv3x3(x, self._packed, self.bias, self.K, self.C, out, stream)
+        if r.__class__ is not int:
+            return r
+        if r != ERR_UNSUPPORTED:
+            raise SdAttnError(r, "sd_winograd_direct_forward")
+        return self._transformed(x, out, stream)
+
+    def _transformed(self, x, out, stream):
+        import torch
         N, H, W, _ = (int(v) for v in x.shape)
+        s = stream if stream is not None else torch.cuda.current_stream(x.device).cuda_stream
+        with torch.cuda.stream(torch.cuda.ExternalStream(s, device=x.device)):
+            U = self.U   # (its first use is ordered before this call)
         need = sd_winograd_workspace_bytes(N, H, W, self.C, self.K)
         if self._workspace is None or self._workspace.numel() < need:
             self._workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=x.device)
         if out is None:
             out = torch.empty(N, H, W, self.K, dtype=torch.float16, device=x.device)
-        s = stream if stream is not None else torch.cuda.current_stream(x.device).cuda_stream
-        rc = sd_winograd_conv3x3_forward(x.data_ptr(), self.U.data_ptr(),
-                                         self.bias.data_ptr() if self.bias is not None else 0, out.data_ptr(),
-                                         self._workspace.data_ptr(), self._workspace.numel(), N, H, W, self.C, self.K, s)
+        rc = sd_winograd_conv3x3_forward(x.data_ptr(), U.data_ptr(), self.bias.data_ptr() if self.bias is not None else 0,
+                                         out.data_ptr(), self._workspace.data_ptr(), self._workspace.numel(), N, H, W, self.C,
+                                         self.K, s)
         if rc != OK:
             raise SdAttnError(rc, "sd_winograd_conv3x3_forward")
         return out

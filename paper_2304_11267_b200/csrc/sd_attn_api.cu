@@ -17,6 +17,7 @@
 #include "../../include/sd_groupnorm.h"
 #include "../../include/sd_winograd.h"
 #include "cross_kernel.cuh"
+#include "conv_direct_kernel.cuh"
 #include "cross2_kernel.cuh"
 #include "geglu_kernel.cuh"
 #include "groupnorm_kernel.cuh"
@@ -1343,6 +1344,8 @@ struct WinogradDeviceState {
     int ready;
     int* status;
     encode_tiled_fn encode_tiled;
+    int sm_count;
+    int max_clusters[CD_MAX_SPLIT + 1];   // clusters of that many conv_direct_kernel CTAs the device holds at once
 };
 static WinogradDeviceState g_wg_state[STATIC_MAX_DEVICES];
 
@@ -1366,6 +1369,22 @@ static int winograd_setup(WinogradDeviceState** out) {
             return cuda_fail(nullptr, e != cudaSuccess ? e : cudaErrorUnknown);
         e = raise_smem_limit(winograd_gemm_kernel, winograd_gemm_smem_bytes(WG_MAX_N_CHUNK, WG_MAX_STAGES));
         if (e == cudaSuccess) e = cudaMemset(status, 0, sizeof(int) * DEV_STATUS_INTS);
+        if (e == cudaSuccess) e = raise_smem_limit(conv_direct_kernel<false>, CD_SMEM_BUDGET + 1024);
+        if (e == cudaSuccess) e = raise_smem_limit(conv_direct_kernel<true>, CD_SMEM_BUDGET + 1024);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&st->sm_count, cudaDevAttrMultiProcessorCount, dev);
+        for (int c = 2; c <= CD_MAX_SPLIT && e == cudaSuccess; ++c) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(c, 64, 1);
+            cfg.blockDim = dim3(CD_THREADS);
+            cfg.dynamicSmemBytes = CD_SMEM_BUDGET + 1024;
+            cudaLaunchAttribute attr;
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = c;
+            attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            e = cudaOccupancyMaxActiveClusters(&st->max_clusters[c], conv_direct_kernel<true>, &cfg);
+        }
         if (e != cudaSuccess) return cuda_fail(nullptr, e);
         st->status = (int*)status;
         st->encode_tiled = (encode_tiled_fn)fn;
@@ -1461,6 +1480,139 @@ extern "C" int sd_winograd_conv3x3_forward(const void* x, const void* U, const v
     if (e != cudaSuccess) return cuda_fail(nullptr, e);
     e = launch_overlapped_if(overlap, winograd_output_kernel, dim3((unsigned)((out_threads + 127) / 128)), dim3(128), 0, s,
                              (const float*)M, (const __half*)bias, (__half*)y, a);
+    return e == cudaSuccess ? SD_ATTN_OK : cuda_fail(nullptr, e);
+}
+
+// ------------------------------------------------------------------------------------------------
+// The same convolution as one implicit matrix product (conv_direct_kernel.cuh).
+struct ConvDirectPlan {
+    int n_tile, n_tiles, m_tiles, split, stages;
+};
+
+static bool conv_direct_fits(int N, int H, int W, int C, int K) {
+    return W <= CD_MAX_W && C % 8 == 0 && K % 8 == 0 && ((long long)N * (H + 1) + 1) * (W + 2) + TILE_M < (1ll << 30) &&
+           ((long long)N * (H + 1) * (W + 2) + TILE_M - 1) / TILE_M <= 65535 && (long long)N * H * W <= (1ll << 31) / 8;
+}
+
+// Filter rows per CTA and CTAs per tile.  Clocks of a (64 channels, tap) step: the tensor core's 2 n, its operand reads from
+// shared memory (128 bytes a clock: 128 + n), the fetch of n filter rows of 128 bytes and a ninth of the patch at about
+// 80 bytes a clock and SM, and half of what an issuing thread needs for one; times the steps of a CTA and the waves, plus
+// the ramp of a CTA (first fetch, accumulator out) and, for a split, the cluster's exchange.
+static ConvDirectPlan plan_conv_direct(const WinogradDeviceState* st, int N, int H, int W, int C, int K) {
+    const int pw = W + 2, steps = 9 * ((C + CHUNK_COLS - 1) / CHUNK_COLS), patch_bytes = cd_patch_bytes(pw);
+    ConvDirectPlan best = {};
+    double best_cost = -1.0;
+    const int n_max = (K + 15) / 16 * 16 < CD_MAX_N ? (K + 15) / 16 * 16 : CD_MAX_N;
+    ConvDirectPlan p;
+    p.m_tiles = (int)(((long long)N * (H + 1) * pw + TILE_M - 1) / TILE_M);
+    for (int n = n_max < 64 ? n_max : 64; n <= n_max; n += 16) {
+        p.n_tile = n;
+        p.n_tiles = (K + n - 1) / n;
+        p.stages = (CD_SMEM_BUDGET - 2 * patch_bytes) / (n * CHUNK_ROW_BYTES);
+        if (p.stages > CD_MAX_STAGES) p.stages = CD_MAX_STAGES;
+        if (p.stages < 2) continue;
+        const double fetch = (n * CHUNK_ROW_BYTES + patch_bytes / 9.0) / 80.0;
+        double step = n > 128 ? 2.0 * n : 128.0 + n;
+        if (fetch > step) step = fetch;
+        if (step < 280.0) step = 280.0;
+        if (p.stages < 4) step *= 1.15;
+        for (p.split = 1; p.split <= CD_MAX_SPLIT && steps / p.split >= 9; ++p.split) {
+            const int at_once = p.split == 1 ? st->sm_count : st->max_clusters[p.split] * p.split;
+            if (at_once <= 0 || cd_staging_bytes(n, p.split) > 2 * patch_bytes + p.stages * n * CHUNK_ROW_BYTES) continue;
+            const long ctas = (long)p.n_tiles * p.m_tiles * p.split;
+            const double waves = (double)((ctas + at_once - 1) / at_once);
+            const double cost = waves * (((steps + p.split - 1) / p.split) * step + 5000.0 + (p.split > 1 ? 2500.0 : 0.0));
+            if (best_cost < 0 || cost < best_cost) {
+                best_cost = cost;
+                best = p;
+            }
+        }
+    }
+    return best;
+}
+
+extern "C" int sd_winograd_direct_supported(int N, int H, int W, int C, int K) {
+    return N > 0 && H > 0 && W > 0 && C > 0 && K > 0 && conv_direct_fits(N, H, W, C, K) ? 1 : 0;
+}
+
+extern "C" size_t sd_winograd_direct_filter_elems(int K, int C) { return K > 0 && C > 0 ? conv_packed_elems(K, C) : 0; }
+
+extern "C" int sd_winograd_direct_pack_filter(const void* w, void* packed, int K, int C, void* stream) {
+    if (!w || !packed || K <= 0 || C <= 0) return SD_ATTN_ERR_INVALID_VALUE;
+    if (K % 8 != 0 || C % 8 != 0) return SD_ATTN_ERR_UNSUPPORTED;
+    if (((uintptr_t)w & 15u) || ((uintptr_t)packed & 15u)) return SD_ATTN_ERR_ALIGNMENT;
+    int sms = 0;
+    const int rc = device_is_sm100(&sms);
+    if (rc != SD_ATTN_OK) return rc;
+    const long long pieces = (long long)(conv_packed_elems(K, C) / 8);
+    conv_pack_kernel<<<(unsigned)((pieces + 255) / 256), 256, 0, (cudaStream_t)stream>>>((const __half*)w, (__half*)packed, K, C);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? SD_ATTN_OK : cuda_fail(nullptr, e);
+}
+
+extern "C" int sd_winograd_direct_forward(const void* x, const void* packed, const void* bias, void* y, int N, int H, int W, int C, int K,
+                                          void* stream) {
+    if (N < 0 || H <= 0 || W <= 0 || C <= 0 || K <= 0) return SD_ATTN_ERR_INVALID_VALUE;
+    if (C % 8 != 0 || K % 8 != 0) return SD_ATTN_ERR_UNSUPPORTED;
+    if (N == 0) return SD_ATTN_OK;
+    if (!x || !packed || !y) return SD_ATTN_ERR_INVALID_VALUE;
+    if (((uintptr_t)x & 15u) || ((uintptr_t)packed & 15u) || ((uintptr_t)y & 15u) || ((uintptr_t)bias & 3u)) return SD_ATTN_ERR_ALIGNMENT;
+    if (!conv_direct_fits(N, H, W, C, K)) return SD_ATTN_ERR_UNSUPPORTED;
+    WinogradDeviceState* st = nullptr;
+    const int rc = winograd_setup(&st);
+    if (rc != SD_ATTN_OK) return rc;
+    // (the plan depends on the shape only: a layer's next call finds its own)
+    struct Known { int N, H, W, C, K; const WinogradDeviceState* st; ConvDirectPlan plan; };
+    static thread_local Known known[8];
+    static thread_local int known_next = 0;
+    const ConvDirectPlan* plan = nullptr;
+    for (const Known& k : known)
+        if (k.st == st && k.N == N && k.H == H && k.W == W && k.C == C && k.K == K) plan = &k.plan;
+    if (!plan) {
+        Known& k = known[known_next];
+        known_next = (known_next + 1) % 8;
+        k = {N, H, W, C, K, st, plan_conv_direct(st, N, H, W, C, K)};
+        plan = &k.plan;
+    }
+    if (plan->n_tiles == 0) return SD_ATTN_ERR_UNSUPPORTED;
+
+    ConvDirectArgs a;
+    a.y = (__half*)y; a.bias = (const __half*)bias;
+    a.H = H; a.W = W; a.K = K;
+    a.pw = W + 2;
+    a.padded_rows = N * (H + 1);
+    a.chunks = (C + CHUNK_COLS - 1) / CHUNK_COLS;
+    a.n_tile = plan->n_tile;
+    a.tmem_cols = next_pow2_cols(2 * plan->n_tile);
+    a.split = plan->split;
+    a.stages = plan->stages;
+    a.patch_bytes = cd_patch_bytes(a.pw);
+    a.filter = (const __half*)packed;
+    a.k_padded = (K + 15) / 16 * 16;
+    a.by_pw = make_fast_div((uint32_t)a.pw);
+    a.by_h1 = make_fast_div((uint32_t)(H + 1));
+    a.status = st->status;
+    CUtensorMap tx;
+    const cuuint64_t xd[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
+    const cuuint64_t xs[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
+    const cuuint32_t xb[4] = {(cuuint32_t)CHUNK_COLS, (cuuint32_t)a.pw, 1, 1}, ones[4] = {1, 1, 1, 1};
+    if (st->encode_tiled(&tx, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(x), xd, xs, xb, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                         CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return SD_ATTN_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)plan->split, (unsigned)plan->n_tiles, (unsigned)plan->m_tiles);
+    cfg.blockDim = dim3(CD_THREADS);
+    cfg.dynamicSmemBytes = (size_t)2 * a.patch_bytes + (size_t)plan->stages * plan->n_tile * CHUNK_ROW_BYTES + 1024;
+    cfg.stream = (cudaStream_t)stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)plan->split;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = plan->split > 1 ? 2 : 1;
+    const cudaError_t e = plan->split > 1 ? cudaLaunchKernelEx(&cfg, conv_direct_kernel<true>, tx, a) : cudaLaunchKernelEx(&cfg, conv_direct_kernel<false>, tx, a);
     return e == cudaSuccess ? SD_ATTN_OK : cuda_fail(nullptr, e);
 }
 

@@ -18,6 +18,7 @@
 #include "../../include/sd_attn.h"
 #include "../../include/sd_geglu.h"
 #include "../../include/sd_groupnorm.h"
+#include "../../include/sd_winograd.h"
 
 namespace {
 
@@ -179,6 +180,32 @@ PyObject* groupnorm_impl(PyObject* const* a) {
     return result(a[5], std::move(made));
 }
 
+// conv3x3(x, packed filter, bias or None, K, C, out or None, stream or None) -> out, or an int status
+PyObject* conv3x3_impl(PyObject* const* a) {
+    const Tensor *x = tensor_of(a[0], "x"), *packed = x ? tensor_of(a[1], "packed") : nullptr;
+    if (!packed) return nullptr;
+    const Tensor* bias = nullptr;
+    if (a[2] != Py_None && !(bias = tensor_of(a[2], "bias"))) return nullptr;
+    const long K = PyLong_AsLong(a[3]), C = PyLong_AsLong(a[4]);
+    if (PyErr_Occurred()) return nullptr;
+    if (!x->is_cuda() || x->scalar_type() != at::kHalf || !x->is_contiguous() || x->dim() != 4 || x->size(3) != C) {
+        PyErr_Format(PyExc_ValueError, "x must be a contiguous float16 CUDA tensor [N,H,W,%ld]", C);
+        return nullptr;
+    }
+    const int64_t N = x->size(0), H = x->size(1), W = x->size(2);
+    void* stream;
+    if (!stream_of(a[6], *x, &stream)) return nullptr;
+    if (N > 0 && !sd_winograd_direct_supported((int)N, (int)H, (int)W, (int)C, (int)K)) return PyLong_FromLong(SD_ATTN_ERR_UNSUPPORTED);
+    Tensor made;
+    const Tensor* out = &made;
+    if (a[5] == Py_None) made = empty_on(*x, {N, H, W, (int64_t)K});
+    else if (!(out = tensor_of(a[5], "out"))) return nullptr;
+    const int rc = sd_winograd_direct_forward(x->data_ptr(), packed->data_ptr(), bias ? bias->data_ptr() : nullptr, out->data_ptr(), (int)N,
+                                              (int)H, (int)W, (int)C, (int)K, stream);
+    if (rc != SD_ATTN_OK) return PyLong_FromLong(rc);
+    return result(a[5], std::move(made));
+}
+
 // A C++ exception (out of memory in the caching allocator, say) becomes the Python error torch itself would raise.
 template <PyObject* (*IMPL)(PyObject* const*), int N_ARGS>
 PyObject* entry(PyObject*, PyObject* const* args, Py_ssize_t n) {
@@ -195,6 +222,7 @@ PyMethodDef methods[] = {
     {"attention", (PyCFunction)(void*)entry<attention_impl, 8>, METH_FASTCALL, "sd_attn_forward on torch tensors"},
     {"geglu", (PyCFunction)(void*)entry<geglu_impl, 3>, METH_FASTCALL, "sd_geglu_forward on torch tensors"},
     {"groupnorm", (PyCFunction)(void*)entry<groupnorm_impl, 7>, METH_FASTCALL, "sd_groupnorm_forward on torch tensors"},
+    {"conv3x3", (PyCFunction)(void*)entry<conv3x3_impl, 7>, METH_FASTCALL, "sd_winograd_direct_forward on torch tensors"},
     {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_sd_torch", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};

@@ -1,0 +1,84 @@
+"""The direct 3x3 convolution at the edges of its tiles and of its plan, and the transformed domain behind the same class
+for images it does not cover, against the oracle.
+
+The direct kernel multiplies the binary16 values as they are, accumulates in binary32 and rounds once: |err| <= 2^-11 |y|
+plus binary32 accumulation over 9 C products (2e-6 of the sum of their magnitudes, about sqrt(9 C) r.m.s. here).
+"""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import test_gpu_winograd as wg  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def bd():
+    from paper_2304_11267_b200 import binding
+    from paper_2304_11267_b200 import build
+    build.build()
+    binding.load()
+    return binding
+
+
+# one position and one channel group; just under, at and over 128 positions of the padded raster (W + 2) (H + 1); three
+# images in one tile; the widest image (126) and rows that leave a tile one position; channel counts around 64 and K around
+# the 16-filter granule, one and several filter tiles; few tiles and many channels (the steps split two- to eightfold)
+@pytest.mark.parametrize("N,H,W,C,K", [
+    (1, 1, 1, 8, 8), (1, 6, 15, 8, 8), (1, 7, 14, 16, 24), (1, 7, 15, 64, 40), (3, 3, 3, 72, 16), (2, 2, 126, 64, 32),
+    (1, 1, 126, 8, 264), (2, 5, 125, 56, 72), (1, 8, 8, 1280, 64), (2, 9, 12, 640, 328), (1, 16, 16, 320, 1280),
+    (1, 33, 43, 128, 200), (4, 12, 11, 320, 320), (2, 31, 29, 192, 648),
+])
+def test_against_the_oracle(bd, N, H, W, C, K):
+    assert bd.sd_winograd_direct_supported(N, H, W, C, K)
+    x, w, b = wg.make(500 + H + W + C + K, N, H, W, C, K)
+    ref = oracle.conv3x3_forward(x, w, b)
+    got = wg.run(bd, x, w, b).astype(np.float64)
+    err = np.abs(got - ref)
+    assert np.all(err <= 2.0 ** -11 * np.abs(ref) + 2e-5), float((err - 2.0 ** -11 * np.abs(ref)).max())
+
+
+def test_guard_bytes_and_repeated_bits(bd):
+    x, w, b = wg.make(3, 2, 9, 13, 640, 72)
+    layer = bd.WinogradConv3x3(torch.from_numpy(w).cuda(), torch.from_numpy(b).cuda())
+    tx = torch.from_numpy(x).cuda()
+    n, guard = 2 * 9 * 13 * 72, 4096
+    buf = torch.full((n + 2 * guard,), 55.0, dtype=torch.float16, device="cuda")
+    out = buf[guard:guard + n].view(2, 9, 13, 72)
+    layer(tx, out=out)
+    again = layer(tx)
+    torch.cuda.synchronize()
+    assert torch.equal(out, again)
+    assert bool((buf[:guard] == 55.0).all()) and bool((buf[guard + n:] == 55.0).all())
+
+
+def test_wide_images_take_the_transformed_domain(bd):
+    assert not bd.sd_winograd_direct_supported(1, 6, 127, 72, 40)
+    x, w, b = wg.make(11, 1, 6, 127, 72, 40)
+    wg.check(wg.run(bd, x, w, b), oracle.conv3x3_forward(x, w, b), "127 wide")
+
+
+@pytest.mark.parametrize("N,H,W,C,K", [(2, 32, 32, 320, 320), (1, 13, 10, 40, 24), (3, 7, 9, 200, 328), (1, 1, 5, 16, 16)])
+def test_the_transformed_domain_itself(bd, N, H, W, C, K):
+    x, w, b = wg.make(700 + H + C, N, H, W, C, K)
+    layer = bd.WinogradConv3x3(torch.from_numpy(w).cuda(), torch.from_numpy(b).cuda())
+    assert torch.equal(layer._filter().cpu(), torch.from_numpy(w))
+    y = layer._transformed(torch.from_numpy(x).cuda(), None, None)
+    rc, detail = bd.sd_winograd_query_status()
+    assert rc == bd.OK, detail
+    wg.check(y.cpu().numpy(), oracle.conv3x3_forward(x, w, b), str((N, H, W, C, K)))
+
+
+def test_arguments(bd):
+    f = bd.sd_winograd_direct_forward
+    assert f(256, 256, 0, 256, 1, 8, 8, 0, 16, 0) == bd.ERR_INVALID_VALUE
+    assert f(256, 256, 0, 256, 1, 8, 8, 12, 16, 0) == bd.ERR_UNSUPPORTED
+    assert f(256, 256, 0, 256, 1, 8, 127, 16, 16, 0) == bd.ERR_UNSUPPORTED
+    assert f(256, 256, 0, 256, 0, 8, 8, 16, 16, 0) == bd.OK
+    assert f(0, 256, 0, 256, 1, 8, 8, 16, 16, 0) == bd.ERR_INVALID_VALUE
+    assert f(264, 256, 0, 256, 1, 8, 8, 16, 16, 0) == bd.ERR_ALIGNMENT
+    assert bd.sd_winograd_direct_pack_filter(0, 256, 16, 16, 0) == bd.ERR_INVALID_VALUE
+    assert bd.sd_winograd_direct_pack_filter(256, 256, 12, 16, 0) == bd.ERR_UNSUPPORTED
