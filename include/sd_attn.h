@@ -54,14 +54,15 @@ typedef enum {
 
 typedef enum {
     SD_ATTN_F16 = 0, /* IEEE binary16 q/k/v/out, binary32 accumulation            */
-    SD_ATTN_F32 = 1, /* binary32 throughout (plain FMA arithmetic, no TF32)        */
+    SD_ATTN_F32 = 1, /* binary32 throughout: plain FMAs, or (AUTO, d % 4 == 0) products of operands split exactly into
+                        three bfloat16 parts on the tensor cores, accumulated in binary32; never TF32        */
     SD_ATTN_BF16 = 2 /* bfloat16 q/k/v/out, binary32 accumulation; the softmax weights enter the second product
                         rounded to bfloat16 (8 significant bits), so results are about 8x coarser than F16's.
                         Implemented by FUSED, CROSS and SIMT; TWOPASS mode answers UNSUPPORTED.              */
 } sd_attn_dtype;
 
 typedef enum {
-    SD_ATTN_MODE_AUTO = 0,    /* F16: CROSS when Nk fits one key tile, else FUSED.  F32: SIMT */
+    SD_ATTN_MODE_AUTO = 0,    /* F16: CROSS when Nk fits one key tile, else FUSED.  F32: reported as SIMT */
     SD_ATTN_MODE_FUSED = 1,   /* single-pass online softmax (FlashAttention, Sec. 3.2.2)      */
     SD_ATTN_MODE_CROSS = 2,   /* all keys in one shared-memory tile, plain softmax            */
     SD_ATTN_MODE_TWOPASS = 3, /* partially fused softmax of Sec. 3.2.1: scores and [L,S] in HBM */

@@ -22,6 +22,7 @@
 #include "geglu_kernel.cuh"
 #include "groupnorm_kernel.cuh"
 #include "winograd_kernel.cuh"
+#include "f32_kernel.cuh"
 #include "fused4s_kernel.cuh"
 #include "selftest_kernel.cuh"
 #include "simt_kernel.cuh"
@@ -79,6 +80,7 @@ struct sd_attn_handle {
     encode_tiled_fn encode_tiled;
     cudaError_t last_cuda_error;
     int sm_count;
+    int f32_ok;               // likewise (see below) for the f32_attention_kernel
     int fused4s_ok;           // the register hand-over inside these kernels fits their launch allocation
     int cross2_four_ok;
     // sd_attn_forward_host: copies of one slice of heads overlap the kernel of another (see there)
@@ -226,6 +228,15 @@ static cudaError_t check_register_pools(sd_attn_handle* h) {
     return e;
 }
 
+template <typename SH>
+static cudaError_t prepare_f32_kernel(sd_attn_handle* h) {
+    cudaFuncAttributes fa;
+    cudaError_t e = raise_smem_limit(f32_attention_kernel<SH>, SH::SMEM);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, f32_attention_kernel<SH>);
+    if (e == cudaSuccess && SH::THREADS * fa.numRegs < SH::POOL) h->f32_ok = 0;
+    return e;
+}
+
 extern "C" int sd_attn_create_ex(const sd_attn_options* options, sd_attn_handle** out) {
     if (!out) return SD_ATTN_ERR_INVALID_VALUE;
     *out = nullptr;
@@ -286,6 +297,11 @@ extern "C" int sd_attn_create_ex(const sd_attn_options* options, sd_attn_handle*
         h->cross2_four_ok = 1;
         e = check_register_pools<false>(h);
         if (e == cudaSuccess) e = check_register_pools<true>(h);
+        h->f32_ok = 1;
+        if (e == cudaSuccess) e = prepare_f32_kernel<F32Two>(h);
+        if (e == cudaSuccess) e = prepare_f32_kernel<F32One>(h);
+        if (e == cudaSuccess) e = prepare_f32_kernel<F32Mid>(h);
+        if (e == cudaSuccess) e = prepare_f32_kernel<F32Wide>(h);
     }
     if (e == cudaSuccess) e = cudaMalloc((void**)&h->dev_status, sizeof(int) * DEV_STATUS_INTS);
     if (e == cudaSuccess) e = cudaMemset(h->dev_status, 0, sizeof(int) * DEV_STATUS_INTS);
@@ -490,6 +506,36 @@ static int launch_simt(sd_attn_handle* h, const Problem& p) {
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->launches += 1;
     return SD_ATTN_OK;
+}
+
+template <typename SH>
+static int launch_f32_as(sd_attn_handle* h, const Problem& p, F32Args& a) {
+    const int tiles = (p.Nq + TILE_M - 1) / TILE_M;
+    a.units_per_head = (tiles + SH::T - 1) / SH::T;
+    const cudaError_t e = launch_overlapped(h, f32_attention_kernel<SH>, dim3((unsigned)(a.units_per_head * p.BH)), dim3(SH::THREADS), SH::SMEM,
+                                            p.stream, a);
+    if (e != cudaSuccess) return cuda_fail(h, e);
+    h->launches += 1;
+    return SD_ATTN_OK;
+}
+
+// binary32 tensors with d % 4 == 0: three-way split operands on the tensor cores.  Two query tiles per CTA (d <= 48) as soon
+// as the tiles outnumber the SMs: they share the conversion of K and V, and one's softmax runs under the other's products.
+static int launch_f32(sd_attn_handle* h, const Problem& p) {
+    F32Args a;
+    a.q = (const float*)p.q; a.k = (const float*)p.k; a.v = (const float*)p.v; a.out = (float*)p.out;
+    a.lq = head_layout(p.heads, p.BH, p.Nq, p.d);
+    a.lk = head_layout(p.heads, p.BH, p.Nk, p.d);
+    a.Nq = p.Nq; a.Nk = p.Nk; a.d = p.d;
+    a.scale_log2e = fabsf(p.scale) * LOG2E;
+    a.negate = p.scale < 0.f;
+    a.by_pieces = make_fast_div((uint32_t)(p.d + 7) / 8);
+    a.status = h->dev_status;
+    const long long tiles = (long long)((p.Nq + TILE_M - 1) / TILE_M) * p.BH;
+    if (p.d <= 48 && tiles > h->sm_count) return launch_f32_as<F32Two>(h, p, a);
+    if (p.d <= 64) return launch_f32_as<F32One>(h, p, a);
+    if (p.d <= 96) return launch_f32_as<F32Mid>(h, p, a);
+    return launch_f32_as<F32Wide>(h, p, a);
 }
 
 // 65..80 keys (the 77 text tokens): one persistent CTA per SM walks a range of (head, tile) items of `n` problems of
@@ -807,6 +853,8 @@ static Problem make_problem(const sd_attn_handle* h, const void* q, const void* 
 static int launch_one(sd_attn_handle* h, const Problem& p, int mode, int dtype) {
     switch (mode) {
         case SD_ATTN_MODE_SIMT:
+            // AUTO's binary32 kernel; the CUDA-core kernel serves the other types, d % 4 != 0 and callers that ask for it
+            if (dtype == SD_ATTN_F32 && h->mode == SD_ATTN_MODE_AUTO && p.d % 4 == 0 && h->f32_ok) return launch_f32(h, p);
             return dtype == SD_ATTN_F16    ? launch_simt<__half>(h, p)
                    : dtype == SD_ATTN_BF16 ? launch_simt<__nv_bfloat16>(h, p)
                                            : launch_simt<float>(h, p);

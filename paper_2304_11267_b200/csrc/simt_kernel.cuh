@@ -2,8 +2,8 @@
 //
 // It evaluates Eq. 3 with the single-pass running (max, sum) form of the softmax reductions of
 // Eq. 4 (the FlashAttention recurrence of Sec. 3.2.2) using plain FMAs -- no tensor cores, hence
-// no TF32 rounding -- and is the library's binary32 path and the on-device cross-check of the
-// tensor-core kernels.
+// no TF32 rounding -- and serves head dims the tensor-core kernels do not take (16-bit tensors with d % 8 != 0, binary32
+// with d % 4 != 0) and is the on-device cross-check of those kernels.
 //
 // Work split: a block owns 32 query rows (8 warps x 4 rows); keys stream through shared memory
 // in chunks of 32.  In the score phase lane j owns key j of the chunk; in the P.V phase lane c

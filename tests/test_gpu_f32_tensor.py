@@ -1,0 +1,84 @@
+"""AUTO's binary32 kernel (three-way split operands on the tensor cores) at the edges of its variants, against the oracle.
+
+Bounds: the split products are exact to 2^-24 and every tile's sum is rounded to nearest, so the error is binary32's: 2e-6 of
+max |V| and 2e-6 relative L2 (measured at most 5e-7), a fifth of the path's stated tolerance.  Scores in the hundreds carry
+their own rounding (2^-24 of a score of 500 moves a weight by 3e-5): those cases use the stated 1e-5 against a softmax whose
+weights sit on few keys."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def bd():
+    from paper_2304_11267_b200 import binding
+    from paper_2304_11267_b200 import build
+    build.build()
+    binding.load()
+    return binding
+
+
+def draw(seed, B, H, Nq, Nk, d):
+    g = np.random.default_rng(seed)
+    return tuple(g.standard_normal((B, H, n, d), dtype=np.float32) for n in (Nq, Nk, Nk))
+
+
+def run(bd, q, k, v, scale, tokens_first=False):
+    a = bd.Attention(layout=bd.LAYOUT_BNHD if tokens_first else bd.LAYOUT_BHND)
+    t = [torch.from_numpy(np.ascontiguousarray(x.transpose(0, 2, 1, 3)) if tokens_first else x).cuda() for x in (q, k, v)]
+    out = a.forward(*t, scale=scale)
+    a.check()
+    assert a.last_mode == bd.MODE_SIMT
+    out = out.cpu().numpy()
+    return out.transpose(0, 2, 1, 3) if tokens_first else out
+
+
+def check(got, ref, v, bound=2e-6):
+    got = got.astype(np.float64)
+    assert np.all(np.isfinite(got))
+    err, rel = np.abs(got - ref).max() / np.abs(v).max(), np.linalg.norm(got - ref) / np.linalg.norm(ref)
+    assert err <= bound and rel <= bound, (err, rel)
+
+
+# head dims at the edges of the variants (48, 64, 96, 160) and of the 4-, 8- and 16-column granules; rows around one and two
+# query tiles; keys around the 32- and 64-key tiles
+@pytest.mark.parametrize("d", [4, 8, 20, 40, 44, 48, 52, 64, 68, 80, 96, 100, 160])
+@pytest.mark.parametrize("Nq,Nk", [(1, 1), (127, 64), (129, 65), (257, 33), (300, 191)])
+def test_variants(bd, d, Nq, Nk):
+    q, k, v = draw(d + Nq, 1, 3, Nq, Nk, d)
+    scale = float(np.float32(d ** -0.5))
+    check(run(bd, q, k, v, scale), oracle.forward(q, k, v, scale)[0], v)
+
+
+@pytest.mark.parametrize("d,Nq", [(40, 1300), (36, 2500)])
+def test_two_query_tiles_per_cta(bd, d, Nq):
+    q, k, v = draw(d, 2, 8, Nq, 200, d)   # more tiles than SMs; the last CTA of a head has one
+    scale = float(np.float32(d ** -0.5))
+    ref = oracle.forward(q, k, v, scale)[0]
+    check(run(bd, q, k, v, scale), ref, v)
+    check(run(bd, q, k, v, scale, tokens_first=True), ref, v)
+
+
+@pytest.mark.parametrize("d", [40, 80, 160])
+@pytest.mark.parametrize("scale", [-0.4, 0.0])
+def test_negative_and_zero_scale(bd, d, scale):
+    q, k, v = draw(d, 1, 2, 150, 150, d)
+    check(run(bd, q, k, v, scale), oracle.forward(q, k, v, scale)[0], v, 1e-5)
+
+
+@pytest.mark.parametrize("d", [40, 80, 160])
+def test_scores_that_leave_the_anchor_behind(bd, d):
+    """The anchor is the first key tile's maximum; keys that grow 40-fold twice raise some rows' scores by hundreds, past the
+    2^64 at which a row is re-anchored (and lower others', whose weights vanish)."""
+    q, k, v = draw(d, 1, 2, 260, 260, d)
+    k[:, :, 100:] *= 40.0
+    k[:, :, 210:] *= 6.0
+    scale = float(np.float32(d ** -0.5))
+    ref = oracle.forward(q, k, v, scale)[0]
+    scores = np.einsum("bhid,bhjd->bhij", q.astype(np.float64), k.astype(np.float64)) * scale
+    assert (scores[..., 210:].max(-1) - scores[..., :32].max(-1)).max() > 64 * np.log(2.0)
+    check(run(bd, q, k, v, scale), ref, v, 1e-4)
