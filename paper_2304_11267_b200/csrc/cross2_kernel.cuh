@@ -224,7 +224,8 @@ cross2_attention_kernel(const __grid_constant__ Cross2ArgsT<NP> args) {
                 const int s = i % stages, g = gh - bh0;
                 const int pi = GROUPED ? gh / args.BH : 0, bh = gh - pi * args.BH;   // problem, head inside it
                 const Cross2Problem& pr = args.prob[pi];
-                const int bz = bh / args.lay.heads, hz = bh - bz * args.lay.heads;
+                int bz, hz;
+                split_head(args.lay, bh, bz, hz);
                 if (g != g_prev) {
                     // a new head: its K and V go into buffer g & 1 once the head two back has been consumed
                     if (g >= 2 && !mbar_wait(smem_u32(&bar_kv_empty[g & 1]), ((g >> 1) - 1) & 1, abort_p, args.status,
@@ -287,7 +288,8 @@ cross2_attention_kernel(const __grid_constant__ Cross2ArgsT<NP> args) {
                 // K and V of the CTA's first head, while the producer thread fetches the first Q tiles: a copy
                 // instruction holds its thread for several hundred clocks, and the first scores wait for all three.
                 const uint32_t bar = smem_u32(&bar_kv_full[0]);
-                const int bz0 = hb0 / args.lay.heads, hz0 = hb0 - bz0 * args.lay.heads;
+                int bz0, hz0;
+                split_head(args.lay, hb0, bz0, hz0);
                 mbar_arrive_expect_tx(bar, 2 * kv_bytes);
                 for (int ch = 0; ch < nch; ++ch)
                     tma_load_4d(kv_smem + ch * X2_KN * CHUNK_ROW_BYTES, &args.prob[prob0].tk, bar, ch * CHUNK_COLS, 0, hz0, bz0);
@@ -535,7 +537,8 @@ cross2_attention_kernel(const __grid_constant__ Cross2ArgsT<NP> args) {
                     int rows = args.Nq - tile * TILE_M;
                     if (rows > TILE_M) rows = TILE_M;
                     if (args.strided_rows) {   // rows past Nq are clipped by the hardware
-                        const int bz = bh / args.lay.heads, hz = bh - bz * args.lay.heads;
+                        int bz, hz;
+                        split_head(args.lay, bh, bz, hz);
                         tma_store_4d(&pr.tout_rows, stage, 0, tile * TILE_M, hz, bz);
                     } else {
                         bulk_store(pr.out + ((size_t)bh * args.Nq + (size_t)tile * TILE_M) * args.d, stage,

@@ -92,7 +92,8 @@ cross_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
     bool ok = true;
 
     if (tid == 0) {
-        const int bz = bh / args.lay.heads, hz = bh - bz * args.lay.heads;
+        int bz, hz;
+        split_head(args.lay, bh, bz, hz);
         mbar_arrive_expect_tx(bar_qk, (uint32_t)(nch * (TILE_M + kn) * CHUNK_ROW_BYTES));
         for (int ch = 0; ch < nch; ++ch)
             tma_load_4d(q_smem + ch * TILE_M * CHUNK_ROW_BYTES, &tmap_q, bar_qk, ch * CHUNK_COLS, row0, hz, bz);

@@ -88,7 +88,7 @@ __device__ __noinline__ void f4s_combine_pieces(const Fused4Args& args, int t, i
     for (int c = c_first; c <= c_last; ++c)
         l_all += ex2_approx(__ldcg(piece_of(c) + dpad * TILE_M) - m_all) * __ldcg(piece_of(c) + (dpad + 1) * TILE_M);
     const float inv = 1.f / l_all;
-    const int quad = unit % args.units_per_head, bh = unit / args.units_per_head;
+    const int bh = (int)fast_div((uint32_t)unit, args.by_units_per_head), quad = unit - bh * args.units_per_head;
     const int row = quad * args.tiles_per_cta * TILE_M + t * TILE_M + r;
     __half* orow = head_row(args.prob[prob_i].out, args.lay, bh, row);
     // 24 columns at a time (d is a multiple of 8), the loads of two pieces in flight together
@@ -156,7 +156,8 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     struct Barriers {
         uint64_t s_full[F4_TILES][F4S_BUFFERS], p_full[F4_TILES][F4S_BUFFERS];   // p_full: 4 arrivals, one per softmax warp
         uint64_t q_full[F4_TILES], pv_done[F4_TILES], o_final[F4_TILES];
-        uint64_t kv_full[F4_STAGES];
+        uint64_t k_first;                 // K of the first key tile, which the first scores need before anything of V
+        uint64_t kv_full[F4_STAGES];      // (the first key tile: its V)
         uint64_t buf_free[F4S_BUFFERS];   // SPLIT > 1: the products reading a buffer's weights are done
         uint64_t kv_empty[F4_STAGES];     // one commit per issuer: as many arrivals as the unit has query tiles
     };
@@ -169,6 +170,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     auto& bar_q_full = bars.q_full;
     auto& bar_pv_done = bars.pv_done;
     auto& bar_o_final = bars.o_final;
+    auto& bar_k_first = bars.k_first;
     auto& bar_kv_full = bars.kv_full;
     auto& bar_kv_empty = bars.kv_empty;
     auto& bar_buf_free = bars.buf_free;
@@ -188,10 +190,10 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     if (threadIdx.x == 0) pdl_launch_dependents();   // the next kernel of the stream may start its set-up
     const int n_kv_all = args.n_kv;
     if (threadIdx.x == 32) {   // the tensor maps are kernel parameters: their fetch need not wait for anything
-        const int p0 = args.shares ? 0 : (int)(blockIdx.x / args.n_units);
-        tma_prefetch_desc(&args.prob[p0].tq);
-        tma_prefetch_desc(&args.prob[p0].tk);
-        tma_prefetch_desc(&args.prob[p0].tv);
+        const Fused4Problem& p0 = args.prob[blockIdx.y];   // (shares: one row of CTAs)
+        tma_prefetch_desc(&p0.tq);
+        tma_prefetch_desc(&p0.tk);
+        tma_prefetch_desc(&p0.tv);
     }
     const int dpad = args.dpad;
     constexpr int nch = NCH;
@@ -222,35 +224,43 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
         mbar_init_fence();
         __syncwarp();
     };
-    // The scheduling warp (an otherwise idle control warp, all lanes in step) walks this CTA's steps: [w_begin, w_end)
-    // of the W = units x key tiles of a problem -- of every problem in turn when the launch deals shares out.
+    // The scheduling warp (an otherwise idle control warp, all lanes in step) publishes the CTA's segments.  Whole units: the
+    // grid says which one, (unit, problem) = (blockIdx.x, blockIdx.y).  Shares: it walks this CTA's steps [w_begin, w_end) of the
+    // W = units x key tiles of a problem, of every problem in turn.  (The 64-bit divisions of that walk, done by every thread
+    // in either mode, were 1500 of the 2500 clocks before the first copy was issued.)
     constexpr int SCHED_WARP = 21;
-    const int W = args.n_units * n_kv_all;                             // (the host keeps it below 2^31)
-    const int G = args.shares ? (int)gridDim.x : args.n_units;         // CTAs among which a problem's steps are dealt out
-    const int cta = args.shares ? (int)blockIdx.x : (int)(blockIdx.x % args.n_units);   // this CTA among them
-    const int w_begin = (int)((long long)cta * W / G), w_end = (int)((long long)(cta + 1) * W / G);
-    int sched_w = w_begin, sched_prob = args.shares ? 0 : (int)(blockIdx.x / args.n_units);
-    const int sched_prob_end = args.shares ? args.n_prob : sched_prob + 1;
+    int sched_w = 0, sched_w_end = 0, sched_w_begin = 0, sched_prob = 0;
     // publishes the next segment (or "none") and (re-)initialises the barriers for it
     auto next_segment = [&](bool again) {
-        if (!(sched_w < w_end)) {   // on to this CTA's share of the next problem
-            sched_w = w_begin;
-            ++sched_prob;
+        int unit, j0, n;
+        if (!args.shares) {
+            unit = blockIdx.x; j0 = 0; n = n_kv_all; sched_prob = blockIdx.y;
+        } else {
+            if (!again) {
+                const int W = args.n_units * n_kv_all, G = (int)gridDim.x;   // (the host keeps W below 2^31)
+                sched_w = sched_w_begin = (int)((long long)blockIdx.x * W / G);
+                sched_w_end = (int)((long long)(blockIdx.x + 1) * W / G);
+            }
+            if (!(sched_w < sched_w_end)) {   // on to this CTA's share of the next problem
+                sched_w = sched_w_begin;
+                ++sched_prob;
+            }
+            if (sched_prob >= args.n_prob || !(sched_w_begin < sched_w_end)) {
+                if (lane == 0) seg_desc[0] = 0;
+                return;
+            }
+            unit = sched_w / n_kv_all;
+            j0 = sched_w - unit * n_kv_all;
+            n = (sched_w_end - sched_w) < (n_kv_all - j0) ? (sched_w_end - sched_w) : (n_kv_all - j0);
+            sched_w += n;
         }
-        if (sched_prob >= sched_prob_end || !(w_begin < w_end)) {
-            if (lane == 0) seg_desc[0] = 0;
-            return;
-        }
-        const int unit = sched_w / n_kv_all, j0 = sched_w - unit * n_kv_all;
-        const int n = (w_end - sched_w) < (n_kv_all - j0) ? (w_end - sched_w) : (n_kv_all - j0);
-        const int quad = unit % args.units_per_head;
+        const int bh = (int)fast_div((uint32_t)unit, args.by_units_per_head), quad = unit - bh * args.units_per_head;
         int tiles = (args.Nq - quad * args.tiles_per_cta * TILE_M + TILE_M - 1) / TILE_M;
         if (tiles > args.tiles_per_cta) tiles = args.tiles_per_cta;
-        sched_w += n;
         if (lane == 0) {
             seg_desc[0] = 1; seg_desc[1] = sched_prob; seg_desc[2] = unit; seg_desc[3] = j0; seg_desc[4] = n;
             seg_desc[5] = tiles;
-            seg_desc[6] = !(sched_w < w_end) && sched_prob + 1 == sched_prob_end;
+            seg_desc[6] = !args.shares || (!(sched_w < sched_w_end) && sched_prob + 1 == args.n_prob);
         }
         init_barriers(tiles, again);
     };
@@ -266,9 +276,6 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    // Set-up (barriers, tensor memory) overlapped the tail of the previous kernel of the stream; global memory and
-    // every bounded wait come after it has completed.
-    pdl_wait();
     const uint32_t tmem_base = tmem_base_slot;
     // columns: the score buffers | O_0 .. O_{T-1} (SPLIT > 1: the parts' O_0 .. O_{SPLIT-1})
     const uint32_t tmem_o0 = tmem_base + (SPLIT > 1 ? args.split_buffers : args.tiles_per_cta + 1) * BN;
@@ -280,7 +287,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
         named_barrier(2 + t, TILE_M);                // everybody has read the box
         const int r = tid & (TILE_M - 1);
         if (r == 0) piece_ticket[t][3] = 0;
-        const long long u0 = (long long)unit * n_kv_all;
+        const long long u0 = (long long)unit * n_kv_all, W = (long long)args.n_units * n_kv_all, G = gridDim.x;
         const int c_first = (int)(((u0 + 1) * G - 1) / W), c_last = (int)(((u0 + n_kv_all) * G - 1) / W);
         if (ticket != c_last - c_first) return;
         __threadfence();
@@ -288,6 +295,18 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
         f4s_combine_pieces<BF>(args, t, r, prob_i, unit, c_first, c_last);
     };
 
+    // Every role's set-up (barriers, tensor memory, registers, what it reads of the parameters, whose first touch misses the
+    // constant cache: 700-1100 clocks of a role's first instructions) overlaps the tail of the previous kernel of the stream;
+    // global memory and every bounded wait come after that kernel has completed.
+    auto role_ready = [](int a, int b, int c) {
+        asm volatile("" ::"r"(a), "r"(b), "r"(c));   // computed by now
+        pdl_wait();
+    };
+    // ... and what the epilogue reads, 150 K clocks later
+    auto touch_output = [&](const Fused4Problem& pr) {
+        asm volatile("" ::"l"(pr.out), "r"(args.lay.heads), "r"(args.lay.ld), "l"(args.lay.head_stride), "l"(args.lay.batch_stride),
+                     "r"(args.lay.by_heads.m), "r"(args.lay.by_heads.shift), "r"(args.d), "r"(args.Nq));
+    };
     // One setmaxnreg site per kind, executed by whole warpgroups; the budget is the CTA's launch allocation.  The
     // control warps and the softmax warps each walk the CTA's segments in a loop of their own (the code behind a
     // setmaxnreg must be reachable from that one only) and meet at the CTA-wide barriers between segments.
@@ -298,7 +317,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     if (!seg_desc[0]) break;
     const int prob_i = seg_desc[1], unit = seg_desc[2], j0 = seg_desc[3], n_kv = seg_desc[4], T = seg_desc[5];
     const bool last_segment = seg_desc[6] != 0;
-    const int quad = unit % args.units_per_head, bh = unit / args.units_per_head;
+    const int bh = (int)fast_div((uint32_t)unit, args.by_units_per_head), quad = unit - bh * args.units_per_head;
     const Fused4Problem& pr = args.prob[prob_i];
     const int row_base = quad * args.tiles_per_cta * TILE_M;
     const int NB = SPLIT > 1 ? args.split_buffers : T + 1;   // score buffers in the rotation
@@ -307,7 +326,9 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
         if (elect_one()) {
             // In the order the issuers need them: Q_0 and the first key tile first (a tile of 80-byte rows costs the
             // TMA unit about 7 clocks per row, so the order decides when the first scores can start).
-            const int bz = bh / args.lay.heads, hz = bh - bz * args.lay.heads;
+            int bz, hz;
+            split_head(args.lay, bh, bz, hz);
+            role_ready(bz, hz, row_base);
             auto load_q = [&](int t) {
                 const uint32_t bar = smem_u32(&bar_q_full[t]);
                 mbar_arrive_expect_tx(bar, q_tile_bytes);
@@ -315,9 +336,18 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     tma_load_4d(q_smem + t * q_tile_bytes + ch * TILE_M * CHUNK_ROW_BYTES, &pr.tq, bar, ch * CHUNK_COLS,
                                 row_base + t * TILE_M, hz, bz);
             };
+            auto load_tile = [&](const CUtensorMap* map, uint32_t dst, uint32_t bar, int j) {
+                for (int ch = 0; ch < nch; ++ch)
+                    tma_load_4d(dst + ch * BN * CHUNK_ROW_BYTES, map, bar, ch * CHUNK_COLS, (j0 + j) * BN, hz, bz);
+            };
             load_q(0);
-            int s = 0, pe = 1;   // stage of key tile j; parity of the kv_empty phase that frees it (from j = stages on)
-            for (int j = 0; j < n_kv; ++j, ++s) {
+            mbar_arrive_expect_tx(smem_u32(&bar_k_first), kv_tile_bytes);
+            load_tile(&pr.tk, kv_smem, smem_u32(&bar_k_first), 0);
+            for (int t = 1; t < T; ++t) load_q(t);
+            mbar_arrive_expect_tx(smem_u32(&bar_kv_full[0]), kv_tile_bytes);
+            load_tile(&pr.tv, kv_smem + kv_tile_bytes, smem_u32(&bar_kv_full[0]), 0);
+            int s = 1, pe = 1;   // stage of key tile j; parity of the kv_empty phase that frees it (from j = stages on)
+            for (int j = 1; j < n_kv; ++j, ++s) {
                 if (s == stages) { s = 0; pe ^= 1; }
                 // (eight stages ahead of the issuers: it sleeps between polls, which is worth 1% of the call)
                 if (j >= stages && !mbar_wait_lazy(smem_u32(&bar_kv_empty[s]), pe, abort_p, args.status, SITE_G_EMPTY, j))
@@ -325,12 +355,8 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 const uint32_t k_dst = kv_smem + s * 2 * kv_tile_bytes, v_dst = k_dst + kv_tile_bytes;
                 const uint32_t bar = smem_u32(&bar_kv_full[s]);
                 mbar_arrive_expect_tx(bar, 2 * kv_tile_bytes);
-                for (int ch = 0; ch < nch; ++ch)
-                    tma_load_4d(k_dst + ch * BN * CHUNK_ROW_BYTES, &pr.tk, bar, ch * CHUNK_COLS, (j0 + j) * BN, hz, bz);
-                for (int ch = 0; ch < nch; ++ch)
-                    tma_load_4d(v_dst + ch * BN * CHUNK_ROW_BYTES, &pr.tv, bar, ch * CHUNK_COLS, (j0 + j) * BN, hz, bz);
-                if (j == 0)
-                    for (int t = 1; t < T; ++t) load_q(t);
+                load_tile(&pr.tk, k_dst, bar, j);
+                load_tile(&pr.tv, v_dst, bar, j);
             }
             // Another segment follows: the issuers' last commits on the ring (never waited for above) must have
             // landed before the barriers are initialised again.
@@ -397,6 +423,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 }
             };
 
+            role_ready(ksteps_s, (int)idesc_s, (int)idesc_o);
             if (SPLIT > 1) {
                 // One tile, NB score buffers: step j uses buffer j % NB.  A lone issuing thread needs about 1000 clocks
                 // per key tile (two waits, seven to nine MMAs, three commits) and would pace the kernel, so the work
@@ -410,10 +437,10 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     int b = 0, ph = 0;                 // buffer and its bar_buf_free phase
                     int sn = 0, pn = 0;                // stage and phase of the key tile whose scores are requested
                     for (int jn = 0; jn < n_kv && ok; ++jn) {
-                        ok = mbar_wait(smem_u32(&bar_kv_full[sn]), pn, abort_p, args.status, SITE_G_KV, jn);
-                        if (ok && jn >= NB) {          // the products of key tile jn - NB have read their weights
-                            ok = mbar_wait(smem_u32(&bar_buf_free[b]), ph, abort_p, args.status, SITE_G_PV, jn);
-                        }
+                        // (the buffer first: once product jn - NB has completed, V(0) has landed, which makes the parity wait
+                        // for the second filling of stage 0 sound)
+                        if (jn >= NB) ok = mbar_wait(smem_u32(&bar_buf_free[b]), ph, abort_p, args.status, SITE_G_PV, jn);
+                        ok = ok && mbar_wait(smem_u32(jn == 0 ? &bar_k_first : &bar_kv_full[sn]), pn, abort_p, args.status, SITE_G_KV, jn);
                         if (!ok) break;
                         tc_fence_after_sync();
                         issue_s(q_desc_own_split, 0, sn, b);
@@ -424,7 +451,8 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     int b = 0, ph = 0;
                     int sj = 0;                        // stage of key tile j
                     for (int j = 0; j < n_kv && ok; ++j) {
-                        ok = mbar_wait(smem_u32(&bar_p_full[0][b]), ph, abort_p, args.status, SITE_G_P, j);
+                        if (j == 0) ok = mbar_wait(smem_u32(&bar_kv_full[0]), 0, abort_p, args.status, SITE_G_KV, 0);
+                        ok = ok && mbar_wait_eager(smem_u32(&bar_p_full[0][b]), ph, abort_p, args.status, SITE_G_P, j);
                         if (!ok) break;
                         tc_fence_after_sync();
                         issue_o(j, sj, b);
@@ -437,7 +465,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     }
                 }
             }
-            bool ok = SPLIT == 1 && mbar_wait(smem_u32(&bar_kv_full[0]), 0, abort_p, args.status, SITE_G_KV, 0) &&
+            bool ok = SPLIT == 1 && mbar_wait(smem_u32(&bar_k_first), 0, abort_p, args.status, SITE_G_KV, 0) &&
                       mbar_wait(smem_u32(&bar_q_full[t]), 0, abort_p, args.status, SITE_G_Q, t);
             if (ok) {
                 // the first T+1 steps fill the buffers: step t (own tile, key tile 0) into buffer t; the last issuer
@@ -457,6 +485,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
             // warps); it requests step k + NB = (tn, jn) into the same buffer
             int b = t, ph = 0, jm = 0;
             const int jn_off = (t + 1 == T) ? 2 : 1;
+            if (ok) ok = mbar_wait(smem_u32(&bar_kv_full[0]), 0, abort_p, args.status, SITE_G_KV, 0);   // V of key tile 0
             int sj = 0;                                 // stage of key tile j
             int sn = jn_off % stages, pn = (jn_off / stages) & 1;   // stage and phase of key tile jn = j + jn_off
             for (int j = 0; j < n_kv && ok; ++j) {
@@ -497,7 +526,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     if (!seg_desc[0]) break;
     const int prob_i = seg_desc[1], unit = seg_desc[2], j0 = seg_desc[3], n_kv = seg_desc[4], T = seg_desc[5];
     const bool last_segment = seg_desc[6] != 0;
-    const int quad = unit % args.units_per_head, bh = unit / args.units_per_head;
+    const int bh = (int)fast_div((uint32_t)unit, args.by_units_per_head), quad = unit - bh * args.units_per_head;
     const Fused4Problem& pr = args.prob[prob_i];
     const int row_base = quad * args.tiles_per_cta * TILE_M;
     const int NB = SPLIT > 1 ? args.split_buffers : T + 1;   // score buffers in the rotation
@@ -515,9 +544,13 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 const float c2 = pr.scale_log2e;
                 float m_run = 0.f, l_run = 0.f;   // anchor and row sum over this part's keys
                 bool ok = true;
-                // NB is a multiple of SPLIT, so buffer b = j % NB always meets the same part: one consumer per barrier.
-                // The part's i-th key tile uses buffer (g + SPLIT i) % NB, phase ((g + SPLIT i) / NB) & 1.
+                // The part's i-th key tile j = g + SPLIT i uses buffer j % NB, phase (j / NB) & 1.  (Parts take turns at a buffer's
+                // barrier when NB is no multiple of SPLIT; the parity wait stays sound: the buffer's next scores need this
+                // tile's product, and its last ones, S(j - NB), completed before S(j - SPLIT), which this part has seen --
+                // NB >= SPLIT, and one thread's MMAs and commits complete in order.)
                 int b = g, ph = 0;
+                touch_output(pr);
+                role_ready(args.Nk, __float_as_int(c2), NB);
                 for (int j = g, i = 0; j < n_kv; j += SPLIT, ++i) {
                     const uint32_t tmem_s = tmem_base + b * BN + lane_off;
                     ok = mbar_wait(smem_u32(&bar_s_full[0][b]), ph, abort_p, args.status, SITE_G_S, j);
@@ -586,13 +619,10 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     l_run += tile_sum;
                     tmem_st32(tmem_s, packed);   // P(j) over the first columns of the buffer, whose scores sit in registers
                     tmem_wait_st();
-                    // every phase of the part's completion barrier is consumed in order, one own key tile late: the
-                    // product of key tile j - SPLIT has had SPLIT tiles' time to finish
-                    if (i > 0) {
-                        ok = mbar_wait(b_pvdone, (i - 1) & 1, abort_p, args.status, SITE_G_PV, j);
-                        ok = __all_sync(0xffffffffu, ok);
-                        if (!ok) break;
-                    }
+                    // (No phase of the part's completion barrier is waited for here.  The rare path above waits for the product of
+                    // the part's previous key tile; the one before that is complete by then -- there are at most two
+                    // buffers per part, so its buffer, or one freed behind it, holds the scores this thread has --, which keeps
+                    // that parity wait from being two phases behind.)
                     tc_fence_before_sync();
                     if (lane == 0) mbar_arrive(smem_u32(&bar_p_full[0][b]));
                     b += SPLIT;
@@ -618,9 +648,9 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     const float inv = 1.f / l_all;
 #pragma unroll
                     for (int p2 = 0; p2 < SPLIT; ++p2) f[p2] *= inv;
-                    const int row = row_base + r;
-                    __half* orow = head_row(pr.out, args.lay, bh, row);
-                    // the column groups of 16 are shared out among the parts; a thread reads its row of every O_p
+                    // The column groups of 16 are shared out among the parts, a thread reads its row of every O_p; the rows meet in
+                    // the query tile's shared memory (no score needs it any more) and leave as whole lines.
+                    const uint32_t pitch = (uint32_t)args.d * 2, rows = q_smem + (warp & 3) * 32 * pitch;
                     for (int cg = g; cg < (dpad >> 4); cg += SPLIT) {
                         float acc[16];
 #pragma unroll
@@ -639,10 +669,13 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                         lo.z = pack_16x2<BF>(acc[4], acc[5]);   lo.w = pack_16x2<BF>(acc[6], acc[7]);
                         hi.x = pack_16x2<BF>(acc[8], acc[9]);   hi.y = pack_16x2<BF>(acc[10], acc[11]);
                         hi.z = pack_16x2<BF>(acc[12], acc[13]); hi.w = pack_16x2<BF>(acc[14], acc[15]);
-                        if (row < args.Nq) {
-                            if (cg * 16 + 8 <= args.d) *reinterpret_cast<uint4*>(orow + cg * 16) = lo;
-                            if (cg * 16 + 16 <= args.d) *reinterpret_cast<uint4*>(orow + cg * 16 + 8) = hi;
-                        }
+                        st_shared_v4(rows + lane * pitch + cg * 32, lo);
+                        if (cg * 16 + 16 <= args.d) st_shared_v4(rows + lane * pitch + cg * 32 + 16, hi);
+                    }
+                    named_barrier(2, SPLIT * 128);
+                    if (g == 0) {
+                        const int at = row_base + (warp & 3) * 32;
+                        store_staged_rows(head_row(pr.out, args.lay, bh, at), args.lay.ld, rows, args.d >> 3, min(32, args.Nq - at), lane);
                     }
                 }
             }
@@ -652,6 +685,8 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
             const uint32_t tmem_o = tmem_o0 + t * dpad + lane_off;
             const uint32_t b_pvdone = smem_u32(&bar_pv_done[t]);
             const float c2 = pr.scale_log2e;
+            touch_output(pr);
+            role_ready(args.Nk, __float_as_int(c2), NB);
             float m_run = 0.f;   // anchor of the exponent: a bound on the running max, times scale*log2(e)
             float l_run = 0.f;   // running sum of p (relative to m_run)
             bool ok = true;
@@ -748,11 +783,11 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
             // (the last phase of the product barrier, never consumed above: nothing of this segment is in flight after it)
             if (ok) ok = mbar_wait(b_pvdone, (n_kv - 1) & 1, abort_p, args.status, SITE_G_PV, n_kv);
             ok = __all_sync(0xffffffffu, ok);
-            const int row = row_base + t * TILE_M + r;
-            __half* orow = head_row(pr.out, args.lay, bh, row);
             if (ok && j0 == 0 && n_kv == n_kv_all) {   // all key tiles of the unit: no pieces to combine
                 tc_fence_after_sync();
                 const float inv = 1.f / l_run;
+                // rows to the query tile's shared memory (no score needs it any more), and out as whole lines
+                const uint32_t pitch = (uint32_t)args.d * 2, rows = q_smem + t * q_tile_bytes + (warp & 3) * 32 * pitch;
                 for (int g = 0; g < (dpad >> 4); ++g) {
                     uint32_t x[16];
                     tmem_ld16(tmem_o + g * 16, x);
@@ -766,11 +801,13 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     hi.y = pack_16x2<BF>(__uint_as_float(x[10]) * inv, __uint_as_float(x[11]) * inv);
                     hi.z = pack_16x2<BF>(__uint_as_float(x[12]) * inv, __uint_as_float(x[13]) * inv);
                     hi.w = pack_16x2<BF>(__uint_as_float(x[14]) * inv, __uint_as_float(x[15]) * inv);
-                    if (row < args.Nq) {
-                        if (g * 16 + 8 <= args.d) *reinterpret_cast<uint4*>(orow + g * 16) = lo;
-                        if (g * 16 + 16 <= args.d) *reinterpret_cast<uint4*>(orow + g * 16 + 8) = hi;
-                    }
+                    st_shared_v4(rows + lane * pitch + g * 32, lo);
+                    if (g * 16 + 16 <= args.d) st_shared_v4(rows + lane * pitch + g * 32 + 16, hi);
                 }
+                __syncwarp();
+                const int at = row_base + t * TILE_M + (warp & 3) * 32;
+                store_staged_rows(head_row(pr.out, args.lay, bh, at), args.lay.ld, rows, args.d >> 3, min(32, args.Nq - at), lane);
+                if (!last_segment) fence_proxy_async_smem();   // the next segment's Q comes to the same place
             } else if (ok) {
                 // ---- a piece of the unit's key range: (O, anchor, row sum) of the thread's row to the scratch.  A CTA
                 // has at most two pieces per problem (its first segment may begin and its last may end inside a
@@ -805,6 +842,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 16 && lane == 0 && abort_flag) {
+        mbar_drain(smem_u32(&bar_k_first), 0);
         for (int s = 0; s < F4_STAGES; ++s) mbar_drain(smem_u32(&bar_kv_full[s]), 0);
     }
     __syncthreads();

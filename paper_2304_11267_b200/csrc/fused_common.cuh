@@ -47,6 +47,7 @@ struct Fused4Args {
     int nch;             // 64-column chunks per row (1..3)
     int stages;          // K/V ring depth (2..8)
     int split_buffers;   // split variant only: score buffers of the lone tile (2..5)
+    FastDiv by_units_per_head;
     int* status;
     // pieces of units whose key tiles are cut between CTAs (shares only): per problem two slots of part_slot_floats
     // per CTA, each [tile][dpad + 2 columns: O, anchor, row sum][128 rows]; arrival counters per (problem, unit,

@@ -201,6 +201,7 @@ static cudaError_t raise_layout_kernels() {
     if (e == cudaSuccess) e = raise_smem_limit(fused4s_attention_kernel<F4S_POLY_PER8, 1, 4, BF>, F4S_SMEM_BUDGET + 1024);
     if (e == cudaSuccess) e = raise_smem_limit(fused4s_attention_kernel<F4S_POLY_PER8, 1, 2, BF>, F4S_SMEM_BUDGET + 1024);
     if (e == cudaSuccess) e = raise_smem_limit(fused4s_attention_kernel<F4S_POLY_PER8, 2, 2, BF>, F4S_SMEM_BUDGET + 1024);
+    if (e == cudaSuccess) e = raise_smem_limit(fused4s_attention_kernel<F4S_POLY_PER8, 2, 3, BF>, F4S_SMEM_BUDGET + 1024);
     if (e == cudaSuccess) e = raise_smem_limit(fused4s_attention_kernel<F4S_POLY_PER8, 3, 2, BF>, F4S_SMEM_BUDGET + 1024);
     return e;
 }
@@ -210,12 +211,12 @@ template <bool BF>
 static cudaError_t check_register_pools(sd_attn_handle* h) {
     cudaFuncAttributes fa;
     cudaError_t e = cudaSuccess;
-    const void* f4s[8] = {(const void*)fused4s_attention_kernel<F4S_POLY_PER8, 1, 1, BF>, (const void*)fused4s_attention_kernel<0, 1, 1, BF>,
+    const void* f4s[9] = {(const void*)fused4s_attention_kernel<F4S_POLY_PER8, 1, 1, BF>, (const void*)fused4s_attention_kernel<0, 1, 1, BF>,
                           (const void*)fused4s_attention_kernel<0, 2, 1, BF>, (const void*)fused4s_attention_kernel<0, 3, 1, BF>,
                           (const void*)fused4s_attention_kernel<F4S_POLY_PER8, 1, 4, BF>, (const void*)fused4s_attention_kernel<F4S_POLY_PER8, 1, 2, BF>,
-                          (const void*)fused4s_attention_kernel<F4S_POLY_PER8, 2, 2, BF>,
+                          (const void*)fused4s_attention_kernel<F4S_POLY_PER8, 2, 2, BF>, (const void*)fused4s_attention_kernel<F4S_POLY_PER8, 2, 3, BF>,
                           (const void*)fused4s_attention_kernel<F4S_POLY_PER8, 3, 2, BF>};
-    for (int i = 0; i < 8 && e == cudaSuccess; ++i) {
+    for (int i = 0; i < 9 && e == cudaSuccess; ++i) {
         e = cudaFuncGetAttributes(&fa, f4s[i]);
         if (e == cudaSuccess && F4_THREADS * fa.numRegs < 512 * F4S_SOFTMAX_REGS + 256 * F4S_CONTROL_REGS) h->fused4s_ok = 0;
     }
@@ -417,6 +418,7 @@ static HeadLayout head_layout(int heads, int BH, int N, int d) {
     } else {
         l.heads = BH; l.ld = d; l.head_stride = (long long)N * d; l.batch_stride = (long long)BH * N * d;
     }
+    l.by_heads = make_fast_div((uint32_t)l.heads);
     return l;
 }
 
@@ -644,6 +646,8 @@ static void dispatch_fused4s(sd_attn_handle* h, int split, const Fused4Args& a, 
         launch_overlapped(h, fused4s_attention_kernel<F4S_POLY_PER8, 1, 4, BF>, grid, block, smem, stream, a);
     else if (split == 2 && a.nch == 1)
         launch_overlapped(h, fused4s_attention_kernel<F4S_POLY_PER8, 1, 2, BF>, grid, block, smem, stream, a);
+    else if (split == 3 && a.nch == 2)
+        launch_overlapped(h, fused4s_attention_kernel<F4S_POLY_PER8, 2, 3, BF>, grid, block, smem, stream, a);
     else if (split == 2 && a.nch == 2)
         launch_overlapped(h, fused4s_attention_kernel<F4S_POLY_PER8, 2, 2, BF>, grid, block, smem, stream, a);
     else if (split == 2 && a.nch == 3)
@@ -744,6 +748,7 @@ static int launch_fused_group(sd_attn_handle* h, const Problem* ps, int n) {
     a.part = h->part;
     a.part_count = h->part_count;
     a.part_slot_floats = plan.slot_floats;
+    a.by_units_per_head = make_fast_div((uint32_t)plan.units_per_head);
     const int q_tile_bytes = a.nch * TILE_M * CHUNK_ROW_BYTES, stage_bytes = 2 * a.nch * F4_BN * CHUNK_ROW_BYTES;
     // one chunk per row: the kernel lays out four tile slots and eight stages whatever tiles_per_cta is (192 KB)
     const int tile_slots = a.nch == 1 ? F4_TILES : a.tiles_per_cta;
@@ -762,17 +767,21 @@ static int launch_fused_group(sd_attn_handle* h, const Problem* ps, int n) {
         fp.scale_log2e = fabsf(pi.scale) * LOG2E;
         fp.negate = pi.scale < 0.f;
     }
-    dim3 grid(plan.shares ? plan.grid : plan.n_units * n), block(F4_THREADS);
-    // One tile per unit: its key tiles are dealt out among 4 or 2 warpgroups (parts), each with an accumulator of its
-    // own in tensor memory next to the score buffers, whose number is a multiple of the parts (a buffer then always
-    // meets the same part) and smaller than the K/V ring (a buffer ahead is a key tile ahead).
+    dim3 grid(plan.shares ? plan.grid : plan.n_units, plan.shares ? 1 : n), block(F4_THREADS);
+    // One tile per unit: its key tiles are dealt out among 4, 3 or 2 warpgroups (parts), each with an accumulator of its own in
+    // tensor memory, next to as many score buffers as fit behind them (five at most): a part then finds its next scores
+    // requested while it still works on the last ones.
     int split = 1;
     a.split_buffers = 2;
     if (a.tiles_per_cta == 1 && h->opt.fused_split != 1) {
-        split = 4 * F4_BN + 4 * a.dpad <= 512 ? 4 : 2;
+        split = 4 * F4_BN + 4 * a.dpad <= 512 ? 4 : 3 * F4_BN + 3 * a.dpad <= 512 && a.nch == 2 ? 3 : 2;
         if (h->opt.fused_split == 2) split = 2;
-        a.split_buffers = (4 * F4_BN + split * a.dpad <= 512 && a.stages >= 5) ? 4 : 2;
-        if (a.split_buffers < split || 2 * F4_BN + 2 * a.dpad > 512) split = 1;   // (no room: d > 192)
+        a.split_buffers = (512 - split * a.dpad) / F4_BN;
+        // (and no more than two per part: a part may wait for its last product only when the one before it has completed)
+        if (a.split_buffers > 2 * split) a.split_buffers = 2 * split;
+        if (a.split_buffers > F4S_BUFFERS) a.split_buffers = F4S_BUFFERS;
+        if (a.split_buffers > a.stages) a.split_buffers = a.stages;
+        if (a.split_buffers < split) split = 1;   // (cannot happen for d <= SD_ATTN_MAX_D)
     }
     if (p.bf16)
         dispatch_fused4s<true>(h, split, a, grid, block, smem, p.stream);

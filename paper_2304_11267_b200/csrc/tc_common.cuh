@@ -185,6 +185,19 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, uint
         "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(x), "r"(y), "r"(z)
         : "memory");
 }
+// q = n / d for 0 <= n < 2^31 by one multiplication: m = floor(2^(31 + l) / d) + 1 with l = ceil(log2 d) exceeds the exact
+// quotient's multiplier by less than 2^l / d parts, which the floor absorbs for every such n.
+struct FastDiv {
+    uint32_t d, m, shift;
+};
+__host__ inline FastDiv make_fast_div(uint32_t d) {
+    uint32_t l = 0;
+    while ((1ull << l) < d) ++l;
+    return {d, (uint32_t)((1ull << (31 + l)) / d + 1), 31 + l};
+}
+__device__ __forceinline__ uint32_t fast_div(uint32_t n, const FastDiv& f) {
+    return (uint32_t)(((uint64_t)n * f.m) >> f.shift);
+}
 // Where the heads of a tensor lie.  A (batch, head) index bh splits into batch = bh / heads and head = bh % heads;
 // row r of that head starts batch * batch_stride + head * head_stride + r * ld elements into the tensor.
 // Head-major [B][H][N][d] is {heads = B*H, ld = d, head_stride = N*d} (the batch index is always 0); token-major
@@ -195,10 +208,16 @@ struct HeadLayout {
     int ld;
     long long head_stride;
     long long batch_stride;
+    FastDiv by_heads;
 };
+__device__ __forceinline__ void split_head(const HeadLayout& lay, int bh, int& batch, int& head) {
+    batch = (int)fast_div((uint32_t)bh, lay.by_heads);
+    head = bh - batch * lay.heads;
+}
 template <typename T>
 __device__ __forceinline__ T* head_row(T* base, const HeadLayout& lay, int bh, int row) {
-    const int batch = bh / lay.heads, head = bh - batch * lay.heads;
+    int batch, head;
+    split_head(lay, bh, batch, head);
     return base + batch * lay.batch_stride + head * lay.head_stride + (long long)row * lay.ld;
 }
 // 4-D tile load global -> shared: (x = innermost element, y = row, z = head, w = batch); x as for the 3-D load.
@@ -209,6 +228,21 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint
         " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w)
         : "memory");
+}
+// A warp's rows of 16-bit results, staged densely in shared memory by their threads (row r at rows + r * pieces * 16), to
+// global memory as whole lines: `out_row` is row 0, a row `pieces` 16-byte pieces, the next one ld elements on.  (Each thread
+// storing its own row costs an LSU wavefront per thread and piece: 2500 clocks for four tiles of 128 rows at d = 40.)
+__device__ __forceinline__ void store_staged_rows(void* out_row, int ld, uint32_t rows, int pieces, int n_rows, int lane) {
+    uint4* out = reinterpret_cast<uint4*>(out_row);
+    if (ld == pieces * 8) {   // head-major: one contiguous run
+#pragma unroll 4
+        for (int i = lane; i < n_rows * pieces; i += 32) out[i] = ld_shared_v4(rows + i * 16);
+    } else {   // a row's pieces by neighbouring lanes
+        const int wide = pieces > 16 ? 32 : pieces > 8 ? 16 : 8, step = 32 / wide, p = lane & (wide - 1);
+        if (p < pieces)
+#pragma unroll 4
+            for (int r = lane / wide; r < n_rows; r += step) out[(long long)r * (ld >> 3) + p] = ld_shared_v4(rows + (r * pieces + p) * 16);
+    }
 }
 // Untiled bulk copy global -> shared, completion counted in bytes on `bar`.  Both addresses 16-byte aligned, the
 // size a multiple of 16 bytes.
@@ -408,19 +442,6 @@ __host__ __device__ constexpr uint32_t idesc_f16(int m, int n, bool a_mn_major, 
 }
 
 // ------------------------------------------------------------------ small math helpers
-// q = n / d for 0 <= n < 2^31 by one multiplication: m = floor(2^(31 + l) / d) + 1 with l = ceil(log2 d) exceeds the exact
-// quotient's multiplier by less than 2^l / d parts, which the floor absorbs for every such n.
-struct FastDiv {
-    uint32_t d, m, shift;
-};
-__host__ inline FastDiv make_fast_div(uint32_t d) {
-    uint32_t l = 0;
-    while ((1ull << l) < d) ++l;
-    return {d, (uint32_t)((1ull << (31 + l)) / d + 1), 31 + l};
-}
-__device__ __forceinline__ uint32_t fast_div(uint32_t n, const FastDiv& f) {
-    return (uint32_t)(((uint64_t)n * f.m) >> f.shift);
-}
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

@@ -1,0 +1,46 @@
+"""The lone query tile's variants of the single-pass kernel: two, three and four parts, score buffers that are no multiple of
+the parts, a K/V ring as deep as the buffers, against the oracle (tolerances of test_gpu_parity.py)."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import test_gpu_parity as parity  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def bd():
+    from paper_2304_11267_b200 import binding
+    from paper_2304_11267_b200 import build
+    build.build()
+    binding.load()
+    return binding
+
+
+# head dims at the edges of the parts (64 -> 4, 72..96 -> 3, 104..160 -> 2); key tiles from one per launch to several times
+# round the buffers and the ring (3 at d = 160), the last one ragged or not
+@pytest.mark.parametrize("d", [8, 40, 64, 72, 80, 96, 104, 128, 136, 160])
+@pytest.mark.parametrize("Nk", [129, 192, 257, 320, 400, 1000])
+def test_parts_buffers_and_ring(bd, d, Nk):
+    a = bd.Attention()
+    q, k, v = parity.rand_qkv(d + Nk, 1, 3, 150, Nk, d, qmult=2.0)
+    scale = float(np.float32(d ** -0.5))
+    ref, _, _ = oracle.forward(q, k, v, scale)
+    parity.check(parity.run(a, bd, bd.MODE_AUTO, q, k, v, scale), ref, v, what="d=%d Nk=%d" % (d, Nk))
+    a.close()
+
+
+@pytest.mark.parametrize("d", [40, 80, 160])
+def test_parts_that_re_anchor_at_every_key_tile(bd, d):
+    """Scores that rise along the keys: the rescale of a part's accumulator waits for its own last product."""
+    a = bd.Attention()
+    q, k, v = parity.rand_qkv(d, 1, 4, 128, 1024, d)
+    k = (k.astype(np.float32) * np.repeat(np.geomspace(0.1, 12.0, 16), 64)[None, None, :, None].astype(np.float32)).astype(np.float16)
+    scale = float(np.float32(d ** -0.5))
+    ref, _, _ = oracle.forward(q, k, v, scale)
+    for _ in range(5):
+        parity.check(parity.run(a, bd, bd.MODE_FUSED, q, k, v, scale), ref, v, what="rising d=%d" % d)
+    a.close()
