@@ -31,7 +31,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "cross_kernel.cuh"  // TILE_M, CHUNK_COLS, CHUNK_ROW_BYTES
+#include "cross_common.cuh"  // TILE_M, CHUNK_COLS, CHUNK_ROW_BYTES
 #include "tc_common.cuh"
 
 namespace sd_attn {

@@ -2,7 +2,7 @@
 // text tokens), any head dim up to 160.  Memory-bound: per tile of 128 query rows it reads Q and writes O
 // once; K and V (12-50 KB per head) stay in L2.
 //
-// cross_kernel.cuh runs one tile per CTA, start to finish, and leans on CTA-level overlap; its launch,
+// cross1_kernel.cuh runs one tile per CTA, start to finish, and leans on CTA-level overlap; its launch,
 // tensor-memory allocation, descriptor fetch and drain are paid per tile and HBM sits idle meanwhile.
 // Here ONE CTA per SM walks a contiguous range of (head, tile) items with every stage overlapped:
 //   warps 0 .. 4*NWG-1   NWG softmax groups; group w owns items w, w+NWG, ... (thread = query row): exp2, row sum,
@@ -31,7 +31,7 @@
 #pragma once
 #include <cuda.h>
 
-#include "cross_kernel.cuh"  // TILE_M, CHUNK_COLS, CHUNK_ROW_BYTES
+#include "cross_common.cuh"  // TILE_M, CHUNK_COLS, CHUNK_ROW_BYTES
 #include "softmax_math.cuh"
 #include "tc_common.cuh"
 

@@ -30,7 +30,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "cross_kernel.cuh"   // TILE_M
+#include "cross_common.cuh"  // TILE_M
 #include "softmax_math.cuh"
 #include "tc_common.cuh"
 

@@ -650,7 +650,8 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     for (int p2 = 0; p2 < SPLIT; ++p2) f[p2] *= inv;
                     // The column groups of 16 are shared out among the parts, a thread reads its row of every O_p; the rows meet in
                     // the query tile's shared memory (no score needs it any more) and leave as whole lines.
-                    const uint32_t pitch = (uint32_t)args.d * 2, rows = q_smem + (warp & 3) * 32 * pitch;
+                    const int pieces = args.d >> 3, swz = stage_swizzle(lane, pieces);
+                    const uint32_t rows = q_smem + (warp & 3) * 32 * pieces * 16, own = rows + lane * pieces * 16;
                     for (int cg = g; cg < (dpad >> 4); cg += SPLIT) {
                         float acc[16];
 #pragma unroll
@@ -669,13 +670,13 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                         lo.z = pack_16x2<BF>(acc[4], acc[5]);   lo.w = pack_16x2<BF>(acc[6], acc[7]);
                         hi.x = pack_16x2<BF>(acc[8], acc[9]);   hi.y = pack_16x2<BF>(acc[10], acc[11]);
                         hi.z = pack_16x2<BF>(acc[12], acc[13]); hi.w = pack_16x2<BF>(acc[14], acc[15]);
-                        st_shared_v4(rows + lane * pitch + cg * 32, lo);
-                        if (cg * 16 + 16 <= args.d) st_shared_v4(rows + lane * pitch + cg * 32 + 16, hi);
+                        st_shared_v4(own + ((2 * cg) ^ swz) * 16, lo);
+                        if (cg * 16 + 16 <= args.d) st_shared_v4(own + ((2 * cg + 1) ^ swz) * 16, hi);
                     }
                     named_barrier(2, SPLIT * 128);
                     if (g == 0) {
                         const int at = row_base + (warp & 3) * 32;
-                        store_staged_rows(head_row(pr.out, args.lay, bh, at), args.lay.ld, rows, args.d >> 3, min(32, args.Nq - at), lane);
+                        store_staged_rows(head_row(pr.out, args.lay, bh, at), args.lay, rows, args.d >> 3, min(32, args.Nq - at), lane);
                     }
                 }
             }
@@ -787,7 +788,8 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 tc_fence_after_sync();
                 const float inv = 1.f / l_run;
                 // rows to the query tile's shared memory (no score needs it any more), and out as whole lines
-                const uint32_t pitch = (uint32_t)args.d * 2, rows = q_smem + t * q_tile_bytes + (warp & 3) * 32 * pitch;
+                const int pieces = args.d >> 3, swz = stage_swizzle(lane, pieces);
+                const uint32_t rows = q_smem + t * q_tile_bytes + (warp & 3) * 32 * pieces * 16, own = rows + lane * pieces * 16;
                 for (int g = 0; g < (dpad >> 4); ++g) {
                     uint32_t x[16];
                     tmem_ld16(tmem_o + g * 16, x);
@@ -801,12 +803,12 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     hi.y = pack_16x2<BF>(__uint_as_float(x[10]) * inv, __uint_as_float(x[11]) * inv);
                     hi.z = pack_16x2<BF>(__uint_as_float(x[12]) * inv, __uint_as_float(x[13]) * inv);
                     hi.w = pack_16x2<BF>(__uint_as_float(x[14]) * inv, __uint_as_float(x[15]) * inv);
-                    st_shared_v4(rows + lane * pitch + g * 32, lo);
-                    if (g * 16 + 16 <= args.d) st_shared_v4(rows + lane * pitch + g * 32 + 16, hi);
+                    st_shared_v4(own + ((2 * g) ^ swz) * 16, lo);
+                    if (g * 16 + 16 <= args.d) st_shared_v4(own + ((2 * g + 1) ^ swz) * 16, hi);
                 }
                 __syncwarp();
                 const int at = row_base + t * TILE_M + (warp & 3) * 32;
-                store_staged_rows(head_row(pr.out, args.lay, bh, at), args.lay.ld, rows, args.d >> 3, min(32, args.Nq - at), lane);
+                store_staged_rows(head_row(pr.out, args.lay, bh, at), args.lay, rows, args.d >> 3, min(32, args.Nq - at), lane);
                 if (!last_segment) fence_proxy_async_smem();   // the next segment's Q comes to the same place
             } else if (ok) {
                 // ---- a piece of the unit's key range: (O, anchor, row sum) of the thread's row to the scratch.  A CTA

@@ -2,7 +2,7 @@
 #pragma once
 #include <cuda.h>
 
-#include "cross_kernel.cuh"  // TILE_M, CHUNK_COLS, CHUNK_ROW_BYTES
+#include "cross_common.cuh"  // TILE_M, CHUNK_COLS, CHUNK_ROW_BYTES
 #include "softmax_math.cuh"
 #include "tc_common.cuh"
 

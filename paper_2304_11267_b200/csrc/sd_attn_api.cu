@@ -16,8 +16,8 @@
 #include "../../include/sd_geglu.h"
 #include "../../include/sd_groupnorm.h"
 #include "../../include/sd_winograd.h"
-#include "cross_kernel.cuh"
 #include "conv_direct_kernel.cuh"
+#include "cross1_kernel.cuh"
 #include "cross2_kernel.cuh"
 #include "geglu_kernel.cuh"
 #include "groupnorm_kernel.cuh"
@@ -185,9 +185,24 @@ static void destroy_host_overlap(sd_attn_handle* h) {   // the handle was calloc
 }
 
 // The kernels AUTO selects exist for binary16 and for bfloat16 tensors (BF); each needs its shared-memory limit raised.
+template <bool BF, int KN, int NP>
+static cudaError_t raise_cross1() {
+    cudaError_t e = raise_smem_limit(cross1_attention_kernel<KN, 1, false, BF, NP>, x1_smem_bytes(1, KN));
+    if (e == cudaSuccess) e = raise_smem_limit(cross1_attention_kernel<KN, 2, false, BF, NP>, x1_smem_bytes(2, KN));
+    if (e == cudaSuccess) e = raise_smem_limit(cross1_attention_kernel<KN, 3, false, BF, NP>, x1_smem_bytes(3, KN));
+    if constexpr (KN <= 80) {
+        if (e == cudaSuccess) e = raise_smem_limit(cross1_attention_kernel<KN, 1, true, BF, NP>, x1_smem_bytes(1, KN));
+    }
+    return e;
+}
 template <bool BF>
 static cudaError_t raise_layout_kernels() {
-    cudaError_t e = raise_smem_limit(cross_attention_kernel<BF>, cross_smem_bytes(3, 128));
+    cudaError_t e = raise_cross1<BF, 64, 1>();
+    if (e == cudaSuccess) e = raise_cross1<BF, 80, 1>();
+    if (e == cudaSuccess) e = raise_cross1<BF, 128, 1>();
+    if (e == cudaSuccess) e = raise_cross1<BF, 64, X1_GROUP_MAX>();
+    if (e == cudaSuccess) e = raise_cross1<BF, 80, X1_GROUP_MAX>();
+    if (e == cudaSuccess) e = raise_cross1<BF, 128, X1_GROUP_MAX>();
     if (e == cudaSuccess) e = raise_smem_limit(cross2_attention_kernel<2, BF, 1>, X2_SMEM_BUDGET + 1024);
     if (e == cudaSuccess) e = raise_smem_limit(cross2_attention_kernel<3, BF, 1>, X2_SMEM_BUDGET + 1024);
     if (e == cudaSuccess) e = raise_smem_limit(cross2_attention_kernel<4, BF, 1>, X2_SMEM_BUDGET + 1024);
@@ -419,6 +434,7 @@ static HeadLayout head_layout(int heads, int BH, int N, int d) {
         l.heads = BH; l.ld = d; l.head_stride = (long long)N * d; l.batch_stride = (long long)BH * N * d;
     }
     l.by_heads = make_fast_div((uint32_t)l.heads);
+    l.piece_inv = d >= 8 ? 65536u / (uint32_t)(d / 8) + 1u : 0u;
     return l;
 }
 
@@ -608,35 +624,75 @@ static int launch_cross2_group(sd_attn_handle* h, const Problem* ps, int n) {
     return n == 1 ? launch_cross2_np<1>(h, ps, 1) : launch_cross2_np<X2_GROUP_MAX>(h, ps, n);
 }
 
-static int launch_cross2(sd_attn_handle* h, const Problem& p) { return launch_cross2_group(h, &p, 1); }
+template <int KN, int NCH, bool DENSE, int NP>
+static cudaError_t launch_cross1_as(sd_attn_handle* h, const Problem& p, int n, const Cross1ArgsT<NP>& a) {
+    const dim3 grid((p.Nq + a.tile_rows - 1) / a.tile_rows, p.BH, n), block(X1_THREADS);
+    const size_t smem = x1_smem_bytes(NCH, KN);
+    return p.bf16 ? launch_overlapped(h, cross1_attention_kernel<KN, NCH, DENSE, true, NP>, grid, block, smem, p.stream, a)
+                  : launch_overlapped(h, cross1_attention_kernel<KN, NCH, DENSE, false, NP>, grid, block, smem, p.stream, a);
+}
 
-static int launch_cross(sd_attn_handle* h, const Problem& p) {
-    if (cross2_supports(p.Nk, p.d) && !h->opt.cross_one_tile) return launch_cross2(h, p);
-    CrossArgs a;
-    a.out = (__half*)p.out;
+// One tile per CTA, for `n` problems of ONE shape (BH, Nq, Nk, d, layout, dtype alike): one launch.
+template <int NP>
+static int launch_cross1_np(sd_attn_handle* h, const Problem* ps, int n) {
+    const Problem& p = ps[0];
+    const int kn = x1_key_tile(p.Nk), nch = (p.d + CHUNK_COLS - 1) / CHUNK_COLS;
+    const bool dense = x1_dense(p.d, kn, p.heads == 0);
+    Cross1ArgsT<NP> a;
+    a.tmem_cols = x1_tmem_cols(kn, (p.d + 15) / 16 * 16);
+    // 64-row tiles when they fit the GPU at once: as many CTAs per SM as tensor memory and shared memory take, four at most
+    int resident = 512 / a.tmem_cols;
+    const int by_smem = (int)((size_t)227 * 1024 / (x1_smem_bytes(nch, kn) + 1024));
+    if (by_smem < resident) resident = by_smem;
+    if (resident > 4) resident = 4;
+    a.tile_rows = (long long)((p.Nq + 63) / 64) * p.BH <= (long long)resident * h->sm_count ? 64 : TILE_M;
+    for (int i = 0; i < n; ++i) {
+        const Problem& pi = ps[i];
+        Cross1Problem& c = a.prob[i];
+        c.q = (const __half*)pi.q; c.k = (const __half*)pi.k; c.v = (const __half*)pi.v; c.out = (__half*)pi.out;
+        if (!dense) {
+            int rc = make_tmap(h, &c.tq, pi.q, pi.BH, pi.Nq, pi.d, a.tile_rows, pi.heads, pi.bf16);
+            if (rc == SD_ATTN_OK) rc = make_tmap(h, &c.tk, pi.k, pi.BH, pi.Nk, pi.d, kn, pi.heads, pi.bf16);
+            if (rc == SD_ATTN_OK) rc = make_tmap(h, &c.tv, pi.v, pi.BH, pi.Nk, pi.d, kn, pi.heads, pi.bf16);
+            if (rc != SD_ATTN_OK) return rc;
+        }
+        c.scale_log2e = fabsf(pi.scale) * LOG2E;
+        c.negate = pi.scale < 0.f;
+    }
     a.lay = head_layout(p.heads, p.BH, p.Nq, p.d);
     a.Nq = p.Nq; a.Nk = p.Nk; a.d = p.d;
-    a.kn = (p.Nk + 15) / 16 * 16;
-    a.dpad = (p.d + 15) / 16 * 16;
-    a.nch = (p.d + CHUNK_COLS - 1) / CHUNK_COLS;
-    a.tmem_cols = next_pow2_cols(a.kn + a.dpad);
-    a.scale_log2e = fabsf(p.scale) * LOG2E;
-    a.negate = p.scale < 0.f;
     a.status = h->dev_status;
-    CUtensorMap tq, tk, tv;
-    int rc = make_tmap(h, &tq, p.q, p.BH, p.Nq, p.d, TILE_M, p.heads, p.bf16);
-    if (rc == SD_ATTN_OK) rc = make_tmap(h, &tk, p.k, p.BH, p.Nk, p.d, a.kn, p.heads, p.bf16);
-    if (rc == SD_ATTN_OK) rc = make_tmap(h, &tv, p.v, p.BH, p.Nk, p.d, a.kn, p.heads, p.bf16);
-    if (rc != SD_ATTN_OK) return rc;
-    dim3 grid((p.Nq + TILE_M - 1) / TILE_M, p.BH), block(CROSS_THREADS);
-    if (p.bf16)
-        launch_overlapped(h, cross_attention_kernel<true>, grid, block, cross_smem_bytes(a.nch, a.kn), p.stream, tq, tk, tv, a);
-    else
-        launch_overlapped(h, cross_attention_kernel<false>, grid, block, cross_smem_bytes(a.nch, a.kn), p.stream, tq, tk, tv, a);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e;
+#define SD_X1(KN) (nch == 1 ? launch_cross1_as<KN, 1, false, NP>(h, p, n, a) : nch == 2 ? launch_cross1_as<KN, 2, false, NP>(h, p, n, a) \
+                                                                                 : launch_cross1_as<KN, 3, false, NP>(h, p, n, a))
+    if (kn == 64) e = dense ? launch_cross1_as<64, 1, true, NP>(h, p, n, a) : SD_X1(64);
+    else if (kn == 80) e = dense ? launch_cross1_as<80, 1, true, NP>(h, p, n, a) : SD_X1(80);
+    else e = SD_X1(128);
+#undef SD_X1
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->launches += 1;
     return SD_ATTN_OK;
+}
+
+static int launch_cross1_group(sd_attn_handle* h, const Problem* ps, int n) {
+    if (n < 1 || n > X1_GROUP_MAX) return SD_ATTN_ERR_INVALID_VALUE;
+    return n == 1 ? launch_cross1_np<1>(h, ps, 1) : launch_cross1_np<X1_GROUP_MAX>(h, ps, n);
+}
+
+// The persistent kernel (65..80 keys) keeps K and V of a head for all its tiles and hides a tile's chain behind other tiles';
+// one CTA per tile has the shorter chain.  The line: four tiles per SM, about what is resident at once (5525 x 77 d = 40, 704
+// tiles: 8.4 us either way; 2304 x 77 d = 80 B = 4, 576 tiles: 9.6 against 9.9 persistent; B = 16: 32.4 against 28.1), and
+// token-major tensors of d <= 48, whose K and V rows are the costly ones to fetch (4096 x 77 d = 40: 8.1 against 7.4).  The two
+// kernels give the same bits (the same products, exponents and order of additions), so a group may take the other one than
+// its problems would alone.
+static bool cross_is_persistent(const sd_attn_handle* h, const Problem& p, int n) {
+    if (!cross2_supports(p.Nk, p.d) || h->opt.cross_one_tile) return false;
+    return (long long)((p.Nq + TILE_M - 1) / TILE_M) * p.BH * n > 4ll * h->sm_count || (p.heads > 0 && p.d <= 48);
+}
+
+// `n` problems of one shape (BH, Nq, Nk, d, layout, dtype alike) in one launch.
+static int launch_cross_group(sd_attn_handle* h, const Problem* ps, int n) {
+    return cross_is_persistent(h, ps[0], n) ? launch_cross2_group(h, ps, n) : launch_cross1_group(h, ps, n);
 }
 
 template <bool BF>
@@ -867,7 +923,7 @@ static int launch_one(sd_attn_handle* h, const Problem& p, int mode, int dtype) 
             return dtype == SD_ATTN_F16    ? launch_simt<__half>(h, p)
                    : dtype == SD_ATTN_BF16 ? launch_simt<__nv_bfloat16>(h, p)
                                            : launch_simt<float>(h, p);
-        case SD_ATTN_MODE_CROSS: return launch_cross(h, p);
+        case SD_ATTN_MODE_CROSS: return launch_cross_group(h, &p, 1);
         case SD_ATTN_MODE_FUSED: return launch_fused(h, p);
         case SD_ATTN_MODE_TWOPASS: return launch_twopass(h, p);
         default: return SD_ATTN_ERR_INVALID_VALUE;
@@ -900,6 +956,7 @@ static double group_cost_us(const Problem& p, int n, int dtype) {
     return c > 8.0 ? c : 8.0;
 }
 
+static_assert(X1_GROUP_MAX == X2_GROUP_MAX, "one group size for CROSS");
 constexpr int BATCH_MAX_GROUP = F4_GROUP_MAX > X2_GROUP_MAX ? F4_GROUP_MAX : X2_GROUP_MAX;
 
 extern "C" int sd_attn_forward_batch(sd_attn_handle* h, const sd_attn_problem* problems, int count, int dtype,
@@ -961,8 +1018,7 @@ extern "C" int sd_attn_forward_batch(sd_attn_handle* h, const sd_attn_problem* p
     for (int i = 0; i < count; ++i) {
         if (taken[i]) continue;
         const sd_attn_problem& p0 = problems[i];
-        const bool x2 = modes[i] == SD_ATTN_MODE_CROSS && cross2_supports(p0.Nk, p0.d) && !h->opt.cross_one_tile;
-        int cap = x2 ? X2_GROUP_MAX : 1;
+        int cap = modes[i] == SD_ATTN_MODE_CROSS ? X1_GROUP_MAX : 1;
         if (modes[i] == SD_ATTN_MODE_FUSED)
             cap = plan_fused(h, make_problem(h, p0.q, p0.k, p0.v, p0.out, p0.B, p0.H, p0.Nq, p0.Nk, p0.d, p0.scale, dtype, s)).max_group;
         first[n_groups] = n_members;
@@ -991,7 +1047,6 @@ extern "C" int sd_attn_forward_batch(sd_attn_handle* h, const sd_attn_problem* p
         const int g = k == 0 ? biggest : (k <= biggest ? k - 1 : k);
         const int i = member[first[g]], n = first[g + 1] - first[g];
         const sd_attn_problem& p0 = problems[i];
-        const bool x2 = modes[i] == SD_ATTN_MODE_CROSS && cross2_supports(p0.Nk, p0.d) && !h->opt.cross_one_tile;
         Problem group[BATCH_MAX_GROUP];
         for (int m = 0; m < n; ++m) {
             const sd_attn_problem& p = problems[member[first[g] + m]];
@@ -1009,7 +1064,7 @@ extern "C" int sd_attn_forward_batch(sd_attn_handle* h, const sd_attn_problem* p
         cudaStream_t target = lane == 0 ? s : h->batch_lane[lane - 1];
         for (int m = 0; m < n; ++m) group[m].stream = target;
         if (modes[i] == SD_ATTN_MODE_FUSED) rc = launch_fused_group(h, group, n);
-        else if (x2) rc = launch_cross2_group(h, group, n);
+        else if (modes[i] == SD_ATTN_MODE_CROSS) rc = launch_cross_group(h, group, n);
         else rc = launch_one(h, group[0], modes[i], dtype);
         if (rc == SD_ATTN_OK) h->last_mode = modes[i];
     }

@@ -209,6 +209,7 @@ struct HeadLayout {
     long long head_stride;
     long long batch_stride;
     FastDiv by_heads;
+    uint32_t piece_inv;   // 65536 / (d / 8) + 1: i / (d / 8) == (i * piece_inv) >> 16 for the slots of 32 rows
 };
 __device__ __forceinline__ void split_head(const HeadLayout& lay, int bh, int& batch, int& head) {
     batch = (int)fast_div((uint32_t)bh, lay.by_heads);
@@ -229,19 +230,21 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint
         "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w)
         : "memory");
 }
-// A warp's rows of 16-bit results, staged densely in shared memory by their threads (row r at rows + r * pieces * 16), to
-// global memory as whole lines: `out_row` is row 0, a row `pieces` 16-byte pieces, the next one ld elements on.  (Each thread
-// storing its own row costs an LSU wavefront per thread and piece: 2500 clocks for four tiles of 128 rows at d = 40.)
-__device__ __forceinline__ void store_staged_rows(void* out_row, int ld, uint32_t rows, int pieces, int n_rows, int lane) {
-    uint4* out = reinterpret_cast<uint4*>(out_row);
-    if (ld == pieces * 8) {   // head-major: one contiguous run
+// A warp's rows of 16-bit results go through shared memory to leave as whole lines.  (Each thread storing its own row costs an
+// LSU wavefront per thread and piece: 2500 clocks for four tiles of 128 rows at d = 40.)  Row r is `pieces` slots of 16 bytes
+// at slot r * pieces; piece p lies in slot p ^ stage_swizzle(r), which keeps the writes of eight neighbouring threads (same p, a
+// row each) on different banks whatever the row's length: a row of 20 pieces would put them on two.
+__device__ __forceinline__ int stage_swizzle(int r, int pieces) {
+    const int tz = min(__ffs(pieces) - 1, 3);   // the largest power of two, up to 8, that divides a row
+    return (r >> (3 - tz)) & ((1 << tz) - 1);
+}
+__device__ __forceinline__ void store_staged_rows(void* out_row0, const HeadLayout& lay, uint32_t rows, int pieces, int n_rows, int lane) {
+    uint4* out = reinterpret_cast<uint4*>(out_row0);
+    const int ld = lay.ld >> 3, n = n_rows * pieces;
 #pragma unroll 4
-        for (int i = lane; i < n_rows * pieces; i += 32) out[i] = ld_shared_v4(rows + i * 16);
-    } else {   // a row's pieces by neighbouring lanes
-        const int wide = pieces > 16 ? 32 : pieces > 8 ? 16 : 8, step = 32 / wide, p = lane & (wide - 1);
-        if (p < pieces)
-#pragma unroll 4
-            for (int r = lane / wide; r < n_rows; r += step) out[(long long)r * (ld >> 3) + p] = ld_shared_v4(rows + (r * pieces + p) * 16);
+    for (int i = lane; i < n; i += 32) {
+        const int r = (int)(((uint32_t)i * lay.piece_inv) >> 16), q = i - r * pieces;
+        out[r * ld + (q ^ stage_swizzle(r, pieces))] = ld_shared_v4(rows + i * 16);
     }
 }
 // Untiled bulk copy global -> shared, completion counted in bytes on `bar`.  Both addresses 16-byte aligned, the

@@ -1,0 +1,55 @@
+"""The one-tile cross-attention kernel over its key tiles, row tiles, fetches and head dims, against the oracle (tolerances of
+test_gpu_parity.py), and both CROSS kernels on the same problem."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import test_gpu_parity as parity  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def bd():
+    from paper_2304_11267_b200 import binding
+    from paper_2304_11267_b200 import build
+    build.build()
+    binding.load()
+    return binding
+
+
+def run(bd, q, k, v, scale, tokens_first=False, **options):
+    a = bd.Attention(layout=bd.LAYOUT_BNHD if tokens_first else bd.LAYOUT_BHND, options=bd.Options(**options))
+    t = [torch.from_numpy(np.ascontiguousarray(x.transpose(0, 2, 1, 3)) if tokens_first else x).cuda() for x in (q, k, v)]
+    out = a.forward(*t, scale=float(scale))
+    a.check()
+    assert a.last_mode == bd.MODE_CROSS
+    out = out.cpu().numpy()
+    a.close()
+    return out.transpose(0, 2, 1, 3) if tokens_first else out
+
+
+# keys around the tiles of 64, 80 and 128; head dims at the edges of the chunks and of the untiled fetch; rows that leave a
+# tile of 64 with one row, a warp with none
+@pytest.mark.parametrize("Nk", [1, 16, 63, 64, 65, 77, 80, 81, 127, 128])
+@pytest.mark.parametrize("d,Nq", [(8, 65), (40, 64), (48, 97), (56, 129), (64, 33), (80, 200), (128, 64), (136, 31), (160, 130)])
+def test_key_tiles_and_head_dims(bd, d, Nq, Nk):
+    q, k, v = parity.rand_qkv(d + Nk, 2, 3, Nq, Nk, d, qmult=3.0)   # (some rows' maximum lies far above their first score)
+    scale = np.float32(d ** -0.5)
+    ref, _, _ = oracle.forward(q, k, v, scale)
+    got = run(bd, q, k, v, scale, cross_one_tile=1)
+    parity.check(got, ref, v, what="d=%d Nq=%d Nk=%d" % (d, Nq, Nk))
+    assert np.array_equal(got, run(bd, q, k, v, scale, tokens_first=True, cross_one_tile=1))
+
+
+# more tiles than the GPU holds at once: 128-row tiles; the problem right at the line between the two kernels
+@pytest.mark.parametrize("B,Nq,d", [(2, 4733, 40), (2, 2304, 80), (2, 4736, 40), (3, 1500, 160)])
+def test_row_tiles_and_the_line_between_the_kernels(bd, B, Nq, d):
+    q, k, v = parity.rand_qkv(Nq, B, 8, Nq, 77, d)
+    scale = np.float32(d ** -0.5)
+    rows = np.arange(0, B * 8 * Nq, 11, dtype=np.int64)
+    ref, _, _ = oracle.forward(q, k, v, scale, rows=rows)
+    for opts in ({}, {"cross_one_tile": 1}):
+        parity.check(run(bd, q, k, v, scale, **opts).reshape(-1, d)[rows], ref, v, what="%d x 77 d=%d %s" % (Nq, d, opts))
