@@ -19,11 +19,13 @@
 // patch is double-buffered per 64 channels.  The filter is laid out once per layer in the order it is used, swizzle included,
 // so that a step's tile is one contiguous bulk copy.  Small images leave too few tiles for the GPU: the (64 channels, tap)
 // steps are then split among the CTAs of a cluster, which exchange their accumulators through distributed shared memory.
-//   warp 0 filter producer   warp 1 MMA issuer of the even steps   warp 2 patch producer   warp 3 MMA issuer of the odd steps
-// What bounds it is the tensor core only if the thread that feeds it keeps up: a step is 320 clocks of it at 160 channels,
-// but one thread's waits, descriptors, MMAs and commits of a step take 600 (measured: 224 wait, 56 for the four MMAs, 72
-// commit, the rest loop).  So two threads take the steps in turn, each into an accumulator of its own (products of different
-// threads are not ordered), added when they are read out.
+//   warps 0, 4 filter producers   warps 1, 3 MMA issuers (of the even and the odd steps each)   warp 2 patch producer
+// What bounds it is the tensor core only if the threads that feed it keep up: a step is 320 clocks of it at 160 channels, but
+// one issuing thread's waits, descriptors, MMAs and commits of a step take 600 and one producing thread's wait and copy 300.  So
+// two of either take the steps in turn; the issuers each have an accumulator of their own (products of different threads are
+// not ordered), added when they are read out.  With the second producer a step of 80 channels went from 320 to 230 clocks
+// (2 x 32 x 32, 640 -> 640: 17.0 -> 14.8 us; 2 x 33 x 43: 24.3 -> 18.2); 160 channels are at the tensor core's rate either way
+// (2 x 64 x 64, 320 -> 320: 14.9k of a CTA's 24k clocks are products, 4k the ramp, 2.4k stores at 17 bytes a clock).
 // Every wait is bounded and reports to the status block.
 #pragma once
 #include <cuda.h>
@@ -42,7 +44,7 @@ constexpr int CD_MAX_SPLIT = 8;
 constexpr int CD_MAX_N = 256;            // output channels per CTA, at most (one MMA)
 constexpr int CD_MAX_W = 126;            // two patch buffers and the filter ring fit shared memory up to here
 constexpr int CD_SMEM_BUDGET = 222 * 1024;
-enum { SITE_D_AEMPTY = 60, SITE_D_AFULL = 61, SITE_D_BEMPTY = 62, SITE_D_BFULL = 63, SITE_D_DONE = 64, SITE_D_RECV = 65 };
+enum { SITE_D_AEMPTY = 60, SITE_D_AFULL = 61, SITE_D_BEMPTY = 62, SITE_D_BFULL = 63, SITE_D_DONE = 64, SITE_D_FIRST = 65 };
 
 struct ConvDirectArgs {
     __half* y;
@@ -64,11 +66,11 @@ struct ConvDirectArgs {
 // Padded rows a tile's patch spans, at most: 128 positions and 2 pw + 2 more, from anywhere in a row.
 __host__ inline int cd_patch_rows(int pw) { return (TILE_M + 2 * pw + 2 + pw - 1 + pw - 1) / pw; }
 __host__ inline int cd_patch_bytes(int pw) { return (cd_patch_rows(pw) * pw * CHUNK_ROW_BYTES + 1023) & ~1023; }
-// The accumulator on its way out: binary16 rows of n_tile + 8 (one CTA per tile), or binary32 rows of n_tile + 4 and, behind
-// them, those of this CTA's share of the rows from every other CTA of the cluster.
+// The accumulator on its way out: binary16 rows of n_tile + 8 (one CTA per tile), or, of every CTA of the cluster, the
+// binary32 rows of n_tile + 4 that this CTA finishes.
 __host__ __device__ inline int cd_share_rows(int split) { return (TILE_M + split - 1) / split; }
 __host__ inline int cd_staging_bytes(int n_tile, int split) {
-    return split == 1 ? TILE_M * (n_tile + 8) * 2 : (TILE_M + (split - 1) * cd_share_rows(split)) * (n_tile + 4) * 4;
+    return split == 1 ? TILE_M * (n_tile + 8) * 2 : split * cd_share_rows(split) * (n_tile + 4) * 4;
 }
 
 __device__ __forceinline__ void cd_cluster_sync() {
@@ -80,11 +82,8 @@ __device__ __forceinline__ uint32_t cd_map_to_rank(uint32_t addr, int rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
     return remote;
 }
-// Bulk copy of this CTA's shared memory into another one of the cluster, completion counted on a barrier there.
-__device__ __forceinline__ void cd_push(uint32_t remote_dst, uint32_t src, uint32_t bytes, uint32_t remote_bar) {
-    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(remote_dst), "r"(src),
-                 "r"(bytes), "r"(remote_bar)
-                 : "memory");
+__device__ __forceinline__ void cd_store_remote(uint32_t addr, float a, float b, float c, float d) {
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
 // w [K][3][3][C] -> packed [ceil(C / 64)][9][K rounded up to 16][64], zeros in the padding, the eight 16-byte pieces of row k
@@ -109,7 +108,7 @@ template <bool CLUSTER>   // the steps of a tile are split among the CTAs of a c
 __global__ void __launch_bounds__(CD_THREADS, 1)
 conv_direct_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDirectArgs args) {
     extern __shared__ uint8_t cd_smem_raw[];
-    __shared__ __align__(8) uint64_t bar_a_full[2], bar_a_empty[2], bar_b_full[CD_MAX_STAGES], bar_b_empty[CD_MAX_STAGES], bar_done, bar_recv;
+    __shared__ __align__(8) uint64_t bar_a_full[2], bar_a_empty[2], bar_b_full[CD_MAX_STAGES], bar_b_empty[CD_MAX_STAGES], bar_done, bar_first;
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
     __shared__ float bias_s[CD_MAX_N];
@@ -138,7 +137,7 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDirectA
             mbar_init(smem_u32(&bar_b_empty[s]), 1);
         }
         mbar_init(smem_u32(&bar_done), 2);
-        mbar_init(smem_u32(&bar_recv), 1);
+        mbar_init(smem_u32(&bar_first), 1);
         mbar_init_fence();
         tma_prefetch_desc(&tmap_x);
     }
@@ -153,24 +152,27 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDirectA
     const uint32_t tmem_d = tmem_base_slot;
     volatile int* abort_p = &abort_flag;
 
-    if (warp == 0) {
+    if (warp == 0 || warp == 4) {
         if (elect_one()) {
-            // ---------------------------------------------------------------- filter producer
-            // (the last tile of channels may be short: the accumulator columns behind it are not stored)
+            // ---------------------------------------------------------------- filter producers: every second step each
+            // (the last tile of channels may be short: the accumulator columns behind it are not stored).  Behind the first
+            // step's filters the first patch goes out, which those products wait for too, and only then the rest of the ring.
+            const int mine = warp >> 2;
             const uint32_t bytes = (uint32_t)(min(n_tile, args.k_padded - k0) * CHUNK_ROW_BYTES);
-            const __half* src = args.filter + ((size_t)q_begin * args.k_padded + k0) * CHUNK_COLS;
-            const size_t step = (size_t)args.k_padded * CHUNK_COLS;
-            uint32_t dst = ring_smem;
-            int s = 0, pe = 1;
+            const __half* src = args.filter + ((size_t)(q_begin + mine) * args.k_padded + k0) * CHUNK_COLS;
+            const size_t step = 2 * (size_t)args.k_padded * CHUNK_COLS;
+            uint32_t dst = ring_smem + mine * stage_pitch;
+            int s = mine, pe = 1;
             bool filled = false;
-            for (int q = q_begin; q < q_end; ++q) {
+            for (int q = q_begin + mine; q < q_end; q += 2) {
+                if (q == q_begin + mine + 2 && !mbar_wait(smem_u32(&bar_first), 0, abort_p, args.status, SITE_D_FIRST, q)) break;
                 if (filled && !mbar_wait(smem_u32(&bar_b_empty[s]), pe, abort_p, args.status, SITE_D_BEMPTY, q)) break;
                 const uint32_t bar = smem_u32(&bar_b_full[s]);
                 mbar_arrive_expect_tx(bar, bytes);
                 bulk_load(dst, src, bytes, bar);
                 src += step;
-                dst += stage_pitch;
-                if (++s == stages) { s = 0; pe ^= 1; dst = ring_smem; filled = true; }
+                dst += 2 * stage_pitch;
+                if ((s += 2) >= stages) { s = mine; pe ^= 1; dst = ring_smem + mine * stage_pitch; filled = true; }
             }
         }
     } else if (warp == 2) {
@@ -189,46 +191,52 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDirectA
                     tma_load_4d(patch_smem + b * args.patch_bytes + r * pw * CHUNK_ROW_BYTES, &tmap_x, bar, c * CHUNK_COLS, -1, img_y,
                                 pr < args.padded_rows ? n : 0);
                 }
+                if (i == 0) mbar_arrive(smem_u32(&bar_first));
             }
         }
     } else if (warp == 1 || warp == 3) {
-        if (elect_one()) {
-            // ---------------------------------------------------------------- MMA issuers: every second step each
-            // Descriptors are 32-bit additions to their address field (16-byte units), nothing is divided in the loop.
-            const int mine = warp >> 1;
-            const uint32_t idesc = idesc_f16(TILE_M, n_tile, false, false, false);
-            constexpr uint64_t DESC = smem_desc_sw128(0, 16, 1024);
-            const uint32_t a0 = (patch_smem + col0 * CHUNK_ROW_BYTES) >> 4, a_buf = (uint32_t)args.patch_bytes >> 4;
-            const uint32_t b0 = ring_smem >> 4, b_stage = stage_pitch >> 4, tmem_acc = tmem_d + mine * n_tile;
-            int s = mine, pf = 0, chunk_i = 0, tap = q_begin % 9 + mine;
-            uint32_t b_at = b0 + mine * b_stage, a_at = a0;
-            bool ok = mbar_wait(smem_u32(&bar_a_full[0]), 0, abort_p, args.status, SITE_D_AFULL, q_begin);
-            for (int q = q_begin + mine; q < q_end && ok; q += 2) {
-                if (tap >= 9) {   // the next 64 channels
-                    tc_commit(smem_u32(&bar_a_empty[chunk_i & 1]));
-                    tap -= 9;
-                    ++chunk_i;
-                    a_at = a0 + (chunk_i & 1) * a_buf;
-                    ok = mbar_wait(smem_u32(&bar_a_full[chunk_i & 1]), (chunk_i >> 1) & 1, abort_p, args.status, SITE_D_AFULL, q);
-                }
-                ok = ok && mbar_wait(smem_u32(&bar_b_full[s]), pf, abort_p, args.status, SITE_D_BFULL, q);
-                if (!ok) break;
-                tc_fence_after_sync();
-                const uint32_t a_tap = a_at + (uint32_t)(((tap * 11) >> 5) * (pw - 3) + tap) * 8;   // (tap * 11) >> 5 = tap / 3
+        // ------------------------------------------------------------------- MMA issuers: every second step each
+        // Descriptors are 32-bit additions to their address field (16-byte units), nothing is divided in the loop; the whole
+        // warp runs it and one thread issues, which keeps descriptors in uniform registers.
+        const bool leader = elect_one();
+        auto wait = [&](uint64_t& bar, int parity, int site, int q) {
+            return __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar), parity, abort_p, args.status, site, q)) != 0;
+        };
+        const int mine = warp >> 1;
+        const uint32_t idesc = idesc_f16(TILE_M, n_tile, false, false, false);
+        constexpr uint64_t DESC = smem_desc_sw128(0, 16, 1024);
+        const uint32_t a0 = (patch_smem + col0 * CHUNK_ROW_BYTES) >> 4, a_buf = (uint32_t)args.patch_bytes >> 4;
+        const uint32_t b0 = ring_smem >> 4, b_stage = stage_pitch >> 4, tmem_acc = tmem_d + mine * n_tile;
+        int s = mine, pf = 0, chunk_i = 0, tap = q_begin % 9 + mine;
+        uint32_t b_at = b0 + mine * b_stage, a_at = a0;
+        bool ok = wait(bar_a_full[0], 0, SITE_D_AFULL, q_begin);
+        for (int q = q_begin + mine; q < q_end && ok; q += 2) {
+            if (tap >= 9) {   // the next 64 channels
+                if (leader) tc_commit(smem_u32(&bar_a_empty[chunk_i & 1]));
+                tap -= 9;
+                ++chunk_i;
+                a_at = a0 + (chunk_i & 1) * a_buf;
+                ok = wait(bar_a_full[chunk_i & 1], (chunk_i >> 1) & 1, SITE_D_AFULL, q);
+            }
+            ok = ok && wait(bar_b_full[s], pf, SITE_D_BFULL, q);
+            if (!ok) break;
+            tc_fence_after_sync();
+            const uint32_t a_tap = a_at + (uint32_t)(((tap * 11) >> 5) * (pw - 3) + tap) * 8;   // (tap * 11) >> 5 = tap / 3
+            if (leader) {
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
                     mma_f16_ss(tmem_acc, DESC | (a_tap + (uint32_t)(kk * 2)), DESC | (b_at + (uint32_t)(kk * 2)), idesc,
                                q > q_begin + mine || kk > 0);
                 tc_commit(smem_u32(&bar_b_empty[s]));
-                tap += 2;
-                s += 2;
-                b_at += 2 * b_stage;
-                if (s >= stages) { s -= stages; b_at -= stages * b_stage; pf ^= 1; }
             }
-            if (ok) tc_commit(smem_u32(&bar_done));
+            tap += 2;
+            s += 2;
+            b_at += 2 * b_stage;
+            if (s >= stages) { s -= stages; b_at -= stages * b_stage; pf ^= 1; }
         }
+        if (ok && leader) tc_commit(smem_u32(&bar_done));
     } else {
-        for (int c = tid - 128; c < n_tile; c += 128) bias_s[c] = args.bias && k0 + c < args.K ? __half2float(args.bias[k0 + c]) : 0.f;
+        for (int c = tid - 160; c < n_tile; c += 96) bias_s[c] = args.bias && k0 + c < args.K ? __half2float(args.bias[k0 + c]) : 0.f;
     }
     __syncwarp();
 
@@ -237,12 +245,18 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDirectA
     __syncthreads();   // (bias_s; the roles are done)
     bool ok = mbar_wait(smem_u32(&bar_done), 0, abort_p, args.status, SITE_D_DONE, blockIdx.z);
     ok = __all_sync(0xffffffffu, ok);
+    if (CLUSTER) cd_cluster_sync();   // every CTA of the cluster is done with its rings
     uint8_t* staging = cd_smem_raw + (smem_base - smem_u32(cd_smem_raw));
     const int pitch = CLUSTER ? n_tile + 4 : n_tile + 8;   // floats, halves
+    const int share_rows = cd_share_rows(split);
     if (ok) {
         tc_fence_after_sync();
         const int row = (warp & 3) * 32 + lane, groups = n_tile >> 4, g_begin = warp < 4 ? 0 : groups >> 1, g_end = warp < 4 ? groups >> 1 : groups;
         const uint32_t src = tmem_d + ((uint32_t)((warp & 3) * 32) << 16);
+        // CLUSTER: CTA o finishes rows 128 o / split .. 128 (o + 1) / split - 1; every thread stores its row where it is finished
+        // (straight from registers: bulk copies of staged rows took 4000 clocks for 42 KB)
+        const int owner = CLUSTER ? ((row + 1) * split - 1) >> 7 : 0, in_share = CLUSTER ? row - TILE_M * owner / split : row;
+        const uint32_t remote = CLUSTER ? cd_map_to_rank(smem_base + (uint32_t)((rank * share_rows + in_share) * pitch * 4), owner) : 0u;
         for (int g = g_begin; g < g_end; ++g) {
             uint32_t x[16], y[16];
             tmem_ld16(src + g * 16, x);
@@ -252,9 +266,8 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDirectA
 #pragma unroll
             for (int c = 0; c < 16; ++c) v[c] = __uint_as_float(x[c]) + __uint_as_float(y[c]);
             if (CLUSTER) {
-                float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(staging) + row * pitch + g * 16);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) dst[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+                for (int c = 0; c < 16; c += 4) cd_store_remote(remote + (g * 16 + c) * 4, v[c], v[c + 1], v[c + 2], v[c + 3]);
             } else {
                 uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<__half*>(staging) + row * pitch + g * 16);
 #pragma unroll
@@ -263,34 +276,23 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDirectA
                 dst[1] = make_uint4(pack_half2(v[8], v[9]), pack_half2(v[10], v[11]), pack_half2(v[12], v[13]), pack_half2(v[14], v[15]));
             }
         }
-        if (CLUSTER) fence_proxy_async_smem();
     }
-    tc_fence_before_sync();
-    __syncthreads();
     if (abort_flag && tid == 0) {   // gave up: let copies in flight land before shared memory is released
         for (int s = 0; s < stages; ++s) mbar_drain(smem_u32(&bar_b_full[s]), 0);
         for (int b = 0; b < 2; ++b) mbar_drain(smem_u32(&bar_a_full[b]), 0);
     }
-    // This CTA finishes rows r_begin .. r_end - 1 of the tile
-    const int r_begin = CLUSTER ? TILE_M * rank / split : 0, r_end = CLUSTER ? TILE_M * (rank + 1) / split : TILE_M;
-    const uint32_t recv_off = (uint32_t)(TILE_M * pitch * 4), slot_bytes = (uint32_t)(cd_share_rows(split) * pitch * 4);
-    if (CLUSTER) {
-        if (tid == 0) mbar_arrive_expect_tx(smem_u32(&bar_recv), (uint32_t)((split - 1) * (r_end - r_begin) * pitch * 4));
-        cd_cluster_sync();   // every CTA of the cluster is done with its rings
-        if (tid < split && tid != rank && !abort_flag) {   // thread o sends CTA o its rows
-            const int o = tid, ob = TILE_M * o / split, oe = TILE_M * (o + 1) / split;
-            cd_push(cd_map_to_rank(smem_base + recv_off + (rank < o ? rank : rank - 1) * slot_bytes, o), smem_base + (uint32_t)(ob * pitch * 4),
-                    (uint32_t)((oe - ob) * pitch * 4), cd_map_to_rank(smem_u32(&bar_recv), o));
-        }
-        __syncwarp();
-        ok = ok && mbar_wait(smem_u32(&bar_recv), 0, abort_p, args.status, SITE_D_RECV, blockIdx.z);
-        ok = __all_sync(0xffffffffu, ok);
-    }
+    tc_fence_before_sync();
+    __syncthreads();
+    if (CLUSTER) cd_cluster_sync();   // every row is where it is finished; nobody touches another CTA's memory from here on
     if (ok && !abort_flag) {
-        // eight channels (16 bytes) a thread at a time
-        const int per_row = min(n_tile, args.K - k0) >> 3, pieces = (r_end - r_begin) * per_row;
-        for (int idx = tid; idx < pieces; idx += CD_THREADS) {
-            const int rr = idx / per_row, row = r_begin + rr, c = (idx - rr * per_row) * 8;
+        // eight channels (16 bytes) a thread at a time: thread = (piece of a row, row modulo the rows done at once)
+        const int r_begin = TILE_M * rank / split, r_end = TILE_M * (rank + 1) / split;
+        const int per_row = min(n_tile, args.K - k0) >> 3, at_once = CD_THREADS / per_row, first = tid / per_row, c = (tid - first * per_row) * 8;
+        float b8[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) b8[i] = CLUSTER ? bias_s[c + i] : 0.f;
+        __half* y = args.y + k0 + c;
+        for (int row = r_begin + first; row < r_end && first < at_once; row += at_once) {
             const int p = p0 + row, pr = (int)fast_div((uint32_t)p, args.by_pw), xx = p - pr * pw;
             const int n = (int)fast_div((uint32_t)pr, args.by_h1), yy = pr - n * (args.H + 1);
             if (xx >= args.W || yy >= args.H || pr >= args.padded_rows) continue;
@@ -298,10 +300,9 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDirectA
             if (CLUSTER) {
                 float v[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) v[i] = bias_s[c + i];
-                for (int o = 0; o < split; ++o) {   // in rank order, so that the bits repeat
-                    const float* part = reinterpret_cast<const float*>(
-                        o == rank ? staging + (row * pitch + c) * 4 : staging + recv_off + (o < rank ? o : o - 1) * slot_bytes + (rr * pitch + c) * 4);
+                for (int i = 0; i < 8; ++i) v[i] = b8[i];
+                const float* part = reinterpret_cast<const float*>(staging) + (row - r_begin) * pitch + c;
+                for (int o = 0; o < split; ++o, part += share_rows * pitch) {   // in rank order, so that the bits repeat
                     const float4 lo = *reinterpret_cast<const float4*>(part), hi = *reinterpret_cast<const float4*>(part + 4);
                     v[0] += lo.x; v[1] += lo.y; v[2] += lo.z; v[3] += lo.w;
                     v[4] += hi.x; v[5] += hi.y; v[6] += hi.z; v[7] += hi.w;
@@ -310,11 +311,9 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap tmap_x, const ConvDirectA
             } else {
                 o8 = *reinterpret_cast<const uint4*>(reinterpret_cast<const __half*>(staging) + row * pitch + c);
             }
-            *reinterpret_cast<uint4*>(args.y + (((long long)n * args.H + yy) * args.W + xx) * args.K + k0 + c) = o8;
+            *reinterpret_cast<uint4*>(y + (size_t)((uint32_t)(n * args.H + yy) * (uint32_t)args.W + xx) * args.K) = o8;
         }
     }
-    __syncthreads();
-    if (CLUSTER) cd_cluster_sync();   // this CTA's shared memory is the source of copies until every CTA has received its rows
     if (warp == 3) tmem_dealloc(tmem_d, (uint32_t)args.tmem_cols);
 }
 

@@ -30,7 +30,7 @@ def bd():
 @pytest.mark.parametrize("N,H,W,C,K", [
     (1, 1, 1, 8, 8), (1, 6, 15, 8, 8), (1, 7, 14, 16, 24), (1, 7, 15, 64, 40), (3, 3, 3, 72, 16), (2, 2, 126, 64, 32),
     (1, 1, 126, 8, 264), (2, 5, 125, 56, 72), (1, 8, 8, 1280, 64), (2, 9, 12, 640, 328), (1, 16, 16, 320, 1280),
-    (1, 33, 43, 128, 200), (4, 12, 11, 320, 320), (2, 31, 29, 192, 648),
+    (1, 33, 43, 128, 200), (4, 12, 11, 320, 320), (2, 31, 29, 192, 648), (1, 9, 9, 832, 640), (1, 16, 16, 512, 968),
 ])
 def test_against_the_oracle(bd, N, H, W, C, K):
     assert bd.sd_winograd_direct_supported(N, H, W, C, K)
