@@ -24,7 +24,11 @@
 // The exponents are anchored at the row maximum of the FIRST key tile: bf16 parts have binary32's range, so a later score may
 // lie 2^64 above it before anything overflows; only then (the sum of a tile's weights says so) is the row re-anchored and the
 // tile redone.
-// Operands in shared memory are [part h, m, l][32-column chunk][row][64 bytes].  V is used as it lies (MN-major).
+// Operands in shared memory are [part h, m, l][32-column chunk][row][64 bytes].  V is used as it lies (MN-major).  Where one
+// query tile leaves room in tensor memory, its Q goes there: read from shared memory, 128 rows for each product of 32 or 64 keys
+// were most of the product's time.
+// us, operands of S in shared memory, undivided issuing loops, rows stored one by one -> now: 16 x 4096 x 4096, d = 40 285 -> 265;
+// 16 x 1024, d = 80 40.1 -> 34.8; 16 x 256, d = 160 35.6 -> 27.8; 16 x 256 x 77, d = 160 21.1 -> 16.1.
 // Every wait is bounded and reports to the status block.
 #pragma once
 #include <cuda_runtime.h>
@@ -54,10 +58,13 @@ struct F32Args {
 };
 
 // NC: 32-column chunks of a row (d <= 32 NC).  BN: keys per key tile.  T: query tiles per CTA.  ACC: output columns per
-// softmax thread.  KS, VS: depth of the K and V rings.  NO: buffers for the product of a key tile.
-template <int NC_, int BN_, int T_, int ACC_, int KS_, int VS_, int NO_>
+// softmax thread.  KS, VS: depth of the K and V rings.  NO: buffers for the product of a key tile.  MAX_FIRST: whether a key tile
+// fits the anchor is decided from its maximum before the exponentials, so that the weights replace the scores in registers,
+// not from the weights' sum behind them (measured: d = 80 43 -> 36 us; the other shapes lose 2% to 12% by it).
+template <int NC_, int BN_, int T_, int ACC_, int KS_, int VS_, int NO_, bool MAX_FIRST_>
 struct F32Shape {
     static constexpr int NC = NC_, BN = BN_, T = T_, ACC = ACC_, KS = KS_, VS = VS_, NO = NO_;
+    static constexpr bool MAX_FIRST = MAX_FIRST_;
     static constexpr int MAX_D = NC * F3_CHUNK < 2 * ACC ? NC * F3_CHUNK : 2 * ACC;
     static constexpr int N_CONV = T == 2 ? 1 : 2;   // warpgroups that convert K; as many for V
     static constexpr int WG_CONVERT = 2 * T, WG_ISSUE = WG_CONVERT + 2 * N_CONV, THREADS = (WG_ISSUE + 1) * 128;
@@ -67,7 +74,10 @@ struct F32Shape {
     // buffers for the product.  A softmax thread's weights go over its own scores (h, m) and behind all scores (l), so the
     // halves of a row need not wait for one another: word `off` of part (h, m) of half x at x BN/2 + (0, BN/4) + off, of
     // part l at BN + x BN/4 + off.
-    static constexpr int HALF = BN / 2, SLOT = 3 * BN / 2, O_COLS = 2 * ACC, TILE_COLS = 2 * SLOT + NO * O_COLS;
+    static constexpr int HALF = BN / 2, SLOT = 3 * BN / 2, O_COLS = 2 * ACC;
+    static constexpr bool Q_TMEM = T == 1;             // (two query tiles leave 32 columns)
+    static constexpr int Q_COLS = NC * F3_CHUNK / 2;   // of a part
+    static constexpr int TILE_COLS = 2 * SLOT + NO * O_COLS + (Q_TMEM ? 3 * Q_COLS : 0);
     static_assert(T * TILE_COLS <= 512, "tensor memory");
     // registers: the pools of setmaxnreg must not exceed what the CTA was launched with
     static constexpr int LAUNCH_REGS = 65536 / THREADS / 8 * 8;
@@ -75,11 +85,12 @@ struct F32Shape {
     static constexpr int POOL = 128 * (2 * T * SOFTMAX_REGS + 2 * N_CONV * CONVERT_REGS + ISSUE_REGS);
     static_assert(POOL <= THREADS * LAUNCH_REGS, "setmaxnreg budget");
 };
-using F32Two = F32Shape<2, 64, 2, 24, 2, 2, 1>;     // d <= 48, two query tiles
-using F32One = F32Shape<2, 64, 1, 32, 3, 3, 2>;     // d <= 64
-using F32Mid = F32Shape<3, 64, 1, 48, 2, 2, 2>;     // d <= 96
-using F32Wide = F32Shape<5, 32, 1, 80, 2, 1, 2>;    // d <= 160
+using F32Two = F32Shape<2, 64, 2, 24, 2, 2, 1, false>;     // d <= 48, two query tiles
+using F32One = F32Shape<2, 64, 1, 32, 3, 3, 2, false>;     // d <= 64
+using F32Mid = F32Shape<3, 64, 1, 48, 2, 2, 1, true>;     // d <= 96
+using F32Wide = F32Shape<5, 32, 1, 80, 2, 1, 1, true>;    // d <= 160
 constexpr float F32_TILE_SUM_LIMIT = 1.8446744e19f; // 2^64: no weight above it reaches the products
+constexpr float F32_MAX_LIMIT = 58.f;               // log2 of the largest weight where the maximum decides: 64 of them stay below the sum
 
 // Shared-memory matrix descriptor of a 64-byte-swizzled tile (rows of 64 bytes, eight to a 512-byte atom).
 __host__ __device__ constexpr uint64_t smem_desc_sw64(uint32_t byte_addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
@@ -225,14 +236,15 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
     const uint32_t tmem_base = tmem_base_slot;
     auto tmem_slot = [&](int t, int b) { return tmem_base + t * SH::TILE_COLS + b * SH::SLOT; };
     auto tmem_o = [&](int t, int b) { return tmem_base + t * SH::TILE_COLS + 2 * SH::SLOT + b * SH::O_COLS; };
+    auto tmem_q = [&](int t) { return tmem_base + t * SH::TILE_COLS + 2 * SH::SLOT + NO * SH::O_COLS; };
     // Q_t, by the 256 threads that will work on its scores: thread i of them
     auto convert_q = [&](int t, int i) {
-        constexpr int n = 256;
+        constexpr int n = 256, U = SH::T == 1 ? 5 : 4;
         const float* qb = head_row(args.q, args.lq, bh, 0);
-        for (int first = i; first < TILE_M * pieces; first += 4 * n) {
-            float4 lo[4], hi[4];
+        for (int first = i; first < TILE_M * pieces; first += U * n) {
+            float4 lo[U], hi[U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const int idx = first + u * n, r = (int)fast_div((uint32_t)idx, args.by_pieces), c = (idx - r * pieces) * 8;
                 const int row = row_base + t * TILE_M + r;
                 lo[u] = hi[u] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -243,7 +255,7 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                 }
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const int idx = first + u * n, r = (int)fast_div((uint32_t)idx, args.by_pieces);
                 const int p = idx - r * pieces;
                 if (idx < TILE_M * pieces)
@@ -251,7 +263,25 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                                  lo[u], hi[u]);
             }
         }
-        fence_proxy_async_smem();
+        if constexpr (SH::Q_TMEM) {   // thread = row: its steps of 16 columns, every second one
+            named_barrier(1 + t, 256);
+            const int row = i & 127, sw = (row >> 1) & 3;
+            const uint32_t src = q_smem + t * SH::Q_TILE + row * 64, dst = tmem_q(t) + ((uint32_t)((warp & 3) * 32) << 16);
+#pragma unroll
+            for (int part = 0; part < 3; ++part)
+#pragma unroll
+                for (int kk = 0; kk < 2 * NC; ++kk) {
+                    if ((kk & 1) != i >> 7 || kk * 16 >= d) continue;
+                    const uint32_t at = src + part * SH::Q_PART + (kk >> 1) * (TILE_M * 64);
+                    const uint4 a = ld_shared_v4(at + ((((kk & 1) * 2) ^ sw) << 4)), b = ld_shared_v4(at + ((((kk & 1) * 2 + 1) ^ sw) << 4));
+                    const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+                    tmem_st8(dst + part * SH::Q_COLS + kk * 8, w);
+                }
+            tmem_wait_st();
+            tc_fence_before_sync();
+        } else {
+            fence_proxy_async_smem();
+        }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bars.q_full[t]));
     };
@@ -259,8 +289,13 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
     if (wg == SH::WG_ISSUE) {
         setmaxnreg_dec<SH::ISSUE_REGS>();
         const int t = (warp & 3) >> 1;
-        if (t < T && elect_one()) {
+        if (t < T) {
+            // the whole warp runs the loops and one thread issues, which keeps descriptors in uniform registers
+            const bool leader = elect_one();
             bool ok = true;
+            auto wait = [&](uint64_t& bar, int parity, int site, int j) {
+                return __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar), parity, abort_p, args.status, site, j)) != 0;
+            };
             // parts of the six products, small ones first
             constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};
             if ((warp & 1) == 0) {
@@ -268,26 +303,32 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                 const uint32_t idesc = idesc_f16(TILE_M, BN, false, false, args.negate != 0, true);
                 const int ksteps = (d + 15) / 16;
                 const uint64_t q_desc = smem_desc_sw64(q_smem + t * SH::Q_TILE, 16, 512), k_desc = smem_desc_sw64(k_smem, 16, 512);
-                ok = mbar_wait(smem_u32(&bars.q_full[t]), 0, abort_p, args.status, SITE_F_Q, t);
+                ok = wait(bars.q_full[t], 0, SITE_F_Q, t);
                 int s = 0, pk = 0;
                 for (int j = 0; j < n_kv && ok; ++j) {
                     const int b = j & 1;
-                    ok = mbar_wait(smem_u32(&bars.k_full[s]), pk, abort_p, args.status, SITE_F_K, j);
-                    if (ok && j >= 2) ok = mbar_wait(smem_u32(&bars.slot_free[t][b]), ((j >> 1) - 1) & 1, abort_p, args.status, SITE_F_SLOT, j);
+                    ok = wait(bars.k_full[s], pk, SITE_F_K, j);
+                    if (ok && j >= 2) ok = wait(bars.slot_free[t][b], ((j >> 1) - 1) & 1, SITE_F_SLOT, j);
                     if (!ok) break;
                     tc_fence_after_sync();
                     const uint64_t kd = k_desc + (uint64_t)(s * (SH::KV_STAGE >> 4));
                     const uint32_t ts = tmem_slot(t, b);
+                    if (leader) {
 #pragma unroll
-                    for (int p = 0; p < 6; ++p)
+                        for (int p = 0; p < 6; ++p)
 #pragma unroll
-                        for (int kk = 0; kk < 2 * NC; ++kk)   // (offsets are constants; a loop over the steps there are took four times as long)
-                            if (kk < ksteps)
-                                mma_f16_ss(ts, q_desc + (uint64_t)((PA[p] * SH::Q_PART + (kk >> 1) * (TILE_M * 64) + (kk & 1) * 32) >> 4),
-                                           kd + (uint64_t)((PB[p] * SH::KV_PART + (kk >> 1) * (BN * 64) + (kk & 1) * 32) >> 4), idesc,
-                                           p > 0 || kk > 0);
-                    tc_commit(smem_u32(&bars.s_full[t][b]));
-                    tc_commit(smem_u32(&bars.k_empty[s]));
+                            for (int kk = 0; kk < 2 * NC; ++kk)   // (offsets are constants)
+                                if (kk < ksteps) {
+                                    const uint64_t kt = kd + (uint64_t)((PB[p] * SH::KV_PART + (kk >> 1) * (BN * 64) + (kk & 1) * 32) >> 4);
+                                    if constexpr (SH::Q_TMEM)
+                                        mma_f16_ts(ts, tmem_q(t) + PA[p] * SH::Q_COLS + kk * 8, kt, idesc, p > 0 || kk > 0);
+                                    else
+                                        mma_f16_ss(ts, q_desc + (uint64_t)((PA[p] * SH::Q_PART + (kk >> 1) * (TILE_M * 64) + (kk & 1) * 32) >> 4),
+                                                   kt, idesc, p > 0 || kk > 0);
+                                }
+                        tc_commit(smem_u32(&bars.s_full[t][b]));
+                        tc_commit(smem_u32(&bars.k_empty[s]));
+                    }
                     if (++s == KS) { s = 0; pk ^= 1; }
                 }
             } else {
@@ -303,21 +344,23 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                 for (int j = 0; j < n_kv && ok; ++j) {
                     const int b = j & 1, ob = j % NO;
                     const uint32_t tp = tmem_slot(t, b), to = tmem_o(t, ob);
-                    ok = mbar_wait(smem_u32(&bars.v_full[s]), pv, abort_p, args.status, SITE_F_V, j);
-                    if (ok && j >= NO) ok = mbar_wait(smem_u32(&bars.o_free[t][ob]), (j / NO - 1) & 1, abort_p, args.status, SITE_F_OFREE, j);
-                    if (ok) ok = mbar_wait_eager(smem_u32(&bars.p_full[t][b]), (j >> 1) & 1, abort_p, args.status, SITE_F_P, j);
+                    ok = wait(bars.v_full[s], pv, SITE_F_V, j);
+                    if (ok && j >= NO) ok = wait(bars.o_free[t][ob], (j / NO - 1) & 1, SITE_F_OFREE, j);
+                    if (ok) ok = __all_sync(0xffffffffu, mbar_wait_eager(smem_u32(&bars.p_full[t][b]), (j >> 1) & 1, abort_p, args.status, SITE_F_P, j));
                     if (!ok) break;
                     tc_fence_after_sync();
                     const uint64_t vd = v_desc + (uint64_t)(s * (SH::KV_STAGE >> 4));
+                    if (leader) {
 #pragma unroll
-                    for (int p = 0; p < 6; ++p)
+                        for (int p = 0; p < 6; ++p)
 #pragma unroll
-                        for (int kk = 0; kk < BN / 16; ++kk)
-                            mma_f16_ts(to, tp + weights_at(PA[p], kk), vd + (uint64_t)((PB[p] * SH::KV_PART + kk * 1024) >> 4), idesc,
-                                       p > 0 || kk > 0);
-                    tc_commit(smem_u32(&bars.pv_done[t][ob]));
-                    tc_commit(smem_u32(&bars.slot_free[t][b]));
-                    tc_commit(smem_u32(&bars.v_empty[s]));
+                            for (int kk = 0; kk < BN / 16; ++kk)
+                                mma_f16_ts(to, tp + weights_at(PA[p], kk), vd + (uint64_t)((PB[p] * SH::KV_PART + kk * 1024) >> 4), idesc,
+                                           p > 0 || kk > 0);
+                        tc_commit(smem_u32(&bars.pv_done[t][ob]));
+                        tc_commit(smem_u32(&bars.slot_free[t][b]));
+                        tc_commit(smem_u32(&bars.v_empty[s]));
+                    }
                     if (++s == VS) { s = 0; pv ^= 1; }
                 }
             }
@@ -396,7 +439,7 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
             bool ok = true;
             for (int j = 0; j < n_kv; ++j) {
                 const int b = j & 1;
-                ok = mbar_wait(smem_u32(&bars.s_full[t][b]), (j >> 1) & 1, abort_p, args.status, SITE_F_S, j);
+                ok = ok && mbar_wait(smem_u32(&bars.s_full[t][b]), (j >> 1) & 1, abort_p, args.status, SITE_F_S, j);
                 ok = __all_sync(0xffffffffu, ok);
                 const uint32_t slot = tmem_slot(t, b) + lane_off;
                 const int valid = args.Nk - j * BN - half * HALF;   // columns past it are zero-filled keys
@@ -414,10 +457,7 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                     m_run = row_max_of_halves(row_max_masked<HALF>(s, valid));
                     nm_run = -m_run * c2;
                 }
-                float tile_sum;
-                bool live = true;
-#pragma unroll 1
-                for (int attempt = 0; attempt < 2; ++attempt) {
+                auto sweep = [&]() -> float {   // weights of the anchor in use, to tensor memory; their sum
                     const uint64_t c2c2 = pack_b64(__float_as_uint(c2), __float_as_uint(c2));
                     const uint64_t nmnm = pack_b64(__float_as_uint(nm_run), __float_as_uint(nm_run));
                     uint64_t sum[2] = {0ull, 0ull};
@@ -452,13 +492,10 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                         tmem_st4(own + BN / 4, m);
                         tmem_st4(slot + BN + half * (BN / 4) + c / 2, l);
                     }
-                    tile_sum = sum_f32x2(sum[0], sum[1]);
-                    if (attempt == 0 && j > 0 && ok) ok = add_product(j - 1);
-                    // One decision for the query tile's 256 threads: go on, give up (a wait expired), or redo the tile.
-                    if (attempt == 1 || named_barrier_and(1 + t, 256, ok && tile_sum <= F32_TILE_SUM_LIMIT)) break;
-                    live = named_barrier_and(1 + t, 256, ok);
-                    if (!live) break;
-                    // Rare: a score far above the anchor.  Everything summed so far is rescaled to the new one.
+                    return sum_f32x2(sum[0], sum[1]);
+                };
+                // Rare: a score far above the anchor.  Everything summed so far is rescaled to the new one.
+                auto reanchor = [&]() {
                     const float m_new = fmaxf(m_run, row_max_of_halves(row_max_masked<HALF>(s, valid)));
                     const float nm_new = -m_new * c2, alpha = ex2_approx(nm_new - nm_run);
                     m_run = m_new;
@@ -467,9 +504,41 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                     const uint64_t aa = pack_b64(__float_as_uint(alpha), __float_as_uint(alpha));
 #pragma unroll
                     for (int c = 0; c < ACC / 2; ++c) o[c] = fma_f32x2(o[c], aa, 0ull);
-                    tmem_wait_st();
+                };
+                // One decision for the query tile's 256 threads: go on, give up (a wait expired), or re-anchor.  The product of the
+                // key tile before is added ahead of handing this one's weights over: once their product runs, loads from
+                // tensor memory take three times as long.
+                float tile_sum;
+                if constexpr (SH::MAX_FIRST) {
+                    bool added = j == 0;
+                    if (j > 0) {
+                        float top[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                        for (int c = 0; c < HALF; ++c) top[c & 3] = fmaxf(top[c & 3], __uint_as_float(s[c]));
+                        const float mx = fmaxf(fmaxf(top[0], top[1]), fmaxf(top[2], top[3]));
+                        if (!named_barrier_and(1 + t, 256, ok && fmaf(mx, c2, nm_run) <= F32_MAX_LIMIT)) {
+                            if (!named_barrier_and(1 + t, 256, ok)) { ok = false; break; }
+                            ok = add_product(j - 1);
+                            added = true;
+                            reanchor();
+                        }
+                    }
+                    tile_sum = sweep();
+                    if (!added && ok) ok = add_product(j - 1);
+                } else {
+                    bool live = true;
+#pragma unroll 1
+                    for (int attempt = 0; attempt < 2; ++attempt) {
+                        tile_sum = sweep();
+                        if (attempt == 0 && j > 0 && ok) ok = add_product(j - 1);
+                        if (attempt == 1 || named_barrier_and(1 + t, 256, ok && tile_sum <= F32_TILE_SUM_LIMIT)) break;
+                        live = named_barrier_and(1 + t, 256, ok);
+                        if (!live) break;
+                        reanchor();
+                        tmem_wait_st();
+                    }
+                    if (!live) { ok = false; break; }
                 }
-                if (!live) { ok = false; break; }
                 l_run += tile_sum;
                 tmem_wait_st();
                 tc_fence_before_sync();
@@ -479,18 +548,31 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
             if (ok) ok = add_product(n_kv - 1);
             half_s[t][half][wt] = l_run;
             ok = named_barrier_and(1 + t, 256, ok);
-            const int row = row_base + t * TILE_M + wt;
-            if (ok && row < args.Nq) {
+            if (ok) {
+                // A thread's columns are 4 ACC bytes of a row of its own: through shared memory (the query tile's, which no product
+                // reads any more), so that a warp's stores run along the rows (row by row they took 9000 clocks at d = 160).
+                constexpr int PITCH = ACC + 4;   // floats
+                static_assert(8 * 32 * PITCH * 4 <= SH::Q_TILE, "staging");
                 const float inv = 1.f / (half_s[t][0][wt] + half_s[t][1][wt]);
-                float* orow = head_row(args.out, args.lq, bh, row) + c0;
+                const uint32_t stage = q_smem + t * SH::Q_TILE + (uint32_t)((half * 4 + (warp & 3)) * 32 * PITCH * 4);
 #pragma unroll
                 for (int c = 0; c < ACC; c += 4) {
-                    if (c + 4 <= cols) {   // (d and c0 are multiples of 4)
-                        uint32_t x0, x1, x2, x3;
-                        unpack_b64(o[c / 2], x0, x1);
-                        unpack_b64(o[c / 2 + 1], x2, x3);
-                        *reinterpret_cast<float4*>(orow + c) = make_float4(__uint_as_float(x0) * inv, __uint_as_float(x1) * inv,
-                                                                          __uint_as_float(x2) * inv, __uint_as_float(x3) * inv);
+                    uint32_t x[4];
+                    unpack_b64(o[c / 2], x[0], x[1]);
+                    unpack_b64(o[c / 2 + 1], x[2], x[3]);
+                    st_shared_v4(stage + (lane * PITCH + c) * 4,
+                                 make_uint4(__float_as_uint(__uint_as_float(x[0]) * inv), __float_as_uint(__uint_as_float(x[1]) * inv),
+                                            __float_as_uint(__uint_as_float(x[2]) * inv), __float_as_uint(__uint_as_float(x[3]) * inv)));
+                }
+                __syncwarp();
+                const int row0 = row_base + t * TILE_M + (warp & 3) * 32, rows = args.Nq - row0 < 32 ? args.Nq - row0 : 32;
+                // lane = (piece of four columns, row modulo the rows done at once); d and c0 are multiples of 4
+                const int per_row = cols > 0 ? cols >> 2 : 1, at_once = 32 / per_row, first = lane / per_row, c = (lane - first * per_row) * 4;
+                if (cols > 0 && first < at_once) {
+                    float* out = head_row(args.out, args.lq, bh, row0) + c0 + c;
+                    for (int r = first; r < rows; r += at_once) {
+                        const uint4 v = ld_shared_v4(stage + (r * PITCH + c) * 4);
+                        *reinterpret_cast<uint4*>(out + (long long)r * args.lq.ld) = v;
                     }
                 }
             }
