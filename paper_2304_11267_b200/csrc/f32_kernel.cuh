@@ -27,7 +27,7 @@
 // Operands in shared memory are [part h, m, l][32-column chunk][row][64 bytes].  V is used as it lies (MN-major).  Where one
 // query tile leaves room in tensor memory, its Q goes there: read from shared memory, 128 rows for each product of 32 or 64 keys
 // were most of the product's time.
-// us, operands of S in shared memory, undivided issuing loops, rows stored one by one -> now: 16 x 4096 x 4096, d = 40 285 -> 265;
+// us, operands of S in shared memory, undivided issuing loops, rows stored one by one -> now: 16 x 4096 x 4096, d = 40 285 -> 261;
 // 16 x 1024, d = 80 40.1 -> 34.8; 16 x 256, d = 160 35.6 -> 27.8; 16 x 256 x 77, d = 160 21.1 -> 16.1.
 // Every wait is bounded and reports to the status block.
 #pragma once
@@ -81,7 +81,8 @@ struct F32Shape {
     static_assert(T * TILE_COLS <= 512, "tensor memory");
     // registers: the pools of setmaxnreg must not exceed what the CTA was launched with
     static constexpr int LAUNCH_REGS = 65536 / THREADS / 8 * 8;
-    static constexpr int ISSUE_REGS = 40, CONVERT_REGS = 56, SOFTMAX_REGS = T == 2 ? 88 : 120;
+    // (a few spilled registers in the softmax loop of two query tiles cost 10%: 96 for it, what the others can spare)
+    static constexpr int ISSUE_REGS = T == 2 ? 24 : 40, CONVERT_REGS = T == 2 ? 48 : 56, SOFTMAX_REGS = T == 2 ? 96 : 120;
     static constexpr int POOL = 128 * (2 * T * SOFTMAX_REGS + 2 * N_CONV * CONVERT_REGS + ISSUE_REGS);
     static_assert(POOL <= THREADS * LAUNCH_REGS, "setmaxnreg budget");
 };
