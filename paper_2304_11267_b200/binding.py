@@ -31,7 +31,7 @@ EXPORTS = ["sd_attn_create", "sd_attn_create_ex", "sd_attn_static_query_status",
            "sd_attn_forward_host", "sd_attn_host_staging_bytes",
            "sd_attn_forward_twopass_static", "sd_geglu_forward", "sd_groupnorm_forward", "sd_attn_set_layout", "sd_attn_forward_batch",
            "sd_winograd_filter_elems", "sd_winograd_transform_filter", "sd_winograd_workspace_bytes",
-           "sd_winograd_conv3x3_forward", "sd_winograd_direct_supported",
+           "sd_winograd_conv3x3_forward", "sd_winograd_direct_supported", "sd_winograd_direct_preferred",
            "sd_winograd_direct_filter_elems", "sd_winograd_direct_pack_filter", "sd_winograd_direct_forward",
            "sd_winograd_query_status"]
 
@@ -106,6 +106,8 @@ def load() -> ctypes.CDLL:
     lib.sd_winograd_conv3x3_forward.argtypes = [vp, vp, vp, vp, vp, sz, ci, ci, ci, ci, ci, vp]
     lib.sd_winograd_direct_supported.restype = ci
     lib.sd_winograd_direct_supported.argtypes = [ci] * 5
+    lib.sd_winograd_direct_preferred.restype = ci
+    lib.sd_winograd_direct_preferred.argtypes = [ci] * 5
     lib.sd_winograd_direct_filter_elems.restype = sz
     lib.sd_winograd_direct_filter_elems.argtypes = [ci, ci]
     lib.sd_winograd_direct_pack_filter.restype = ci
@@ -273,6 +275,10 @@ def sd_winograd_direct_supported(N, H, W, C, K) -> bool:
     return bool(load().sd_winograd_direct_supported(N, H, W, C, K))
 
 
+def sd_winograd_direct_preferred(N, H, W, C, K) -> bool:
+    return bool(load().sd_winograd_direct_preferred(N, H, W, C, K))
+
+
 def sd_winograd_direct_filter_elems(K: int, C: int) -> int:
     return int(load().sd_winograd_direct_filter_elems(K, C))
 
@@ -295,8 +301,8 @@ class WinogradConv3x3:
     """A layer's prepared filter plus torch-tensor marshalling: ``WinogradConv3x3(w, bias)(x)`` with
     w [K,3,3,C], bias [K] or None, x [N,H,W,C] float16 CUDA tensors (channels-last memory) -> y [N,H,W,K].
 
-    Images the direct convolution covers go there (it is the faster one on this GPU); the others through the
-    transformed domain, whose filter ``U`` is made when the first of them comes."""
+    Images go to the direct convolution where it is the faster one; the others (the largest calls, and images too wide for it)
+    through the transformed domain, whose filter ``U`` is made when the first of them comes."""
 
     def __init__(self, w, bias=None, stream: Optional[int] = None):
         import torch
@@ -331,6 +337,8 @@ class WinogradConv3x3:
                                               torch.cuda.current_stream(w.device).cuda_stream)
             if rc != OK:
                 raise SdAttnError(rc, "sd_winograd_transform_filter")
+            if not torch.cuda.is_current_stream_capturing():
+                torch.cuda.current_stream(w.device).synchronize()   # (once: later calls may come on any stream)
             self._U = U
         return self._U
 
@@ -346,8 +354,10 @@ class WinogradConv3x3:
         import torch
         N, H, W, _ = (int(v) for v in x.shape)
         s = stream if stream is not None else torch.cuda.current_stream(x.device).cuda_stream
-        with torch.cuda.stream(torch.cuda.ExternalStream(s, device=x.device)):
-            U = self.U   # (its first use is ordered before this call)
+        U = self._U
+        if U is None:
+            with torch.cuda.stream(torch.cuda.ExternalStream(s, device=x.device)):
+                U = self.U   # (its first use is ordered before this call)
         need = sd_winograd_workspace_bytes(N, H, W, self.C, self.K)
         if self._workspace is None or self._workspace.numel() < need:
             self._workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=x.device)

@@ -1599,6 +1599,7 @@ extern "C" int sd_winograd_conv3x3_forward(const void* x, const void* U, const v
 // The same convolution as one implicit matrix product (conv_direct_kernel.cuh).
 struct ConvDirectPlan {
     int n_tile, n_tiles, m_tiles, split, stages;
+    double clocks;   // the cost the plan was chosen by
 };
 
 static bool conv_direct_fits(int N, int H, int W, int C, int K) {
@@ -1639,10 +1640,47 @@ static ConvDirectPlan plan_conv_direct(const WinogradDeviceState* st, int N, int
             if (best_cost < 0 || cost < best_cost) {
                 best_cost = cost;
                 best = p;
+                best.clocks = cost;
             }
         }
     }
     return best;
+}
+
+// The plan of a shape and whether it is expected to beat the transformed domain: both depend on the shape only, so a layer's
+// next call finds its own.
+struct ConvDirectChoice {
+    int N, H, W, C, K;
+    const WinogradDeviceState* st;
+    ConvDirectPlan plan;
+    bool preferred;
+};
+static const ConvDirectChoice* conv_direct_choice(const WinogradDeviceState* st, int N, int H, int W, int C, int K) {
+    static thread_local ConvDirectChoice known[8];
+    static thread_local int known_next = 0;
+    for (const ConvDirectChoice& k : known)
+        if (k.st == st && k.N == N && k.H == H && k.W == W && k.C == C && k.K == K) return &k;
+    ConvDirectChoice& k = known[known_next];
+    known_next = (known_next + 1) % 8;
+    k = {N, H, W, C, K, st, plan_conv_direct(st, N, H, W, C, K), false};
+    // Microseconds, fitted to 29 shapes of 25 to 220 GFLOP run back to back over three sets of tensors.  The direct kernel: its
+    // plan's clocks and, for the clock rate under a full tensor core, its operations.  The transformed domain: its
+    // intermediates (binary16 V of 36 tiles x C, binary32 M of 36 tiles x K), written and read, and its filter.  The choice costs
+    // 0.6% on average over those shapes, 8% at most; always taking the direct kernel cost up to 39% (4 x 48 x 48, 1920 -> 640:
+    // 180 us against 130), always the transformed domain up to three times (small images).
+    const double tiles = (double)N * ((H + 3) / 4) * ((W + 3) / 4);
+    const double direct = 3.5 + 0.473e-3 * k.plan.clocks + 0.189e-9 * 18.0 * N * (H + 1) * (W + 2) * C * K;
+    const double transformed = 3.5 + 0.674e-6 * 36.0 * tiles * (2.0 * C + 4.0 * K) + 0.202e-6 * 72.0 * C * K;
+    // (small images: three dependent kernels take 18 us whatever their size)
+    k.preferred = k.plan.n_tiles > 0 && direct <= (transformed > 18.0 ? transformed : 18.0);
+    return &k;
+}
+
+extern "C" int sd_winograd_direct_preferred(int N, int H, int W, int C, int K) {
+    if (N <= 0 || H <= 0 || W <= 0 || C <= 0 || K <= 0 || !conv_direct_fits(N, H, W, C, K)) return 0;
+    WinogradDeviceState* st = nullptr;
+    if (winograd_setup(&st) != SD_ATTN_OK) return 0;
+    return conv_direct_choice(st, N, H, W, C, K)->preferred ? 1 : 0;
 }
 
 extern "C" int sd_winograd_direct_supported(int N, int H, int W, int C, int K) {
@@ -1675,19 +1713,7 @@ extern "C" int sd_winograd_direct_forward(const void* x, const void* packed, con
     WinogradDeviceState* st = nullptr;
     const int rc = winograd_setup(&st);
     if (rc != SD_ATTN_OK) return rc;
-    // (the plan depends on the shape only: a layer's next call finds its own)
-    struct Known { int N, H, W, C, K; const WinogradDeviceState* st; ConvDirectPlan plan; };
-    static thread_local Known known[8];
-    static thread_local int known_next = 0;
-    const ConvDirectPlan* plan = nullptr;
-    for (const Known& k : known)
-        if (k.st == st && k.N == N && k.H == H && k.W == W && k.C == C && k.K == K) plan = &k.plan;
-    if (!plan) {
-        Known& k = known[known_next];
-        known_next = (known_next + 1) % 8;
-        k = {N, H, W, C, K, st, plan_conv_direct(st, N, H, W, C, K)};
-        plan = &k.plan;
-    }
+    const ConvDirectPlan* plan = &conv_direct_choice(st, N, H, W, C, K)->plan;
     if (plan->n_tiles == 0) return SD_ATTN_ERR_UNSUPPORTED;
 
     ConvDirectArgs a;

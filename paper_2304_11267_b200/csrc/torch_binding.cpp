@@ -195,7 +195,7 @@ PyObject* conv3x3_impl(PyObject* const* a) {
     const int64_t N = x->size(0), H = x->size(1), W = x->size(2);
     void* stream;
     if (!stream_of(a[6], *x, &stream)) return nullptr;
-    if (N > 0 && !sd_winograd_direct_supported((int)N, (int)H, (int)W, (int)C, (int)K)) return PyLong_FromLong(SD_ATTN_ERR_UNSUPPORTED);
+    if (N > 0 && !sd_winograd_direct_preferred((int)N, (int)H, (int)W, (int)C, (int)K)) return PyLong_FromLong(SD_ATTN_ERR_UNSUPPORTED);
     Tensor made;
     const Tensor* out = &made;
     if (a[5] == Py_None) made = empty_on(*x, {N, H, W, (int64_t)K});

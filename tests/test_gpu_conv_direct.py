@@ -82,3 +82,21 @@ def test_arguments(bd):
     assert f(264, 256, 0, 256, 1, 8, 8, 16, 16, 0) == bd.ERR_ALIGNMENT
     assert bd.sd_winograd_direct_pack_filter(0, 256, 16, 16, 0) == bd.ERR_INVALID_VALUE
     assert bd.sd_winograd_direct_pack_filter(256, 256, 12, 16, 0) == bd.ERR_UNSUPPORTED
+
+
+def test_the_faster_of_the_two(bd):
+    """Small images and few channels go to the direct kernel, the largest calls to the transformed domain."""
+    assert bd.sd_winograd_direct_preferred(2, 64, 64, 320, 320) and bd.sd_winograd_direct_preferred(2, 8, 8, 1280, 1280)
+    assert not bd.sd_winograd_direct_preferred(1, 6, 127, 72, 40) and not bd.sd_winograd_direct_preferred(0, 8, 8, 64, 64)
+    N, H, W, C, K = 4, 24, 24, 2560, 1280
+    assert not bd.sd_winograd_direct_preferred(N, H, W, C, K)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn(N, H, W, C, generator=g, device="cuda").half()
+    w = (torch.randn(K, 3, 3, C, generator=g, device="cuda") / (9 * C) ** 0.5).half()
+    layer = bd.WinogradConv3x3(w)
+    y = layer(x)
+    assert torch.equal(y, layer._transformed(x, None, None))
+    direct = torch.empty_like(y)
+    assert bd.sd_winograd_direct_forward(x.data_ptr(), layer._packed.data_ptr(), 0, direct.data_ptr(), N, H, W, C, K,
+                                         torch.cuda.current_stream().cuda_stream) == bd.OK
+    assert float((y.float() - direct.float()).norm() / direct.float().norm()) < 6e-3
