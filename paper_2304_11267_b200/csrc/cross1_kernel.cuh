@@ -18,6 +18,10 @@
 // output and bank traffic of a tile halve (256 x 77, d = 160, B = 2: 5.8 -> 5.2 us; 32 rows gain nothing more).
 // Measured against the persistent kernel (cross2) and the one-tile kernel before it: 4096 x 77 d = 40 7.3 -> 6.1 us, 1024 x 77
 // d = 80 5.7 -> 5.0, 256 x 77 d = 160 6.2 -> 5.2, 64 x 64 d = 160 5.3 -> 4.4 (CUDA graphs).
+// The maximum as anchor, where a weight above it needs no second look, against an anchor at the first score (CUDA graphs, us):
+// 64 keys 4.4 -> 4.4 (16 x 64 rows, d = 160), 17.1 -> 17.4 (64 x 4096, d = 40); 16 keys 4.55 -> 4.7; 128 keys 5.35 -> 5.4, 35.1 ->
+// 37.2.  The largest weight is then exact; the error that the weights' rounding leaves in the result falls from 2.0e-4 to 1.6e-4 for
+// logits of deviation 1, from 1.8e-4 to 6.8e-5 for 4 (64 keys, binary16, simulated).
 // Tensor memory: S takes KN columns; the weights P (packed 16-bit) go over its first KN / 2 and O behind them, over scores
 // that sit in registers.
 #pragma once
@@ -31,7 +35,7 @@ namespace sd_attn {
 
 constexpr int X1_THREADS = 192;            // four softmax warps (thread = query row), two MMA issuers
 constexpr int X1_GROUP_MAX = 5;            // problems of one shape per launch
-constexpr float X1_HEADROOM_LOG2 = 8.0f;   // exponents are anchored 2^8 above the first key's weight (see cross2_kernel.cuh)
+constexpr float X1_HEADROOM_LOG2 = 8.0f;   // 65..80 keys: exponents are anchored 2^8 above the first key's weight (see cross2_kernel.cuh)
 constexpr float X1_SUM_LIMIT = 4096.0f;    // no weight above 2^12 reaches the 16-bit pack
 enum { SITE_X1_QK = 90, SITE_X1_V = 91, SITE_X1_S = 92, SITE_X1_P = 93, SITE_X1_O = 94 };
 
@@ -204,7 +208,7 @@ cross1_attention_kernel(const __grid_constant__ Cross1ArgsT<NP> args) {
                 tma_load_4d(v_smem + ch * KN * CHUNK_ROW_BYTES, &pr.tv, bar_v, ch * CHUNK_COLS, 0, hz, bz);
         }
         __syncwarp();
-        // ---- softmax: thread = query row = TMEM lane; 32 scores at a time, the weights stay in registers
+        // ---- softmax: thread = query row = TMEM lane; the weights stay in registers
         const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
         const int valid = args.Nk;
         const float c2 = pr.scale_log2e;
@@ -215,40 +219,73 @@ cross1_attention_kernel(const __grid_constant__ Cross1ArgsT<NP> args) {
         ok = __all_sync(0xffffffffu, ok);
         if (ok) {
             tc_fence_after_sync();
-#pragma unroll 1
-            for (int attempt = 0; attempt < 2; ++attempt) {
-                uint64_t acc[2] = {0ull, 0ull};
-                float tail = 0.f;
-#pragma unroll
-                for (int c = 0; c < KN; c += 32) {
-                    uint32_t s[32];
-                    if (c + 32 <= KN) tmem_ld32(tmem_s + lane_off + c, s);
-                    else tmem_ld16(tmem_s + lane_off + c, *reinterpret_cast<uint32_t(*)[16]>(s));
-                    tmem_wait_ld();
-                    if (c == 0 && attempt == 0) anchor = __uint_as_float(s[0]) * c2 + X1_HEADROOM_LOG2;
-                    const float neg_mc = -anchor;
-                    const uint64_t c2c2 = pack_b64(__float_as_uint(c2), __float_as_uint(c2));
-                    const uint64_t nmnm = pack_b64(__float_as_uint(neg_mc), __float_as_uint(neg_mc));
-                    if (c + 32 <= KN) {
-                        if (valid >= c + 32) exp2_pack_32<0, 16, BF>(s, c2c2, nmnm, &packed[c / 2], acc);
-                        else exp2_pack_32_masked<16, BF>(s, c2, neg_mc, c, valid, &packed[c / 2], tail);   // (keys past Nk: zeros)
-                    } else {
-                        exp2_pack_32_masked<8, BF>(s, c2, neg_mc, c, valid, &packed[c / 2], tail);
-                    }
-                }
-                row_sum = sum_f32x2(acc[0], acc[1]) + tail;   // S_i of Eq. 4, relative to the anchor
-                const bool over = !(row_sum <= X1_SUM_LIMIT);
-                if (attempt == 1 || !__any_sync(0xffffffffu, over)) break;
-                // rare: the row maximum lies far above the first score.  Nothing has been stored yet: take L_i of Eq. 4
-                // from the scores and redo the row.
+            uint64_t acc[2] = {0ull, 0ull};
+            float tail = 0.f;
+            auto load_32 = [&](int c, uint32_t* s) {   // scores c .. c + 31 (fewer at the end of 80)
+                if (c + 32 <= KN) tmem_ld32(tmem_s + lane_off + c, *reinterpret_cast<uint32_t(*)[32]>(s));
+                else tmem_ld16(tmem_s + lane_off + c, *reinterpret_cast<uint32_t(*)[16]>(s));
+            };
+            auto weights_32 = [&](int c, const uint32_t* s) {   // their weights, packed, and the weights' sum
+                const float neg_mc = -anchor;
+                const uint64_t c2c2 = pack_b64(__float_as_uint(c2), __float_as_uint(c2));
+                const uint64_t nmnm = pack_b64(__float_as_uint(neg_mc), __float_as_uint(neg_mc));
+                if (c + 32 > KN) exp2_pack_32_masked<8, BF>(s, c2, neg_mc, c, valid, &packed[c / 2], tail);
+                else if (valid >= c + 32) exp2_pack_32<0, 16, BF>(s, c2c2, nmnm, &packed[c / 2], acc);
+                else exp2_pack_32_masked<16, BF>(s, c2, neg_mc, c, valid, &packed[c / 2], tail);   // (keys past Nk: zeros)
+            };
+            if constexpr (KN != 80) {
+                // Anchored at the maximum, L_i of Eq. 4: the largest weight is 1, which 16 bits hold exactly.  A block of scores is
+                // held in registers (DENSE: of 32, so that a fourth CTA fits); only 128 keys, and DENSE, fetch one again.
+                constexpr int HELD = DENSE ? 32 : 64;
+                uint32_t s[HELD];
                 float row_max = -INFINITY;
-                for (int c = 0; c < KN; c += 16) {
-                    uint32_t s[16];
-                    tmem_ld16(tmem_s + lane_off + c, s);
+#pragma unroll
+                for (int c = 0; c < KN; c += HELD) {
+#pragma unroll
+                    for (int u = 0; u < HELD; u += 32) load_32(c + u, &s[u]);
                     tmem_wait_ld();
-                    row_max = fmaxf(row_max, row_max_masked<16>(s, valid - c));
+                    row_max = fmaxf(row_max, valid >= c + HELD ? row_max_3<HELD>(s) : row_max_first<HELD>(s, valid - c));
                 }
                 anchor = row_max * c2;
+#pragma unroll
+                for (int c = KN - HELD; c >= 0; c -= HELD) {   // (from the end: the last block is there)
+                    if (c < KN - HELD) {
+#pragma unroll
+                        for (int u = 0; u < HELD; u += 32) load_32(c + u, &s[u]);
+                        tmem_wait_ld();
+                    }
+#pragma unroll
+                    for (int u = HELD - 32; u >= 0; u -= 32) weights_32(c + u, &s[u]);
+                }
+                row_sum = sum_f32x2(acc[0], acc[1]) + tail;   // S_i of Eq. 4, relative to the anchor
+            } else {
+                // as the persistent kernel anchors them, so that the two give the same bits
+#pragma unroll 1
+                for (int attempt = 0; attempt < 2; ++attempt) {
+                    acc[0] = acc[1] = 0ull;
+                    tail = 0.f;
+#pragma unroll
+                    for (int c = 0; c < KN; c += 32) {
+                        uint32_t s[32];
+                        load_32(c, s);
+                        tmem_wait_ld();
+                        if (c == 0 && attempt == 0) anchor = __uint_as_float(s[0]) * c2 + X1_HEADROOM_LOG2;
+                        weights_32(c, s);
+                    }
+                    row_sum = sum_f32x2(acc[0], acc[1]) + tail;
+                    const bool over = !(row_sum <= X1_SUM_LIMIT);
+                    if (attempt == 1 || !__any_sync(0xffffffffu, over)) break;
+                    // rare: the row maximum lies far above the first score.  Nothing has been stored yet: take the maximum
+                    // from the scores and redo the row.
+                    float row_max = -INFINITY;
+                    for (int c = 0; c < KN; c += 16) {
+                        uint32_t s[16];
+                        tmem_ld16(tmem_s + lane_off + c, s);
+                        tmem_wait_ld();
+                        row_max = fmaxf(row_max, row_max_masked<16>(s, valid - c));
+                    }
+                    anchor = row_max * c2;
+                }
             }
 #pragma unroll
             for (int c = 0; c < KN / 2; c += 8) tmem_st8(tmem_s + lane_off + c, *reinterpret_cast<uint32_t(*)[8]>(&packed[c]));

@@ -67,6 +67,34 @@ __device__ __forceinline__ float row_max_masked(const uint32_t* s, int valid) {
     return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
 }
 
+// Maximum of N scores (a multiple of 8), two per instruction.
+__device__ __forceinline__ float max_3(float a, uint32_t b, uint32_t c) {
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(__uint_as_float(b)), "f"(__uint_as_float(c)));
+    return d;
+}
+template <int N>
+__device__ __forceinline__ float row_max_3(const uint32_t* s) {
+    float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+    for (int c = 0; c < N; c += 2) m[(c >> 1) & 3] = max_3(m[(c >> 1) & 3], s[c], s[c + 1]);
+    return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+}
+// Maximum over the first `valid` of N scores; -inf where there are none.  The mask's bits become predicates eight at a time.
+template <int N>
+__device__ __forceinline__ float row_max_first(const uint32_t* s, int valid) {
+    float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+    for (int c0 = 0; c0 < N; c0 += 32) {
+        const int n = valid - c0;
+        const uint32_t mask = n >= 32 ? 0xffffffffu : n <= 0 ? 0u : (1u << n) - 1u;
+#pragma unroll
+        for (int c = 0; c < 32; ++c)
+            if ((mask >> c) & 1u) m[c & 3] = fmaxf(m[c & 3], __uint_as_float(s[c0 + c]));
+    }
+    return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+}
+
 __device__ __forceinline__ uint64_t add_rm_f32x2(uint64_t a, uint64_t b) {   // round toward -inf
     uint64_t d;
     asm("add.rm.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));

@@ -53,3 +53,24 @@ def test_row_tiles_and_the_line_between_the_kernels(bd, B, Nq, d):
     ref, _, _ = oracle.forward(q, k, v, scale, rows=rows)
     for opts in ({}, {"cross_one_tile": 1}):
         parity.check(run(bd, q, k, v, scale, **opts).reshape(-1, d)[rows], ref, v, what="%d x 77 d=%d %s" % (Nq, d, opts))
+
+
+@pytest.mark.parametrize("dtype", ["float16", "bfloat16"])
+@pytest.mark.parametrize("Nk", [2, 64, 81, 128])
+def test_the_largest_weight_is_exact(bd, Nk, dtype):
+    """Up to 64 and from 81 keys a row's exponents are anchored at its maximum, so the largest weight is 1 and only the others
+    are rounded, by u = 2^-11 (bfloat16: 2^-8) of themselves.  Where the others make up less than a quarter of the row's sum, a
+    constant V = 1 comes back as 1 +- u / 4 (+ 128 half steps of binary16's subnormals, 2^-18), which rounds to 1: the next value
+    below is u away.  With the anchor at another score the largest weight itself is off by up to u, and a fifth of the rows are
+    not 1.  Here the second key leads the first by 1.5 to 2.25 and the others by 7.5 to 11.25."""
+    r = 1.0 + 0.5 * torch.rand(2, 4, 512, 1, generator=torch.Generator().manual_seed(Nk))
+    q = (r * torch.ones(64)).to(getattr(torch, dtype))
+    k = torch.full((2, 4, Nk, 64), -6.0 / 8.0).to(q.dtype)
+    k[:, :, 0], k[:, :, 1] = 0.0, 1.5 / 8.0
+    p = torch.softmax(q.double() @ k.double().transpose(-1, -2) / 8.0, -1)
+    assert p.max(-1).values.min() > 0.75
+    a = bd.Attention()
+    out = a.forward(q.cuda(), k.cuda(), torch.ones_like(k).cuda())
+    a.check()
+    assert a.last_mode == bd.MODE_CROSS
+    assert bool((out == 1.0).all())
