@@ -301,8 +301,9 @@ class WinogradConv3x3:
     """A layer's prepared filter plus torch-tensor marshalling: ``WinogradConv3x3(w, bias)(x)`` with
     w [K,3,3,C], bias [K] or None, x [N,H,W,C] float16 CUDA tensors (channels-last memory) -> y [N,H,W,K].
 
-    Images go to the direct convolution where it is the faster one; the others (the largest calls, and images too wide for it)
-    through the transformed domain, whose filter ``U`` is made when the first of them comes."""
+    Images go to the direct convolution where it is the faster one, the others (the largest calls, and images too wide for it)
+    through the transformed domain.  Both forms of the filter, and what a device needs once, are made here: a later call may be
+    the first of its kind and under stream capture, where nothing can be made that an uncaptured call could rely on."""
 
     def __init__(self, w, bias=None, stream: Optional[int] = None):
         import torch
@@ -311,11 +312,14 @@ class WinogradConv3x3:
         self.K, self.C = int(w.shape[0]), int(w.shape[3])
         self.bias = bias.contiguous() if bias is not None else None
         self._packed = torch.empty(sd_winograd_direct_filter_elems(self.K, self.C), dtype=torch.float16, device=w.device)
+        self.U = torch.empty(sd_winograd_filter_elems(self.K, self.C), dtype=torch.float16, device=w.device)
         s = stream if stream is not None else torch.cuda.current_stream(w.device).cuda_stream
         rc = sd_winograd_direct_pack_filter(w.data_ptr(), self._packed.data_ptr(), self.K, self.C, s)
         if rc != OK:
             raise SdAttnError(rc, "sd_winograd_direct_pack_filter")
-        self._U = None
+        rc = sd_winograd_transform_filter(w.data_ptr(), self.U.data_ptr(), self.K, self.C, s)
+        if rc != OK:
+            raise SdAttnError(rc, "sd_winograd_transform_filter")
         self._workspace = None
 
     def _filter(self):
@@ -325,22 +329,6 @@ class WinogradConv3x3:
         at = torch.arange(8, device=p.device)[None, :] ^ (torch.arange(p.shape[2], device=p.device) & 7)[:, None]
         p = torch.gather(p, 3, at[None, None, :, :, None].expand(p.shape))
         return p.permute(2, 1, 0, 3, 4).reshape(p.shape[2], 3, 3, -1)[:self.K, :, :, :self.C].contiguous()
-
-    @property
-    def U(self):
-        """The filter in the transformed domain (made on the current stream at first use)."""
-        import torch
-        if self._U is None:
-            w = self._filter()
-            U = torch.empty(sd_winograd_filter_elems(self.K, self.C), dtype=torch.float16, device=w.device)
-            rc = sd_winograd_transform_filter(w.data_ptr(), U.data_ptr(), self.K, self.C,
-                                              torch.cuda.current_stream(w.device).cuda_stream)
-            if rc != OK:
-                raise SdAttnError(rc, "sd_winograd_transform_filter")
-            if not torch.cuda.is_current_stream_capturing():
-                torch.cuda.current_stream(w.device).synchronize()   # (once: later calls may come on any stream)
-            self._U = U
-        return self._U
 
     def __call__(self, x, out=None, stream: Optional[int] = None):
         r = (_torch_ext or _ext()).conv3x3(x, self._packed, self.bias, self.K, self.C, out, stream)
@@ -354,16 +342,12 @@ class WinogradConv3x3:
         import torch
         N, H, W, _ = (int(v) for v in x.shape)
         s = stream if stream is not None else torch.cuda.current_stream(x.device).cuda_stream
-        U = self._U
-        if U is None:
-            with torch.cuda.stream(torch.cuda.ExternalStream(s, device=x.device)):
-                U = self.U   # (its first use is ordered before this call)
         need = sd_winograd_workspace_bytes(N, H, W, self.C, self.K)
         if self._workspace is None or self._workspace.numel() < need:
             self._workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=x.device)
         if out is None:
             out = torch.empty(N, H, W, self.K, dtype=torch.float16, device=x.device)
-        rc = sd_winograd_conv3x3_forward(x.data_ptr(), U.data_ptr(), self.bias.data_ptr() if self.bias is not None else 0,
+        rc = sd_winograd_conv3x3_forward(x.data_ptr(), self.U.data_ptr(), self.bias.data_ptr() if self.bias is not None else 0,
                                          out.data_ptr(), self._workspace.data_ptr(), self._workspace.numel(), N, H, W, self.C,
                                          self.K, s)
         if rc != OK:

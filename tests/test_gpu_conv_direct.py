@@ -100,3 +100,20 @@ def test_the_faster_of_the_two(bd):
     assert bd.sd_winograd_direct_forward(x.data_ptr(), layer._packed.data_ptr(), 0, direct.data_ptr(), N, H, W, C, K,
                                          torch.cuda.current_stream().cuda_stream) == bd.OK
     assert float((y.float() - direct.float()).norm() / direct.float().norm()) < 6e-3
+
+
+@pytest.mark.parametrize("N,H,W,C,K", [(1, 6, 130, 72, 40), (1, 16, 16, 64, 64)])   # through either domain
+def test_a_layers_first_call_may_be_captured(bd, N, H, W, C, K):
+    """What the capture leaves behind must serve an eager call although the graph has not run yet."""
+    x, w, b = wg.make(90, N, H, W, C, K)
+    layer = bd.WinogradConv3x3(torch.from_numpy(w).cuda(), torch.from_numpy(b).cuda())
+    tx = torch.from_numpy(x).cuda()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        captured = layer(tx)
+    ref = oracle.conv3x3_forward(x, w, b)
+    wg.check(layer(tx).cpu().numpy(), ref, "eager call after the capture")
+    g.replay()
+    wg.check(captured.cpu().numpy(), ref, "replay")
+    rc, detail = bd.sd_winograd_query_status()
+    assert rc == bd.OK, detail
