@@ -320,7 +320,6 @@ class WinogradConv3x3:
         rc = sd_winograd_transform_filter(w.data_ptr(), self.U.data_ptr(), self.K, self.C, s)
         if rc != OK:
             raise SdAttnError(rc, "sd_winograd_transform_filter")
-        self._workspace = None
 
     def _filter(self):
         """The filter [K,3,3,C] back from the packed one (pieces of eight channels, swizzled by the filter's number)."""
@@ -343,13 +342,17 @@ class WinogradConv3x3:
         N, H, W, _ = (int(v) for v in x.shape)
         s = stream if stream is not None else torch.cuda.current_stream(x.device).cuda_stream
         need = sd_winograd_workspace_bytes(N, H, W, self.C, self.K)
-        if self._workspace is None or self._workspace.numel() < need:
-            self._workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=x.device)
         if out is None:
             out = torch.empty(N, H, W, self.K, dtype=torch.float16, device=x.device)
-        rc = sd_winograd_conv3x3_forward(x.data_ptr(), self.U.data_ptr(), self.bias.data_ptr() if self.bias is not None else 0,
-                                         out.data_ptr(), self._workspace.data_ptr(), self._workspace.numel(), N, H, W, self.C,
-                                         self.K, s)
+        # The workspace comes from the caching allocator, for this call and in the order of its stream: one kept by the layer would be
+        # shared by calls on other streams, and one that grows would leave a captured graph with memory that is someone else's.
+        workspace = torch.cuda.caching_allocator_alloc(need, x.device, s) if need else 0
+        try:
+            rc = sd_winograd_conv3x3_forward(x.data_ptr(), self.U.data_ptr(), self.bias.data_ptr() if self.bias is not None else 0,
+                                             out.data_ptr(), workspace, need, N, H, W, self.C, self.K, s)
+        finally:
+            if need:
+                torch.cuda.caching_allocator_delete(workspace)
         if rc != OK:
             raise SdAttnError(rc, "sd_winograd_conv3x3_forward")
         return out

@@ -117,3 +117,34 @@ def test_a_layers_first_call_may_be_captured(bd, N, H, W, C, K):
     wg.check(captured.cpu().numpy(), ref, "replay")
     rc, detail = bd.sd_winograd_query_status()
     assert rc == bd.OK, detail
+
+
+def test_the_transformed_domains_workspace_belongs_to_one_call(bd):
+    """Calls on two streams at once do not share it, nor does a captured call keep memory that a larger one has given back."""
+    g = torch.Generator(device="cuda").manual_seed(5)
+    w = (torch.randn(64, 3, 3, 64, generator=g, device="cuda") / 24.0).half()
+    layer = bd.WinogradConv3x3(w)
+    small, large = (torch.randn(1, h, 200, 64, generator=g, device="cuda").half() for h in (24, 96))
+    want_small, want_large = layer(small), layer(large)
+    assert not bd.sd_winograd_direct_supported(*large.shape, 64)
+    side = torch.cuda.Stream()
+    outs = [torch.empty_like(small) for _ in range(40)]
+    torch.cuda.synchronize()
+    got = []
+    for out in outs:
+        with torch.cuda.stream(side):
+            got.append((layer(large), want_large))
+        got.append((layer(small), want_small))
+        got.append((layer(small, out=out, stream=side.cuda_stream), want_small))
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in got)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        captured = layer(small)
+    layer(large)
+    held = [torch.full((1 << 20,), 7.0, device="cuda") for _ in range(40)]   # whatever was given back is someone else's now
+    captured.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(captured, want_small)
+    assert all(bool((t == 7.0).all()) for t in held)
