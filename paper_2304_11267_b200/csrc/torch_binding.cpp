@@ -55,6 +55,13 @@ Tensor empty_on(const Tensor& like, at::IntArrayRef sizes) {
     return at::detail::empty_cuda(sizes, like.scalar_type(), like.device(), std::nullopt);
 }
 
+// Lets other Python threads run: an allocation may wait for the device, and a launch waits where its queue is full -- perhaps for
+// a host function that itself needs the interpreter.  No Python call inside.
+struct OtherThreadsRun {
+    PyThreadState* state = PyEval_SaveThread();
+    ~OtherThreadsRun() { PyEval_RestoreThread(state); }
+};
+
 // The result object: the caller's `out` where one was given, else the new tensor.
 PyObject* result(PyObject* out, Tensor&& made) {
     if (out == Py_None) return THPVariable_Wrap(std::move(made));
@@ -100,10 +107,14 @@ PyObject* attention_impl(PyObject* const* a) {
     if (!stream_of(a[7], *q, &stream)) return nullptr;
     Tensor made;
     const Tensor* out = &made;
-    if (a[6] == Py_None) made = empty_on(*q, s);
-    else if (!(out = tensor_of(a[6], "out"))) return nullptr;
-    const int rc = sd_attn_forward(h, q->data_ptr(), k->data_ptr(), v->data_ptr(), out->data_ptr(), (int)s[0], (int)H, (int)Nq,
-                                   (int)Nk, (int)d, (float)scale, dtype, stream);
+    if (a[6] != Py_None && !(out = tensor_of(a[6], "out"))) return nullptr;
+    int rc;
+    {
+        OtherThreadsRun scope;
+        if (out == &made) made = empty_on(*q, s);
+        rc = sd_attn_forward(h, q->data_ptr(), k->data_ptr(), v->data_ptr(), out->data_ptr(), (int)s[0], (int)H, (int)Nq, (int)Nk,
+                             (int)d, (float)scale, dtype, stream);
+    }
     if (rc != SD_ATTN_OK) return PyLong_FromLong(rc);
     return result(a[6], std::move(made));
 }
@@ -127,14 +138,17 @@ PyObject* geglu_impl(PyObject* const* a) {
     if (!stream_of(a[2], *x, &stream)) return nullptr;
     Tensor made;
     const Tensor* out = &made;
-    if (a[1] == Py_None) {
-        c10::SmallVector<int64_t, 5> sizes(x->sizes().begin(), x->sizes().end());
-        sizes[dim - 1] = C;
-        made = empty_on(*x, sizes);
-    } else if (!(out = tensor_of(a[1], "out"))) {
-        return nullptr;
+    if (a[1] != Py_None && !(out = tensor_of(a[1], "out"))) return nullptr;
+    int rc;
+    {
+        OtherThreadsRun scope;
+        if (out == &made) {
+            c10::SmallVector<int64_t, 5> sizes(x->sizes().begin(), x->sizes().end());
+            sizes[dim - 1] = C;
+            made = empty_on(*x, sizes);
+        }
+        rc = sd_geglu_forward(x->data_ptr(), out->data_ptr(), rows, (int)C, dtype, stream);
     }
-    const int rc = sd_geglu_forward(x->data_ptr(), out->data_ptr(), rows, (int)C, dtype, stream);
     if (rc != SD_ATTN_OK) return PyLong_FromLong(rc);
     return result(a[1], std::move(made));
 }
@@ -172,10 +186,14 @@ PyObject* groupnorm_impl(PyObject* const* a) {
     if (!stream_of(a[6], *x, &stream)) return nullptr;
     Tensor made;
     const Tensor* out = &made;
-    if (a[5] == Py_None) made = empty_on(*x, x->sizes());
-    else if (!(out = tensor_of(a[5], "out"))) return nullptr;
-    const int rc = sd_groupnorm_forward(x->data_ptr(), affine[0], affine[1], out->data_ptr(), (int)N, (int)C, HW, (int)groups,
-                                        (float)eps, dtype, stream);
+    if (a[5] != Py_None && !(out = tensor_of(a[5], "out"))) return nullptr;
+    int rc;
+    {
+        OtherThreadsRun scope;
+        if (out == &made) made = empty_on(*x, x->sizes());
+        rc = sd_groupnorm_forward(x->data_ptr(), affine[0], affine[1], out->data_ptr(), (int)N, (int)C, HW, (int)groups, (float)eps, dtype,
+                                  stream);
+    }
     if (rc != SD_ATTN_OK) return PyLong_FromLong(rc);
     return result(a[5], std::move(made));
 }
@@ -195,13 +213,18 @@ PyObject* conv3x3_impl(PyObject* const* a) {
     const int64_t N = x->size(0), H = x->size(1), W = x->size(2);
     void* stream;
     if (!stream_of(a[6], *x, &stream)) return nullptr;
-    if (N > 0 && !sd_winograd_direct_preferred((int)N, (int)H, (int)W, (int)C, (int)K)) return PyLong_FromLong(SD_ATTN_ERR_UNSUPPORTED);
     Tensor made;
     const Tensor* out = &made;
-    if (a[5] == Py_None) made = empty_on(*x, {N, H, W, (int64_t)K});
-    else if (!(out = tensor_of(a[5], "out"))) return nullptr;
-    const int rc = sd_winograd_direct_forward(x->data_ptr(), packed->data_ptr(), bias ? bias->data_ptr() : nullptr, out->data_ptr(), (int)N,
-                                              (int)H, (int)W, (int)C, (int)K, stream);
+    if (a[5] != Py_None && !(out = tensor_of(a[5], "out"))) return nullptr;
+    int rc = SD_ATTN_ERR_UNSUPPORTED;
+    {
+        OtherThreadsRun scope;
+        if (N == 0 || sd_winograd_direct_preferred((int)N, (int)H, (int)W, (int)C, (int)K)) {
+            if (out == &made) made = empty_on(*x, {N, H, W, (int64_t)K});
+            rc = sd_winograd_direct_forward(x->data_ptr(), packed->data_ptr(), bias ? bias->data_ptr() : nullptr, out->data_ptr(), (int)N,
+                                            (int)H, (int)W, (int)C, (int)K, stream);
+        }
+    }
     if (rc != SD_ATTN_OK) return PyLong_FromLong(rc);
     return result(a[5], std::move(made));
 }
