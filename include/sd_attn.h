@@ -55,7 +55,11 @@ typedef enum {
 typedef enum {
     SD_ATTN_F16 = 0, /* IEEE binary16 q/k/v/out, binary32 accumulation            */
     SD_ATTN_F32 = 1, /* binary32 throughout: plain FMAs, or (AUTO, d % 4 == 0) products of operands split exactly into
-                        three bfloat16 parts on the tensor cores, accumulated in binary32; never TF32        */
+                        three bfloat16 parts on the tensor cores, accumulated in binary32; never TF32.  Rows that
+                        come out infinite or NaN on the tensor cores (inputs above the largest bfloat16, products that
+                        overflow on the way) are computed once more with plain FMAs, so the upper end of the range,
+                        infinities and NaNs behave as there; inputs below 2^-109 in magnitude are read with an
+                        absolute error of up to 2^-134                                                        */
     SD_ATTN_BF16 = 2 /* bfloat16 q/k/v/out, binary32 accumulation; the softmax weights enter the second product
                         rounded to bfloat16 (8 significant bits), so results are about 8x coarser than F16's.
                         Implemented by FUSED, CROSS and SIMT; TWOPASS mode answers UNSUPPORTED.              */

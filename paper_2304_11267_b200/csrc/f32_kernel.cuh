@@ -24,6 +24,10 @@
 // The exponents are anchored at the row maximum of the FIRST key tile: bf16 parts have binary32's range, so a later score may
 // lie 2^64 above it before anything overflows; only then (the sum of a tile's weights says so) is the row re-anchored and the
 // tile redone.
+// The ends of binary32's range: a value above the largest bfloat16 (or an infinity) has no three parts, and weights of up to 2^64 may
+// overflow a product whose result is finite.  Either leaves an infinity or a NaN in the row's output, never a wrong finite value:
+// rows whose output is not finite are computed once more by the warp that holds them, with plain FMAs.  Values below 2^-109 lose
+// their lowest bits (the parts end at bfloat16's smallest subnormal, 2^-133).
 // Operands in shared memory are [part h, m, l][32-column chunk][row][64 bytes].  V is used as it lies (MN-major).  Where one
 // query tile leaves room in tensor memory, its Q goes there: read from shared memory, 128 rows for each product of 32 or 64 keys
 // were most of the product's time.
@@ -51,6 +55,7 @@ struct F32Args {
     HeadLayout lq, lk;      // heads of q and out (Nq rows each), of k and v (Nk rows)
     int Nq, Nk, d;
     int units_per_head;     // ceil(query tiles of a head / T)
+    float scale;
     float scale_log2e;      // |scale| * log2(e)
     int negate;             // scale < 0: the tensor core negates Q
     FastDiv by_pieces;      // division by the eight-column pieces of a row
@@ -163,6 +168,67 @@ struct F32Converter {
             if (at_s[u] >= 0) f32_store_at(tile + (at_s[u] & ~1), NC * ROWS * 64, lo[u], hi[u]);
     }
 };
+
+// Columns c0 .. c0 + cols - 1 of one output row by one warp, with the operations of simt_kernel.cuh in their order.  For the rows the
+// split operands cannot serve (see above), whose loads come straight from global memory: with a NaN in every head, so that all rows of
+// 16 x 4096 x 4096, d = 40, are redone, a call takes 21.7 ms (the CUDA-core kernel 3.9); without one 294 us before and after.
+template <int ACC>
+__device__ __forceinline__ void f32_plain_row(const F32Args& a, int bh, int row, int c0, int cols, int lane) {
+    constexpr int CC = (ACC + 31) / 32, GROUP = 8;
+    const float* q = head_row(a.q, a.lq, bh, row);
+    const float* k = head_row(a.k, a.lk, bh, 0);
+    const float* v = head_row(a.v, a.lk, bh, 0) + c0 + lane;
+    const long long ld = a.lk.ld;
+    float m = -INFINITY, l = 0.f, o[CC];
+#pragma unroll
+    for (int cc = 0; cc < CC; ++cc) o[cc] = 0.f;
+#pragma unroll 1
+    for (int j0 = 0; j0 < a.Nk; j0 += 32) {
+        float score = -INFINITY;
+        if (j0 + lane < a.Nk) {   // lane = key
+            const float* kj = k + (j0 + lane) * ld;
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+            for (int c = 0; c < a.d; c += 4) {
+                const float4 qq = __ldg(reinterpret_cast<const float4*>(q + c)), kk = __ldg(reinterpret_cast<const float4*>(kj + c));
+                acc.x = fmaf(qq.x, kk.x, acc.x);
+                acc.y = fmaf(qq.y, kk.y, acc.y);
+                acc.z = fmaf(qq.z, kk.z, acc.z);
+                acc.w = fmaf(qq.w, kk.w, acc.w);
+            }
+            score = a.scale * ((acc.x + acc.y) + (acc.z + acc.w));
+        }
+        float mx = score;
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
+        const float m_new = fmaxf(m, mx), alpha = expf(m - m_new), p = expf(score - m_new);
+        m = m_new;
+        l = l * alpha + p;
+#pragma unroll
+        for (int cc = 0; cc < CC; ++cc) o[cc] *= alpha;
+#pragma unroll 1
+        for (int g = 0; g < 32; g += GROUP) {   // lane = column
+            float x[GROUP][CC];
+#pragma unroll
+            for (int u = 0; u < GROUP; ++u)
+#pragma unroll
+                for (int cc = 0; cc < CC; ++cc)
+                    x[u][cc] = j0 + g + u < a.Nk && cc * 32 + lane < cols ? __ldg(v + (j0 + g + u) * ld + cc * 32) : 0.f;
+#pragma unroll
+            for (int u = 0; u < GROUP; ++u) {
+                const float pj = __shfl_sync(0xffffffffu, p, g + u);
+#pragma unroll
+                for (int cc = 0; cc < CC; ++cc) o[cc] = fmaf(pj, x[u][cc], o[cc]);
+            }
+        }
+    }
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) l += __shfl_xor_sync(0xffffffffu, l, s);
+    float* out = head_row(a.out, a.lq, bh, row) + c0 + lane;
+#pragma unroll
+    for (int cc = 0; cc < CC; ++cc)
+        if (cc * 32 + lane < cols) out[cc * 32] = o[cc] / l;
+}
 
 template <typename SH>
 __global__ void __launch_bounds__(SH::THREADS, 1)
@@ -556,14 +622,19 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                 static_assert(8 * 32 * PITCH * 4 <= SH::Q_TILE, "staging");
                 const float inv = 1.f / (half_s[t][0][wt] + half_s[t][1][wt]);
                 const uint32_t stage = q_smem + t * SH::Q_TILE + (uint32_t)((half * 4 + (warp & 3)) * 32 * PITCH * 4);
+                float zero = 0.f;   // (until a value is not finite)
 #pragma unroll
                 for (int c = 0; c < ACC; c += 4) {
                     uint32_t x[4];
                     unpack_b64(o[c / 2], x[0], x[1]);
                     unpack_b64(o[c / 2 + 1], x[2], x[3]);
-                    st_shared_v4(stage + (lane * PITCH + c) * 4,
-                                 make_uint4(__float_as_uint(__uint_as_float(x[0]) * inv), __float_as_uint(__uint_as_float(x[1]) * inv),
-                                            __float_as_uint(__uint_as_float(x[2]) * inv), __float_as_uint(__uint_as_float(x[3]) * inv)));
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float y = __uint_as_float(x[i]) * inv;
+                        zero = fmaf(y, 0.f, zero);
+                        x[i] = __float_as_uint(y);
+                    }
+                    st_shared_v4(stage + (lane * PITCH + c) * 4, make_uint4(x[0], x[1], x[2], x[3]));
                 }
                 __syncwarp();
                 const int row0 = row_base + t * TILE_M + (warp & 3) * 32, rows = args.Nq - row0 < 32 ? args.Nq - row0 : 32;
@@ -576,6 +647,8 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                         *reinterpret_cast<uint4*>(out + (long long)r * args.lq.ld) = v;
                     }
                 }
+                uint32_t again = __ballot_sync(0xffffffffu, !(zero == 0.f) && lane < rows);
+                for (; again; again &= again - 1) f32_plain_row<ACC>(args, bh, row0 + __ffs(again) - 1, c0, cols, lane);
             }
         }
     }

@@ -545,6 +545,7 @@ static int launch_f32(sd_attn_handle* h, const Problem& p) {
     a.lq = head_layout(p.heads, p.BH, p.Nq, p.d);
     a.lk = head_layout(p.heads, p.BH, p.Nk, p.d);
     a.Nq = p.Nq; a.Nk = p.Nk; a.d = p.d;
+    a.scale = p.scale;
     a.scale_log2e = fabsf(p.scale) * LOG2E;
     a.negate = p.scale < 0.f;
     a.by_pieces = make_fast_div((uint32_t)(p.d + 7) / 8);

@@ -82,3 +82,47 @@ def test_scores_that_leave_the_anchor_behind(bd, d):
     scores = np.einsum("bhid,bhjd->bhij", q.astype(np.float64), k.astype(np.float64)) * scale
     assert (scores[..., 210:].max(-1) - scores[..., :32].max(-1)).max() > 64 * np.log(2.0)
     check(run(bd, q, k, v, scale), ref, v, 1e-4)
+
+
+@pytest.mark.parametrize("d,H,Nq", [(40, 2, 150), (40, 8, 2500), (80, 2, 150), (160, 2, 150)])   # the four variants
+@pytest.mark.parametrize("what", ["inf in V", "largest V", "inf in K", "largest K", "nan in Q", "V and rising scores"])
+def test_the_ends_of_the_range(bd, what, d, H, Nq):
+    """Values without three bfloat16 parts, and weights whose products overflow although the result is finite: what the plain kernel
+    returns comes back, infinities and NaNs included."""
+    g = torch.Generator().manual_seed(d + Nq)
+    q, k, v = (torch.randn(1, H, n, d, generator=g) for n in (Nq, 200, 200))
+    if what == "inf in V":
+        v[0, 1, 70, 3] = float("inf")
+        v[0, 1, 9, d - 1] = float("-inf")
+    elif what == "largest V":
+        v[0, 1, 70, 3] = v[0, 0, 9, d - 1] = torch.finfo(torch.float32).max
+    elif what == "inf in K":        # a score of -inf: weight zero
+        q[0, 1, :, 5] = q[0, 1, :, 5].abs() + 0.1
+        k[0, 1, 70, 5] = float("-inf")
+    elif what == "largest K":       # scores of some 1e38, of either sign
+        k[0, 1, 70, 5] = torch.finfo(torch.float32).max
+        q[0, 1, :, 5] *= 0.1
+    elif what == "nan in Q":
+        q[0, 0, Nq - 1, 0] = q[0, 1, 17, 2] = float("nan")
+    else:                           # weights near 2^47 against the first key tile's maximum times V near 2^90
+        q = 0.5 + 0.5 * torch.rand(q.shape, generator=g)
+        k *= 0.01
+        k[:, :, 150] += 33.0 / 0.75 / d ** 0.5
+        v *= 2.0 ** 90
+    q, k, v = q.cuda(), k.cuda(), v.cuda()
+    plain = bd.Attention(mode=bd.MODE_SIMT).forward(q, k, v)
+    a = bd.Attention()
+    got = a.forward(q, k, v)
+    a.check()
+    assert bool(torch.isfinite(plain).all()) == (what not in ("inf in V", "nan in Q"))
+    torch.testing.assert_close(got, plain, rtol=1e-5, atol=1e-5 * float(v[v.isfinite() & (v.abs() < 1e37)].abs().max()), equal_nan=True)
+
+
+@pytest.mark.parametrize("d", [40, 80, 160])
+def test_small_values(bd, d):
+    """V near 2^-100 has its three parts, and Q near 2^-60 against K near 2^60."""
+    q, k, v = draw(d + 1, 1, 2, 150, 150, d)
+    scale = float(np.float32(d ** -0.5))
+    ref = oracle.forward(q, k, v, scale)[0]
+    got = run(bd, q * np.float32(2.0 ** -60), k * np.float32(2.0 ** 60), v * np.float32(2.0 ** -100), scale)
+    check(got.astype(np.float64) * 2.0 ** 100, ref, v)
