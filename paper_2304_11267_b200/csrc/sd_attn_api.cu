@@ -540,6 +540,7 @@ static int launch_f32_as(sd_attn_handle* h, const Problem& p, F32Args& a) {
 // binary32 tensors with d % 4 == 0: three-way split operands on the tensor cores.  Two query tiles per CTA (d <= 48) as soon
 // as the tiles outnumber the SMs: they share the conversion of K and V, and one's softmax runs under the other's products.
 static int launch_f32(sd_attn_handle* h, const Problem& p) {
+    if (!h->f32_ok) return SD_ATTN_ERR_UNSUPPORTED;   // (an error, not the plain kernel: that one takes thirteen times as long)
     F32Args a;
     a.q = (const float*)p.q; a.k = (const float*)p.k; a.v = (const float*)p.v; a.out = (float*)p.out;
     a.lq = head_layout(p.heads, p.BH, p.Nq, p.d);
@@ -920,7 +921,7 @@ static int launch_one(sd_attn_handle* h, const Problem& p, int mode, int dtype) 
     switch (mode) {
         case SD_ATTN_MODE_SIMT:
             // AUTO's binary32 kernel; the CUDA-core kernel serves the other types, d % 4 != 0 and callers that ask for it
-            if (dtype == SD_ATTN_F32 && h->mode == SD_ATTN_MODE_AUTO && p.d % 4 == 0 && h->f32_ok) return launch_f32(h, p);
+            if (dtype == SD_ATTN_F32 && h->mode == SD_ATTN_MODE_AUTO && p.d % 4 == 0) return launch_f32(h, p);
             return dtype == SD_ATTN_F16    ? launch_simt<__half>(h, p)
                    : dtype == SD_ATTN_BF16 ? launch_simt<__nv_bfloat16>(h, p)
                                            : launch_simt<float>(h, p);

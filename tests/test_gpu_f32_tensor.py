@@ -1,9 +1,10 @@
 """AUTO's binary32 kernel (three-way split operands on the tensor cores) at the edges of its variants, against the oracle.
 
 Bounds: the split products are exact to 2^-24 and every tile's sum is rounded to nearest, so the error is binary32's: 2e-6 of
-max |V| and 2e-6 relative L2 (measured at most 5e-7), a fifth of the path's stated tolerance.  Scores in the hundreds carry
-their own rounding (2^-24 of a score of 500 moves a weight by 3e-5): those cases use the stated 1e-5 against a softmax whose
-weights sit on few keys."""
+max |V| and 2e-6 relative L2 (measured at most 5e-7), a fifth of the path's stated tolerance.  Scores carry their own
+rounding into the weights, 2^-24 of a score: those cases have bounds of their own, the stated 1e-5 for scores of up to 20 (1e-6 of a
+weight) and 1e-4 for scores of up to a thousand (6e-5).  AUTO reports SIMT for both binary32 kernels and the plain one would meet these
+bounds too; which one ran shows in the bits."""
 import numpy as np
 import pytest
 
@@ -116,6 +117,18 @@ def test_the_ends_of_the_range(bd, what, d, H, Nq):
     a.check()
     assert bool(torch.isfinite(plain).all()) == (what not in ("inf in V", "nan in Q"))
     torch.testing.assert_close(got, plain, rtol=1e-5, atol=1e-5 * float(v[v.isfinite() & (v.abs() < 1e37)].abs().max()), equal_nan=True)
+
+
+@pytest.mark.parametrize("d,H,Nq", [(40, 2, 150), (40, 8, 2500), (80, 2, 150), (160, 2, 150)])   # the four variants
+def test_auto_runs_on_the_tensor_cores(bd, d, H, Nq):
+    """The two kernels add in different orders and round differently: over thousands of values their bits differ; the plain
+    kernel in AUTO's place would give its own."""
+    t = [torch.from_numpy(x).cuda() for x in draw(d + 7, 1, H, Nq, 400, d)]
+    auto, plain = bd.Attention(), bd.Attention(mode=bd.MODE_SIMT)
+    got, want = auto.forward(*t), plain.forward(*t)
+    assert auto.last_mode == plain.last_mode == bd.MODE_SIMT
+    assert float((got != want).float().mean()) > 0.1
+    torch.testing.assert_close(got, want, rtol=1e-5, atol=1e-5)
 
 
 @pytest.mark.parametrize("d", [40, 80, 160])
