@@ -1650,7 +1650,9 @@ static ConvDirectPlan plan_conv_direct(const WinogradDeviceState* st, int N, int
 }
 
 // The plan of a shape and whether it is expected to beat the transformed domain: both depend on the shape only, so a layer's
-// next call finds its own.
+// next call finds its own.  A plan is a hundred candidates, 0.7 us; a denoising step has some twenty shapes of 3x3
+// convolution at one image size, and the table holds three such sizes.
+constexpr int CD_KNOWN_SHAPES = 64;
 struct ConvDirectChoice {
     int N, H, W, C, K;
     const WinogradDeviceState* st;
@@ -1658,12 +1660,12 @@ struct ConvDirectChoice {
     bool preferred;
 };
 static const ConvDirectChoice* conv_direct_choice(const WinogradDeviceState* st, int N, int H, int W, int C, int K) {
-    static thread_local ConvDirectChoice known[8];
+    static thread_local ConvDirectChoice known[CD_KNOWN_SHAPES];
     static thread_local int known_next = 0;
     for (const ConvDirectChoice& k : known)
         if (k.st == st && k.N == N && k.H == H && k.W == W && k.C == C && k.K == K) return &k;
     ConvDirectChoice& k = known[known_next];
-    known_next = (known_next + 1) % 8;
+    known_next = (known_next + 1) % CD_KNOWN_SHAPES;
     k = {N, H, W, C, K, st, plan_conv_direct(st, N, H, W, C, K), false};
     // Microseconds, fitted to 29 shapes of 25 to 220 GFLOP run back to back over three sets of tensors.  The direct kernel: its
     // plan's clocks and, for the clock rate under a full tensor core, its operations.  The transformed domain: its
