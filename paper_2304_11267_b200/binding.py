@@ -276,7 +276,10 @@ def sd_winograd_direct_supported(N, H, W, C, K) -> bool:
 
 
 def sd_winograd_direct_preferred(N, H, W, C, K) -> bool:
-    return bool(load().sd_winograd_direct_preferred(N, H, W, C, K))
+    r = load().sd_winograd_direct_preferred(N, H, W, C, K)
+    if r < 0:
+        raise SdAttnError(-r, "sd_winograd_direct_preferred")
+    return r == 1
 
 
 def sd_winograd_direct_filter_elems(K: int, C: int) -> int:

@@ -1683,7 +1683,8 @@ static const ConvDirectChoice* conv_direct_choice(const WinogradDeviceState* st,
 extern "C" int sd_winograd_direct_preferred(int N, int H, int W, int C, int K) {
     if (N <= 0 || H <= 0 || W <= 0 || C <= 0 || K <= 0 || !conv_direct_fits(N, H, W, C, K)) return 0;
     WinogradDeviceState* st = nullptr;
-    if (winograd_setup(&st) != SD_ATTN_OK) return 0;
+    const int rc = winograd_setup(&st);
+    if (rc != SD_ATTN_OK) return -rc;
     return conv_direct_choice(st, N, H, W, C, K)->preferred ? 1 : 0;
 }
 

@@ -216,10 +216,12 @@ PyObject* conv3x3_impl(PyObject* const* a) {
     Tensor made;
     const Tensor* out = &made;
     if (a[5] != Py_None && !(out = tensor_of(a[5], "out"))) return nullptr;
-    int rc = SD_ATTN_ERR_UNSUPPORTED;
+    int rc;
     {
         OtherThreadsRun scope;
-        if (N == 0 || sd_winograd_direct_preferred((int)N, (int)H, (int)W, (int)C, (int)K)) {
+        const int preferred = N == 0 ? 1 : sd_winograd_direct_preferred((int)N, (int)H, (int)W, (int)C, (int)K);
+        rc = preferred < 0 ? -preferred : SD_ATTN_ERR_UNSUPPORTED;
+        if (preferred > 0) {
             if (out == &made) made = empty_on(*x, {N, H, W, (int64_t)K});
             rc = sd_winograd_direct_forward(x->data_ptr(), packed->data_ptr(), bias ? bias->data_ptr() : nullptr, out->data_ptr(), (int)N,
                                             (int)H, (int)W, (int)C, (int)K, stream);

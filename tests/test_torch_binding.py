@@ -31,3 +31,12 @@ def test_bad_tensors_raise(bd, call):
     else:
         with pytest.raises(TypeError):
             bd._ext().geglu(x)
+
+
+@pytest.mark.skipif(torch.cuda.is_available(), reason="needs a machine whose CUDA calls fail")
+def test_a_failing_device_is_an_error_and_not_an_answer(bd):
+    """Which convolution is the faster one depends on the device; sizes that neither takes are answered without it."""
+    assert not bd.sd_winograd_direct_preferred(1, 6, 127, 72, 40)
+    with pytest.raises(bd.SdAttnError) as raised:
+        bd.sd_winograd_direct_preferred(2, 64, 64, 320, 320)
+    assert raised.value.status in (bd.ERR_CUDA, bd.ERR_ARCH)
