@@ -58,8 +58,9 @@ int sd_winograd_conv3x3_forward(const void *x, const void *U, const void *bias, 
  * binary32 and rounded once -- no scratch and no error of the transforms.  It is supported for images up to 126 positions wide
  * (sd_winograd_direct_supported answers 1 or 0 for a shape, without a device) and the faster of the two up to some 50 billion
  * operations a call: sd_winograd_direct_preferred answers 1 where it is supported and expected to be the faster one on the
- * current device, 0 where it is not, and minus an sd_attn_status where the device could not be asked.  The filter w [K][3][3][C] is laid out once per layer in the order the kernel reads it
- * (sd_winograd_direct_pack_filter: sd_winograd_direct_filter_elems(K, C) binary16 values, 9 K C up to padding).
+ * current device, 0 where it is not, and minus an sd_attn_status where the device could not be asked.  The filter w
+ * [K][3][3][C] is laid out once per layer in the order the kernel reads it (sd_winograd_direct_pack_filter:
+ * sd_winograd_direct_filter_elems(K, C) binary16 values, 9 K C up to padding).
  * Errors: INVALID_VALUE, UNSUPPORTED (C or K not a multiple of 8, or a shape it does not cover), ALIGNMENT, ARCH, CUDA; a
  * bounded wait that expires is reported by sd_winograd_query_status.
  */

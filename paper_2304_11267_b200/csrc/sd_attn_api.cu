@@ -682,14 +682,21 @@ static int launch_cross1_group(sd_attn_handle* h, const Problem* ps, int n) {
 }
 
 // The persistent kernel (65..80 keys) keeps K and V of a head for all its tiles and hides a tile's chain behind other tiles';
-// one CTA per tile has the shorter chain.  The line: four tiles per SM, about what is resident at once (5525 x 77 d = 40, 704
-// tiles: 8.4 us either way; 2304 x 77 d = 80 B = 4, 576 tiles: 9.6 against 9.9 persistent; B = 16: 32.4 against 28.1), and
-// token-major tensors of d <= 48, whose K and V rows are the costly ones to fetch (4096 x 77 d = 40: 8.1 against 7.4).  The two
-// kernels give the same bits (the same products, exponents and order of additions), so a group may take the other one than
+// one CTA per tile has the shorter chain.  The line, in tiles of all the launch's problems:
+//   four per SM, about what is resident at once (5525 x 77 d = 40, 704 tiles: 8.4 us either way; 2304 x 77 d = 80 B = 4, 576 tiles:
+//     9.6 against 9.9 persistent; B = 16: 32.4 against 28.1);
+//   token-major tensors of d <= 48, whose K and V rows are the costly ones to fetch: half an SM, where the one-tile kernel's tiles of
+//     64 rows still have an SM each (d = 40, one-tile against persistent: 64 tiles 4.6 / 5.1 us, 72 4.6 / 5.1, 80 5.3 / 5.3, 128
+//     6.9 / 5.4, 512 11.0 / 7.5; at 88 to 120 tiles either may be ahead, by 0.4);
+//   several such problems in one launch, whose argument block costs the persistent kernel 2 us more: two per SM (five of 256 rows,
+//     80 tiles 5.9 / 7.6, five of 512, 160 tiles 6.8 / 8.4, five of 1024, 320 tiles 9.2 / 9.35).
+// The two kernels give the same bits (the same products, exponents and order of additions), so a group may take the other one than
 // its problems would alone.
 static bool cross_is_persistent(const sd_attn_handle* h, const Problem& p, int n) {
     if (!cross2_supports(p.Nk, p.d) || h->opt.cross_one_tile) return false;
-    return (long long)((p.Nq + TILE_M - 1) / TILE_M) * p.BH * n > 4ll * h->sm_count || (p.heads > 0 && p.d <= 48);
+    const long long tiles = (long long)((p.Nq + TILE_M - 1) / TILE_M) * p.BH * n, sms = h->sm_count;
+    if (p.heads > 0 && p.d <= 48) return n == 1 ? 2 * tiles > sms : tiles > 2 * sms;
+    return tiles > 4 * sms;
 }
 
 // `n` problems of one shape (BH, Nq, Nk, d, layout, dtype alike) in one launch.

@@ -55,6 +55,31 @@ def test_row_tiles_and_the_line_between_the_kernels(bd, B, Nq, d):
         parity.check(run(bd, q, k, v, scale, **opts).reshape(-1, d)[rows], ref, v, what="%d x 77 d=%d %s" % (Nq, d, opts))
 
 
+# token-major calls at the line between the kernels: one tile, half an SM's worth of tiles and one more; groups at two per SM
+@pytest.mark.parametrize("dtype", ["float16", "bfloat16"])
+@pytest.mark.parametrize("n,Nq,Nk,d", [(1, 1, 65, 40), (1, 1153, 77, 40), (1, 1183, 80, 48), (1, 1185, 77, 8), (3, 700, 77, 40),
+                                       (5, 947, 80, 24), (4, 1300, 65, 48)])
+def test_token_major_line_between_the_kernels(bd, n, Nq, Nk, d, dtype):
+    g = torch.Generator(device="cuda").manual_seed(Nq + d)
+    sets = [tuple(torch.randn(1, m, 8, d, generator=g, device="cuda").to(getattr(torch, dtype)) for m in (Nq, Nk, Nk)) for _ in range(n)]
+    results = []
+    for options in ({}, {"cross_one_tile": 1}):
+        a = bd.Attention(layout=bd.LAYOUT_BNHD, options=bd.Options(**options))
+        outs = [torch.zeros_like(q) for q, _, _ in sets]
+        problems = bd.make_problems([(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), 1, 8, Nq, Nk, d, d ** -0.5)
+                                     for (q, k, v), o in zip(sets, outs)])
+        code = bd.F16 if dtype == "float16" else bd.BF16
+        assert bd.sd_attn_forward_batch(a.handle, problems, code, torch.cuda.current_stream().cuda_stream) == bd.OK
+        results.append(outs + [a.forward(*t) for t in sets])
+        a.check()
+    for i in range(n):
+        assert torch.equal(results[0][i], results[0][n + i])                                              # the group and the call alone
+        assert torch.equal(results[0][i], results[1][i]) and torch.equal(results[0][i], results[1][n + i])   # either kernel
+        q, k, v = (t.transpose(1, 2).double() for t in sets[i])
+        ref = (torch.softmax(q @ k.transpose(-1, -2) * d ** -0.5, -1) @ v).transpose(1, 2)
+        assert float((results[0][i].double() - ref).norm() / ref.norm()) < (2e-3 if dtype == "float16" else 1.6e-2)
+
+
 @pytest.mark.parametrize("dtype", ["float16", "bfloat16"])
 @pytest.mark.parametrize("Nk", [2, 64, 81, 128])
 def test_the_largest_weight_is_exact(bd, Nk, dtype):
