@@ -538,7 +538,11 @@ static int launch_f32_as(sd_attn_handle* h, const Problem& p, F32Args& a) {
 }
 
 // binary32 tensors with d % 4 == 0: three-way split operands on the tensor cores.  Two query tiles per CTA (d <= 48) as soon
-// as the tiles outnumber the SMs: they share the conversion of K and V, and one's softmax runs under the other's products.
+// as the tiles outnumber the SMs: they share the conversion of K and V, and one's softmax runs under the other's products.  One
+// wave of two-tile CTAs takes 1.2 to 1.4 times a wave of one-tile ones, so the line is where the latter need a second wave (d = 40,
+// two tiles against one, us: 148 tiles 131 / 93 at 4096 keys, 40 / 30 at 1024, 11.9 / 9.9 at 77; 152 tiles 131 / 183, 40 / 55, 11.8 /
+// 16.8; 304 263 / 273, 77 / 83, 22 / 25; 592 78 / 113 at 1024; only at 296 tiles, all 148 SMs with two, are two waves of one ahead:
+// 227 / 185, 67 / 57, 20 / 19).
 static int launch_f32(sd_attn_handle* h, const Problem& p) {
     if (!h->f32_ok) return SD_ATTN_ERR_UNSUPPORTED;   // (an error, not the plain kernel: that one takes thirteen times as long)
     F32Args a;
