@@ -39,7 +39,7 @@ ROTATING_SETS = 8   # 8 x 42 MB of q/k/v/out for the two variants = 336 MB, abov
 # ncu capture of the kernel instance named here (profiles/fused4s_c2_self_4096_d40.md): q, k, v read once (15.73 MB
 # algorithmic) and next to nothing written during the launch -- the 5.2 MB of output are still in the 126 MB L2 when
 # the kernel ends.  A constant from a capture: it moves only when the capture is redone.
-FUSED_TRAFFIC = {"bytes_per_launch": 15801344, "kernel_instance": "fused4s_attention_kernel<2, 1, 1, 0>(Fused4Args)",
+FUSED_TRAFFIC = {"bytes_per_launch": 15804928, "kernel_instance": "fused4s_attention_kernel<2, 1, 1, 0>(Fused4Args)",
                  "capture": "profiles/fused4s_c2_self_4096_d40.md"}
 # Of every 8 exponentials of the d = 40 kernel this many go to the FMA pipe (F4S_POLY_PER8 in fused4s_kernel.cuh), and
 # FMA-pipe results per score element: scale, row sum, half a pack on the special-function path; 6 more on the
@@ -268,7 +268,8 @@ def run_ours(args):
         for i in range(max(args.warmup, 3) + args.steps):
             layer(xs[i % 4], out=y, stream=stream)
         torch.cuda.synchronize()
-        print(json.dumps({"kernel_loop_only": True, "workload": "winograd", "launches": 3 * (max(args.warmup, 3) + args.steps)}))
+        per_call = 1 if bd.sd_winograd_direct_preferred(N, H, W, C, K) else 3
+        print(json.dumps({"kernel_loop_only": True, "workload": "winograd", "launches": per_call * (max(args.warmup, 3) + args.steps)}))
         return 0
     if args.workload == "geglu":
         sets = geglu_sets(device, 4)
@@ -797,16 +798,23 @@ WG_SHAPE = (2, 64, 64, 320, 320)      # N, H, W, C, K: a 3x3 convolution of the 
 
 
 def winograd_numbers(bd, device, stream, peaks):
-    """The Winograd 3x3 convolution (Sec. 3.3) on one UNet layer shape: microseconds per call (input transform, 36
-    GEMMs, output transform), the rate in terms of the direct convolution's FLOPs, and the oracle on a sample."""
+    """The 3x3 convolution (Sec. 3.3) on one UNet layer shape, through the domain the layer chooses for it: microseconds per
+    call, the rates in terms of the direct convolution's FLOPs and of the products that domain has, and the oracle on a sample."""
     import torch
     import oracle
     N, H, W, C, K = WG_SHAPE
+
+    def domain(n):
+        """Of a batch of n: the name, kernels per call, products on the tensor cores, filter values per channel pair."""
+        if bd.sd_winograd_direct_preferred(n, H, W, C, K):
+            return "direct", 1, 2.0 * n * H * W * 9 * C * K, 9
+        return "transformed", 3, 2.0 * 36 * n * ((H + 3) // 4) * ((W + 3) // 4) * C * K, 36
+
     g = torch.Generator(device=device).manual_seed(11)
     w = (torch.randn(K, 3, 3, C, device=device, generator=g) / (9.0 * C) ** 0.5).to(torch.float16)
     b = (0.1 * torch.randn(K, device=device, generator=g)).to(torch.float16)
     layer = bd.WinogradConv3x3(w, b, stream)
-    n_sets = 16       # 16 x (5.2 MB in + 5.2 MB out): with the 7.4 MB filter and 35 MB of scratch, more than the L2
+    n_sets = 16       # 16 x (5.2 MB in + 5.2 MB out): more than the L2
     xs = [torch.randn(N, H, W, C, device=device, generator=g).to(torch.float16) for _ in range(n_sets)]
     ys = [torch.empty(N, H, W, K, device=device, dtype=torch.float16) for _ in range(n_sets)]
     for i in range(4):
@@ -824,9 +832,9 @@ def winograd_numbers(bd, device, stream, peaks):
         raise bd.SdAttnError(rc, "winograd device status %s" % detail)
     us = 1e3 * start.elapsed_time(end) / iters
     direct_flops = 2.0 * N * H * W * K * C * 9
-    tiles = N * ((H + 3) // 4) * ((W + 3) // 4)
-    gemm_flops = 2.0 * 36 * tiles * K * C
-    io_bytes = 2.0 * (N * H * W * C + N * H * W * K + 36 * K * C)
+    name, launches, tensor_flops, filter_values = domain(N)
+    io_bytes = 2.0 * (N * H * W * C + N * H * W * K + filter_values * K * C)
+    us_tensor, us_hbm = tensor_flops / (peaks["tflops"] * 1e6), io_bytes / (peaks["hbm_gbs"] * 1e3)
     # the oracle, timed on the first rows of the first image (a few seconds of CPU work)
     hs, ws_ = 9, 64
     x0 = xs[0][:1, :hs + 1].cpu().numpy()
@@ -835,9 +843,9 @@ def winograd_numbers(bd, device, stream, peaks):
     cpu_s = time.perf_counter() - t0
     got = ys[0][:1, :hs].cpu().numpy().astype("float64")
     rel = float(((got - ref) ** 2).sum() ** 0.5 / ((ref ** 2).sum() ** 0.5))
-    # the same layer at 16 times the batch: enough tiles for many waves of GEMM CTAs (the rate of the kernels
-    # themselves, where the UNet's own shape is a chain of three short kernels)
+    # the same layer at 16 times the batch: enough tiles for many waves of CTAs
     NB = 16 * N
+    name_b, launches_b, tensor_flops_b, _ = domain(NB)
     xb = torch.randn(NB, H, W, C, device=device, generator=g).to(torch.float16)
     yb = torch.empty(NB, H, W, K, device=device, dtype=torch.float16)
     for _ in range(2):
@@ -850,15 +858,17 @@ def winograd_numbers(bd, device, stream, peaks):
     torch.cuda.synchronize()
     us_b = 1e3 * start.elapsed_time(end) / 5
     del xb, yb
-    return {"us_per_call": us, "launches_per_call": 3,
-            "at_16x_batch": {"us_per_call": us_b, "direct_conv_tflops_equivalent": 16 * direct_flops / (us_b * 1e-6) / 1e12,
-                             "gemm_tflops": 16 * gemm_flops / (us_b * 1e-6) / 1e12},
+    return {"us_per_call": us, "domain": name, "launches_per_call": launches,
+            "at_16x_batch": {"us_per_call": us_b, "domain": name_b, "launches_per_call": launches_b,
+                             "direct_conv_tflops_equivalent": 16 * direct_flops / (us_b * 1e-6) / 1e12,
+                             "gemm_tflops": tensor_flops_b / (us_b * 1e-6) / 1e12},
             "direct_conv_tflops_equivalent": direct_flops / (us * 1e-6) / 1e12,
-            "gemm_tflops": gemm_flops / (us * 1e-6) / 1e12,
-            "bound": "hbm", "algorithmic_bytes": io_bytes, "achieved_gbs": io_bytes / (us * 1e-6) / 1e9,
-            "peak_gbs": peaks["hbm_gbs"], "frac": io_bytes / (us * 1e-6) / 1e9 / peaks["hbm_gbs"],
-            "peak_source": peaks["source"],
-            "note": "x + y + transformed filter are the algorithmic bytes; V and M (35 MB) go through the L2",
+            "gemm_tflops": tensor_flops / (us * 1e-6) / 1e12,
+            "bound": "tensor" if us_tensor > us_hbm else "hbm", "frac": max(us_tensor, us_hbm) / us,
+            "algorithmic_bytes": io_bytes, "achieved_gbs": io_bytes / (us * 1e-6) / 1e9,
+            "peak_gbs": peaks["hbm_gbs"], "peak_tflops": peaks["tflops"], "peak_source": peaks["source"],
+            "note": "x + y + the filter in the form that runs are the algorithmic bytes; frac is of the larger of their time and "
+                    "that of the products",
             "rel_l2_vs_oracle_on_sample": rel,
             "cpu_oracle_gflops": 2.0 * 1 * (hs + 1) * ws_ * K * C * 9 / cpu_s / 1e9,
             "cpu_oracle_sample": "%d of %d rows of one image" % (hs + 1, H)}
