@@ -70,7 +70,7 @@ typedef enum {
     SD_ATTN_MODE_FUSED = 1,   /* single-pass online softmax (FlashAttention, Sec. 3.2.2)      */
     SD_ATTN_MODE_CROSS = 2,   /* all keys in one shared-memory tile, plain softmax            */
     SD_ATTN_MODE_TWOPASS = 3, /* partially fused softmax of Sec. 3.2.1: scores and [L,S] in HBM */
-    SD_ATTN_MODE_SIMT = 4     /* CUDA-core kernel, F16 or F32 storage, fp32 arithmetic        */
+    SD_ATTN_MODE_SIMT = 4     /* CUDA-core kernel, any storage, fp32 arithmetic               */
 } sd_attn_mode;
 
 typedef enum {
@@ -98,7 +98,7 @@ typedef struct {
                               complete before it reads or writes global memory, so stream order is kept      */
     int fused_tiles;       /* 1..4: fixed number of query tiles per CTA of the FUSED kernel (0: by problem size) */
     int fused_split;       /* FUSED with one query tile per CTA: 2 or 4 warpgroups share its key tiles, 1 none
-                              (0: by head dim)                                                                */
+                              (0: by head dim: 4 up to 64, 3 up to 96, else 2)                                 */
     int fused_shares;      /* 1: FUSED deals the (group of query tiles, key tile) steps of a problem out in equal
                               shares to one CTA per SM, so that no SM idles in a last, partly filled wave; a group
                               whose key range is cut between CTAs is finished through scratch the handle then owns

@@ -31,7 +31,8 @@
 // Operands in shared memory are [part h, m, l][32-column chunk][row][64 bytes].  V is used as it lies (MN-major).  Where one
 // query tile leaves room in tensor memory, its Q goes there: read from shared memory, 128 rows for each product of 32 or 64 keys
 // were most of the product's time.
-// us, operands of S in shared memory, undivided issuing loops, rows stored one by one -> now: 16 x 4096 x 4096, d = 40 285 -> 261;
+// us in a graph, operands of S in shared memory, undivided issuing loops, rows stored one by one -> now: 16 x 4096 x 4096, d = 40 285 ->
+// 262 (293 a call through the entry point with other work between);
 // 16 x 1024, d = 80 40.1 -> 34.8; 16 x 256, d = 160 35.6 -> 27.8; 16 x 256 x 77, d = 160 21.1 -> 16.1.
 // Every wait is bounded and reports to the status block.
 #pragma once

@@ -141,8 +141,8 @@ __device__ __noinline__ void f4s_store_piece(float* piece, uint32_t tmem_o, int 
 // (tcgen05.ld -> exp2 -> tcgen05.st -> hand-over: 1400-1500 clocks per key tile, measured, against 600 per tile
 // with four tiles resident); the parts work on different key tiles at the same time, so their chains overlap as
 // those of four query tiles do, and they need no agreement on an anchor because their products never share an
-// accumulator.  The score buffers run ahead of the products (NB of them, a multiple of SPLIT), and the MMAs come from
-// two threads: the products of key tile j from one, the scores of key tile j + NB from the other.
+// accumulator.  The score buffers run ahead of the products (NB of them, SPLIT to 2 SPLIT: 4 of 3 parts at d = 80, 5 of 4 at d = 40), and the MMAs
+// come from two threads: the products of key tile j from one, the scores of key tile j + NB from the other.
 template <int POLY, int NCH, int SPLIT = 1, bool BF = false>   // NCH: 64-column chunks per row (head dim <= 64 * NCH); BF: bfloat16 tensors
 __global__ void __launch_bounds__(F4_THREADS, 1)
 fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {

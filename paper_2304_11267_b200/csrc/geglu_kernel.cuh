@@ -11,9 +11,9 @@
 // reciprocal, one exp2, a dozen FMAs.  The form keeps its RELATIVE accuracy for very negative gates, where 1 + erf
 // would cancel.  A thread takes UNROLL pairs of 16-byte pieces (one of each half of a row), all fetched before it computes
 // anything, and ends; finding a piece's row is one multiplication (a 64-bit division per piece was a third of the
-// instructions).  Two elements at a time on the packed binary32 pipe come to about 16 instructions per element.
-// 8192 x 1280 fp16 (63 MB): 12.3 us = 5.1 TB/s (16.4 with the division, a grid-stride loop and 28 instructions per
-// element, launched without overlap); fp32: 19.2 us = 6.55 TB/s, the copy rate (22.3).
+// instructions).  Two elements at a time on the packed binary32 pipe come to 20 instructions per element (ncu), about 16 of them arithmetic.
+// 8192 x 1280 fp16 (63 MB): 13.0 us a call through the entry point = 4.8 TB/s, 11.9 in a graph (16.4 with the division, a grid-stride
+// loop and 28 instructions per element, launched without overlap); fp32: 19.2 us = 6.55 TB/s, the copy rate (22.3).
 #pragma once
 #include <cuda_fp16.h>
 #include <stdint.h>

@@ -994,7 +994,8 @@ extern "C" int sd_attn_forward_batch(sd_attn_handle* h, const sd_attn_problem* p
         free(modes);
         return SD_ATTN_ERR_INVALID_VALUE;
     }
-    // TWOPASS lends ONE workspace to every call and the CUDA-core kernel gains nothing from company: one after another
+    // One after another: TWOPASS lends ONE workspace to every call, and the CUDA-core kernel gains nothing from company.  (AUTO's
+    // binary32 kernel counts as SIMT and goes the same way, although its small calls leave SMs idle that others could use.)
     bool serial = !h->batch_lanes_ok || count == 1;
     for (int i = 0; i < count; ++i)
         if (modes[i] == SD_ATTN_MODE_TWOPASS || modes[i] == SD_ATTN_MODE_SIMT) serial = true;
@@ -1332,7 +1333,7 @@ static cudaError_t launch_geglu_as(const void* x, void* out, long long pieces, i
 }
 
 // Pieces per thread: two of binary16 once that still leaves every SM its eight resident blocks (8192 x 1280: 12.3 us
-// against 13.3 with one, 12.9 with four; 512 x 5120: 4.4 against 3.5), one of binary32, whose pieces hold half the values
+// against 13.3 with one, 12.9 with four, timed side by side in a loop; 512 x 5120: 4.4 against 3.5), one of binary32, whose pieces hold half the values
 // (8192 x 1280: 19.2 us = the copy rate, against 20.8 with two).
 template <typename T, int VEC>
 static cudaError_t launch_geglu(const void* x, void* out, long long pieces, int pieces_per_row, int sms, cudaStream_t s) {
