@@ -1,5 +1,4 @@
-// Single-pass attention of binary32 tensors on the bf16 tensor cores, at binary32 precision: one query tile per CTA.  (Two, d <= 48:
-// f32_two_kernel.cuh.)
+// Single-pass attention of binary32 tensors on the bf16 tensor cores, at binary32 precision.
 //
 // A binary32 value is the sum of three bfloat16 values, h = bf16(x), m = bf16(x - h), l = bf16(x - h - m): 3 x 8 bits hold
 // its 24-bit significand exactly.  A product of two such sums is taken as the six of its nine terms that reach its last
@@ -9,10 +8,10 @@
 // goes into a fresh accumulator and is added to the running output on the CUDA cores, rounded to nearest -- and inside a
 // tile the small terms are issued first.  (4096 tokens, d = 40: relative error 2.9e-7, with plain binary32 FMAs 1.2e-6.)
 //
-// Bound: six bf16 products per binary32 one, 1152 tensor clocks per 128 x 64 tile of scores at d = 40, against 6000
-// clocks of the FMA pipe.
+// Bound: six bf16 products per binary32 one, 1152 tensor clocks per 128 x 64 tile of scores at d = 40 (and reads of Q and K
+// from shared memory that make it about 1440) against 6000 clocks of the FMA pipe.
 //
-// One CTA: a query tile of 128 rows (T = 1).  Warpgroups (four warps each):
+// One CTA: T query tiles of 128 rows.  Warpgroups (four warps each):
 //   softmax     two per query tile, thread = half a query row: its scores from tensor memory into registers, exp2, row sum; the
 //               weights are split into three packed bf16 operands and stored over the scores.  Two such slots per query tile:
 //               the next key tile's scores are computed meanwhile.  The same threads hold the row's output columns, half
@@ -29,10 +28,11 @@
 // overflow a product whose result is finite.  Either leaves an infinity or a NaN in the row's output, never a wrong finite value:
 // rows whose output is not finite are computed once more by the warp that holds them, with plain FMAs.  Values below 2^-109 lose
 // their lowest bits (the parts end at bfloat16's smallest subnormal, 2^-133).
-// Operands in shared memory are [part h, m, l][32-column chunk][row][64 bytes].  V is used as it lies (MN-major).  Q goes to
-// tensor memory: read from shared memory, 128 rows for each product of 32 or 64 keys
+// Operands in shared memory are [part h, m, l][32-column chunk][row][64 bytes].  V is used as it lies (MN-major).  Where one
+// query tile leaves room in tensor memory, its Q goes there: read from shared memory, 128 rows for each product of 32 or 64 keys
 // were most of the product's time.
-// us in a graph, operands of S in shared memory, undivided issuing loops, rows stored one by one -> now:
+// us in a graph, operands of S in shared memory, undivided issuing loops, rows stored one by one -> now: 16 x 4096 x 4096, d = 40 285 ->
+// 262 (293 a call through the entry point with other work between);
 // 16 x 1024, d = 80 40.1 -> 34.8; 16 x 256, d = 160 35.6 -> 27.8; 16 x 256 x 77, d = 160 21.1 -> 16.1.
 // Every wait is bounded and reports to the status block.
 #pragma once
@@ -46,6 +46,7 @@
 namespace sd_attn {
 
 constexpr int F3_CHUNK = 32;        // columns per 64-byte swizzled row
+constexpr int F3_MAX_TILES = 2;
 enum { SITE_F_Q = 70, SITE_F_K = 71, SITE_F_KEMPTY = 72, SITE_F_V = 73, SITE_F_VEMPTY = 74, SITE_F_S = 75, SITE_F_SLOT = 76,
        SITE_F_P = 77, SITE_F_PV = 78, SITE_F_OFREE = 79 };
 
@@ -57,24 +58,21 @@ struct F32Args {
     int units_per_head;     // ceil(query tiles of a head / T)
     float scale;
     float scale_log2e;      // |scale| * log2(e)
-    // f32_two_kernel: |scale| * log2(e), and what the tensor core's truncation takes away from a score, as (scale_hi + scale_lo) scale_power
-    // with the significand in [1, 2) (or zero) and a power of two; the share of a product P V that it takes away
-    float scale_hi, scale_lo, scale_power, truncated;
     int negate;             // scale < 0: the tensor core negates Q
     FastDiv by_pieces;      // division by the eight-column pieces of a row
     int* status;
 };
 
-// NC: 32-column chunks of a row (d <= 32 NC).  BN: keys per key tile.  T: query tiles per CTA (one).  ACC: output columns per
+// NC: 32-column chunks of a row (d <= 32 NC).  BN: keys per key tile.  T: query tiles per CTA.  ACC: output columns per
 // softmax thread.  KS, VS: depth of the K and V rings.  NO: buffers for the product of a key tile.  MAX_FIRST: whether a key tile
 // fits the anchor is decided from its maximum before the exponentials, so that the weights replace the scores in registers,
 // not from the weights' sum behind them (measured: d = 80 43 -> 36 us; the other shapes lose 2% to 12% by it).
-template <int NC_, int BN_, int ACC_, int KS_, int VS_, int NO_, bool MAX_FIRST_>
+template <int NC_, int BN_, int T_, int ACC_, int KS_, int VS_, int NO_, bool MAX_FIRST_>
 struct F32Shape {
-    static constexpr int NC = NC_, BN = BN_, T = 1, ACC = ACC_, KS = KS_, VS = VS_, NO = NO_;
+    static constexpr int NC = NC_, BN = BN_, T = T_, ACC = ACC_, KS = KS_, VS = VS_, NO = NO_;
     static constexpr bool MAX_FIRST = MAX_FIRST_;
     static constexpr int MAX_D = NC * F3_CHUNK < 2 * ACC ? NC * F3_CHUNK : 2 * ACC;
-    static constexpr int N_CONV = 2;   // warpgroups that convert K; as many for V
+    static constexpr int N_CONV = T == 2 ? 1 : 2;   // warpgroups that convert K; as many for V
     static constexpr int WG_CONVERT = 2 * T, WG_ISSUE = WG_CONVERT + 2 * N_CONV, THREADS = (WG_ISSUE + 1) * 128;
     static constexpr int Q_PART = NC * TILE_M * 64, Q_TILE = 3 * Q_PART, KV_PART = NC * BN * 64, KV_STAGE = 3 * KV_PART;
     static constexpr int SMEM = T * Q_TILE + (KS + VS) * KV_STAGE + 1024;
@@ -83,18 +81,21 @@ struct F32Shape {
     // halves of a row need not wait for one another: word `off` of part (h, m) of half x at x BN/2 + (0, BN/4) + off, of
     // part l at BN + x BN/4 + off.
     static constexpr int HALF = BN / 2, SLOT = 3 * BN / 2, O_COLS = 2 * ACC;
+    static constexpr bool Q_TMEM = T == 1;             // (two query tiles leave 32 columns)
     static constexpr int Q_COLS = NC * F3_CHUNK / 2;   // of a part
-    static constexpr int TILE_COLS = 2 * SLOT + NO * O_COLS + 3 * Q_COLS;
+    static constexpr int TILE_COLS = 2 * SLOT + NO * O_COLS + (Q_TMEM ? 3 * Q_COLS : 0);
     static_assert(T * TILE_COLS <= 512, "tensor memory");
     // registers: the pools of setmaxnreg must not exceed what the CTA was launched with
     static constexpr int LAUNCH_REGS = 65536 / THREADS / 8 * 8;
-    static constexpr int ISSUE_REGS = 40, CONVERT_REGS = 56, SOFTMAX_REGS = 120;
+    // (a few spilled registers in the softmax loop of two query tiles cost 10%: 96 for it, what the others can spare)
+    static constexpr int ISSUE_REGS = T == 2 ? 24 : 40, CONVERT_REGS = T == 2 ? 48 : 56, SOFTMAX_REGS = T == 2 ? 96 : 120;
     static constexpr int POOL = 128 * (2 * T * SOFTMAX_REGS + 2 * N_CONV * CONVERT_REGS + ISSUE_REGS);
     static_assert(POOL <= THREADS * LAUNCH_REGS, "setmaxnreg budget");
 };
-using F32One = F32Shape<2, 64, 32, 3, 3, 2, false>;     // d <= 64
-using F32Mid = F32Shape<3, 64, 48, 2, 2, 1, true>;     // d <= 96
-using F32Wide = F32Shape<5, 32, 80, 2, 1, 1, true>;    // d <= 160
+using F32Two = F32Shape<2, 64, 2, 24, 2, 2, 1, false>;     // d <= 48, two query tiles
+using F32One = F32Shape<2, 64, 1, 32, 3, 3, 2, false>;     // d <= 64
+using F32Mid = F32Shape<3, 64, 1, 48, 2, 2, 1, true>;     // d <= 96
+using F32Wide = F32Shape<5, 32, 1, 80, 2, 1, 1, true>;    // d <= 160
 constexpr float F32_TILE_SUM_LIMIT = 1.8446744e19f; // 2^64: no weight above it reaches the products
 constexpr float F32_MAX_LIMIT = 58.f;               // log2 of the largest weight where the maximum decides: 64 of them stay below the sum
 
@@ -306,7 +307,7 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
     auto tmem_q = [&](int t) { return tmem_base + t * SH::TILE_COLS + 2 * SH::SLOT + NO * SH::O_COLS; };
     // Q_t, by the 256 threads that will work on its scores: thread i of them
     auto convert_q = [&](int t, int i) {
-        constexpr int n = 256, U = 5;
+        constexpr int n = 256, U = SH::T == 1 ? 5 : 4;
         const float* qb = head_row(args.q, args.lq, bh, 0);
         for (int first = i; first < TILE_M * pieces; first += U * n) {
             float4 lo[U], hi[U];
@@ -330,22 +331,25 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                                  lo[u], hi[u]);
             }
         }
-        // to tensor memory: thread = row, its steps of 16 columns, every second one
-        named_barrier(1 + t, 256);
-        const int row = i & 127, sw = (row >> 1) & 3;
-        const uint32_t src = q_smem + t * SH::Q_TILE + row * 64, dst = tmem_q(t) + ((uint32_t)((warp & 3) * 32) << 16);
+        if constexpr (SH::Q_TMEM) {   // thread = row: its steps of 16 columns, every second one
+            named_barrier(1 + t, 256);
+            const int row = i & 127, sw = (row >> 1) & 3;
+            const uint32_t src = q_smem + t * SH::Q_TILE + row * 64, dst = tmem_q(t) + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll
-        for (int part = 0; part < 3; ++part)
+            for (int part = 0; part < 3; ++part)
 #pragma unroll
-            for (int kk = 0; kk < 2 * NC; ++kk) {
-                if ((kk & 1) != i >> 7 || kk * 16 >= d) continue;
-                const uint32_t at = src + part * SH::Q_PART + (kk >> 1) * (TILE_M * 64);
-                const uint4 a = ld_shared_v4(at + ((((kk & 1) * 2) ^ sw) << 4)), b = ld_shared_v4(at + ((((kk & 1) * 2 + 1) ^ sw) << 4));
-                const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-                tmem_st8(dst + part * SH::Q_COLS + kk * 8, w);
-            }
-        tmem_wait_st();
-        tc_fence_before_sync();
+                for (int kk = 0; kk < 2 * NC; ++kk) {
+                    if ((kk & 1) != i >> 7 || kk * 16 >= d) continue;
+                    const uint32_t at = src + part * SH::Q_PART + (kk >> 1) * (TILE_M * 64);
+                    const uint4 a = ld_shared_v4(at + ((((kk & 1) * 2) ^ sw) << 4)), b = ld_shared_v4(at + ((((kk & 1) * 2 + 1) ^ sw) << 4));
+                    const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+                    tmem_st8(dst + part * SH::Q_COLS + kk * 8, w);
+                }
+            tmem_wait_st();
+            tc_fence_before_sync();
+        } else {
+            fence_proxy_async_smem();
+        }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bars.q_full[t]));
     };
@@ -366,7 +370,7 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                 // ------------------------------------------------------------ S_t(j) = Q_t K(j)^T
                 const uint32_t idesc = idesc_f16(TILE_M, BN, false, false, args.negate != 0, true);
                 const int ksteps = (d + 15) / 16;
-                const uint64_t k_desc = smem_desc_sw64(k_smem, 16, 512);
+                const uint64_t q_desc = smem_desc_sw64(q_smem + t * SH::Q_TILE, 16, 512), k_desc = smem_desc_sw64(k_smem, 16, 512);
                 ok = wait(bars.q_full[t], 0, SITE_F_Q, t);
                 int s = 0, pk = 0;
                 for (int j = 0; j < n_kv && ok; ++j) {
@@ -384,7 +388,11 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                             for (int kk = 0; kk < 2 * NC; ++kk)   // (offsets are constants)
                                 if (kk < ksteps) {
                                     const uint64_t kt = kd + (uint64_t)((PB[p] * SH::KV_PART + (kk >> 1) * (BN * 64) + (kk & 1) * 32) >> 4);
-                                    mma_f16_ts(ts, tmem_q(t) + PA[p] * SH::Q_COLS + kk * 8, kt, idesc, p > 0 || kk > 0);
+                                    if constexpr (SH::Q_TMEM)
+                                        mma_f16_ts(ts, tmem_q(t) + PA[p] * SH::Q_COLS + kk * 8, kt, idesc, p > 0 || kk > 0);
+                                    else
+                                        mma_f16_ss(ts, q_desc + (uint64_t)((PA[p] * SH::Q_PART + (kk >> 1) * (TILE_M * 64) + (kk & 1) * 32) >> 4),
+                                                   kt, idesc, p > 0 || kk > 0);
                                 }
                         tc_commit(smem_u32(&bars.s_full[t][b]));
                         tc_commit(smem_u32(&bars.k_empty[s]));

@@ -64,18 +64,21 @@ def test_two_query_tiles_per_cta(bd, d, Nq):
     check(run(bd, q, k, v, scale, tokens_first=True), ref, v)
 
 
-@pytest.mark.parametrize("d", [40, 80, 160])
+FOUR = pytest.mark.parametrize("d,H,Nq", [(40, 2, 150), (40, 16, 1250), (80, 2, 150), (160, 2, 150)])   # the variants
+
+
+@FOUR
 @pytest.mark.parametrize("scale", [-0.4, 0.0])
-def test_negative_and_zero_scale(bd, d, scale):
-    q, k, v = draw(d, 1, 2, 150, 150, d)
+def test_negative_and_zero_scale(bd, d, H, Nq, scale):
+    q, k, v = draw(d, 1, H, Nq, 150, d)
     check(run(bd, q, k, v, scale), oracle.forward(q, k, v, scale)[0], v, 1e-5)
 
 
-@pytest.mark.parametrize("d", [40, 80, 160])
-def test_scores_that_leave_the_anchor_behind(bd, d):
+@pytest.mark.parametrize("d,H,Nq", [(40, 2, 260), (40, 16, 1250), (80, 2, 260), (160, 2, 260)])   # the four variants
+def test_scores_that_leave_the_anchor_behind(bd, d, H, Nq):
     """The anchor is the first key tile's maximum; keys that grow 40-fold twice raise some rows' scores by hundreds, past the
     2^64 at which a row is re-anchored (and lower others', whose weights vanish)."""
-    q, k, v = draw(d, 1, 2, 260, 260, d)
+    q, k, v = draw(d, 1, H, Nq, 260, d)
     k[:, :, 100:] *= 40.0
     k[:, :, 210:] *= 6.0
     scale = float(np.float32(d ** -0.5))
@@ -131,10 +134,10 @@ def test_auto_runs_on_the_tensor_cores(bd, d, H, Nq):
     torch.testing.assert_close(got, want, rtol=1e-5, atol=1e-5)
 
 
-@pytest.mark.parametrize("d", [40, 80, 160])
-def test_small_values(bd, d):
+@FOUR
+def test_small_values(bd, d, H, Nq):
     """V near 2^-100 has its three parts, and Q near 2^-60 against K near 2^60."""
-    q, k, v = draw(d + 1, 1, 2, 150, 150, d)
+    q, k, v = draw(d + 1, 1, H, Nq, 150, d)
     scale = float(np.float32(d ** -0.5))
     ref = oracle.forward(q, k, v, scale)[0]
     got = run(bd, q * np.float32(2.0 ** -60), k * np.float32(2.0 ** 60), v * np.float32(2.0 ** -100), scale)
@@ -143,9 +146,7 @@ def test_small_values(bd, d):
 
 @pytest.mark.parametrize("d,Nq,Nk", [(40, 2500, 65), (48, 1250, 200), (4, 1250, 64), (44, 1250, 130)])   # two query tiles per CTA
 def test_columns_of_v_far_apart(bd, d, Nq, Nk):
-    """Two query tiles per CTA: V's columns are scaled one by one before they are split into two binary16 parts (2^-23 of a value at
-    most, 2^-17 of a key tile's largest below which the second part thins out), so a column's error is relative to that column.
-    Columns from 2^-90 to 2^90, keys that grow 2^10-fold: the first key tile's scale must not reach into the next one's."""
+    """Columns of V from 2^-90 to 2^90, keys that grow 2^10-fold: a column's error is relative to that column."""
     q, k, v = draw(d + Nq, 1, 16, Nq, Nk, d)
     v *= np.float32(2.0) ** np.linspace(-90, 90, d).round().astype(np.float32)
     v[:, :, 64:] *= np.float32(2.0 ** 10)
@@ -158,8 +159,8 @@ def test_columns_of_v_far_apart(bd, d, Nq, Nk):
 
 @pytest.mark.parametrize("growth", [2.0 ** 5, 2.0 ** 12, 2.0 ** 15])
 def test_weights_past_the_range_of_a_part(bd, growth):
-    """Two query tiles per CTA: the first key tile's largest weight is 2^2 and binary16 ends at 2^16.  Keys along q itself give the second
-    and third key tiles' weights a largest one of about `growth` and its square times that, in rows of some warps only."""
+    """Two query tiles per CTA: keys along q itself give the second and third key tiles a largest weight of about `growth` times the first
+    one's and its square, in rows of some warps only."""
     q, k, v = draw(77, 1, 16, 1300, 190, 40)
     q /= np.linalg.norm(q, axis=-1, keepdims=True)
     k *= 0.01
@@ -167,3 +168,59 @@ def test_weights_past_the_range_of_a_part(bd, growth):
         k[:, :, at] = q[:, :, 640] * np.float32(np.log(x) * 40 ** 0.5)
     scale = float(np.float32(40 ** -0.5))
     check(run(bd, q, k, v, scale), oracle.forward(q, k, v, scale)[0], v, 1e-5)
+
+
+def around_one_key(seed, Nk, at, spread):
+    """Sixteen heads in which key `at` lies 10 to 40 binary orders above all the others (`spread`: their deviation, in such orders).
+    More query tiles than SMs; d = 40."""
+    g = np.random.default_rng(seed)
+    q, k = np.zeros((1, 16, 1250, 40), np.float32), g.standard_normal((1, 16, Nk, 40), dtype=np.float32)
+    scale = float(np.float32(40 ** -0.5))
+    order = np.float32(np.log(2.0) / scale)
+    q[..., 0] = g.uniform(0.95, 1.05, q.shape[:3])
+    k[..., 0] *= spread * order
+    k[0, :, at, 0] = np.linspace(10, 40, 16) * order
+    return q, k, scale
+
+
+@pytest.mark.parametrize("Nk,at,spread", [(4096, 0, 0), (4096, 0, 1), (4096, 2000, 0), (9216, 5, 0)])
+@pytest.mark.parametrize("value", [0.01, 0.0])
+def test_keys_far_below_one(bd, Nk, at, spread, value):
+    """Thousands of keys far below a dominant one whose V is small, or zero: each weighs next to nothing, and together they are the
+    output.  The result is right relative to itself, head by head: 1e-5, the path's bound (scores of up to 40 binary orders carry 4e-6 of a
+    weight)."""
+    q, k, scale = around_one_key(Nk + at, Nk, at, spread)
+    v = np.random.default_rng(1).uniform(0.5, 1.0, k.shape).astype(np.float32)
+    v[:, :, at] = value
+    rows = (np.arange(16)[:, None] * 1250 + np.arange(0, 1250, 25)).ravel()
+    ref = oracle.forward(q, k, v, scale, rows=rows)[0].reshape(16, -1, 40)
+    got = run(bd, q, k, v, scale)[0, :, ::25].astype(np.float64)
+    assert np.abs(got - ref).max() <= 2e-6
+    rel = np.linalg.norm(got - ref, axis=(1, 2)) / np.linalg.norm(ref, axis=(1, 2))
+    assert rel.max() <= 1e-5, rel
+
+
+@pytest.mark.parametrize("outlier", [2.0 ** 26, 2.0 ** 30])
+def test_an_outlier_in_v_without_weight(bd, outlier):
+    """A column of V whose largest value, by far, belongs to a key without weight: the others' products are as exact as ever."""
+    q, k, v = draw(11, 1, 16, 1250, 200, 40)
+    q[..., 0], k[..., 0] = 1.0, 0.0
+    k[:, :, 3, 0] = -100.0 * 40 ** 0.5 * np.log(2.0)
+    v[:, :, 3, ::3] = outlier
+    scale = float(np.float32(40 ** -0.5))
+    check(run(bd, q, k, v, scale), oracle.forward(q, k, v, scale)[0], np.delete(v, 3, axis=2))
+
+
+def test_one_key_comes_back_as_it_is(bd):
+    """One key of weight one: V's three parts add up to V, bit by bit."""
+    q, k, v = draw(5, 1, 16, 1250, 1, 40)
+    assert np.array_equal(run(bd, q, k, v, 0.0), np.broadcast_to(v, q.shape))
+
+
+# two query tiles per CTA: a last half or whole key tile without a key, head dims around the 4-, 8- and 16-column granules
+@pytest.mark.parametrize("d", [4, 8, 20, 28, 44, 48])
+@pytest.mark.parametrize("Nk", [1, 31, 33, 63, 97])
+def test_two_query_tiles_at_the_edges(bd, d, Nk):
+    q, k, v = draw(d + Nk, 1, 16, 1250, Nk, d)
+    scale = float(np.float32(d ** -0.5))
+    check(run(bd, q, k, v, scale), oracle.forward(q, k, v, scale)[0], v)
