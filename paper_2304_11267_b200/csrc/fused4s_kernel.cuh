@@ -143,7 +143,13 @@ __device__ __noinline__ void f4s_store_piece(float* piece, uint32_t tmem_o, int 
 // those of four query tiles do, and they need no agreement on an anchor because their products never share an
 // accumulator.  The score buffers run ahead of the products (NB of them, SPLIT to 2 SPLIT: 4 of 3 parts at d = 80, 5 of 4 at d = 40), and the MMAs
 // come from two threads: the products of key tile j from one, the scores of key tile j + NB from the other.
-template <int POLY, int NCH, int SPLIT = 1, bool BF = false>   // NCH: 64-column chunks per row (head dim <= 64 * NCH); BF: bfloat16 tensors
+//
+// How closely the roles follow one another (FORM).  F4_PACED, whole units of 80 < d <= 128: a softmax warp takes its tile's last product on
+// the way to the hand-over, and the loading thread sleeps between polls.  Two tiles of such heads fall into step without:
+// us paced / plain, 16 x 2304 x 2304, d = 72 38.1 / 36.6, 80 37.4 / 35.3, 88 39.6 / 43.5, 96 38.0 / 43.1, 112 39.0 / 46.1, 128 41.6 / 47.4 (runs of
+// one side differ by 0.5%); 8 x 4096, d = 128 64.9 / 74.3.  (Only at 3.5 waves of CTAs does d = 96 gain without: 32 x 4096 231 / 224, d = 128 242 / 245.)
+enum { F4_PLAIN, F4_PACED };
+template <int POLY, int NCH, int SPLIT = 1, bool BF = false, int FORM = F4_PLAIN>   // NCH: 64-column chunks per row (head dim <= 64 * NCH); BF: bfloat16 tensors
 __global__ void __launch_bounds__(F4_THREADS, 1)
 fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     constexpr int BN = F4_BN;
@@ -156,6 +162,9 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     // us with no test, 24, 4096: 4 x 8 x 9216 x 9216, d = 40, 674, 665, 671; 2 x 8 x 2304 x 2304, d = 80, 39.3, 34.4, 33.6; in parts 1419,
     // d = 80, 16.0, 16.3, 15.8, and 256, d = 160, 7.88, 7.99, 8.04.
     constexpr uint32_t P_TESTS = KV_APART ? 0 : SPLIT == 1 && NCH == 1 ? 24 : 4096;
+    constexpr bool PACED = FORM == F4_PACED;
+    static_assert(!PACED || SPLIT == 1, "forms");
+    constexpr int PRODUCTS = PACED ? 1 : F4S_BUFFERS;
     extern __shared__ uint8_t f4s_smem_raw[];
     // per (tile, buffer): S ready (MMA) | P ready (softmax) | product done.  per tile: Q landed | all of O_t done.
     // The score barriers are per tile AND buffer so that every barrier has ONE consumer that takes its phases in order (a parity wait is only sound for a waiter exactly one phase behind): tile t meets buffer b
@@ -163,11 +172,13 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     // (one block of memory, so that a warp can (re-)initialise them side by side: see init_barriers)
     struct Barriers {
         uint64_t s_full[F4_TILES][F4S_BUFFERS], p_full[F4_TILES][F4S_BUFFERS];   // p_full: 4 arrivals, one per softmax warp
-        uint64_t q_full[F4_TILES], o_final[F4_TILES];
+        uint64_t q_full[F4_TILES];
         // one per tile and buffer, so that a softmax warp need not take every phase on its way to the hand-over, which the next
         // tile's scores wait behind: with a wait there 82.7 us for 2 x 8 x 4096 x 4096, d = 40, without 80.9
-        // (4 x 8 x 9216 x 9216: 750 and 739)
-        uint64_t pv_done[F4_TILES][F4S_BUFFERS];   // (SPLIT > 1: [part][0])
+        // (4 x 8 x 9216 x 9216: 750 and 739).  Paced: one per tile; with as many as the others have, unused, 41.6 us for
+        // 16 x 2304 x 2304, d = 128, are 44.8.
+        uint64_t pv_done[F4_TILES][PRODUCTS];   // (SPLIT > 1: [part][0])
+        uint64_t o_final[F4_TILES];
         uint64_t k_first;                 // K of the first key tile, which the first scores need before anything of V
         uint64_t kv_full[F4_STAGES];      // (the first key tile: its V)
         uint64_t buf_free[F4S_BUFFERS];   // SPLIT > 1: the products reading a buffer's weights are done
@@ -379,7 +390,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 if (s == stages) { s = 0; pe ^= 1; }
                 // (Eight stages ahead of the issuers it sleeps between polls, which is worth 1% of the call; a shorter ring's next load
                 // is waited for: 1024, d = 80, five stages: 12.4 us with sleep, 12.2 without; 2304: 21.8 and 21.5.)
-                if (j >= stages && !(stages == F4_STAGES ? mbar_wait_lazy(smem_u32(&bar_kv_empty[s]), pe, abort_p, args.status, SITE_G_EMPTY, j)
+                if (j >= stages && !(PACED || stages == F4_STAGES ? mbar_wait_lazy(smem_u32(&bar_kv_empty[s]), pe, abort_p, args.status, SITE_G_EMPTY, j)
                                                          : mbar_wait(smem_u32(&bar_kv_empty[s]), pe, abort_p, args.status, SITE_G_EMPTY, j)))
                     break;
                 const uint32_t k_dst = kv_smem + s * 2 * kv_tile_bytes, v_dst = k_dst + kv_tile_bytes;
@@ -547,7 +558,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 tc_fence_after_sync();
                 issue_o(j, sj, b);
                 if (more) issue_s(q_desc, tn, sn, b);               // into the buffer P is read from: behind it, in order
-                tc_commit(b_pvdone + b * 8);                        // O_t holds key tiles 0..j
+                tc_commit(PACED ? b_pvdone : b_pvdone + b * 8);     // O_t holds key tiles 0..j
                 tc_commit(smem_u32(&bar_kv_empty[sj]));             // this issuer is done with K(j), V(j)
                 if (j == n_kv - 1) tc_commit(smem_u32(&bar_o_final[t]));
                 b = (b == 0) ? NB - 1 : b - 1;              // k += NB - 1
@@ -780,13 +791,14 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     // Rare: a row of this warp met a score far above its anchor.  O_t may be touched once the P V
                     // product of key tile j-1 has completed; nothing of P_t(j) has been stored yet, so the scores are
                     // still in tensor memory.  The first registers of the row are borrowed for O_t.
-                    // (Nothing waits for the phases of the products' barriers in between, so there is one per buffer: the scores
+                    // (Where nothing waits for the phases of the products' barriers in between, there is one per buffer: the scores
                     // S_t(j) in hand came behind the product of step k - NB in their buffer, that product's scores behind the one
                     // of k - 2 NB, and T such steps back stands P_t V(j - NB), the last before j in the barrier of j's buffer.
                     // So of every barrier of this tile at most the newest phase is open, and a parity wait is sound.)
                     if (j > 0) {
                         const int bp = b + 1 == NB ? 0 : b + 1;   // buffer of key tile j - 1
-                        ok = mbar_wait(b_pvdone + bp * 8, jm > 0 ? ph : ph ^ 1, abort_p, args.status, SITE_G_PV, j);
+                        ok = PACED ? mbar_wait(b_pvdone, (j - 1) & 1, abort_p, args.status, SITE_G_PV, j)
+                                   : mbar_wait(b_pvdone + bp * 8, jm > 0 ? ph : ph ^ 1, abort_p, args.status, SITE_G_PV, j);
                         ok = __all_sync(0xffffffffu, ok);
                         if (!ok) break;
                         tc_fence_after_sync();
@@ -818,6 +830,12 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 l_run += tile_sum;
                 tmem_st32(tmem_s, packed);   // P_t(j) over the first columns of the buffer, whose scores sit in registers
                 tmem_wait_st();
+                // (paced: every phase, before P V(j) can complete; P V(j-1) has had a whole step to finish)
+                if (PACED && j > 0) {
+                    ok = mbar_wait(b_pvdone, (j - 1) & 1, abort_p, args.status, SITE_G_PV, j);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                }
                 tc_fence_before_sync();
                 if (lane == 0) mbar_arrive(smem_u32(&bar_p_full[t][b]));
                 b = (b == 0) ? NB - 1 : b - 1;              // k += NB - 1
@@ -825,7 +843,9 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
             }
             if (ok) ok = mbar_wait(smem_u32(&bar_o_final[t]), 0, abort_p, args.status, SITE_G_O, t);
             // (another segment follows: the last phase of every product barrier must have landed before they start over)
-            if (!last_segment)
+            if (PACED) {
+                if (ok) ok = mbar_wait(b_pvdone, (n_kv - 1) & 1, abort_p, args.status, SITE_G_PV, n_kv);
+            } else if (!last_segment)
                 for (int j = n_kv > NB ? n_kv - NB : 0; j < n_kv && ok; ++j)
                     ok = mbar_wait(b_pvdone + ((t + (NB - 1) * j) % NB) * 8, (j / NB) & 1, abort_p, args.status, SITE_G_PV, n_kv);
             ok = __all_sync(0xffffffffu, ok);

@@ -58,3 +58,17 @@ def test_tiles_that_re_anchor_at_every_key_tile(bd, tiles, shares, Nk):
     for _ in range(5):
         parity.check(parity.run(a, bd, bd.MODE_FUSED, q, k, v, scale), ref, v, what="tiles=%d Nk=%d" % (tiles, Nk))
     a.close()
+
+
+@pytest.mark.parametrize("tiles,d", [(2, 72), (3, 80), (1, 88), (2, 88), (1, 128), (2, 128), (2, 136), (2, 160)])
+@pytest.mark.parametrize("Nk", [65, 193, 257, 449])   # around the score buffers (2 to 4) and the K/V ring (3 to 6)
+def test_whole_units_of_wide_heads(bd, tiles, d, Nk):
+    """80 < d <= 128 takes every phase of the products' barriers, the others only where a row is re-anchored, here at every key tile."""
+    a = bd.Attention(bd.MODE_FUSED, options=bd.Options(fused_tiles=tiles, fused_split=1))
+    q, k, v = parity.rand_qkv(d + Nk, 1, 3, 300, Nk, d)
+    scale = float(np.float32(d ** -0.5))
+    for grow in (1.0, 12.0):
+        kk = (k.astype(np.float32) * np.geomspace(0.1 if grow > 1 else 1.0, grow, Nk, dtype=np.float32)[None, None, :, None]).astype(np.float16)
+        ref, _, _ = oracle.forward(q, kk, v, scale)
+        parity.check(parity.run(a, bd, bd.MODE_FUSED, q, kk, v, scale), ref, v, what="tiles=%d d=%d Nk=%d" % (tiles, d, Nk))
+    a.close()
