@@ -148,22 +148,23 @@ __device__ __noinline__ void f4s_store_piece(float* piece, uint32_t tmem_o, int 
 // the way to the hand-over, and the loading thread sleeps between polls.  Two tiles of such heads fall into step without:
 // us paced / plain, 16 x 2304 x 2304, d = 72 38.1 / 36.6, 80 37.4 / 35.3, 88 39.6 / 43.5, 96 38.0 / 43.1, 112 39.0 / 46.1, 128 41.6 / 47.4 (runs of
 // one side differ by 0.5%); 8 x 4096, d = 128 64.9 / 74.3.  (Only at 3.5 waves of CTAs does d = 96 gain without: 32 x 4096 231 / 224, d = 128 242 / 245.)
-enum { F4_PLAIN, F4_PACED };
+// F4_APART, parts of d > 128 whose key tiles outnumber the ring's three stages: K and V have threads and barriers of their own, and a
+// stage's K is free for the next load when its scores are computed, not when its product is.  Where no stage is used twice, the
+// additional waits and commits only cost.  us plain / apart, 16 x N x N, d = 160: 144 6.57 / 6.71, 200 7.87 / 7.76, 256 7.83 / 7.64, 1024 18.0 / 15.8;
+// 32 x 192 6.66 / 6.84, x 300 8.95 / 8.68, x 576 23.1 / 21.4 (runs of one side differ by 0.3%).  At d <= 128 the ring is deeper: 1024, d = 80: 12.4 / 12.8.
+enum { F4_PLAIN, F4_PACED, F4_APART };
 template <int POLY, int NCH, int SPLIT = 1, bool BF = false, int FORM = F4_PLAIN>   // NCH: 64-column chunks per row (head dim <= 64 * NCH); BF: bfloat16 tensors
 __global__ void __launch_bounds__(F4_THREADS, 1)
 fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     constexpr int BN = F4_BN;
-    // Parts of d > 128, whose ring has three stages: K and V have threads and barriers of their own, and a stage's K is free for the
-    // next load when its scores are computed, not when its product is (2 x 8 x 256 x 256, d = 160: 8.5 -> 8.0 us; 4 x 8 x 576 x 576: 24.5 ->
-    // 22.4).  At d <= 128 the ring is deeper, and the issuing threads' additional wait and commit cost more (1024, d = 80: 12.4 -> 12.8).
-    constexpr bool KV_APART = SPLIT > 1 && NCH == 3;
+    constexpr bool KV_APART = FORM == F4_APART;
     constexpr int KV_V_WARP = 19;   // (an issuer that parts leave idle)
     // How often an issuing thread tests plainly for weights before its wait suspends: a suspended thread sees them later, the tests take issue slots.
     // us with no test, 24, 4096: 4 x 8 x 9216 x 9216, d = 40, 674, 665, 671; 2 x 8 x 2304 x 2304, d = 80, 39.3, 34.4, 33.6; in parts 1419,
     // d = 80, 16.0, 16.3, 15.8, and 256, d = 160, 7.88, 7.99, 8.04.
     constexpr uint32_t P_TESTS = KV_APART ? 0 : SPLIT == 1 && NCH == 1 ? 24 : 4096;
     constexpr bool PACED = FORM == F4_PACED;
-    static_assert(!PACED || SPLIT == 1, "forms");
+    static_assert(FORM == F4_PLAIN || PACED == (SPLIT == 1), "forms");
     constexpr int PRODUCTS = PACED ? 1 : F4S_BUFFERS;
     extern __shared__ uint8_t f4s_smem_raw[];
     // per (tile, buffer): S ready (MMA) | P ready (softmax) | product done.  per tile: Q landed | all of O_t done.

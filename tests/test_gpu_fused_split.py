@@ -33,12 +33,12 @@ def test_parts_buffers_and_ring(bd, d, Nk):
     a.close()
 
 
-@pytest.mark.parametrize("d", [40, 80, 160])
-def test_parts_that_re_anchor_at_every_key_tile(bd, d):
+@pytest.mark.parametrize("d,Nk", [(40, 1024), (80, 1024), (160, 1024), (136, 130), (160, 192), (160, 256)])   # (d > 128: a ring of three stages)
+def test_parts_that_re_anchor_at_every_key_tile(bd, d, Nk):
     """Scores that rise along the keys: the rescale of a part's accumulator waits for its own last product."""
     a = bd.Attention()
-    q, k, v = parity.rand_qkv(d, 1, 4, 128, 1024, d)
-    k = (k.astype(np.float32) * np.repeat(np.geomspace(0.1, 12.0, 16), 64)[None, None, :, None].astype(np.float32)).astype(np.float16)
+    q, k, v = parity.rand_qkv(d, 1, 4, 128, Nk, d)
+    k = (k.astype(np.float32) * np.repeat(np.geomspace(0.1, 12.0, 16), 64)[:1024:1024 // Nk][:Nk, None].astype(np.float32)).astype(np.float16)
     scale = float(np.float32(d ** -0.5))
     ref, _, _ = oracle.forward(q, k, v, scale)
     for _ in range(5):
