@@ -144,16 +144,19 @@ __device__ __noinline__ void f4s_store_piece(float* piece, uint32_t tmem_o, int 
 // accumulator.  The score buffers run ahead of the products (NB of them, SPLIT to 2 SPLIT: 4 of 3 parts at d = 80, 5 of 4 at d = 40), and the MMAs
 // come from two threads: the products of key tile j from one, the scores of key tile j + NB from the other.
 //
-// How closely the roles follow one another (FORM).  F4_PACED, whole units of 80 < d <= 128: a softmax warp takes its tile's last product on
-// the way to the hand-over, and the loading thread sleeps between polls.  Two tiles of such heads fall into step without:
-// us paced / plain, 16 x 2304 x 2304, d = 72 38.1 / 36.6, 80 37.4 / 35.3, 88 39.6 / 43.5, 96 38.0 / 43.1, 112 39.0 / 46.1, 128 41.6 / 47.4 (runs of
-// one side differ by 0.5%); 8 x 4096, d = 128 64.9 / 74.3.  (Only at 3.5 waves of CTAs does d = 96 gain without: 32 x 4096 231 / 224, d = 128 242 / 245.)
+// How closely the roles follow one another (FORM).  F4_PACED, whole units of 80 < d <= 128: a softmax warp takes its tile's last
+// product on the way to the hand-over, and the loading thread sleeps between polls.  Two tiles of such heads fall into step without:
+// us paced / plain, 16 x 2304 x 2304, d = 72 38.1 / 36.6, 80 37.4 / 35.3, 88 39.6 / 43.5, 96 38.0 / 43.1, 112 39.0 / 46.1, 128 41.6 / 47.4
+// (runs of one side differ by 0.5%); 8 x 4096, d = 128 64.9 / 74.3.  (Only at 3.5 waves of CTAs does d = 96 gain without: 32 x 4096
+// 231 / 224, d = 128 242 / 245.)
 // F4_APART, parts of d > 128 whose key tiles outnumber the ring's three stages: K and V have threads and barriers of their own, and a
 // stage's K is free for the next load when its scores are computed, not when its product is.  Where no stage is used twice, the
-// additional waits and commits only cost.  us plain / apart, 16 x N x N, d = 160: 144 6.57 / 6.71, 200 7.87 / 7.76, 256 7.83 / 7.64, 1024 18.0 / 15.8;
-// 32 x 192 6.66 / 6.84, x 300 8.95 / 8.68, x 576 23.1 / 21.4 (runs of one side differ by 0.3%).  At d <= 128 the ring is deeper: 1024, d = 80: 12.4 / 12.8.
+// additional waits and commits only cost.  us plain / apart, 16 x N x N, d = 160: 144 6.57 / 6.71, 200 7.87 / 7.76, 256 7.83 / 7.64,
+// 1024 18.0 / 15.8; 32 x 192 6.66 / 6.84, x 300 8.95 / 8.68, x 576 23.1 / 21.4 (runs of one side differ by 0.3%).  At d <= 128 the ring
+// is deeper: 1024, d = 80 12.4 / 12.8.
 enum { F4_PLAIN, F4_PACED, F4_APART };
-template <int POLY, int NCH, int SPLIT = 1, bool BF = false, int FORM = F4_PLAIN>   // NCH: 64-column chunks per row (head dim <= 64 * NCH); BF: bfloat16 tensors
+// NCH: 64-column chunks per row (head dim <= 64 * NCH); BF: bfloat16 tensors
+template <int POLY, int NCH, int SPLIT = 1, bool BF = false, int FORM = F4_PLAIN>
 __global__ void __launch_bounds__(F4_THREADS, 1)
 fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     constexpr int BN = F4_BN;
@@ -168,8 +171,9 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     constexpr int PRODUCTS = PACED ? 1 : F4S_BUFFERS;
     extern __shared__ uint8_t f4s_smem_raw[];
     // per (tile, buffer): S ready (MMA) | P ready (softmax) | product done.  per tile: Q landed | all of O_t done.
-    // The score barriers are per tile AND buffer so that every barrier has ONE consumer that takes its phases in order (a parity wait is only sound for a waiter exactly one phase behind): tile t meets buffer b
-    // every NB key tiles, and the buffer cannot come back to it before its previous contents were consumed.
+    // The score barriers are per tile AND buffer so that every barrier has ONE consumer that takes its phases in order (a parity wait
+    // is only sound for a waiter exactly one phase behind): tile t meets buffer b every NB key tiles, and the buffer cannot come back
+    // to it before its previous contents were consumed.
     // (one block of memory, so that a warp can (re-)initialise them side by side: see init_barriers)
     struct Barriers {
         uint64_t s_full[F4_TILES][F4S_BUFFERS], p_full[F4_TILES][F4S_BUFFERS];   // p_full: 4 arrivals, one per softmax warp
@@ -381,25 +385,26 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     if (++s == stages) { s = 0; pe ^= 1; }
                 }
             } else {
-            mbar_arrive_expect_tx(smem_u32(&bar_k_first), kv_tile_bytes);
-            load_tile(&pr.tk, kv_smem, smem_u32(&bar_k_first), 0);
-            for (int t = 1; t < T; ++t) load_q(t);
-            mbar_arrive_expect_tx(smem_u32(&bar_kv_full[0]), kv_tile_bytes);
-            load_tile(&pr.tv, kv_smem + kv_tile_bytes, smem_u32(&bar_kv_full[0]), 0);
-            int s = 1, pe = 1;   // stage of key tile j; parity of the kv_empty phase that frees it (from j = stages on)
-            for (int j = 1; j < n_kv; ++j, ++s) {
-                if (s == stages) { s = 0; pe ^= 1; }
-                // (Eight stages ahead of the issuers it sleeps between polls, which is worth 1% of the call; a shorter ring's next load
-                // is waited for: 1024, d = 80, five stages: 12.4 us with sleep, 12.2 without; 2304: 21.8 and 21.5.)
-                if (j >= stages && !(PACED || stages == F4_STAGES ? mbar_wait_lazy(smem_u32(&bar_kv_empty[s]), pe, abort_p, args.status, SITE_G_EMPTY, j)
-                                                         : mbar_wait(smem_u32(&bar_kv_empty[s]), pe, abort_p, args.status, SITE_G_EMPTY, j)))
-                    break;
-                const uint32_t k_dst = kv_smem + s * 2 * kv_tile_bytes, v_dst = k_dst + kv_tile_bytes;
-                const uint32_t bar = smem_u32(&bar_kv_full[s]);
-                mbar_arrive_expect_tx(bar, 2 * kv_tile_bytes);
-                load_tile(&pr.tk, k_dst, bar, j);
-                load_tile(&pr.tv, v_dst, bar, j);
-            }
+                mbar_arrive_expect_tx(smem_u32(&bar_k_first), kv_tile_bytes);
+                load_tile(&pr.tk, kv_smem, smem_u32(&bar_k_first), 0);
+                for (int t = 1; t < T; ++t) load_q(t);
+                mbar_arrive_expect_tx(smem_u32(&bar_kv_full[0]), kv_tile_bytes);
+                load_tile(&pr.tv, kv_smem + kv_tile_bytes, smem_u32(&bar_kv_full[0]), 0);
+                int s = 1, pe = 1;   // stage of key tile j; parity of the kv_empty phase that frees it (from j = stages on)
+                for (int j = 1; j < n_kv; ++j, ++s) {
+                    if (s == stages) { s = 0; pe ^= 1; }
+                    // (Eight stages ahead of the issuers it sleeps between polls, which is worth 1% of the call; a shorter ring's next load
+                    // is waited for: 1024, d = 80, five stages: 12.4 us with sleep, 12.2 without; 2304: 21.8 and 21.5.)
+                    const uint32_t empty = smem_u32(&bar_kv_empty[s]);
+                    if (j >= stages && !(PACED || stages == F4_STAGES ? mbar_wait_lazy(empty, pe, abort_p, args.status, SITE_G_EMPTY, j)
+                                                                      : mbar_wait(empty, pe, abort_p, args.status, SITE_G_EMPTY, j)))
+                        break;
+                    const uint32_t k_dst = kv_smem + s * 2 * kv_tile_bytes, v_dst = k_dst + kv_tile_bytes;
+                    const uint32_t bar = smem_u32(&bar_kv_full[s]);
+                    mbar_arrive_expect_tx(bar, 2 * kv_tile_bytes);
+                    load_tile(&pr.tk, k_dst, bar, j);
+                    load_tile(&pr.tv, v_dst, bar, j);
+                }
             }
             // Another segment follows: the issuers' last commits on the ring (never waited for above) must have
             // landed before the barriers are initialised again.
@@ -500,7 +505,8 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                         // (the buffer first: once product jn - NB has completed, V(0) has landed, which makes the parity wait
                         // for the second filling of stage 0 sound)
                         if (jn >= NB) ok = mbar_wait(smem_u32(&bar_buf_free[b]), ph, abort_p, args.status, SITE_G_PV, jn);
-                        ok = ok && mbar_wait(smem_u32(KV_APART ? &bars.k_full[sn] : jn == 0 ? &bar_k_first : &bar_kv_full[sn]), pn, abort_p, args.status, SITE_G_KV, jn);
+                        ok = ok && mbar_wait(smem_u32(KV_APART ? &bars.k_full[sn] : jn == 0 ? &bar_k_first : &bar_kv_full[sn]), pn, abort_p,
+                                             args.status, SITE_G_KV, jn);
                         if (!ok) break;
                         tc_fence_after_sync();
                         issue_s(q_desc_own_split, 0, sn, b);
@@ -554,7 +560,8 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 const bool more = jn < n_kv;
                 if (more)   // landed long ago: keep this wait off the critical path
                     ok = mbar_wait(smem_u32(&bar_kv_full[sn]), pn, abort_p, args.status, SITE_G_KV, jn);
-                    if (ok) ok = mbar_wait_eager<P_TESTS>(smem_u32(&bar_p_full[t][b]), ph, abort_p, args.status, SITE_G_P, j);
+                // (plain tests first, see P_TESTS: every hand-over passes here)
+                if (ok) ok = mbar_wait_eager<P_TESTS>(smem_u32(&bar_p_full[t][b]), ph, abort_p, args.status, SITE_G_P, j);
                 if (!ok) break;
                 tc_fence_after_sync();
                 issue_o(j, sj, b);

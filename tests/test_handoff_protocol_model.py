@@ -169,7 +169,9 @@ def test_one_barrier_per_buffer_is_not_enough():
 # products O_g (+)= P(j) V(j) from one, the scores of key tile j + NB from the other -- whose instructions the tensor
 # pipe does not order against each other.
 
-def simulate_parts(SPLIT, NB, n_kv, stages, seed, warps=4, wait_buf_free=True, limit=400000):
+def simulate_parts(SPLIT, NB, n_kv, stages, seed, warps=4, wait_buf_free=True, limit=400000, apart=False):
+    """apart: K and V by producers of their own, K's stage free when its scores are computed.  The products' barriers are waited for
+    where a row is re-anchored only (at random)."""
     rnd = random.Random(seed)
     s_full = [Bar(1) for _ in range(NB)]
     p_full = [Bar(warps) for _ in range(NB)]
@@ -179,6 +181,8 @@ def simulate_parts(SPLIT, NB, n_kv, stages, seed, warps=4, wait_buf_free=True, l
     q_full = Bar(1)
     kv_full = [Bar(1) for _ in range(stages)]
     kv_empty = [Bar(1) for _ in range(stages)]
+    k_full, k_empty = [Bar(1) for _ in range(stages)], [Bar(1) for _ in range(stages)]   # (apart)
+    k_stage, products = {}, set()
     pipe_a, pipe_b = [], []                      # per issuing thread, each retired in order
     buf = {b: {} for b in range(NB)}             # per buffer and warp: what it holds
     stage, errors = {}, []
@@ -187,35 +191,39 @@ def simulate_parts(SPLIT, NB, n_kv, stages, seed, warps=4, wait_buf_free=True, l
         if not cond:
             errors.append(what)
 
-    def producer():
-        q_full.arrive()
-        yield
+    def producer(holds, full, empty, with_q):
+        if with_q:
+            q_full.arrive()
+            yield
         for j in range(n_kv):
             s = j % stages
             if j >= stages:
-                while not kv_empty[s].done(((j // stages) - 1) & 1):
+                while not empty[s].done(((j // stages) - 1) & 1):
                     yield
-            stage[s] = j
-            kv_full[s].arrive()
+            holds[s] = j
+            full[s].arrive()
             yield
 
     def score_thread():
         while not q_full.done(0):
             yield
+        holds, full = (k_stage, k_full) if apart else (stage, kv_full)
         for jn in range(n_kv):
             b = jn % NB
-            while not kv_full[jn % stages].done((jn // stages) & 1):
+            while not full[jn % stages].done((jn // stages) & 1):
                 yield
             if jn >= NB and wait_buf_free:
                 while not buf_free[b].done(((jn // NB) - 1) & 1):
                     yield
-            check(stage.get(jn % stages) == jn, ("S reads a stale stage", jn))
-            pipe_b.append(("S", jn, b, [s_full[b]]))
+            check(holds.get(jn % stages) == jn, ("S reads a stale stage", jn))
+            pipe_b.append(("S", jn, b, [s_full[b]] + ([k_empty[jn % stages]] if apart else [])))
             yield
 
     def product_thread():
         for j in range(n_kv):
             b = j % NB
+            while apart and not kv_full[j % stages].done((j // stages) & 1):
+                yield
             while not p_full[b].done((j // NB) & 1):
                 yield
             check(stage.get(j % stages) == j, ("P V reads a stale stage", j))
@@ -231,15 +239,18 @@ def simulate_parts(SPLIT, NB, n_kv, stages, seed, warps=4, wait_buf_free=True, l
             check(buf[b].get(w) == ("S", j), ("a part reads the wrong scores", g, w, j, b, buf[b].get(w)))
             yield
             buf[b][w] = ("P", j)
-            if i > 0:          # the product of the part's previous key tile
+            if i > 0 and rnd.random() < 0.3:   # re-anchored behind the product of the part's previous key tile
                 while not pv_done[g].done((i - 1) & 1):
                     yield
+                check(j - SPLIT in products, ("re-anchored before the part's last product", g, j))
             p_full[b].arrive()
             yield
         while not o_final.done(0):
             yield
 
-    procs = [producer(), score_thread(), product_thread()] + [part_warp(g, w) for g in range(SPLIT) for w in range(warps)]
+    procs = [producer(stage, kv_full, kv_empty, not apart), score_thread(), product_thread()]
+    procs += [producer(k_stage, k_full, k_empty, True)] if apart else []
+    procs += [part_warp(g, w) for g in range(SPLIT) for w in range(warps)]
     steps = 0
     while procs and not errors:
         steps += 1
@@ -253,6 +264,7 @@ def simulate_parts(SPLIT, NB, n_kv, stages, seed, warps=4, wait_buf_free=True, l
                         buf[b][w] = ("S", j)
                 else:
                     check(all(buf[b].get(w) == ("P", j) for w in range(warps)), ("P V reads the wrong weights", j, b))
+                    products.add(j)
                 for x in bars:
                     x.arrive()
         i = rnd.randrange(len(procs))
@@ -269,6 +281,12 @@ def test_lone_tile_in_parts_protocol(SPLIT, NB, n_kv):
     for seed in range(4):
         assert simulate_parts(SPLIT, NB, n_kv, 8, seed) == "ok"
         assert simulate_parts(SPLIT, NB, n_kv, NB + 1, seed) == "ok"
+
+
+@pytest.mark.parametrize("n_kv", [1, 3, 4, 5, 8, 16, 17])
+def test_lone_tile_in_parts_with_k_and_v_apart(n_kv):
+    for seed in range(6):
+        assert simulate_parts(2, 3, n_kv, 3, seed, apart=True) == "ok"
 
 
 def test_scores_must_wait_for_the_completion_of_the_products_they_overwrite():
