@@ -162,10 +162,11 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     constexpr int BN = F4_BN;
     constexpr bool KV_APART = FORM == F4_APART;
     constexpr int KV_V_WARP = 19;   // (an issuer that parts leave idle)
-    // How often an issuing thread tests plainly for weights before its wait suspends: a suspended thread sees them later, the tests take issue slots.
-    // us with no test, 24, 4096: 4 x 8 x 9216 x 9216, d = 40, 674, 665, 671; 2 x 8 x 2304 x 2304, d = 80, 39.3, 34.4, 33.6; in parts 1419,
-    // d = 80, 16.0, 16.3, 15.8, and 256, d = 160, 7.88, 7.99, 8.04.
-    constexpr uint32_t P_TESTS = KV_APART ? 0 : SPLIT == 1 && NCH == 1 ? 24 : 4096;
+    // How often an issuing thread tests plainly for weights before its wait suspends: a suspended thread sees them later, the tests take
+    // issue slots.  us with no test / 24 / 4096 (least of three runs, which differ by 0.1 to 0.3%): whole units, 16 x 4096 x 4096,
+    // d = 40 83.7 / 82.6 / 83.2, 32 x 9216 687 / 681 / 686, but 16 x 2304, d = 64 32.8 / 32.8 / 32.4; in parts 8 x 1419, d = 80
+    // 15.71 / 16.12 / 15.55, 16 x 1024 12.07 / 12.37 / 12.07; K and V apart 16 x 256, d = 160 7.63 / 7.73 / 7.79, 32 x 576 21.4 / 21.6 / 21.7.
+    constexpr uint32_t P_TESTS = KV_APART ? 0 : SPLIT == 1 && NCH == 1 && POLY != 0 ? 24 : 4096;
     constexpr bool PACED = FORM == F4_PACED;
     static_assert(FORM == F4_PLAIN || PACED == (SPLIT == 1), "forms");
     constexpr int PRODUCTS = PACED ? 1 : F4S_BUFFERS;
