@@ -178,13 +178,12 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     // (one block of memory, so that a warp can (re-)initialise them side by side: see init_barriers)
     struct Barriers {
         uint64_t s_full[F4_TILES][F4S_BUFFERS], p_full[F4_TILES][F4S_BUFFERS];   // p_full: 4 arrivals, one per softmax warp
-        uint64_t q_full[F4_TILES];
+        uint64_t q_full[F4_TILES], o_final[F4_TILES];
         // one per tile and buffer, so that a softmax warp need not take every phase on its way to the hand-over, which the next
         // tile's scores wait behind: with a wait there 82.7 us for 2 x 8 x 4096 x 4096, d = 40, without 80.9
         // (4 x 8 x 9216 x 9216: 750 and 739).  Paced: one per tile; with as many as the others have, unused, 41.6 us for
         // 16 x 2304 x 2304, d = 128, are 44.8.
         uint64_t pv_done[F4_TILES][PRODUCTS];   // (SPLIT > 1: [part][0])
-        uint64_t o_final[F4_TILES];
         uint64_t k_first;                 // K of the first key tile, which the first scores need before anything of V
         uint64_t kv_full[F4_STAGES];      // (the first key tile: its V)
         uint64_t buf_free[F4S_BUFFERS];   // SPLIT > 1: the products reading a buffer's weights are done
