@@ -169,6 +169,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
     constexpr uint32_t P_TESTS = KV_APART ? 0 : SPLIT == 1 && NCH == 1 && POLY != 0 ? 24 : 4096;
     constexpr bool PACED = FORM == F4_PACED;
     static_assert(FORM == F4_PLAIN || PACED == (SPLIT == 1), "forms");
+    constexpr bool LOADS_AHEAD = PACED || (NCH == 1 && SPLIT > 1);   // the loading thread sleeps between polls
     constexpr int PRODUCTS = PACED ? 1 : F4S_BUFFERS;
     extern __shared__ uint8_t f4s_smem_raw[];
     // per (tile, buffer): S ready (MMA) | P ready (softmax) | product done.  per tile: Q landed | all of O_t done.
@@ -393,11 +394,13 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 int s = 1, pe = 1;   // stage of key tile j; parity of the kv_empty phase that frees it (from j = stages on)
                 for (int j = 1; j < n_kv; ++j, ++s) {
                     if (s == stages) { s = 0; pe ^= 1; }
-                    // (Eight stages ahead of the issuers it sleeps between polls, which is worth 1% of the call; a shorter ring's next load
-                    // is waited for: 1024, d = 80, five stages: 12.4 us with sleep, 12.2 without; 2304: 21.8 and 21.5.)
+                    // (Eight stages ahead of the issuers, one chunk a row, it sleeps between polls, which is worth 1% of the call; a shorter
+                    // ring's next load is waited for: 16 x 1024, d = 80, five stages: 12.27 us with sleep, 12.14 without.  The depth
+                    // decides at run time where that is measured better, for the code it leaves: known at compile time, parts of
+                    // 8 x 1419, d = 80 15.6 -> 16.1, but of 32 x 256, d = 64 5.79 -> 5.75.)
                     const uint32_t empty = smem_u32(&bar_kv_empty[s]);
-                    if (j >= stages && !(PACED || stages == F4_STAGES ? mbar_wait_lazy(empty, pe, abort_p, args.status, SITE_G_EMPTY, j)
-                                                                      : mbar_wait(empty, pe, abort_p, args.status, SITE_G_EMPTY, j)))
+                    if (j >= stages && !(LOADS_AHEAD || stages == F4_STAGES ? mbar_wait_lazy(empty, pe, abort_p, args.status, SITE_G_EMPTY, j)
+                                                                            : mbar_wait(empty, pe, abort_p, args.status, SITE_G_EMPTY, j)))
                         break;
                     const uint32_t k_dst = kv_smem + s * 2 * kv_tile_bytes, v_dst = k_dst + kv_tile_bytes;
                     const uint32_t bar = smem_u32(&bar_kv_full[s]);
