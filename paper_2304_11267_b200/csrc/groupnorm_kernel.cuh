@@ -75,31 +75,32 @@ __device__ __forceinline__ void gn_affine_piece(const uint4& x, float scale, flo
 }
 
 // ------------------------------------------------------------------ statistics of a set of values
-// (count, mean, sum of squared deviations from that mean).  Two sets merge without cancellation (Chan, Golub and
-// LeVeque's pairwise update), so ONE reduction delivers mean and variance: a thread takes its own values' mean and
-// deviations from registers, then warps, the block and the cluster merge triples.
+// (count, mean, sum of squared deviations from that mean).  ONE reduction delivers mean and variance: a thread takes its own
+// values' mean and deviations from registers, then warps, the block and the cluster put theirs together.
 struct GnStat {
     float n, mean, m2;
 };
-__device__ __forceinline__ GnStat gn_merge(const GnStat& a, const GnStat& b) {
+// Of a warp's lanes, by sums about lane 0's mean: that is the mean of a subset, so the sum of squares about it exceeds the one about the
+// common mean by the ratio of the counts at most, 32, which is all the subtraction can lose.
+__device__ __forceinline__ GnStat gn_merge_lanes(const GnStat& s) {
+    const float at = __shfl_sync(0xffffffffu, s.mean, 0), d = s.n > 0.f ? s.mean - at : 0.f;
+    float n = s.n, sum = s.n * d, sq = fmaf(sum, d, s.m2);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        n += __shfl_xor_sync(0xffffffffu, n, o);
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    }
+    const float shift = n > 0.f ? __fdividef(sum, n) : 0.f;
+    return {n, at + shift, fmaxf(fmaf(-sum, shift, sq), 0.f)};
+}
+__device__ __forceinline__ GnStat gn_merge(const GnStat& a, const GnStat& b) {   // Chan, Golub and LeVeque's pairwise update
     const float n = a.n + b.n, w = n > 0.f ? __fdividef(b.n, n) : 0.f, d = b.mean - a.mean;
     GnStat r;
     r.n = n;
     r.mean = fmaf(d, w, a.mean);
     r.m2 = a.m2 + b.m2 + d * d * (a.n * w);
     return r;
-}
-template <int LANES>
-__device__ __forceinline__ GnStat gn_merge_lanes(GnStat s) {
-#pragma unroll
-    for (int o = LANES / 2; o > 0; o >>= 1) {
-        GnStat t;
-        t.n = __shfl_xor_sync(0xffffffffu, s.n, o);
-        t.mean = __shfl_xor_sync(0xffffffffu, s.mean, o);
-        t.m2 = __shfl_xor_sync(0xffffffffu, s.m2, o);
-        s = gn_merge(s, t);
-    }
-    return s;
 }
 
 // Registers form: a group is shared out among the CL blocks of a cluster, a thread holds PPT 16-byte pieces of it in
@@ -108,10 +109,10 @@ __device__ __forceinline__ GnStat gn_merge_lanes(GnStat s) {
 // piece and pieces straddle channels.  The pieces are then those that lie whole inside the group, and the values before
 // the first and behind the last one (fewer than a piece each) go to the first block's first threads one by one.
 // What bounds it is the latency of one pass -- fetch, reduction, exchange, write -- as long as the group is shared out
-// finely enough for every SM to take part; see launch_groupnorm in sd_attn_api.cu for the split and what it measured.
-constexpr int GN_MAX_THREADS = 512;
+// finely enough for every SM to take part, and the instructions of a block that holds a large group; see launch_groupnorm in
+// sd_attn_api.cu for the split and what it measured.
 constexpr int GN_MAX_CLUSTER = 8;
-constexpr int GN_MAX_CPG = 1024;   // channels per group whose affine parameters the block keeps in shared memory
+constexpr int GN_MAX_CPG = 1024;   // channels per group whose scale and shift the block keeps in shared memory
 
 struct GroupNormPlan {
     int log2_cluster, pieces_per_block, cpg;   // blocks per group, 16-byte pieces of each, channels per group
@@ -121,14 +122,14 @@ struct GroupNormPlan {
 __device__ __forceinline__ void gn_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void gn_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-template <typename T, int PPT, bool RAGGED>
-__global__ void __launch_bounds__(GN_MAX_THREADS)
+template <typename T, int THREADS, int PPT, bool RAGGED>
+__global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 1)
 groupnorm_cluster_kernel(const GroupNormArgs a, const GroupNormPlan plan) {
     const int cluster = 1 << plan.log2_cluster, pieces_per_block = plan.pieces_per_block;
-    constexpr int VEC = 16 / (int)sizeof(T);
-    __shared__ GnStat warp_stat[GN_MAX_THREADS / 32];
+    constexpr int VEC = 16 / (int)sizeof(T), WARPS = THREADS / 32;
+    __shared__ GnStat warp_stat[WARPS];
     __shared__ GnStat block_stat[GN_MAX_CLUSTER];
-    __shared__ T affine[2][GN_MAX_CPG];
+    __shared__ float2 affine[GN_MAX_CPG];   // y = x * .x + .y
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = (int)blockIdx.x & (cluster - 1), group = (int)blockIdx.x >> plan.log2_cluster;
     const int cpg = plan.cpg, hw = (int)a.HW, n_elems = cpg * hw;
@@ -136,7 +137,7 @@ groupnorm_cluster_kernel(const GroupNormArgs a, const GroupNormPlan plan) {
     const long long base = (long long)group * n_elems;   // groups follow one another in memory
     const int head = RAGGED ? (int)((VEC - (base & (VEC - 1))) & (VEC - 1)) : 0;   // values before the first whole piece
     const int n_pieces = (n_elems - head) / VEC;                                    // (n_elems >= hw >= VEC > head)
-    const int p_end = min(n_pieces, (rank + 1) * pieces_per_block);
+    const int p0 = rank * pieces_per_block + tid, p_end = min(n_pieces, (rank + 1) * pieces_per_block);
     const T* src = static_cast<const T*>(a.x) + base;
     T* dst = static_cast<T*>(a.y) + base;
 
@@ -145,19 +146,23 @@ groupnorm_cluster_kernel(const GroupNormArgs a, const GroupNormPlan plan) {
     pdl_wait();
 
     uint4 v[PPT];
+    {
+        const uint4* from = reinterpret_cast<const uint4*>(src + head) + p0;
 #pragma unroll
-    for (int k = 0; k < PPT; ++k) {
-        const int p = rank * pieces_per_block + tid + k * (int)blockDim.x;
-        if (p < p_end) v[k] = *reinterpret_cast<const uint4*>(src + head + p * VEC);
+        for (int k = 0; k < PPT; ++k)
+            if (p0 + k * THREADS < p_end) v[k] = from[k * THREADS];
     }
     // RAGGED: this thread's lone value, if it has one
     const int lone = tid < head ? tid : head + n_pieces * VEC + (tid - head);
     const bool has_lone = RAGGED && rank == 0 && tid < 2 * VEC && lone < n_elems;
     float lone_x = has_lone ? gn_to_float(src[lone]) : 0.f;
-    for (int c = tid; c < cpg; c += (int)blockDim.x) {
-        if (a.gamma) affine[0][c] = static_cast<const T*>(a.gamma)[c0 + c];
-        if (a.beta) affine[1][c] = static_cast<const T*>(a.beta)[c0 + c];
-    }
+    // channel c0 + c's parameters: channel `tid`'s now, further ones (more channels than threads) when they are needed
+    auto parameters = [&](int c, float& ga, float& be) {
+        ga = a.gamma ? gn_to_float(static_cast<const T*>(a.gamma)[c0 + c]) : 1.f;
+        be = a.beta ? gn_to_float(static_cast<const T*>(a.beta)[c0 + c]) : 0.f;
+    };
+    float ga = 0.f, be = 0.f;
+    if (tid < cpg) parameters(tid, ga, be);
 
     // ---- statistics: the thread's own values, then warp, block, cluster.  One pass over the registers, about the
     // thread's first value: as that value is one of the set, the sum of squares about it exceeds the one about the mean by
@@ -166,8 +171,7 @@ groupnorm_cluster_kernel(const GroupNormArgs a, const GroupNormPlan plan) {
     uint64_t sum2 = 0ull, sq2 = 0ull;
 #pragma unroll
     for (int k = 0; k < PPT; ++k) {
-        const int p = rank * pieces_per_block + tid + k * (int)blockDim.x;
-        if (p >= p_end) continue;
+        if (p0 + k * THREADS >= p_end) continue;
         const T* e = reinterpret_cast<const T*>(&v[k]);
         if (k == 0) pivot = gn_to_float(e[0]);
         const uint64_t pp = gn_pack(pivot, pivot);
@@ -193,71 +197,70 @@ groupnorm_cluster_kernel(const GroupNormArgs a, const GroupNormPlan plan) {
         s.mean = pivot + shift;
         s.m2 = fmaxf(fmaf(-sum, shift, sq), 0.f);
     }
-    s = gn_merge_lanes<32>(s);
+    s = gn_merge_lanes(s);
     if (lane == 0) warp_stat[warp] = s;
     __syncthreads();
-    const int warps = (int)blockDim.x >> 5;
-    s = lane < warps ? warp_stat[lane] : GnStat{0.f, 0.f, 0.f};
-    s = gn_merge_lanes<GN_MAX_THREADS / 32>(s);   // lanes 0..15 hold it all (and 16..31 nothing: lane 0 counts)
+    const bool prepares = warp * 32 < cpg;   // scale and shift of some channels
+    if (prepares || cluster > 1) {
+        s = lane < WARPS ? warp_stat[lane] : GnStat{0.f, 0.f, 0.f};
+        s = gn_merge_lanes(s);
+    }
     if (cluster > 1) {
         gn_cluster_wait();
-        if (warp == 0 && lane < cluster) {
-            // every lane of the lower half has the block's triple; lane r stores it into block r's slot of this block
-            const GnStat mine = {__shfl_sync((1u << cluster) - 1u, s.n, 0), __shfl_sync((1u << cluster) - 1u, s.mean, 0),
-                                 __shfl_sync((1u << cluster) - 1u, s.m2, 0)};
+        if (warp == 0 && lane < cluster) {   // lane r stores the block's triple into block r's slot of this block
             const uint32_t slot = (uint32_t)__cvta_generic_to_shared(&block_stat[rank]);
             uint32_t remote;
             asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(slot), "r"(lane));
-            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(mine.n) : "memory");
-            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote + 4), "f"(mine.mean) : "memory");
-            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote + 8), "f"(mine.m2) : "memory");
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(s.n) : "memory");
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote + 4), "f"(s.mean) : "memory");
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote + 8), "f"(s.m2) : "memory");
         }
         gn_cluster_arrive();
         gn_cluster_wait();
         s = block_stat[0];
         for (int r = 1; r < cluster; ++r) s = gn_merge(s, block_stat[r]);
-    } else {
-        s.mean = __shfl_sync(0xffffffffu, s.mean, 0);
-        s.m2 = __shfl_sync(0xffffffffu, s.m2, 0);
     }
-    const float rstd = 1.0f / sqrtf(s.m2 / (float)n_elems + a.eps);
 
     // ---- y = x * scale + shift
-    auto affine_of = [&](int c, float& scale, float& shift) {
-        const float ga = a.gamma ? gn_to_float(affine[0][c]) : 1.f, be = a.beta ? gn_to_float(affine[1][c]) : 0.f;
-        scale = rstd * ga;
-        shift = fmaf(-s.mean, scale, be);
-    };
+    if (prepares) {
+        const float rstd = 1.0f / sqrtf(s.m2 / (float)n_elems + a.eps);
+        for (int c = tid; c < cpg; c += THREADS) {
+            if (c != tid) parameters(c, ga, be);
+            const float scale = rstd * ga;
+            affine[c] = make_float2(scale, fmaf(-s.mean, scale, be));
+        }
+    }
+    __syncthreads();
+    uint4* to = reinterpret_cast<uint4*>(dst + head) + p0;
 #pragma unroll
     for (int k = 0; k < PPT; ++k) {
-        const int p = rank * pieces_per_block + tid + k * (int)blockDim.x, e0 = head + p * VEC;
-        if (p >= p_end) continue;
-        const int c = (int)fast_div((uint32_t)e0, plan.by_hw);
-        const int left = (c + 1) * hw - e0;   // values of the piece before the next channel begins
-        float scale, shift;
-        affine_of(c, scale, shift);
+        if (p0 + k * THREADS >= p_end) continue;
+        const int e0 = head + (p0 + k * THREADS) * VEC, c = (int)fast_div((uint32_t)e0, plan.by_hw);
+        const float2 f = affine[c];
         uint4 o;
-        gn_affine_piece<T, VEC>(v[k], scale, shift, o);
-        if (RAGGED && left < VEC) {
-            // a channel boundary inside (one: hw >= VEC), and another channel behind it, as the piece lies inside the group:
-            // the words behind the boundary come from a second evaluation
-            affine_of(c + 1, scale, shift);
-            uint4 o1;
-            gn_affine_piece<T, VEC>(v[k], scale, shift, o1);
-            uint32_t* w = reinterpret_cast<uint32_t*>(&o);
-            const uint32_t* w1 = reinterpret_cast<const uint32_t*>(&o1);
+        gn_affine_piece<T, VEC>(v[k], f.x, f.y, o);
+        if (RAGGED) {
+            const int left = (c + 1) * hw - e0;   // values of the piece before the next channel begins
+            if (left < VEC) {
+                // a channel boundary inside (one: hw >= VEC), and another channel behind it, as the piece lies inside the group:
+                // the words behind the boundary come from a second evaluation
+                const float2 f1 = affine[c + 1];
+                uint4 o1;
+                gn_affine_piece<T, VEC>(v[k], f1.x, f1.y, o1);
+                uint32_t* w = reinterpret_cast<uint32_t*>(&o);
+                const uint32_t* w1 = reinterpret_cast<const uint32_t*>(&o1);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint32_t m = left * (int)sizeof(T) >= 4 * i + 4 ? 0u : left * (int)sizeof(T) > 4 * i ? 0xffff0000u : 0xffffffffu;
-                w[i] = (w[i] & ~m) | (w1[i] & m);
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t m = left * (int)sizeof(T) >= 4 * i + 4 ? 0u : left * (int)sizeof(T) > 4 * i ? 0xffff0000u : 0xffffffffu;
+                    w[i] = (w[i] & ~m) | (w1[i] & m);
+                }
             }
         }
-        *reinterpret_cast<uint4*>(dst + e0) = o;
+        to[k * THREADS] = o;
     }
     if (has_lone) {
-        float scale, shift;
-        affine_of((int)fast_div((uint32_t)lone, plan.by_hw), scale, shift);
-        gn_from_float(dst[lone], fmaf(lone_x, scale, shift));
+        const float2 f = affine[fast_div((uint32_t)lone, plan.by_hw)];
+        gn_from_float(dst[lone], fmaf(lone_x, f.x, f.y));
     }
 }
 

@@ -33,6 +33,17 @@ def test_groupnorm_group_sizes_at_the_edges_of_a_plan(bd, dtype, pieces_times):
     gn.check(gn.run(bd, x, 2, 1e-5, gamma, beta), x, 2, 1e-5, gamma, beta, what=str(pieces_times))
 
 
+# (groups, 16-byte pieces of each): blocks per group and threads per block, on either side of every line of the plan on 148 SMs
+@pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
+@pytest.mark.parametrize("groups,pieces", [(33, 5119), (33, 5120), (34, 5120), (74, 2559), (74, 2560), (75, 2560), (74, 10240), (74, 10241),
+                                           (33, 20480), (33, 20481), (148, 2561), (148, 4097), (148, 6144), (148, 6145), (149, 4097), (149, 6145)])
+@pytest.mark.parametrize("odd", [0, 3])   # values more than whole pieces: ragged groups
+def test_groupnorm_blocks_of_a_group(bd, dtype, groups, pieces, odd):
+    vec = 16 // np.dtype(dtype).itemsize
+    x, gamma, beta = gn.make(groups + pieces, (1, groups, pieces * vec - odd), dtype, scale=0.9, shift=0.5)
+    gn.check(gn.run(bd, x, groups, 1e-5, gamma, beta), x, groups, 1e-5, gamma, beta, what=str((groups, pieces, odd)))
+
+
 @pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
 @pytest.mark.parametrize("C,HW,G", [(12, 9, 3), (6, 5, 1), (40, 31, 8), (10, 5525, 1), (20, 4757, 2), (64, 37, 32), (1030, 9, 1),
                                     (2, 24577, 1), (2, 8, 2), (4, 4, 1)])
