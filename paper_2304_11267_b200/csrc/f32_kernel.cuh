@@ -8,8 +8,13 @@
 // goes into a fresh accumulator and is added to the running output on the CUDA cores, rounded to nearest -- and inside a
 // tile the small terms are issued first.  (4096 tokens, d = 40: relative error 2.9e-7, with plain binary32 FMAs 1.2e-6.)
 //
-// Bound: six bf16 products per binary32 one, 1152 tensor clocks per 128 x 64 tile of scores at d = 40 (and reads of Q and K
-// from shared memory that make it about 1440) against 6000 clocks of the FMA pipe.
+// Eight columns left behind the whole 16-column steps of Q K^T (d = 40: 32 and 8) do not take six half-empty steps but share three: what
+// they contribute is l h + h l, m m + m h and h m + h h, two terms a step, with [l | h], [m | m], [h | h] of Q against [h | l], [m | h],
+// [m | h] of K.
+//
+// Bound: the softmax warps.  A key tile of two query tiles takes about 3900 clocks, of which a sweep is 2500 (clock stamps: exponentials,
+// and on the half-rate integer pipe the splitting of the weights, with four warps a scheduler in it at once) and the rest waits and the
+// addition of the product; six bf16 products per binary32 one are 960 tensor clocks per 128 x 64 tile of scores at d = 40.
 //
 // One CTA: T query tiles of 128 rows.  Warpgroups (four warps each):
 //   softmax     two per query tile, thread = half a query row: its scores from tensor memory into registers, exp2, row sum; the
@@ -31,9 +36,8 @@
 // Operands in shared memory are [part h, m, l][32-column chunk][row][64 bytes].  V is used as it lies (MN-major).  Where one
 // query tile leaves room in tensor memory, its Q goes there: read from shared memory, 128 rows for each product of 32 or 64 keys
 // were most of the product's time.
-// us in a graph, operands of S in shared memory, undivided issuing loops, rows stored one by one -> now: 16 x 4096 x 4096, d = 40 285 ->
-// 262 (293 a call through the entry point with other work between);
-// 16 x 1024, d = 80 40.1 -> 34.8; 16 x 256, d = 160 35.6 -> 27.8; 16 x 256 x 77, d = 160 21.1 -> 16.1.
+// us a call, half-empty steps, steps counted at run time, parts taken out with masks -> now: 16 x 4096 x 4096, d = 40 285 -> 270, 3000
+// 196 -> 177; 16 x 1024, d = 64 29.9 -> 29.2, d = 80 35.7 -> 35.4; 16 x 600, d = 120 50.5 -> 41.1; 16 x 256, d = 160 27.7 -> 24.6.
 // Every wait is bounded and reports to the status block.
 #pragma once
 #include <cuda_runtime.h>
@@ -67,11 +71,13 @@ struct F32Args {
 // softmax thread.  KS, VS: depth of the K and V rings.  NO: buffers for the product of a key tile.  MAX_FIRST: whether a key tile
 // fits the anchor is decided from its maximum before the exponentials, so that the weights replace the scores in registers,
 // not from the weights' sum behind them (measured: d = 80 43 -> 36 us; the other shapes lose 2% to 12% by it).
-template <int NC_, int BN_, int T_, int ACC_, int KS_, int VS_, int NO_, bool MAX_FIRST_>
+template <int NC_, int BN_, int T_, int ACC_, int KS_, int VS_, int NO_, bool MAX_FIRST_, int MIN_PIECES_>
 struct F32Shape {
     static constexpr int NC = NC_, BN = BN_, T = T_, ACC = ACC_, KS = KS_, VS = VS_, NO = NO_;
     static constexpr bool MAX_FIRST = MAX_FIRST_;
+    static constexpr int MIN_PIECES = MIN_PIECES_;   // of eight columns
     static constexpr int MAX_D = NC * F3_CHUNK < 2 * ACC ? NC * F3_CHUNK : 2 * ACC;
+    static constexpr int MAX_PIECES = MAX_D / 8;
     static constexpr int N_CONV = T == 2 ? 1 : 2;   // warpgroups that convert K; as many for V
     static constexpr int WG_CONVERT = 2 * T, WG_ISSUE = WG_CONVERT + 2 * N_CONV, THREADS = (WG_ISSUE + 1) * 128;
     static constexpr int Q_PART = NC * TILE_M * 64, Q_TILE = 3 * Q_PART, KV_PART = NC * BN * 64, KV_STAGE = 3 * KV_PART;
@@ -81,9 +87,10 @@ struct F32Shape {
     // halves of a row need not wait for one another: word `off` of part (h, m) of half x at x BN/2 + (0, BN/4) + off, of
     // part l at BN + x BN/4 + off.
     static constexpr int HALF = BN / 2, SLOT = 3 * BN / 2, O_COLS = 2 * ACC;
-    static constexpr bool Q_TMEM = T == 1;             // (two query tiles leave 32 columns)
+    static constexpr bool Q_TMEM = T == 1;             // (two query tiles leave 32 columns: part h, Q_STEPS steps of it)
     static constexpr int Q_COLS = NC * F3_CHUNK / 2;   // of a part
-    static constexpr int TILE_COLS = 2 * SLOT + NO * O_COLS + (Q_TMEM ? 3 * Q_COLS : 0);
+    static constexpr int Q_STEPS = 2;
+    static constexpr int TILE_COLS = 2 * SLOT + NO * O_COLS + (Q_TMEM ? 3 * Q_COLS : 8 * Q_STEPS);
     static_assert(T * TILE_COLS <= 512, "tensor memory");
     // registers: the pools of setmaxnreg must not exceed what the CTA was launched with
     static constexpr int LAUNCH_REGS = 65536 / THREADS / 8 * 8;
@@ -92,10 +99,10 @@ struct F32Shape {
     static constexpr int POOL = 128 * (2 * T * SOFTMAX_REGS + 2 * N_CONV * CONVERT_REGS + ISSUE_REGS);
     static_assert(POOL <= THREADS * LAUNCH_REGS, "setmaxnreg budget");
 };
-using F32Two = F32Shape<2, 64, 2, 24, 2, 2, 1, false>;     // d <= 48, two query tiles
-using F32One = F32Shape<2, 64, 1, 32, 3, 3, 2, false>;     // d <= 64
-using F32Mid = F32Shape<3, 64, 1, 48, 2, 2, 1, true>;     // d <= 96
-using F32Wide = F32Shape<5, 32, 1, 80, 2, 1, 1, true>;    // d <= 160
+using F32Two = F32Shape<2, 64, 2, 24, 2, 2, 1, false, 1>;     // d <= 48, two query tiles
+using F32One = F32Shape<2, 64, 1, 32, 3, 3, 2, false, 1>;     // d <= 64
+using F32Mid = F32Shape<3, 64, 1, 48, 2, 2, 1, true, 9>;     // d <= 96
+using F32Wide = F32Shape<5, 32, 1, 80, 2, 1, 1, true, 13>;    // d <= 160
 constexpr float F32_TILE_SUM_LIMIT = 1.8446744e19f; // 2^64: no weight above it reaches the products
 constexpr float F32_MAX_LIMIT = 58.f;               // log2 of the largest weight where the maximum decides: 64 of them stay below the sum
 
@@ -105,21 +112,30 @@ __host__ __device__ constexpr uint64_t smem_desc_sw64(uint32_t byte_addr, uint32
            ((uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32) | (1ull << 46) | (4ull << 61);
 }
 
+// x minus a packed bfloat16 value, the low or the high one: one mixed multiply-add on the FMA pipe, exact here.  (Taking the parts out as
+// binary32 values first costs two shifts or masks a pair on the half-rate integer pipe.)
+__device__ __forceinline__ float less_low_bf16(float x, uint32_t packed) {
+    float d;
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tfma.rn.f32.bf16 %0, l, %2, %3;\n\t}" : "=f"(d) : "r"(packed), "h"((unsigned short)0xBF80), "f"(x));
+    return d;
+}
+__device__ __forceinline__ float less_high_bf16(float x, uint32_t packed) {
+    float d;
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tfma.rn.f32.bf16 %0, h, %2, %3;\n\t}" : "=f"(d) : "r"(packed), "h"((unsigned short)0xBF80), "f"(x));
+    return d;
+}
 // The three bf16 parts of a pair of binary32 values, packed (low half = first value), rounded to nearest.
 __device__ __forceinline__ void split_pair_rn(float x0, float x1, uint32_t& h, uint32_t& m, uint32_t& l) {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(x1), "f"(x0));
-    const uint64_t r = sub_f32x2(pack_b64(__float_as_uint(x0), __float_as_uint(x1)), pack_b64(h << 16, h & 0xffff0000u));
-    uint32_t r0, r1;
-    unpack_b64(r, r0, r1);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m) : "f"(__uint_as_float(r1)), "f"(__uint_as_float(r0)));
-    const uint64_t t = sub_f32x2(r, pack_b64(m << 16, m & 0xffff0000u));
-    uint32_t t0, t1;
-    unpack_b64(t, t0, t1);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(__uint_as_float(t1)), "f"(__uint_as_float(t0)));
+    const float r0 = less_low_bf16(x0, h), r1 = less_high_bf16(x1, h);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m) : "f"(r1), "f"(r0));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(less_high_bf16(r1, m)), "f"(less_low_bf16(r0, m)));
 }
 
-// Eight columns, split into their three parts, `part` bytes apart.
-__device__ __forceinline__ void f32_store_at(uint32_t at, uint32_t part, const float4& lo, const float4& hi) {
+// Eight columns, split into their three parts, `part` bytes apart.  PAIRED: what shares their contraction step in each part (see the
+// file's comment), of Q or of K.
+enum F32Paired { F3_ALONE, F3_PAIR_Q, F3_PAIR_K };
+__device__ __forceinline__ void f32_store_at(uint32_t at, uint32_t part, const float4& lo, const float4& hi, F32Paired paired) {
     uint4 h, m, l;
     split_pair_rn(lo.x, lo.y, h.x, m.x, l.x);
     split_pair_rn(lo.z, lo.w, h.y, m.y, l.y);
@@ -127,7 +143,33 @@ __device__ __forceinline__ void f32_store_at(uint32_t at, uint32_t part, const f
     split_pair_rn(hi.z, hi.w, h.w, m.w, l.w);
     st_shared_v4(at, h);
     st_shared_v4(at + part, m);
-    st_shared_v4(at + 2 * part, l);
+    if (paired != F3_PAIR_K) st_shared_v4(at + 2 * part, l);
+    if (paired == F3_PAIR_Q) {          // h h | m m | l h
+        st_shared_v4(at ^ 16, h);
+        st_shared_v4((at + part) ^ 16, m);
+        st_shared_v4((at + 2 * part) ^ 16, h);
+    } else if (paired == F3_PAIR_K) {   // h l | m h
+        st_shared_v4(at ^ 16, l);
+        st_shared_v4((at + part) ^ 16, h);
+    }
+}
+// The contraction of Q K^T: steps of 16 columns of one part each, and whether the eight columns behind them share steps with another part's.
+// (PIECES eight columns; known at compile time, as steps counted at run time spill in the issuing warps: 2 x 8 x 600 x 600, d = 120
+// 63.6 us against 50.2, and 256, d = 160 27.6 against 25.8)
+template <int PIECES>
+struct F32Steps {
+    static constexpr int whole = PIECES / 2;
+    static constexpr bool left = PIECES % 2 != 0;
+};
+template <int LO, int HI, typename F>
+__device__ __forceinline__ void f32_with_steps(int pieces, const F& f) {
+    if constexpr (LO == HI) {
+        f(F32Steps<LO>{});
+    } else {
+        constexpr int MID = (LO + HI) / 2;
+        if (pieces <= MID) f32_with_steps<LO, MID>(pieces, f);
+        else f32_with_steps<MID + 1, HI>(pieces, f);
+    }
 }
 
 // Convert warpgroups: a tile of ROWS rows of d binary32 values as pieces of eight columns; thread i of THREADS takes pieces
@@ -138,9 +180,9 @@ struct F32Converter {
     const float* base;      // row 0 of the head
     long long tile_step;    // elements from one tile to the next
     int rows, d;            // rows of the head
-    int at_g[MAX_PIECES], at_s[MAX_PIECES];   // the piece in global memory and in the tile; at_s < 0: none
+    int at_g[MAX_PIECES], at_s[MAX_PIECES];   // the piece in global memory and in the tile (bit 0: half of it; bit 1: paired); at_s < 0: none
     float4 lo[MAX_PIECES], hi[MAX_PIECES];
-    __device__ __forceinline__ void init(const float* head, int ld, int rows_, int d_, int i, const FastDiv& by_pieces) {
+    __device__ __forceinline__ void init(const float* head, int ld, int rows_, int d_, int i, const FastDiv& by_pieces, bool is_k) {
         base = head; rows = rows_; d = d_;
         tile_step = (long long)ROWS * ld;
 #pragma unroll
@@ -149,6 +191,7 @@ struct F32Converter {
             at_g[u] = r * ld + p * 8;
             at_s[u] = r < ROWS ? (((p >> 2) * ROWS + r) << 6) + (((p & 3) ^ ((r >> 1) & 3)) << 4) : -1;
             if (p * 8 + 8 > d) at_s[u] |= 1;   // half a piece (d is a multiple of 4)
+            if (is_k && !(p & 1) && p == (int)by_pieces.d - 1) at_s[u] |= 2;
         }
     }
     __device__ __forceinline__ void fetch(int j) {
@@ -166,7 +209,7 @@ struct F32Converter {
     __device__ __forceinline__ void store(uint32_t tile) const {
 #pragma unroll
         for (int u = 0; u < MAX_PIECES; ++u)
-            if (at_s[u] >= 0) f32_store_at(tile + (at_s[u] & ~1), NC * ROWS * 64, lo[u], hi[u]);
+            if (at_s[u] >= 0) f32_store_at(tile + (at_s[u] & ~3), NC * ROWS * 64, lo[u], hi[u], at_s[u] & 2 ? F3_PAIR_K : F3_ALONE);
     }
 };
 
@@ -285,18 +328,7 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
         tmem_alloc(smem_u32(&tmem_base_slot), 512);
         tmem_relinquish();
     }
-    // a contraction step is 16 columns, a converted piece eight: where the last step is half real, its other half stays zero
     const int pieces = (d + 7) >> 3;
-    if (pieces & 1) {
-        constexpr int Q_ROWS = SH::T * 3 * TILE_M, K_ROWS = (KS + VS) * 3 * BN;
-        for (int i = tid; i < Q_ROWS + K_ROWS; i += SH::THREADS) {
-            const bool is_q = i < Q_ROWS;
-            const int rows = is_q ? TILE_M : BN, n = is_q ? i : i - Q_ROWS, part = n / rows, r = n - part * rows;
-            const uint32_t base = (is_q ? q_smem : k_smem) + part * (NC * rows * 64);   // parts and stages follow one another
-            st_shared_v4(base + (pieces >> 2) * (rows * 64) + r * 64 + (((pieces & 3) ^ ((r >> 1) & 3)) << 4), make_uint4(0u, 0u, 0u, 0u));
-        }
-        fence_proxy_async_smem();
-    }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -328,17 +360,18 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                 const int p = idx - r * pieces;
                 if (idx < TILE_M * pieces)
                     f32_store_at(q_smem + t * SH::Q_TILE + (p >> 2) * (TILE_M * 64) + r * 64 + (((p & 3) ^ ((r >> 1) & 3)) << 4), SH::Q_PART,
-                                 lo[u], hi[u]);
+                                 lo[u], hi[u], !(p & 1) && p == pieces - 1 ? F3_PAIR_Q : F3_ALONE);
             }
         }
-        if constexpr (SH::Q_TMEM) {   // thread = row: its steps of 16 columns, every second one
+        if (!SH::Q_TMEM) fence_proxy_async_smem();
+        {   // thread = row: its steps of 16 columns, every second one
             named_barrier(1 + t, 256);
             const int row = i & 127, sw = (row >> 1) & 3;
             const uint32_t src = q_smem + t * SH::Q_TILE + row * 64, dst = tmem_q(t) + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll
-            for (int part = 0; part < 3; ++part)
+            for (int part = 0; part < (SH::Q_TMEM ? 3 : 1); ++part)
 #pragma unroll
-                for (int kk = 0; kk < 2 * NC; ++kk) {
+                for (int kk = 0; kk < (SH::Q_TMEM ? 2 * NC : SH::Q_STEPS); ++kk) {
                     if ((kk & 1) != i >> 7 || kk * 16 >= d) continue;
                     const uint32_t at = src + part * SH::Q_PART + (kk >> 1) * (TILE_M * 64);
                     const uint4 a = ld_shared_v4(at + ((((kk & 1) * 2) ^ sw) << 4)), b = ld_shared_v4(at + ((((kk & 1) * 2 + 1) ^ sw) << 4));
@@ -347,8 +380,6 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                 }
             tmem_wait_st();
             tc_fence_before_sync();
-        } else {
-            fence_proxy_async_smem();
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bars.q_full[t]));
@@ -369,36 +400,48 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
             if ((warp & 1) == 0) {
                 // ------------------------------------------------------------ S_t(j) = Q_t K(j)^T
                 const uint32_t idesc = idesc_f16(TILE_M, BN, false, false, args.negate != 0, true);
-                const int ksteps = (d + 15) / 16;
                 const uint64_t q_desc = smem_desc_sw64(q_smem + t * SH::Q_TILE, 16, 512), k_desc = smem_desc_sw64(k_smem, 16, 512);
-                ok = wait(bars.q_full[t], 0, SITE_F_Q, t);
-                int s = 0, pk = 0;
-                for (int j = 0; j < n_kv && ok; ++j) {
-                    const int b = j & 1;
-                    ok = wait(bars.k_full[s], pk, SITE_F_K, j);
-                    if (ok && j >= 2) ok = wait(bars.slot_free[t][b], ((j >> 1) - 1) & 1, SITE_F_SLOT, j);
-                    if (!ok) break;
-                    tc_fence_after_sync();
-                    const uint64_t kd = k_desc + (uint64_t)(s * (SH::KV_STAGE >> 4));
-                    const uint32_t ts = tmem_slot(t, b);
-                    if (leader) {
+                auto scores = [&](auto steps) {
+                    constexpr int whole = decltype(steps)::whole;
+                    constexpr bool left = decltype(steps)::left;
+                    ok = wait(bars.q_full[t], 0, SITE_F_Q, t);
+                    // The second query tile begins when the first has its first weights: in step, both sweep at once and then both
+                    // wait (16 x 4096 x 4096, d = 40 282 -> 280 us).  Tile 0 hands over no further weights through this
+                    // barrier before tile 1 has let go of key tile 0, which the ring of K then waits for.
+                    if (t == 1) ok = ok && wait(bars.p_full[0][0], 0, SITE_F_P, 0);
+                    int s = 0, pk = 0;
+                    for (int j = 0; j < n_kv && ok; ++j) {
+                        const int b = j & 1;
+                        ok = wait(bars.k_full[s], pk, SITE_F_K, j);
+                        if (ok && j >= 2) ok = wait(bars.slot_free[t][b], ((j >> 1) - 1) & 1, SITE_F_SLOT, j);
+                        if (!ok) break;
+                        tc_fence_after_sync();
+                        const uint64_t kd = k_desc + (uint64_t)(s * (SH::KV_STAGE >> 4));
+                        const uint32_t ts = tmem_slot(t, b);
+                        if (leader) {
+                            auto step = [&](int pa, int pb, int kk, bool q_tmem, bool acc) {
+                                const uint64_t kt = kd + (uint64_t)((pb * SH::KV_PART + (kk >> 1) * (BN * 64) + (kk & 1) * 32) >> 4);
+                                if (q_tmem)
+                                    mma_f16_ts(ts, tmem_q(t) + pa * SH::Q_COLS + kk * 8, kt, idesc, acc);
+                                else
+                                    mma_f16_ss(ts, q_desc + (uint64_t)((pa * SH::Q_PART + (kk >> 1) * (TILE_M * 64) + (kk & 1) * 32) >> 4), kt, idesc, acc);
+                            };
+                            if (left) step(2, 0, whole, SH::Q_TMEM, false);       // l h + h l
 #pragma unroll
-                        for (int p = 0; p < 6; ++p)
+                            for (int p = 0; p < 6; ++p) {
+                                if (left && p == 3) step(1, 1, whole, SH::Q_TMEM, true);   // m m + m h
+                                if (left && p == 5) step(0, 1, whole, SH::Q_TMEM, true);   // h m + h h
 #pragma unroll
-                            for (int kk = 0; kk < 2 * NC; ++kk)   // (offsets are constants)
-                                if (kk < ksteps) {
-                                    const uint64_t kt = kd + (uint64_t)((PB[p] * SH::KV_PART + (kk >> 1) * (BN * 64) + (kk & 1) * 32) >> 4);
-                                    if constexpr (SH::Q_TMEM)
-                                        mma_f16_ts(ts, tmem_q(t) + PA[p] * SH::Q_COLS + kk * 8, kt, idesc, p > 0 || kk > 0);
-                                    else
-                                        mma_f16_ss(ts, q_desc + (uint64_t)((PA[p] * SH::Q_PART + (kk >> 1) * (TILE_M * 64) + (kk & 1) * 32) >> 4),
-                                                   kt, idesc, p > 0 || kk > 0);
-                                }
-                        tc_commit(smem_u32(&bars.s_full[t][b]));
-                        tc_commit(smem_u32(&bars.k_empty[s]));
+                                for (int kk = 0; kk < 2 * NC; ++kk)   // (offsets are constants)
+                                    if (kk < whole) step(PA[p], PB[p], kk, SH::Q_TMEM || (PA[p] == 0 && kk < SH::Q_STEPS), left || p > 0 || kk > 0);
+                            }
+                            tc_commit(smem_u32(&bars.s_full[t][b]));
+                            tc_commit(smem_u32(&bars.k_empty[s]));
+                        }
+                        if (++s == KS) { s = 0; pk ^= 1; }
                     }
-                    if (++s == KS) { s = 0; pk ^= 1; }
-                }
+                };
+                f32_with_steps<SH::MIN_PIECES, SH::MAX_PIECES>(pieces, scores);
             } else {
                 // ------------------------------------------------------------ O_t = P_t(j) V(j)
                 auto weights_at = [](int part, int kk) {   // 16 keys of a part (see F32Shape)
@@ -440,7 +483,7 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
         bool ok = true;
         F32Converter<NC, BN, 128 * SH::N_CONV, SH::MAX_D> cv;
         cv.init(head_row(which == 0 ? args.k : args.v, args.lk, bh, 0), args.lk.ld, args.Nk, d, (wg - SH::WG_CONVERT) % SH::N_CONV * 128 + wt,
-                args.by_pieces);
+                args.by_pieces, which == 0);
         const int depth = which == 0 ? KS : VS;
         const uint32_t ring = which == 0 ? k_smem : v_smem;
         uint64_t* full = which == 0 ? bars.k_full : bars.v_full;
@@ -546,14 +589,9 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                             const uint64_t pp = pack_b64(q0, q1);
                             sum[i & 1] = add_f32x2(sum[i & 1], pp);
                             h[i] = high_halves(q0, q1);
-                            const uint64_t r = sub_f32x2(pp, pack_b64(q0 & 0xffff0000u, q1 & 0xffff0000u));
-                            uint32_t r0, r1;
-                            unpack_b64(r, r0, r1);
-                            m[i] = high_halves(r0, r1);
-                            const uint64_t u = sub_f32x2(r, pack_b64(r0 & 0xffff0000u, r1 & 0xffff0000u));
-                            uint32_t u0, u1;
-                            unpack_b64(u, u0, u1);
-                            l[i] = high_halves(u0, u1);
+                            const float r0 = less_low_bf16(p0, h[i]), r1 = less_high_bf16(p1, h[i]);
+                            m[i] = high_halves(__float_as_uint(r0), __float_as_uint(r1));
+                            l[i] = high_halves(__float_as_uint(less_low_bf16(r0, m[i])), __float_as_uint(less_high_bf16(r1, m[i])));
                         }
                         const uint32_t own = slot + half * HALF + c / 2;   // over scores that sit in registers
                         tmem_st4(own, h);
