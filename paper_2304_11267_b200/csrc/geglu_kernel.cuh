@@ -12,8 +12,10 @@
 // would cancel.  A thread takes UNROLL pairs of 16-byte pieces (one of each half of a row), all fetched before it computes
 // anything, and ends; finding a piece's row is one multiplication (a 64-bit division per piece was a third of the
 // instructions).  Two elements at a time on the packed binary32 pipe come to 20 instructions per element (ncu), about 16 of them arithmetic.
-// 8192 x 1280 fp16 (63 MB): 13.0 us a call through the entry point = 4.8 TB/s, 11.9 in a graph (16.4 with the division, a grid-stride
-// loop and 28 instructions per element, launched without overlap); fp32: 19.2 us = 6.55 TB/s, the copy rate (22.3).
+// A block asks for its pieces in the L2 before the stream's previous kernel has completed: the first blocks' fetch from memory then
+// runs under that kernel's end (8192 x 1280 fp16 11.6 -> 10.6 us a call in a loop, 12000 17.6 -> 16.5, 36864 51.5 -> 49.9).
+// 8192 x 1280 fp16 (63 MB): 10.6 us a call through the entry point = 5.9 TB/s (16.4 with the division, a grid-stride
+// loop and 28 instructions per element, launched without overlap); fp32: 19.5 us = 6.5 TB/s, the copy rate (22.3).
 #pragma once
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -118,19 +120,25 @@ template <typename T, int VEC, int UNROLL, bool BIG>
 __global__ void __launch_bounds__(GEGLU_THREADS)
 geglu_vector_kernel(const T* __restrict__ x, T* __restrict__ out, long long pieces, FastDiv row) {
     if (threadIdx.x == 0) pdl_launch_dependents();
-    pdl_wait();   // x may come from the previous kernel of the stream
     const long long p0 = (long long)blockIdx.x * (GEGLU_THREADS * UNROLL) + threadIdx.x;
-    uint4 a[UNROLL], g[UNROLL];
+    const uint4* src[UNROLL];
 #pragma unroll
     for (int u = 0; u < UNROLL; ++u) {
-        const long long p = p0 + u * GEGLU_THREADS;
-        if (p < pieces) {
-            const long long r = BIG ? p / row.d : (long long)fast_div((uint32_t)p, row);
-            const uint4* src = reinterpret_cast<const uint4*>(x) + (p + r * row.d);   // row r starts at piece 2 r d
-            a[u] = __ldg(src);
-            g[u] = __ldg(src + row.d);
+        const long long p = p0 + u * GEGLU_THREADS, r = BIG ? p / row.d : (long long)fast_div((uint32_t)p, row);
+        src[u] = reinterpret_cast<const uint4*>(x) + (p + r * row.d);   // row r starts at piece 2 r d
+        if (p < pieces && (threadIdx.x & 7) == 0) {
+            prefetch_l2(src[u]);
+            prefetch_l2(src[u] + row.d);
         }
     }
+    pdl_wait();   // x may come from the previous kernel of the stream
+    uint4 a[UNROLL], g[UNROLL];
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u)
+        if (p0 + u * GEGLU_THREADS < pieces) {
+            a[u] = __ldg(src[u]);
+            g[u] = __ldg(src[u] + row.d);
+        }
 #pragma unroll
     for (int u = 0; u < UNROLL; ++u) {
         const long long p = p0 + u * GEGLU_THREADS;

@@ -116,6 +116,7 @@ constexpr int GN_MAX_CPG = 1024;   // channels per group whose scale and shift t
 
 struct GroupNormPlan {
     int log2_cluster, pieces_per_block, cpg;   // blocks per group, 16-byte pieces of each, channels per group
+    int ahead;                                 // ask for the values in the L2 before the stream's previous kernel has completed
     FastDiv by_hw, by_groups;
 };
 
@@ -143,11 +144,16 @@ groupnorm_cluster_kernel(const GroupNormArgs a, const GroupNormPlan plan) {
 
     if (tid == 0) pdl_launch_dependents();
     if (cluster > 1) gn_cluster_arrive();   // every block of the cluster has started once the first wait returns
+    const uint4* from = reinterpret_cast<const uint4*>(src + head) + p0;
+    if (plan.ahead && (tid & 7) == 0) {
+#pragma unroll
+        for (int k = 0; k < PPT; ++k)
+            if (p0 + k * THREADS < p_end) prefetch_l2(from + k * THREADS);
+    }
     pdl_wait();
 
     uint4 v[PPT];
     {
-        const uint4* from = reinterpret_cast<const uint4*>(src + head) + p0;
 #pragma unroll
         for (int k = 0; k < PPT; ++k)
             if (p0 + k * THREADS < p_end) v[k] = from[k * THREADS];
