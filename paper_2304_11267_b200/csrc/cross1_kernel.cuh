@@ -188,6 +188,11 @@ cross1_attention_kernel(const __grid_constant__ Cross1ArgsT<NP> args) {
                     mbar_arrive_expect_tx(bar_qk + ch * 8, KV_BYTES / NCH);
                     tma_load_4d(k_smem + ch * KN * CHUNK_ROW_BYTES, &pr.tk, bar_qk + ch * 8, ch * CHUNK_COLS, 0, hz, bz);
                 }
+                // V behind K: its rows would keep the copy engine (about 3 clocks each) from those that the scores wait for
+                mbar_arrive_expect_tx(bar_v, KV_BYTES);
+#pragma unroll
+                for (int ch = 0; ch < NCH; ++ch)
+                    tma_load_4d(v_smem + ch * KN * CHUNK_ROW_BYTES, &pr.tv, bar_v, ch * CHUNK_COLS, 0, hz, bz);
             }
             const uint32_t idesc = idesc_f16(TILE_M, (d + 15) >> 4 << 4, false, true, false, BF);
             const uint64_t v_desc = smem_desc_sw128(v_smem, KN * CHUNK_ROW_BYTES, 1024);
@@ -201,13 +206,6 @@ cross1_attention_kernel(const __grid_constant__ Cross1ArgsT<NP> args) {
             }
         }
     } else {
-        if (!DENSE && warp == 0 && elect_one()) {
-            mbar_arrive_expect_tx(bar_v, KV_BYTES);
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch)
-                tma_load_4d(v_smem + ch * KN * CHUNK_ROW_BYTES, &pr.tv, bar_v, ch * CHUNK_COLS, 0, hz, bz);
-        }
-        __syncwarp();
         // ---- softmax: thread = query row = TMEM lane; the weights stay in registers
         const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
         const int valid = args.Nk;

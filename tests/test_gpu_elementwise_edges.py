@@ -65,3 +65,26 @@ def test_groupnorm_of_an_outlier_in_front(bd, dtype):
 def test_geglu_sizes_at_the_edges(bd, dtype, rows, C):
     x = geglu.make(rows + C, rows, C, dtype)
     geglu.check(bd.geglu(torch.from_numpy(x).cuda()).cpu().numpy(), x, what=str((rows, C)))
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.float32], ids=["f16", "f32"])
+def test_inputs_written_by_the_kernel_before(bd, dtype):
+    """Blocks ask for their input in the L2 while the kernel that writes it still runs: what they read is what it wrote."""
+    g = torch.Generator(device="cuda").manual_seed(3)
+    xs = [torch.randn(4096, 8192, generator=g, device="cuda").to(dtype) for _ in range(3)]
+    gn_x = torch.randn(12, 128, 64, 64, generator=g, device="cuda").to(dtype)
+    want, got = [], []
+    for x in xs:
+        a = bd.geglu(x)
+        torch.cuda.synchronize()
+        want.append(bd.geglu(a))
+        torch.cuda.synchronize()
+    b = bd.groupnorm(gn_x, 32)
+    torch.cuda.synchronize()
+    want.append(bd.groupnorm(b, 32))
+    torch.cuda.synchronize()
+    a, b = torch.empty_like(a), torch.empty_like(b)   # rewritten by every call
+    for x in xs:
+        got.append(bd.geglu(bd.geglu(x, out=a)))
+    got.append(bd.groupnorm(bd.groupnorm(gn_x, 32, out=b), 32))
+    assert all(torch.equal(w, o) for w, o in zip(want, got))
