@@ -36,8 +36,8 @@
 // Operands in shared memory are [part h, m, l][32-column chunk][row][64 bytes].  V is used as it lies (MN-major).  Where one
 // query tile leaves room in tensor memory, its Q goes there: read from shared memory, 128 rows for each product of 32 or 64 keys
 // were most of the product's time.
-// us a call, half-empty steps, steps counted at run time, parts taken out with masks -> now: 16 x 4096 x 4096, d = 40 285 -> 270, 3000
-// 196 -> 177; 16 x 1024, d = 64 29.9 -> 29.2, d = 80 35.7 -> 35.4; 16 x 600, d = 120 50.5 -> 41.1; 16 x 256, d = 160 27.7 -> 24.6.
+// us a call, half-empty steps, steps counted at run time, parts taken out with masks -> now: 16 x 4096 x 4096, d = 40 285 -> 267, 3000
+// 196 -> 176; 16 x 1024, d = 64 29.8 -> 29.0, d = 80 35.9 -> 35.0; 16 x 600, d = 120 50.0 -> 40.8; 16 x 256, d = 160 27.6 -> 24.5.
 // Every wait is bounded and reports to the status block.
 #pragma once
 #include <cuda_runtime.h>
@@ -532,14 +532,18 @@ f32_attention_kernel(const __grid_constant__ F32Args args) {
                 if (!good) return false;
                 tc_fence_after_sync();
                 const uint32_t src = tmem_o(t, ob) + c0 + lane_off;
+                constexpr int TOGETHER = ACC <= 48 ? 16 : 8;   // columns fetched together: a load and its wait are 130 clocks (80 spill)
 #pragma unroll
-                for (int c = 0; c < ACC; c += 8) {
+                for (int c = 0; c < ACC; c += TOGETHER) {
                     if (c < cols) {
-                        uint32_t x[8];
-                        tmem_ld8(src + c, x);
+                        uint32_t x[16];
+                        if (TOGETHER == 16 && c + 16 <= ACC) tmem_ld16(src + c, x);
+                        else tmem_ld8(src + c, *reinterpret_cast<uint32_t(*)[8]>(x));
                         tmem_wait_ld();
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) o[c / 2 + i] = add_f32x2(o[c / 2 + i], pack_b64(x[2 * i], x[2 * i + 1]));
+                        for (int i = 0; i < TOGETHER / 2; ++i)
+                            if (c + 2 * i < ACC && (i < 4 || c + 8 < cols))   // (columns behind d are not real)
+                                o[c / 2 + i] = add_f32x2(o[c / 2 + i], pack_b64(x[2 * i], x[2 * i + 1]));
                     }
                 }
                 tc_fence_before_sync();
