@@ -153,7 +153,8 @@ __device__ __noinline__ void f4s_store_piece(float* piece, uint32_t tmem_o, int 
 // stage's K is free for the next load when its scores are computed, not when its product is.  Where no stage is used twice, the
 // additional waits and commits only cost.  us plain / apart, 16 x N x N, d = 160: 144 6.57 / 6.71, 200 7.87 / 7.76, 256 7.83 / 7.64,
 // 1024 18.0 / 15.8; 32 x 192 6.66 / 6.84, x 300 8.95 / 8.68, x 576 23.1 / 21.4 (runs of one side differ by 0.3%).  At d <= 128 the ring
-// is deeper: 1024, d = 80 12.4 / 12.8.
+// is deeper: 1024, d = 80 12.4 / 12.8.  (Figures with one issuing thread for products and one for scores, as PLAIN has them; APART has
+// one per part.)
 enum { F4_PLAIN, F4_PACED, F4_APART };
 // NCH: 64-column chunks per row (head dim <= 64 * NCH); BF: bfloat16 tensors
 template <int POLY, int NCH, int SPLIT = 1, bool BF = false, int FORM = F4_PLAIN>
@@ -184,16 +185,17 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
         // tile's scores wait behind: with a wait there 82.7 us for 2 x 8 x 4096 x 4096, d = 40, without 80.9
         // (4 x 8 x 9216 x 9216: 750 and 739).  Paced: one per tile; with as many as the others have, unused, 41.6 us for
         // 16 x 2304 x 2304, d = 128, are 44.8.
-        uint64_t pv_done[F4_TILES][PRODUCTS];   // (SPLIT > 1: [part][0])
+        uint64_t pv_done[F4_TILES][PRODUCTS];   // (SPLIT > 1: [part][0]; K and V apart: [part][product modulo PRODUCTS])
         uint64_t k_first;                 // K of the first key tile, which the first scores need before anything of V
         uint64_t kv_full[F4_STAGES];      // (the first key tile: its V)
         uint64_t buf_free[F4S_BUFFERS];   // SPLIT > 1: the products reading a buffer's weights are done
-        uint64_t k_full[KV_APART ? F4_STAGES : 1], k_empty[KV_APART ? F4_STAGES : 1];   // KV_APART: K's (kv_full, kv_empty: V's)
+        // KV_APART: K's (kv_full, kv_empty: V's); "landed" barriers by key tile modulo F4_STAGES, not by stage (see the issuers)
+        uint64_t k_full[KV_APART ? F4_STAGES : 1], k_empty[KV_APART ? F4_STAGES : 1];
         uint64_t kv_empty[F4_STAGES];     // one commit per issuer: as many arrivals as the unit has query tiles
     };
     constexpr int N_BARRIERS = sizeof(Barriers) / sizeof(uint64_t);
     constexpr int P_FULL_FIRST = F4_TILES * F4S_BUFFERS, P_FULL_END = 2 * F4_TILES * F4S_BUFFERS;
-    constexpr int KV_EMPTY_FIRST = N_BARRIERS - F4_STAGES;
+    constexpr int KV_EMPTY_FIRST = N_BARRIERS - F4_STAGES, O_FINAL_FIRST = P_FULL_END + F4_TILES;
     __shared__ __align__(8) Barriers bars;
     auto& bar_s_full = bars.s_full;
     auto& bar_p_full = bars.p_full;
@@ -255,8 +257,14 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
             fence_proxy_async_smem();
             __syncwarp();
         }
-        for (int i = lane; i < N_BARRIERS; i += 32)
-            mbar_init(smem_u32(flat + i), i >= KV_EMPTY_FIRST ? (uint32_t)tiles : (i >= P_FULL_FIRST && i < P_FULL_END) ? 4u : 1u);
+        // (the condition only in the instances that have it: as a constant inside one expression it cost parts at d = 80 1.5%)
+        for (int i = lane; i < N_BARRIERS; i += 32) {
+            uint32_t arrivals = i >= KV_EMPTY_FIRST ? (uint32_t)tiles : (i >= P_FULL_FIRST && i < P_FULL_END) ? 4u : 1u;
+            if constexpr (KV_APART) {
+                if (i == O_FINAL_FIRST) arrivals = (uint32_t)min(SPLIT, n_kv_all);   // one per part
+            }
+            mbar_init(smem_u32(flat + i), arrivals);
+        }
         mbar_init_fence();
         __syncwarp();
     };
@@ -381,8 +389,9 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 int s = 0, pe = 1;
                 for (int j = 0; j < n_kv; ++j) {
                     if (j >= stages && !mbar_wait(smem_u32(&bars.k_empty[s]), pe, abort_p, args.status, SITE_G_EMPTY, j)) break;
-                    mbar_arrive_expect_tx(smem_u32(&bars.k_full[s]), kv_tile_bytes);
-                    load_tile(&pr.tk, kv_smem + s * 2 * kv_tile_bytes, smem_u32(&bars.k_full[s]), j);
+                    const uint32_t bar = smem_u32(&bars.k_full[j % F4_STAGES]);
+                    mbar_arrive_expect_tx(bar, kv_tile_bytes);
+                    load_tile(&pr.tk, kv_smem + s * 2 * kv_tile_bytes, bar, j);
                     if (++s == stages) { s = 0; pe ^= 1; }
                 }
             } else {
@@ -427,15 +436,86 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
             int s = 0, pe = 1;
             for (int j = 0; j < n_kv; ++j) {
                 if (j >= stages && !mbar_wait(smem_u32(&bar_kv_empty[s]), pe, abort_p, args.status, SITE_G_EMPTY, j)) break;
-                mbar_arrive_expect_tx(smem_u32(&bar_kv_full[s]), kv_tile_bytes);
+                const uint32_t bar = smem_u32(&bar_kv_full[j % F4_STAGES]);
+                mbar_arrive_expect_tx(bar, kv_tile_bytes);
                 for (int ch = 0; ch < nch; ++ch)
-                    tma_load_4d(kv_smem + (s * 2 + 1) * kv_tile_bytes + ch * BN * CHUNK_ROW_BYTES, &pr.tv, smem_u32(&bar_kv_full[s]),
-                                ch * CHUNK_COLS, (j0 + j) * BN, hz, bz);
+                    tma_load_4d(kv_smem + (s * 2 + 1) * kv_tile_bytes + ch * BN * CHUNK_ROW_BYTES, &pr.tv, bar, ch * CHUNK_COLS,
+                                (j0 + j) * BN, hz, bz);
                 if (++s == stages) { s = 0; pe ^= 1; }
             }
         }
         __syncwarp();
-    } else if (warp > 16 && warp <= 16 + F4_TILES) {
+    } else if (KV_APART && warp > 16 && warp <= 16 + SPLIT) {
+        // ------------------------------------------------------------ K and V apart: MMA issuers, one per part
+        // Issuer g waits for the weights P(j) of its part's key tile j, issues O_g (+)= P(j) V(j), and behind that product -- same thread, so
+        // in order, into the buffer it frees -- the scores of key tile j + NB, which belong to part (g + NB) % SPLIT.  (With a thread for
+        // all products and one for all scores, which waits for the products' completion: 16 x 256 x 256, d = 160 7.59 -> 7.38 us, 576
+        // 11.16 -> 10.79, 1024 15.6 -> 15.3.  Where K and V share a stage the wait for K(j + NB) holds the product of j up, and heads of fewer columns gain
+        // nothing apart either: 16 x 1024, d = 80 11.7 / 12.1, d = 64 10.5 / 11.4, 8 x 1024, d = 40 10.2 / 10.8.)
+        // Issuers are not ordered among one another, so every barrier has one consumer that takes its phases in order: scores and
+        // weights have one per part and buffer, and a landed key tile n the one of n % F4_STAGES: an even number, so all key tiles of a
+        // barrier are one issuer's, and no less than the stages, so its next load, n + F4_STAGES, comes behind load n + stages,
+        // which waits for what this issuer does with key tile n.
+        const int g = warp - 17;
+        if (elect_one()) {
+            const uint32_t idesc_s = idesc_f16(TILE_M, BN, false, false, pr.negate != 0, BF);
+            const uint32_t idesc_o = idesc_f16(TILE_M, dpad, false, true, false, BF);
+            const int ksteps_s = (args.d + 15) / 16;   // 16 columns each; four to a swizzled 64-column chunk
+            const uint64_t q_desc = smem_desc_sw128(q_smem, 16, 1024), k_desc0 = smem_desc_sw128(kv_smem, 16, 1024);
+            const uint64_t v_desc0 = smem_desc_sw128(kv_smem + kv_tile_bytes, BN * CHUNK_ROW_BYTES, 1024);
+            constexpr uint32_t stage_off = (2 * kv_tile_bytes) >> 4;
+            const uint32_t to = tmem_o0 + g * dpad;
+            const int part_n = (g + NB) % SPLIT;   // whose scores this thread requests
+            auto issue_s = [&](int st, int b) {    // scores of the key tile in stage st into buffer b
+                const uint64_t kd = k_desc0 + (uint64_t)(st * stage_off);
+                const uint32_t ts = tmem_base + b * BN;
+#pragma unroll
+                for (int kk = 0; kk < 4 * NCH; ++kk)
+                    if (kk < ksteps_s)
+                        mma_f16_ss(ts, q_desc + (uint64_t)(((kk >> 2) * TILE_M * CHUNK_ROW_BYTES + (kk & 3) * 32) >> 4),
+                                   kd + (uint64_t)(((kk >> 2) * BN * CHUNK_ROW_BYTES + (kk & 3) * 32) >> 4), idesc_s, kk > 0);
+                tc_commit(smem_u32(&bar_s_full[part_n][b]));
+                tc_commit(smem_u32(&bars.k_empty[st]));   // done with K
+            };
+            auto landed = [&](uint64_t* full, int n) {
+                return mbar_wait(smem_u32(full + n % F4_STAGES), (n / F4_STAGES) & 1, abort_p, args.status, SITE_G_KV, n);
+            };
+            role_ready(ksteps_s, (int)idesc_s, (int)idesc_o);
+            bool ok = mbar_wait(smem_u32(&bar_q_full[0]), 0, abort_p, args.status, SITE_G_Q, 0);
+            for (int n = part_n; n < NB && n < n_kv && ok; n += SPLIT) {   // the first NB key tiles fill the buffers (stages >= NB)
+                ok = landed(bars.k_full, n);
+                if (!ok) break;
+                tc_fence_after_sync();
+                issue_s(n, n);
+            }
+            int b = g, ph = 0, met = 0;                    // buffer of key tile j; the part meets it every NB of its key tiles
+            int sj = g, sn = g + NB, i = 0;                // stages of key tiles j and j + NB, the product's barrier
+            if (sn >= stages) sn -= stages;
+            for (int j = g; j < n_kv && ok; j += SPLIT) {
+                const bool more = j + NB < n_kv;
+                if (more) ok = landed(bars.k_full, j + NB);   // (before the weights: off the way from them to the next scores)
+                ok = ok && landed(bars.kv_full, j);
+                ok = ok && mbar_wait_eager<P_TESTS>(smem_u32(&bar_p_full[g][b]), ph, abort_p, args.status, SITE_G_P, j);
+                if (!ok) break;
+                tc_fence_after_sync();
+                const uint64_t vd = v_desc0 + (uint64_t)(sj * stage_off);
+                const uint32_t tp = tmem_base + b * BN;
+#pragma unroll
+                for (int kk = 0; kk < BN / 16; ++kk)
+                    mma_f16_ts(to, tp + kk * 8, vd + (uint64_t)(kk * ((16 * CHUNK_ROW_BYTES) >> 4)), idesc_o, j >= SPLIT || kk > 0);
+                if (more) issue_s(sn, b);
+                tc_commit(smem_u32(&bar_kv_empty[sj]));     // done with V(j)
+                tc_commit(smem_u32(&bar_pv_done[g][i]));    // O_g holds the part's key tiles up to j
+                if ((b += SPLIT) >= NB) b -= NB;
+                if (++met == NB) { met = 0; ph ^= 1; }
+                if ((sj += SPLIT) >= stages) sj -= stages;
+                if ((sn += SPLIT) >= stages) sn -= stages;
+                if (++i == PRODUCTS) i = 0;
+            }
+            if (ok && g < n_kv) tc_commit(smem_u32(&bar_o_final[0]));
+        }
+        __syncwarp();
+    } else if (!KV_APART && warp > 16 && warp <= 16 + F4_TILES) {
         // ------------------------------------------------------------ MMA issuer of the steps of query tile t
         // Issuer t waits for P of its own tile's step k = T*j + t, issues O_t += P V(j), and then -- behind that
         // product, on the same thread, into the buffer it frees -- the scores of step k + NB, which belong to the
@@ -508,12 +588,11 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                         // (the buffer first: once product jn - NB has completed, V(0) has landed, which makes the parity wait
                         // for the second filling of stage 0 sound)
                         if (jn >= NB) ok = mbar_wait(smem_u32(&bar_buf_free[b]), ph, abort_p, args.status, SITE_G_PV, jn);
-                        ok = ok && mbar_wait(smem_u32(KV_APART ? &bars.k_full[sn] : jn == 0 ? &bar_k_first : &bar_kv_full[sn]), pn, abort_p,
+                        ok = ok && mbar_wait(smem_u32(jn == 0 ? &bar_k_first : &bar_kv_full[sn]), pn, abort_p,
                                              args.status, SITE_G_KV, jn);
                         if (!ok) break;
                         tc_fence_after_sync();
                         issue_s(q_desc_own_split, 0, sn, b);
-                        if (KV_APART) tc_commit(smem_u32(&bars.k_empty[sn]));   // done with K(jn)
                         if (++b == NB) { b = 0; if (jn >= NB) ph ^= 1; }
                         if (++sn == stages) { sn = 0; pn ^= 1; }
                     }
@@ -521,7 +600,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     int b = 0, ph = 0;
                     int sj = 0, pj = 0;                // stage and phase of key tile j
                     for (int j = 0; j < n_kv && ok; ++j) {
-                        if (KV_APART || j == 0) ok = mbar_wait(smem_u32(&bar_kv_full[sj]), pj, abort_p, args.status, SITE_G_KV, j);
+                        if (j == 0) ok = mbar_wait(smem_u32(&bar_kv_full[sj]), pj, abort_p, args.status, SITE_G_KV, j);
                         ok = ok && mbar_wait_eager<P_TESTS>(smem_u32(&bar_p_full[0][b]), ph, abort_p, args.status, SITE_G_P, j);
                         if (!ok) break;
                         tc_fence_after_sync();
@@ -611,6 +690,7 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
                 const uint32_t tmem_og = tmem_o0 + g * dpad + lane_off;
                 const uint32_t b_pvdone = smem_u32(&bar_pv_done[g][0]);   // products of THIS part's key tiles
+                const int own = KV_APART ? g : 0;   // (K and V apart: barriers per part)
                 const float c2 = pr.scale_log2e;
                 float m_run = 0.f, l_run = 0.f;   // anchor and row sum over this part's keys
                 bool ok = true;
@@ -618,12 +698,12 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 // barrier when NB is no multiple of SPLIT; the parity wait stays sound: the buffer's next scores need this
                 // tile's product, and its last ones, S(j - NB), completed before S(j - SPLIT), which this part has seen --
                 // NB >= SPLIT, and one thread's MMAs and commits complete in order.)
-                int b = g, ph = 0;
+                int b = g, ph = 0, met = 0;   // (K and V apart, NB odd: the part meets a buffer every NB of its key tiles)
                 touch_output(pr);
                 role_ready(args.Nk, __float_as_int(c2), NB);
                 for (int j = g, i = 0; j < n_kv; j += SPLIT, ++i) {
                     const uint32_t tmem_s = tmem_base + b * BN + lane_off;
-                    ok = mbar_wait(smem_u32(&bar_s_full[0][b]), ph, abort_p, args.status, SITE_G_S, j);
+                    ok = mbar_wait(smem_u32(&bar_s_full[own][b]), ph, abort_p, args.status, SITE_G_S, j);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     tc_fence_after_sync();
@@ -660,7 +740,8 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                         // product of this part's previous key tile has completed; nothing of this tile's weights is
                         // stored yet.  The first registers of the row are borrowed for O_g.
                         if (i > 0) {
-                            ok = mbar_wait(b_pvdone, (i - 1) & 1, abort_p, args.status, SITE_G_PV, j);
+                            ok = KV_APART ? mbar_wait(b_pvdone + (i - 1) % PRODUCTS * 8, ((i - 1) / PRODUCTS) & 1, abort_p, args.status, SITE_G_PV, j)
+                                          : mbar_wait(b_pvdone, (i - 1) & 1, abort_p, args.status, SITE_G_PV, j);
                             ok = __all_sync(0xffffffffu, ok);
                             if (!ok) break;
                             tc_fence_after_sync();
@@ -692,11 +773,16 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                     // (No phase of the part's completion barrier is waited for here.  The rare path above waits for the product of
                     // the part's previous key tile; the one before that is complete by then -- there are at most two
                     // buffers per part, so its buffer, or one freed behind it, holds the scores this thread has --, which keeps
-                    // that parity wait from being two phases behind.)
+                    // that parity wait from being two phases behind.  K and V apart: every product that is not complete keeps one
+                    // of the three buffers, so the one PRODUCTS before it, the last in its barrier, is.)
                     tc_fence_before_sync();
-                    if (lane == 0) mbar_arrive(smem_u32(&bar_p_full[0][b]));
+                    if (lane == 0) mbar_arrive(smem_u32(&bar_p_full[own][b]));
                     b += SPLIT;
-                    if (b >= NB) { b -= NB; ph ^= 1; }
+                    if (b >= NB) {
+                        b -= NB;
+                        if (!KV_APART) ph ^= 1;
+                    }
+                    if (KV_APART && ++met == NB) { met = 0; ph ^= 1; }
                 }
                 // ---- combine the parts: o = sum_g 2^(m_g - m) O_g / sum_g 2^(m_g - m) l_g, m = max_g m_g
                 part_ml[g][r] = make_float2(m_run, l_run);

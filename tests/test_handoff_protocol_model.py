@@ -293,3 +293,137 @@ def test_scores_must_wait_for_the_completion_of_the_products_they_overwrite():
     """Without the per-buffer completion barrier the second thread's scores can land on weights not yet read."""
     outcomes = {simulate_parts(2, 4, 17, 8, seed, wait_buf_free=False) for seed in range(12)}
     assert outcomes != {"ok"}
+
+
+# ---------------------------------------------------------------------------------------------------------------
+# K and V apart, with an issuing thread per part: it issues the product of key tile j and, behind it, in order, the scores of key tile j + NB
+# into the buffer the product frees.  The threads are not ordered among one another, so every barrier has one consumer:
+# scores and weights one per part and buffer, "K(n) has landed" one of eight, a multiple of the parts and no less than the stages.
+
+def simulate_parts_by_threads(SPLIT, NB, n_kv, stages, seed, warps=4, limit=400000, landed=8, per_part=True, products=5):
+    """per_part: barriers of scores and weights per part and buffer, not per buffer alone."""
+    rnd = random.Random(seed)
+    parts = SPLIT if per_part else 1
+    s_full = [[Bar(1) for _ in range(NB)] for _ in range(parts)]
+    p_full = [[Bar(warps) for _ in range(NB)] for _ in range(parts)]
+    meets = next(m for m in range(1, NB + 1) if m * SPLIT % NB == 0)
+    pv_done = [[Bar(1) for _ in range(products)] for _ in range(SPLIT)]
+    o_final, q_full = Bar(min(SPLIT, n_kv)), Bar(1)
+    kv_full, k_full = ([Bar(1) for _ in range(landed)] for _ in range(2))
+    kv_empty, k_empty = ([Bar(1) for _ in range(stages)] for _ in range(2))
+    pipes = [[] for _ in range(SPLIT)]           # per issuing thread, each retired in order
+    buf = {b: {} for b in range(NB)}
+    k_stage, v_stage, done, errors, in_flight = {}, {}, set(), [], []
+
+    def check(cond, what):
+        if not cond:
+            errors.append(what)
+
+    def phase_of(i, j):   # of a part's i-th key tile in its barrier
+        return (i // meets if per_part else j // NB) & 1
+
+    def loader(holds, full, empty, with_q):
+        if with_q:
+            in_flight.append(([], None, q_full))
+        for j in range(n_kv):
+            s = j % stages
+            if j >= stages:
+                while not empty[s].done(((j // stages) - 1) & 1):
+                    yield
+            in_flight.append(([(h, s) for h in holds], j, full[j % landed]))
+            yield
+
+    def issuer(g):
+        part_n = (g + NB) % SPLIT
+
+        def issue_s(n):
+            check(k_stage.get(n % stages) == n, ("S reads a stale stage", n))
+            check(n % SPLIT == part_n, ("another part's scores", n))
+            pipes[g].append(("S", n, n % NB, [s_full[part_n if per_part else 0][n % NB]] + [k_empty[n % stages]]))
+
+        while not q_full.done(0):
+            yield
+        for n in range(part_n, min(NB, n_kv), SPLIT):
+            while not k_full[n % landed].done(0):
+                yield
+            issue_s(n)
+        for i, j in enumerate(range(g, n_kv, SPLIT)):
+            b, n = j % NB, j + NB
+            while n < n_kv and not k_full[n % landed].done((n // landed) & 1):
+                yield
+            while not kv_full[j % landed].done((j // landed) & 1):
+                yield
+            while not p_full[g if per_part else 0][b].done(phase_of(i, j)):
+                yield
+            check(v_stage.get(j % stages) == j, ("P V reads a stale stage", j))
+            pipes[g].append(("PV", j, b, []))
+            if n < n_kv:
+                issue_s(n)
+            pipes[g].append(("C", j, b, [kv_empty[j % stages], pv_done[g][i % products]] + ([o_final] if j + SPLIT >= n_kv else [])))
+            yield
+
+    def part_warp(g, w):
+        for i, j in enumerate(range(g, n_kv, SPLIT)):
+            b = j % NB
+            while not s_full[g if per_part else 0][b].done(phase_of(i, j)):
+                yield
+            check(buf[b].get(w) == ("S", j), ("a part reads the wrong scores", g, w, j, b, buf[b].get(w)))
+            yield
+            buf[b][w] = ("P", j)
+            if i > 0 and rnd.random() < 0.3:   # re-anchored behind the product of the part's previous key tile
+                while not pv_done[g][(i - 1) % products].done(((i - 1) // products) & 1):
+                    yield
+                check(j - SPLIT in done, ("re-anchored before the part's last product", g, j))
+            p_full[g if per_part else 0][b].arrive()
+            yield
+        while not o_final.done(0):
+            yield
+        check(len(done) == n_kv, ("output before the last product", g))
+
+    procs = [issuer(g) for g in range(SPLIT)]
+    procs += [loader([k_stage], k_full, k_empty, True), loader([v_stage], kv_full, kv_empty, False)]
+    procs += [part_warp(g, w) for g in range(SPLIT) for w in range(warps)]
+    speed = [rnd.choice((0.02, 0.3, 1.0)) for _ in range(len(pipes))]   # a queue may lag far behind the others
+    eager = {id(p): rnd.choice((0.05, 0.5, 1.0)) for p in procs}
+    steps = 0
+    while procs and not errors:
+        steps += 1
+        if steps > limit:
+            return "deadlock"
+        if in_flight and rnd.random() < 0.3:     # copies land in any order
+            holds, j, bar = in_flight.pop(rnd.randrange(len(in_flight)))
+            for h, s in holds:
+                h[s] = j
+            bar.arrive()
+        for pipe, p in zip(pipes, speed):
+            if pipe and rnd.random() < p:
+                kind, j, b, bars = pipe.pop(0)
+                if kind == "S":
+                    for w in range(warps):
+                        buf[b][w] = ("S", j)
+                elif kind == "PV":
+                    check(all(buf[b].get(w) == ("P", j) for w in range(warps)), ("P V reads the wrong weights", j, b))
+                else:
+                    done.add(j)
+                for x in bars:
+                    x.arrive()
+        i = rnd.randrange(len(procs))
+        if rnd.random() < eager[id(procs[i])]:
+            try:
+                next(procs[i])
+            except StopIteration:
+                procs.pop(i)
+    return errors[0] if errors else "ok"
+
+
+@pytest.mark.parametrize("stages", [3, 5, 8])
+@pytest.mark.parametrize("n_kv", [1, 2, 3, 4, 5, 8, 17, 31])
+def test_parts_with_issuing_threads_of_their_own(stages, n_kv):
+    for seed in range(8):
+        assert simulate_parts_by_threads(2, 3, n_kv, stages, seed) == "ok"
+
+
+def test_issuing_threads_of_their_own_need_barriers_of_their_own():
+    """Barriers of scores and weights that parts share fail."""
+    outcomes = {simulate_parts_by_threads(2, 3, 31, 3, seed, per_part=False) for seed in range(80)}
+    assert outcomes != {"ok"}
