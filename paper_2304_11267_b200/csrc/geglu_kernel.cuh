@@ -15,7 +15,8 @@
 // A block asks for its pieces in the L2 before the stream's previous kernel has completed: the first blocks' fetch from memory then
 // runs under that kernel's end (8192 x 1280 fp16 11.6 -> 10.6 us a call in a loop, 12000 17.6 -> 16.5, 36864 51.5 -> 49.9).
 // 8192 x 1280 fp16 (63 MB): 10.6 us a call through the entry point = 5.9 TB/s (16.4 with the division, a grid-stride
-// loop and 28 instructions per element, launched without overlap); fp32: 19.5 us = 6.5 TB/s, the copy rate (22.3).
+// loop and 28 instructions per element, launched without overlap); fp32: 17.4 us = 7.2 TB/s, above the copy rate, as the output
+// stays in the L2 (22.3).
 #pragma once
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -116,7 +117,8 @@ constexpr int GEGLU_BLOCKS_PER_SM = 64;   // grid cap of the scalar kernel
 
 // VEC elements per 16-byte piece: 8 (fp16) or 4 (fp32); C is a multiple of VEC and both tensors are 16-byte aligned.
 // BIG: 2^31 pieces or more (64-bit indices).
-template <typename T, int VEC, int UNROLL, bool BIG>
+// ONCE: the input's lines go first when the L2 makes room (see launch_geglu).
+template <typename T, int VEC, int UNROLL, bool BIG, bool ONCE>
 __global__ void __launch_bounds__(GEGLU_THREADS)
 geglu_vector_kernel(const T* __restrict__ x, T* __restrict__ out, long long pieces, FastDiv row) {
     if (threadIdx.x == 0) pdl_launch_dependents();
@@ -136,8 +138,8 @@ geglu_vector_kernel(const T* __restrict__ x, T* __restrict__ out, long long piec
 #pragma unroll
     for (int u = 0; u < UNROLL; ++u)
         if (p0 + u * GEGLU_THREADS < pieces) {
-            a[u] = __ldg(src[u]);
-            g[u] = __ldg(src[u] + row.d);
+            a[u] = ONCE ? __ldcs(src[u]) : __ldg(src[u]);
+            g[u] = ONCE ? __ldcs(src[u] + row.d) : __ldg(src[u] + row.d);
         }
 #pragma unroll
     for (int u = 0; u < UNROLL; ++u) {

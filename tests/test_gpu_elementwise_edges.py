@@ -88,3 +88,12 @@ def test_inputs_written_by_the_kernel_before(bd, dtype):
         got.append(bd.geglu(bd.geglu(x, out=a)))
     got.append(bd.groupnorm(bd.groupnorm(gn_x, 32, out=b), 32))
     assert all(torch.equal(w, o) for w, o in zip(want, got))
+
+
+@pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
+@pytest.mark.parametrize("more", [-1, 0])
+def test_geglu_input_marked_to_go_first(bd, dtype, more):
+    """Either side of the size from which the input's lines are marked: 16 MB of output."""
+    rows = (16 << 20) // (1024 * np.dtype(dtype).itemsize) + more
+    x = geglu.make(rows, rows, 1024, dtype)
+    geglu.check(bd.geglu(torch.from_numpy(x).cuda()).cpu().numpy(), x, what=str(rows))
