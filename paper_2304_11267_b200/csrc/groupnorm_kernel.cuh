@@ -75,32 +75,46 @@ __device__ __forceinline__ void gn_affine_piece(const uint4& x, float scale, flo
 }
 
 // ------------------------------------------------------------------ statistics of a set of values
-// (count, mean, sum of squared deviations from that mean).  ONE reduction delivers mean and variance: a thread takes its own
-// values' mean and deviations from registers, then warps, the block and the cluster put theirs together.
+// (count, mean, sum of squared deviations from that mean).  Two sets merge without cancellation (Chan, Golub and
+// LeVeque's pairwise update), so ONE reduction delivers mean and variance: a thread takes its own values' mean and
+// deviations from registers, then warps, the block and the cluster merge triples.
 struct GnStat {
     float n, mean, m2;
 };
-// Of a warp's lanes, by sums about lane 0's mean: that is the mean of a subset, so the sum of squares about it exceeds the one about the
-// common mean by the ratio of the counts at most, 32, which is all the subtraction can lose.
-__device__ __forceinline__ GnStat gn_merge_lanes(const GnStat& s) {
-    const float at = __shfl_sync(0xffffffffu, s.mean, 0), d = s.n > 0.f ? s.mean - at : 0.f;
-    float n = s.n, sum = s.n * d, sq = fmaf(sum, d, s.m2);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        n += __shfl_xor_sync(0xffffffffu, n, o);
-        sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    }
-    const float shift = n > 0.f ? __fdividef(sum, n) : 0.f;
-    return {n, at + shift, fmaxf(fmaf(-sum, shift, sq), 0.f)};
-}
-__device__ __forceinline__ GnStat gn_merge(const GnStat& a, const GnStat& b) {   // Chan, Golub and LeVeque's pairwise update
+__device__ __forceinline__ GnStat gn_merge(const GnStat& a, const GnStat& b) {
     const float n = a.n + b.n, w = n > 0.f ? __fdividef(b.n, n) : 0.f, d = b.mean - a.mean;
     GnStat r;
     r.n = n;
     r.mean = fmaf(d, w, a.mean);
     r.m2 = a.m2 + b.m2 + d * d * (a.n * w);
     return r;
+}
+// Of LANES neighbouring lanes; every lane gets the result.  `alike` (the same in the whole warp): their counts are equal, as in every
+// warp that holds no remainder, and the update needs neither the division nor the count.  (Sums about one lane's mean take fewer
+// instructions, but lose up to LANES times the rounding where that lane lies far from the rest.)
+template <int LANES>
+__device__ __forceinline__ GnStat gn_merge_lanes(GnStat s, bool alike) {
+    if (alike) {
+        float half = 0.5f * s.n;
+#pragma unroll
+        for (int o = LANES / 2; o > 0; o >>= 1) {
+            const float mean = __shfl_xor_sync(0xffffffffu, s.mean, o), m2 = __shfl_xor_sync(0xffffffffu, s.m2, o), d = mean - s.mean;
+            s.mean = 0.5f * (s.mean + mean);
+            s.m2 = fmaf(d * d, half, s.m2 + m2);
+            half *= 2.f;
+        }
+        s.n *= (float)LANES;
+        return s;
+    }
+#pragma unroll
+    for (int o = LANES / 2; o > 0; o >>= 1) {
+        GnStat t;
+        t.n = __shfl_xor_sync(0xffffffffu, s.n, o);
+        t.mean = __shfl_xor_sync(0xffffffffu, s.mean, o);
+        t.m2 = __shfl_xor_sync(0xffffffffu, s.m2, o);
+        s = gn_merge(s, t);
+    }
+    return s;
 }
 
 // Registers form: a group is shared out among the CL blocks of a cluster, a thread holds PPT 16-byte pieces of it in
@@ -203,13 +217,15 @@ groupnorm_cluster_kernel(const GroupNormArgs a, const GroupNormPlan plan) {
         s.mean = pivot + shift;
         s.m2 = fmaxf(fmaf(-sum, shift, sq), 0.f);
     }
-    s = gn_merge_lanes(s);
+    // threads below `left` hold a piece more than the others, and the first threads of a ragged group's first block lone values
+    const int left = max(p_end - rank * pieces_per_block, 0) % THREADS, warp0 = warp * 32;
+    const bool lone_values = RAGGED && rank == 0;
+    s = gn_merge_lanes<32>(s, (left <= warp0 || left >= warp0 + 32) && !(lone_values && warp == 0));
     if (lane == 0) warp_stat[warp] = s;
     __syncthreads();
-    const bool prepares = warp * 32 < cpg;   // scale and shift of some channels
+    const bool prepares = warp0 < cpg;   // scale and shift of some channels
     if (prepares || cluster > 1) {
-        s = lane < WARPS ? warp_stat[lane] : GnStat{0.f, 0.f, 0.f};
-        s = gn_merge_lanes(s);
+        s = gn_merge_lanes<WARPS>(warp_stat[lane & (WARPS - 1)], left == 0 && !lone_values);
     }
     if (cluster > 1) {
         gn_cluster_wait();

@@ -92,6 +92,46 @@ def test_large_means_small_variances_and_optional_arguments(bd, dtype):
     check(run(bd, x, 32, 0.0, gamma, beta), x, 32, 0.0, gamma, beta, what="eps = 0")
 
 
+@pytest.mark.parametrize("threads,pieces,groups", [(256, 2, 64), (1024, 5, 96)], ids=["8 warps", "32 warps"])
+@pytest.mark.parametrize("far", ["a lane", "a warp"])
+def test_statistics_of_values_far_from_the_rest(bd, threads, pieces, groups, far):
+    """binary32 groups whose values of one lane (of one warp), or of one whole warp, lie far from the rest, so that how lanes and warps
+    are put together decides the variance.  With u = 2^-24 and k = 8 to 10 pairwise steps: a step's deviation term carries
+    2k + 4 roundings, their sum k more, so the variance is off by at most (3k + 4) u <= 34 u and 1 / sqrt(var + eps), with its own three
+    roundings, by 20 u; scale, shift and y = x * scale + shift add one each, and the mean's own error (k u of it) enters
+    through the shift: |err| <= 24 u (|y| + |mean| / sigma).  (Sums about one lane's mean reach 50 to 70 u.)"""
+    g = np.random.default_rng(7)
+    x = g.standard_normal((groups, pieces, threads // 32, 32, 4), dtype=np.float32)
+    for i in range(groups):
+        by = np.float32(g.uniform(5.0, 1000.0))
+        if far == "a lane":
+            x[i, :, g.integers(threads // 32), 0] += by
+        else:
+            x[i, :, 0] += by
+    x = x.reshape(1, groups, -1)
+    got = run(bd, x, groups, 1e-5, None, None).astype(np.float64)
+    want, mean, rstd = oracle.groupnorm_forward(x, groups, 1e-5, None, None)
+    tol = 24 * 2.0 ** -24 * (np.abs(want) + (np.abs(mean) * rstd).reshape(1, groups, 1))
+    assert np.all(np.abs(got - want) <= tol), "worst %.1f of the bound" % float((np.abs(got - want) / tol).max())
+
+
+@pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
+@pytest.mark.parametrize("shape,groups", [((2, 64, 16, 16), 4), ((2, 4, 8, 8), 4), ((1, 74, 20480), 74), ((2, 6, 77, 31), 2)])
+def test_an_infinity_reaches_its_whole_group(bd, dtype, shape, groups):
+    """The mean of a group with an infinity is infinite and no deviation from it is a number: the group is NaN, wherever the value
+    lies, and the other groups are what they would be without it."""
+    x, gamma, beta = make(80, shape, dtype)
+    per_group = x[0].size // groups
+    for sample, at in enumerate((0, 7, 8, per_group // 2 + 5, per_group - 1)):
+        xi = x.copy()
+        xi.reshape(shape[0], groups, -1)[0, 1, at] = np.inf if sample % 2 == 0 else -np.inf
+        got = run(bd, xi, groups, 1e-5, gamma, beta).reshape(shape[0], groups, -1)
+        assert np.isnan(got[0, 1]).all(), at
+        clean = run(bd, x, groups, 1e-5, gamma, beta).reshape(shape[0], groups, -1)
+        got[0, 1] = clean[0, 1]
+        assert np.array_equal(got, clean), at
+
+
 def test_in_place_side_stream_graph_and_guard_bytes(bd):
     x, gamma, beta = make(70, (2, 320, 32, 32), np.float16)
     want_x = x.copy()
