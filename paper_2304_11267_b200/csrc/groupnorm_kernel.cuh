@@ -176,13 +176,10 @@ groupnorm_cluster_kernel(const GroupNormArgs a, const GroupNormPlan plan) {
     const int lone = tid < head ? tid : head + n_pieces * VEC + (tid - head);
     const bool has_lone = RAGGED && rank == 0 && tid < 2 * VEC && lone < n_elems;
     float lone_x = has_lone ? gn_to_float(src[lone]) : 0.f;
-    // channel c0 + c's parameters: channel `tid`'s now, further ones (more channels than threads) when they are needed
-    auto parameters = [&](int c, float& ga, float& be) {
-        ga = a.gamma ? gn_to_float(static_cast<const T*>(a.gamma)[c0 + c]) : 1.f;
-        be = a.beta ? gn_to_float(static_cast<const T*>(a.beta)[c0 + c]) : 0.f;
-    };
-    float ga = 0.f, be = 0.f;
-    if (tid < cpg) parameters(tid, ga, be);
+#pragma unroll 1
+    for (int c = tid; c < cpg; c += THREADS)   // (read back by the thread itself: gamma and beta)
+        affine[c] = make_float2(a.gamma ? gn_to_float(static_cast<const T*>(a.gamma)[c0 + c]) : 1.f,
+                                a.beta ? gn_to_float(static_cast<const T*>(a.beta)[c0 + c]) : 0.f);
 
     // ---- statistics: the thread's own values, then warp, block, cluster.  One pass over the registers, about the
     // thread's first value: as that value is one of the set, the sum of squares about it exceeds the one about the mean by
@@ -246,10 +243,10 @@ groupnorm_cluster_kernel(const GroupNormArgs a, const GroupNormPlan plan) {
     // ---- y = x * scale + shift
     if (prepares) {
         const float rstd = 1.0f / sqrtf(s.m2 / (float)n_elems + a.eps);
+#pragma unroll 1
         for (int c = tid; c < cpg; c += THREADS) {
-            if (c != tid) parameters(c, ga, be);
-            const float scale = rstd * ga;
-            affine[c] = make_float2(scale, fmaf(-s.mean, scale, be));
+            const float scale = rstd * affine[c].x;
+            affine[c] = make_float2(scale, fmaf(-s.mean, scale, affine[c].y));
         }
     }
     __syncthreads();
