@@ -137,8 +137,9 @@ struct GroupNormPlan {
 __device__ __forceinline__ void gn_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void gn_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-template <typename T, int THREADS, int PPT, bool RAGGED>
-__global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 1)
+// RESIDENT: blocks whose registers an SM holds.
+template <typename T, int THREADS, int PPT, int RESIDENT, bool RAGGED>
+__global__ void __launch_bounds__(THREADS, RESIDENT)
 groupnorm_cluster_kernel(const GroupNormArgs a, const GroupNormPlan plan) {
     const int cluster = 1 << plan.log2_cluster, pieces_per_block = plan.pieces_per_block;
     constexpr int VEC = 16 / (int)sizeof(T), WARPS = THREADS / 32;

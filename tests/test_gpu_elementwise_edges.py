@@ -44,6 +44,16 @@ def test_groupnorm_blocks_of_a_group(bd, dtype, groups, pieces, odd):
     gn.check(gn.run(bd, x, groups, 1e-5, gamma, beta), x, groups, 1e-5, gamma, beta, what=str((groups, pieces, odd)))
 
 
+# (groups, pieces): threads and registers of a block where blocks outnumber the SMs: up to four an SM and more, every count of pieces a thread
+@pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
+@pytest.mark.parametrize("groups,pieces", [(592, 512), (593, 512), (592, 513), (593, 1024), (300, 1025), (300, 1536), (149, 1537), (300, 2048), (300, 2049)])
+@pytest.mark.parametrize("odd", [0, 3])
+def test_groupnorm_small_blocks_in_many_waves(bd, dtype, groups, pieces, odd):
+    vec = 16 // np.dtype(dtype).itemsize
+    x, gamma, beta = gn.make(groups + pieces, (1, groups, pieces * vec - odd), dtype, scale=1.1, shift=-0.2)
+    gn.check(gn.run(bd, x, groups, 1e-5, gamma, beta), x, groups, 1e-5, gamma, beta, what=str((groups, pieces, odd)))
+
+
 @pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
 @pytest.mark.parametrize("C,HW,G", [(12, 9, 3), (6, 5, 1), (40, 31, 8), (10, 5525, 1), (20, 4757, 2), (64, 37, 32), (1030, 9, 1),
                                     (2, 24577, 1), (2, 8, 2), (4, 4, 1)])
