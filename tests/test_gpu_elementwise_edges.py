@@ -54,9 +54,20 @@ def test_groupnorm_small_blocks_in_many_waves(bd, dtype, groups, pieces, odd):
     gn.check(gn.run(bd, x, groups, 1e-5, gamma, beta), x, groups, 1e-5, gamma, beta, what=str((groups, pieces, odd)))
 
 
+# ragged and whole groups on either side of the 16 MB from which blocks ask ahead
+@pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
+@pytest.mark.parametrize("groups", [511, 512])
+@pytest.mark.parametrize("odd", [0, 3])
+def test_groupnorm_asking_ahead(bd, dtype, groups, odd):
+    per_group = (32 << 10) // np.dtype(dtype).itemsize + (8 if odd else 0)
+    x, gamma, beta = gn.make(groups, (1, groups, per_group - odd), dtype, scale=1.2, shift=0.3)
+    gn.check(gn.run(bd, x, groups, 1e-5, gamma, beta), x, groups, 1e-5, gamma, beta, what=str((groups, odd)))
+
+
 @pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
 @pytest.mark.parametrize("C,HW,G", [(12, 9, 3), (6, 5, 1), (40, 31, 8), (10, 5525, 1), (20, 4757, 2), (64, 37, 32), (1030, 9, 1),
-                                    (2, 24577, 1), (2, 8, 2), (4, 4, 1)])
+                                    (2, 24577, 1), (2, 8, 2), (4, 4, 1),
+                                    (300, 16, 1), (300, 13, 1), (1024, 8, 1), (1024, 9, 1)])   # more channels in a group than threads
 def test_groupnorm_ragged_channels(bd, dtype, C, HW, G):
     x, gamma, beta = gn.make(C + HW, (3, C, HW), dtype, scale=0.8, shift=5.0)
     gn.check(gn.run(bd, x, G, 1e-5, gamma, beta), x, G, 1e-5, gamma, beta, what=str((C, HW, G)))
