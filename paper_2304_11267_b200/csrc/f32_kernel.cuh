@@ -70,14 +70,14 @@ struct F32Args {
 // NC: 32-column chunks of a row (d <= 32 NC).  BN: keys per key tile.  T: query tiles per CTA.  ACC: output columns per
 // softmax thread.  KS, VS: depth of the K and V rings.  NO: buffers for the product of a key tile.  MAX_FIRST: whether a key tile
 // fits the anchor is decided from its maximum before the exponentials, so that the weights replace the scores in registers,
-// not from the weights' sum behind them (measured: d = 80 43 -> 36 us; the other shapes lose 2% to 12% by it).
-template <int NC_, int BN_, int T_, int ACC_, int KS_, int VS_, int NO_, bool MAX_FIRST_, int MIN_PIECES_>
+// not from the weights' sum behind them (measured: d = 80 43 -> 36 us; the other shapes lose 2% to 12% by it).  BELOW: head dims up to
+// this one take a smaller shape.
+template <int NC_, int BN_, int T_, int ACC_, int KS_, int VS_, int NO_, bool MAX_FIRST_, int BELOW_>
 struct F32Shape {
     static constexpr int NC = NC_, BN = BN_, T = T_, ACC = ACC_, KS = KS_, VS = VS_, NO = NO_;
     static constexpr bool MAX_FIRST = MAX_FIRST_;
-    static constexpr int MIN_PIECES = MIN_PIECES_;   // of eight columns
     static constexpr int MAX_D = NC * F3_CHUNK < 2 * ACC ? NC * F3_CHUNK : 2 * ACC;
-    static constexpr int MAX_PIECES = MAX_D / 8;
+    static constexpr int MIN_PIECES = BELOW_ / 8 + 1, MAX_PIECES = MAX_D / 8;   // of eight columns
     static constexpr int N_CONV = T == 2 ? 1 : 2;   // warpgroups that convert K; as many for V
     static constexpr int WG_CONVERT = 2 * T, WG_ISSUE = WG_CONVERT + 2 * N_CONV, THREADS = (WG_ISSUE + 1) * 128;
     static constexpr int Q_PART = NC * TILE_M * 64, Q_TILE = 3 * Q_PART, KV_PART = NC * BN * 64, KV_STAGE = 3 * KV_PART;
@@ -99,10 +99,10 @@ struct F32Shape {
     static constexpr int POOL = 128 * (2 * T * SOFTMAX_REGS + 2 * N_CONV * CONVERT_REGS + ISSUE_REGS);
     static_assert(POOL <= THREADS * LAUNCH_REGS, "setmaxnreg budget");
 };
-using F32Two = F32Shape<2, 64, 2, 24, 2, 2, 1, false, 1>;     // d <= 48, two query tiles
-using F32One = F32Shape<2, 64, 1, 32, 3, 3, 2, false, 1>;     // d <= 64
-using F32Mid = F32Shape<3, 64, 1, 48, 2, 2, 1, true, 9>;     // d <= 96
-using F32Wide = F32Shape<5, 32, 1, 80, 2, 1, 1, true, 13>;    // d <= 160
+using F32Two = F32Shape<2, 64, 2, 24, 2, 2, 1, false, 0>;                // d <= 48, two query tiles
+using F32One = F32Shape<2, 64, 1, 32, 3, 3, 2, false, 0>;                // d <= 64
+using F32Mid = F32Shape<3, 64, 1, 48, 2, 2, 1, true, F32One::MAX_D>;     // d <= 96
+using F32Wide = F32Shape<5, 32, 1, 80, 2, 1, 1, true, F32Mid::MAX_D>;    // d <= 160
 constexpr float F32_TILE_SUM_LIMIT = 1.8446744e19f; // 2^64: no weight above it reaches the products
 constexpr float F32_MAX_LIMIT = 58.f;               // log2 of the largest weight where the maximum decides: 64 of them stay below the sum
 

@@ -55,6 +55,15 @@ def test_variants(bd, d, Nq, Nk):
     check(run(bd, q, k, v, scale), oracle.forward(q, k, v, scale)[0], v)
 
 
+# one head dim for every count of eight columns, and some that end in half of one: the contraction of Q K^T is compiled for each
+@pytest.mark.parametrize("d", list(range(8, 168, 8)) + [12, 36, 76, 84, 92, 108, 124, 140, 148, 156])
+def test_every_count_of_columns(bd, d):
+    scale = float(np.float32(d ** -0.5))
+    for H, Nq in ((3, 150),) + (((16, 1250),) if d <= 48 else ()):   # (one and two query tiles a CTA)
+        q, k, v = draw(d, 1, H, Nq, 150, d)
+        check(run(bd, q, k, v, scale), oracle.forward(q, k, v, scale)[0], v)
+
+
 @pytest.mark.parametrize("d,Nq", [(40, 1300), (36, 2500)])
 def test_two_query_tiles_per_cta(bd, d, Nq):
     q, k, v = draw(d, 2, 8, Nq, 200, d)   # more tiles than SMs; the last CTA of a head has one
