@@ -694,11 +694,13 @@ fused4s_attention_kernel(const __grid_constant__ Fused4Args args) {
                 const float c2 = pr.scale_log2e;
                 float m_run = 0.f, l_run = 0.f;   // anchor and row sum over this part's keys
                 bool ok = true;
-                // The part's i-th key tile j = g + SPLIT i uses buffer j % NB, phase (j / NB) & 1.  (Parts take turns at a buffer's
-                // barrier when NB is no multiple of SPLIT; the parity wait stays sound: the buffer's next scores need this
-                // tile's product, and its last ones, S(j - NB), completed before S(j - SPLIT), which this part has seen --
-                // NB >= SPLIT, and one thread's MMAs and commits complete in order.)
-                int b = g, ph = 0, met = 0;   // (K and V apart, NB odd: the part meets a buffer every NB of its key tiles)
+                // The part's i-th key tile j = g + SPLIT i uses buffer j % NB.  K and V in one ring: phase (j / NB) & 1 of a barrier that
+                // parts share, in turns when NB is no multiple of SPLIT; the parity wait stays sound: the buffer's next scores need
+                // this tile's product, and its last ones, S(j - NB), completed before S(j - SPLIT), which this part has seen -- NB >=
+                // SPLIT, and the one thread that issues all scores has them completed in order.  K and V apart: scores come from several
+                // threads, so a part has barriers of its own, whose phases it takes one by one: it meets a buffer every NB of its key tiles,
+                // as the host sees to it that NB and SPLIT have no common factor.
+                int b = g, ph = 0, met = 0;
                 touch_output(pr);
                 role_ready(args.Nk, __float_as_int(c2), NB);
                 for (int j = g, i = 0; j < n_kv; j += SPLIT, ++i) {

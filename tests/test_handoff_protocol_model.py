@@ -300,13 +300,15 @@ def test_scores_must_wait_for_the_completion_of_the_products_they_overwrite():
 # into the buffer the product frees.  The threads are not ordered among one another, so every barrier has one consumer:
 # scores and weights one per part and buffer, "K(n) has landed" one of eight, a multiple of the parts and no less than the stages.
 
-def simulate_parts_by_threads(SPLIT, NB, n_kv, stages, seed, warps=4, limit=400000, landed=8, per_part=True, products=5):
-    """per_part: barriers of scores and weights per part and buffer, not per buffer alone."""
+def simulate_parts_by_threads(SPLIT, NB, n_kv, stages, seed, warps=4, limit=400000, landed=8, per_part=True, products=5, landing=0.3,
+                              anchors=0.3):
+    """per_part: barriers of scores and weights per part and buffer, not per buffer alone.  landing, anchors: how soon a copy lands, how often
+    a row is re-anchored."""
     rnd = random.Random(seed)
     parts = SPLIT if per_part else 1
     s_full = [[Bar(1) for _ in range(NB)] for _ in range(parts)]
     p_full = [[Bar(warps) for _ in range(NB)] for _ in range(parts)]
-    meets = next(m for m in range(1, NB + 1) if m * SPLIT % NB == 0)
+    meets = NB   # (as the kernel counts: a part comes back to a buffer after so many of its key tiles, if SPLIT and NB have no common factor)
     pv_done = [[Bar(1) for _ in range(products)] for _ in range(SPLIT)]
     o_final, q_full = Bar(min(SPLIT, n_kv)), Bar(1)
     kv_full, k_full = ([Bar(1) for _ in range(landed)] for _ in range(2))
@@ -370,7 +372,7 @@ def simulate_parts_by_threads(SPLIT, NB, n_kv, stages, seed, warps=4, limit=4000
             check(buf[b].get(w) == ("S", j), ("a part reads the wrong scores", g, w, j, b, buf[b].get(w)))
             yield
             buf[b][w] = ("P", j)
-            if i > 0 and rnd.random() < 0.3:   # re-anchored behind the product of the part's previous key tile
+            if i > 0 and rnd.random() < anchors:   # re-anchored behind the product of the part's previous key tile
                 while not pv_done[g][(i - 1) % products].done(((i - 1) // products) & 1):
                     yield
                 check(j - SPLIT in done, ("re-anchored before the part's last product", g, j))
@@ -390,7 +392,7 @@ def simulate_parts_by_threads(SPLIT, NB, n_kv, stages, seed, warps=4, limit=4000
         steps += 1
         if steps > limit:
             return "deadlock"
-        if in_flight and rnd.random() < 0.3:     # copies land in any order
+        if in_flight and rnd.random() < landing:     # copies land in any order
             holds, j, bar = in_flight.pop(rnd.randrange(len(in_flight)))
             for h, s in holds:
                 h[s] = j
@@ -427,3 +429,24 @@ def test_issuing_threads_of_their_own_need_barriers_of_their_own():
     """Barriers of scores and weights that parts share fail."""
     outcomes = {simulate_parts_by_threads(2, 3, 31, 3, seed, per_part=False) for seed in range(80)}
     assert outcomes != {"ok"}
+
+
+@pytest.mark.parametrize("NB", [2, 4])
+def test_parts_and_score_buffers_with_a_common_factor_fail(NB):
+    """A part comes back to a buffer after NB of its key tiles only where SPLIT and NB have no common factor."""
+    outcomes = {simulate_parts_by_threads(2, NB, 17, 5, seed) for seed in range(8)}
+    assert "ok" not in outcomes
+
+
+def test_one_products_barrier_a_part_is_not_enough():
+    """A softmax warp that looks now and then can be two phases of one barrier behind."""
+    outcomes = {simulate_parts_by_threads(2, 3, 17, 3, seed, products=1) for seed in range(12)}
+    assert outcomes != {"ok"}
+
+
+def test_a_landed_barrier_has_one_issuer():
+    """Barriers by stage, three of them: successive key tiles of a barrier belong to different issuers, and one that runs ahead takes an earlier
+    copy's phase for its own while its copy is on its way."""
+    outcomes = {simulate_parts_by_threads(2, 3, 17, 3, seed, landed=3, landing=0.005) for seed in range(12)}
+    assert outcomes != {"ok"}
+    assert {simulate_parts_by_threads(2, 3, 17, 3, seed, landing=0.005) for seed in range(12)} == {"ok"}
