@@ -118,3 +118,16 @@ def test_geglu_input_marked_to_go_first(bd, dtype, more):
     rows = (16 << 20) // (1024 * np.dtype(dtype).itemsize) + more
     x = geglu.make(rows, rows, 1024, dtype)
     geglu.check(bd.geglu(torch.from_numpy(x).cuda()).cpu().numpy(), x, what=str(rows))
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.float32], ids=["f16", "f32"])
+@pytest.mark.parametrize("share", [8, 2])
+def test_geglu_either_side_of_the_lines_of_the_l2(bd, dtype, share):
+    """An output of an eighth (of half) of the L2, a row less and a row more: the same bits as by parts, which are far below the lines."""
+    C = 1024
+    line = torch.cuda.get_device_properties(0).L2_cache_size // share // (C * torch.finfo(dtype).bits // 8)
+    g = torch.Generator(device="cuda").manual_seed(share)
+    x = torch.randn(line + 1, 2 * C, generator=g, device="cuda").to(dtype)
+    parts = torch.cat([bd.geglu(p.contiguous()) for p in x.split(1024)])
+    for rows in (line - 1, line, line + 1):
+        assert torch.equal(bd.geglu(x[:rows]), parts[:rows]), rows
