@@ -22,9 +22,9 @@ def bd():
 # (channels per group, values per channel, groups), in values of the dtype; a 16-byte piece is 8 (fp16) or 4 (fp32) of them
 @pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
 @pytest.mark.parametrize("pieces_times", [
-    (1024, 0), (1024, 1),            # 256 threads / 512 threads
-    (6144, 0), (6144, 1),            # one block / a cluster of four
-    (12288, 1), (24576, 0), (24576, 1), (49152, 0), (49152, 1),   # clusters of eight, of larger blocks, streaming form
+    (1024, 0), (1024, 1),            # one block / the same with a remainder
+    (6144, 0), (6144, 1),            # clusters of four, without and with a remainder
+    (12288, 1), (24576, 0), (24576, 1), (49152, 0), (49152, 1),   # clusters of four, of eight, streaming form
 ])
 def test_groupnorm_group_sizes_at_the_edges_of_a_plan(bd, dtype, pieces_times):
     pieces, more = pieces_times
@@ -36,7 +36,9 @@ def test_groupnorm_group_sizes_at_the_edges_of_a_plan(bd, dtype, pieces_times):
 # (groups, 16-byte pieces of each): blocks per group and threads per block, on either side of every line of the plan on 148 SMs
 @pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
 @pytest.mark.parametrize("groups,pieces", [(33, 5119), (33, 5120), (34, 5120), (74, 2559), (74, 2560), (75, 2560), (74, 10240), (74, 10241),
-                                           (33, 20480), (33, 20481), (148, 2561), (148, 4097), (148, 6144), (148, 6145), (149, 4097), (149, 6145)])
+                                           (33, 20480), (33, 20481), (148, 2561), (148, 4097), (148, 6144), (148, 6145), (149, 4097), (149, 6145),
+                                           (33, 8192), (33, 8196), (74, 4096), (74, 4098), (149, 2048), (149, 2049), (149, 3072), (149, 3073), (149, 4096),
+                                           (149, 5120), (149, 5121), (222, 5121), (223, 5121), (75, 8193), (111, 8193), (112, 8193), (149, 6146), (222, 6147)])
 @pytest.mark.parametrize("odd", [0, 3])   # values more than whole pieces: ragged groups
 def test_groupnorm_blocks_of_a_group(bd, dtype, groups, pieces, odd):
     vec = 16 // np.dtype(dtype).itemsize
