@@ -188,7 +188,7 @@ cross1_attention_kernel(const __grid_constant__ Cross1ArgsT<NP> args) {
                     mbar_arrive_expect_tx(bar_qk + ch * 8, KV_BYTES / NCH);
                     tma_load_4d(k_smem + ch * KN * CHUNK_ROW_BYTES, &pr.tk, bar_qk + ch * 8, ch * CHUNK_COLS, 0, hz, bz);
                 }
-                // V behind K: its rows would keep the copy engine (about 3 clocks each) from those that the scores wait for
+                // V behind K: the copy engine takes rows one after the other, and the scores wait for K's
                 mbar_arrive_expect_tx(bar_v, KV_BYTES);
 #pragma unroll
                 for (int ch = 0; ch < NCH; ++ch)

@@ -36,7 +36,7 @@
 // Operands in shared memory are [part h, m, l][32-column chunk][row][64 bytes].  V is used as it lies (MN-major).  Where one
 // query tile leaves room in tensor memory, its Q goes there: read from shared memory, 128 rows for each product of 32 or 64 keys
 // were most of the product's time.
-// us a call, half-empty steps, steps counted at run time, parts taken out with masks -> now: 16 x 4096 x 4096, d = 40 285 -> 267, 3000
+// us a call, half-empty steps, steps counted at run time, parts taken out with masks -> now: 16 x 4096 x 4096, d = 40 291 -> 271, 3000
 // 196 -> 176; 16 x 1024, d = 64 29.8 -> 29.0, d = 80 35.9 -> 35.0; 16 x 600, d = 120 50.0 -> 40.8; 16 x 256, d = 160 27.6 -> 24.5.
 // Every wait is bounded and reports to the status block.
 #pragma once

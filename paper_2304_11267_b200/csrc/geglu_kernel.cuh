@@ -13,10 +13,10 @@
 // anything, and ends; finding a piece's row is one multiplication (a 64-bit division per piece was a third of the
 // instructions).  Two elements at a time on the packed binary32 pipe come to 20 instructions per element (ncu), about 16 of them arithmetic.
 // A block asks for its pieces in the L2 before the stream's previous kernel has completed: the first blocks' fetch from memory then
-// runs under that kernel's end (8192 x 1280 fp16 11.6 -> 10.6 us a call in a loop, 12000 17.6 -> 16.5, 36864 51.5 -> 49.9).
-// 8192 x 1280 fp16 (63 MB): 10.6 us a call through the entry point = 5.9 TB/s (16.4 with the division, a grid-stride
-// loop and 28 instructions per element, launched without overlap); fp32: 17.4 us = 7.2 TB/s, above the copy rate, as the output
-// stays in the L2 (22.3).
+// runs under that kernel's end (us in a graph over three sets of tensors: 8192 x 1280 fp16 12.8 -> 12.0, 12000 18.9 -> 17.9, 36864 54.7 ->
+// 50.3).
+// 8192 x 1280 fp16 (63 MB): 11.9 us a call through the entry point = 5.3 TB/s (16.4 with the division, a grid-stride
+// loop and 28 instructions per element, launched without overlap); fp32 (126 MB): 19.6 us = 6.4 TB/s (22.3).
 #pragma once
 #include <cuda_fp16.h>
 #include <stdint.h>
