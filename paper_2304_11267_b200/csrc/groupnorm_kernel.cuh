@@ -91,7 +91,7 @@ __device__ __forceinline__ GnStat gn_merge(const GnStat& a, const GnStat& b) {
 }
 // Of LANES neighbouring lanes; every lane gets the result.  `alike` (the same in the whole warp): their counts are equal, as in every
 // warp that holds no remainder, and the update needs neither the division nor the count.  (Sums about one lane's mean take fewer
-// instructions, but lose up to LANES times the rounding where that lane lies far from the rest.)
+// instructions, but lose up to LANES times the rounding of the variance where that lane lies far from the rest.)
 template <int LANES>
 __device__ __forceinline__ GnStat gn_merge_lanes(GnStat s, bool alike) {
     if (alike) {
@@ -116,6 +116,10 @@ __device__ __forceinline__ GnStat gn_merge_lanes(GnStat s, bool alike) {
     }
     return s;
 }
+// The means of a warp's lanes, then of a block's warps, are taken about the middle one of three of their values, so that a large common
+// mean is rounded once and not in every step of the reduction, also where one lane or warp lies far from the rest (2 x 1280 x 8 x 8 fp32, a mean of
+// three deviations: relative error 1.1e-7, with the means themselves 1.5e-7).
+__device__ __forceinline__ float gn_middle(float a, float b, float c) { return fmaxf(fminf(a, b), fminf(fmaxf(a, b), c)); }
 
 // Registers form: a group is shared out among the CL blocks of a cluster, a thread holds PPT 16-byte pieces of it in
 // registers from the one read to the one write, and the blocks exchange one triple each through distributed shared
@@ -218,12 +222,19 @@ groupnorm_cluster_kernel(const GroupNormArgs a, const GroupNormPlan plan) {
     // threads below `left` hold a piece more than the others, and the first threads of a ragged group's first block lone values
     const int left = max(p_end - rank * pieces_per_block, 0) % THREADS, warp0 = warp * 32;
     const bool lone_values = RAGGED && rank == 0;
+    const float at = gn_middle(__shfl_sync(0xffffffffu, s.mean, 0), __shfl_sync(0xffffffffu, s.mean, 16), __shfl_sync(0xffffffffu, s.mean, 31));
+    s.mean = s.n > 0.f ? s.mean - at : 0.f;
     s = gn_merge_lanes<32>(s, (left <= warp0 || left >= warp0 + 32) && !(lone_values && warp == 0));
+    s.mean += at;
     if (lane == 0) warp_stat[warp] = s;
     __syncthreads();
     const bool prepares = warp0 < cpg;   // scale and shift of some channels
-    if (prepares || cluster > 1) {
-        s = gn_merge_lanes<WARPS>(warp_stat[lane & (WARPS - 1)], left == 0 && !lone_values);
+    if (cluster > 1 ? warp == 0 : prepares) {
+        const float about = gn_middle(warp_stat[0].mean, warp_stat[WARPS / 2].mean, warp_stat[WARPS - 1].mean);
+        s = warp_stat[lane & (WARPS - 1)];
+        s.mean = s.n > 0.f ? s.mean - about : 0.f;
+        s = gn_merge_lanes<WARPS>(s, left == 0 && !lone_values);
+        s.mean += about;
     }
     if (cluster > 1) {
         gn_cluster_wait();

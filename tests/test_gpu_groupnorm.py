@@ -115,6 +115,18 @@ def test_statistics_of_values_far_from_the_rest(bd, threads, pieces, groups, far
     assert np.all(np.abs(got - want) <= tol), "worst %.1f of the bound" % float((np.abs(got - want) / tol).max())
 
 
+def test_a_large_mean_is_rounded_once(bd):
+    """2048 binary32 groups with a mean of 60 deviations.  The group's mean (in [16, 32), spacing 2^-19) and the shift it enters (in [32, 64),
+    2^-18) are rounded once each, a spacing / sqrt(12) on average; the means of threads and warps average out.  In units of the deviations:
+    sqrt((2^-19 / 0.5)^2 + (2^-18)^2) / sqrt(12) = 1.56e-6, here with 15% for the rest.  (Rounded in each step of the reduction: 2.0e-6.)"""
+    g = np.random.default_rng(9)
+    x = (g.standard_normal((64, 1280, 8, 8), dtype=np.float32) * np.float32(0.5) + np.float32(30.0)).astype(np.float32)
+    got = run(bd, x, 32, 0.0, None, None).astype(np.float64)
+    want = oracle.groupnorm_forward(x, 32, 0.0, None, None)[0]
+    error = np.linalg.norm(got - want) / np.linalg.norm(want)
+    assert error <= 1.15 * 1.56e-6, error
+
+
 @pytest.mark.parametrize("dtype", [np.float16, np.float32], ids=["f16", "f32"])
 @pytest.mark.parametrize("shape,groups", [((2, 64, 16, 16), 4), ((2, 4, 8, 8), 4), ((1, 74, 20480), 74), ((2, 6, 77, 31), 2)])
 def test_an_infinity_reaches_its_whole_group(bd, dtype, shape, groups):
